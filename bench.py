@@ -53,9 +53,6 @@ SERVED_OUT_RING = 4  # output buffers per pool pair (a pair can be in flight mor
 # none: the L2 flushed once before the frame, as in the timed steps); the
 # 8-path frame's from a capture with ncu's default per-launch cache flush.
 MEASURED_TRAFFIC = {
-    # the paired schedule's second stage is two kernels side by side: their sum
-    ("sgm_640x480_d128_p4", "pairs_vh"): (131189248, "f7a7031745fff723"),
-    ("sgm_640x480_d128_p4", "pairs_h_wta"): (59698176 + 73417984, "f7a7031745fff723"),
     ("sgm_1242x375_d128_p8", "sweep_h"): (585012992, "f7a7031745fff723"),
     ("sgm_1242x375_d128_p8", "sweep_diag+"): (311625472, "f7a7031745fff723"),
     ("sgm_1242x375_d128_p8", "sweep_diag-"): (311849088, "f7a7031745fff723"),
@@ -833,13 +830,11 @@ def main():
     elif w.n_paths == 4:
         # the first two schedules: the whole first pair beside the other pair's
         # first halves, then that pair's second halves with the winner-take-all;
-        # the paired-line schedule: the whole vertical pair beside n1 = min(W2, H2)
-        # steps of each horizontal direction, then the rest of the horizontal
-        # directions, and the sums and the minimum of every pixel
-        W2, H2 = W + (W & 1), H + (H & 1)
-        f1 = min(W2, H2) / W2
+        # the paired-line schedule: all four directions, then the sums and the
+        # minimum of every pixel (its second walk of the horizontal pair is not
+        # counted again)
         kernel_stages = {"sweep_v+h1": (3, 1), "sweep_h2": (1, 3), "sweep_h+v1": (3, 1), "sweep_v2": (1, 3),
-                         "pairs_vh": (2 + 2 * f1, 1), "pairs_h_wta": (2 * (1 - f1), 3)}
+                         "pairs_vh": (4, 0), "pairs_h_wta": (0, 4)}
     else:
         kernel_stages = {"sweep_h": (2 + (w.n_paths - 2) // 2, 1), "sweep_v": (1, 3), "sweep_diag+": (1, 2),
                          "sweep_diag-": (1, 2)}

@@ -181,8 +181,10 @@ SGM_API int sgm_compute_ex_async(sgm_ctx *ctx, const uint8_t *left, const uint8_
  * Non-blocking form for device pointers only: enqueues the whole path on the
  * context's stream and returns at once.  `left`, `right` and `disp_out` must
  * be device memory; the caller synchronises the stream before reading
- * `disp_out`.  The launch sequence for one (W, H, D, P1, P2, n_paths) and one
- * set of pointers is captured once into a CUDA graph and replayed.
+ * `disp_out`.  The kernels are launched one by one with programmatic stream
+ * serialization, so that calls follow one another in the stream without gaps;
+ * the blocking calls replay a CUDA graph captured once for one (W, H, D, P1,
+ * P2, n_paths) and one set of pointers.
  * Errors: SGM_EINVAL (including host pointers), SGM_ENOMEM, SGM_ECUDA.
  */
 SGM_API int sgm_compute_async(sgm_ctx *ctx, const uint8_t *left, const uint8_t *right, int W, int H, int D, int P1, int P2,
@@ -295,7 +297,8 @@ SGM_API int sgm_served_reset_stats(sgm_ctx *ctx);
  *   raw      uint8  [H][W]    winner-take-all disparity before the median
  *   disp     uint8  [H][W]    final disparity
  * A 4-path problem runs the schedule forced by sgm_set_schedule, else
- * SGM_SCHED_V_THEN_H (it is not autotuned).  Errors as sgm_compute.
+ * SGM_SCHED_V_THEN_H (it is not autotuned); 2 and 8 paths as sgm_compute.
+ * Errors as sgm_compute.
  */
 SGM_API int sgm_debug_stages(sgm_ctx *ctx, const uint8_t *left, const uint8_t *right, int W, int H, int D, int P1, int P2,
                      int n_paths, void *Fb, void *Fm, uint8_t *MC, uint16_t *S, uint8_t *raw, uint8_t *disp);
@@ -312,7 +315,9 @@ SGM_API int sgm_debug_stages(sgm_ctx *ctx, const uint8_t *left, const uint8_t *r
  * vertical pair beside the first halves of the horizontal pair), sweep_h2
  * (the horizontal second halves with the winner-take-all).  With 8 paths:
  * sweep_h (the horizontal pair with the first halves of the three
- * vertical-type pairs), sweep_diag+, sweep_diag-, sweep_v.
+ * vertical-type pairs), sweep_diag+, sweep_diag-, sweep_v.  A context created
+ * with SGM_FLAG_STAGE_TIMING runs these per-line sweeps for 2 and 8 paths and
+ * for the post form.
  */
 SGM_API int sgm_stage_times(sgm_ctx *ctx, float *ms_out, int n);
 
@@ -352,21 +357,23 @@ SGM_API const char *sgm_stage_label(const sgm_ctx *ctx, int i);
  *   SGM_SCHED_H_THEN_V  the whole horizontal pair beside the vertical first
  *                       halves, then the vertical second halves with the
  *                       winner-take-all;
- *   SGM_SCHED_PAIRS     two lines per warp over 2 x 2 pixel quads: the whole
- *                       vertical pair beside min(W, H) steps of each
- *                       horizontal direction, then the rest of the
- *                       horizontal directions with the winner-take-all
- *                       beside a parallel winner-take-all over the columns
- *                       both horizontal directions passed (the longest
- *                       chain is max(W, H) steps).  Not offered when its
- *                       quad records would pass 4 GiB.
+ *   SGM_SCHED_PAIRS     two lines per warp over 2 x 2 pixel quads: all four
+ *                       directions at once, the vertical pair storing its
+ *                       costs and the horizontal pair its state at every
+ *                       16th column (8th for D > 128); then every segment of
+ *                       a row pair walks the horizontal pair again from
+ *                       those states, sums and takes the winner.  Not
+ *                       offered when its quad cubes would pass 4 GiB.
  * All give bit-identical results.  By default the context autotunes: the
  * first call for a new (W, H, D, Census type, byte-sum) key runs the path
  * with each schedule (once to warm up, then five times timed with CUDA
  * events on the context's stream; that call blocks meanwhile) and keeps the
  * one with the lowest median for the key; a stream under capture is not
  * tuned (the first schedule is used).  sgm_set_schedule(ctx, s) forces
- * schedule s; -1 restores autotuning.
+ * schedule s; -1 restores autotuning.  Paths of 2 and 8 directions and the
+ * post form (sgm_compute_ex) run the paired lines too (with 8 paths the
+ * diagonals store their costs as the vertical pair does), or the per-line
+ * sweeps where the paired cubes do not fit the memory cap or the device.
  * Errors: SGM_EINVAL (null context, unknown schedule).
  */
 #define SGM_SCHED_V_THEN_H 0

@@ -45,7 +45,7 @@ unsigned take_bounds_fault() {
 // sgm_stages.cu: copy n bytes src0 -> dst0 and, when src1 is not null,
 // src1 -> dst1 (pinned host buffers to or from the work arena).
 cudaError_t launch_stage(const uint8_t* src0, uint8_t* dst0, const uint8_t* src1, uint8_t* dst1, size_t n,
-                         cudaStream_t stream);
+                         Stream stream);
 }  // namespace sgm
 
 namespace {
@@ -60,7 +60,12 @@ struct Layout {
     int RB;    // bytes per pixel record (sgm_internal.h): MC, S (room for u16 words), stored L_r fields;
                // the paired-line schedule: bytes of one quad in a cube (4D)
     int n_lx;  // stored-L_r fields per record
-    size_t fs = 0;  // the paired-line schedule: bytes of one cube array
+    // the paired-line schedule: passes side by side (2 with the left-right
+    // check, else 1), bytes of one cube array, the strides between feature
+    // images and between the passes' cubes, raw disparities, states and jump
+    // penalties, and the jump penalties' offset
+    int passes = 1;
+    size_t fs = 0, feat_stride = 0, rec_stride = 0, raw_stride = 0, state_stride = 0, p2map = 0, p2_stride = 0;
 };
 
 // Stored-L_r fields: one per pair of opposite paths whose first halves run
@@ -114,8 +119,8 @@ struct Problem {
     int W, H, D, P1, P2, n_paths;
     int ct62 = 0;  // features: 0 = CSCT (Eq. 1), 1 = the full 9x7 Census (SGM_FLAG_CENSUS_FULL)
     int post = 0;  // 0: the plain path (u8 output); else kPostOut16 | the SGM_POST_* flags of sgm_compute_ex
-    int sched = 0;  // 4-path sweep schedule (SGM_SCHED_*)
-    int n1 = -1;    // SGM_SCHED_PAIRS: horizontal steps in the first launch (-1: the default)
+    int sched = 0;  // sweep schedule (SGM_SCHED_*); 2 and 8 paths and the post form: V_THEN_H (the per-line
+                    // sweeps) or PAIRS
     int check_shrink = 0;  // bounds-checked build, test hook (PairsArgs::check_shrink)
 };
 
@@ -132,8 +137,8 @@ inline int p2_max(const Problem& p) { return (p.post & SGM_POST_ADAPTIVE_P2) ? s
 // S kept as bytes between the sweeps (sum_fits_u8 for this problem).
 inline bool s8_for(const Problem& p) { return sum_fits_u8(p.n_paths, p2_max(p), mc_max(p)); }
 
-// The paired-line schedule (SGM_SCHED_PAIRS) of a 4-path plain problem.
-inline bool pairs_sched(const Problem& p) { return p.n_paths == 4 && !p.post && p.sched == SGM_SCHED_PAIRS; }
+// The paired-line schedule (SGM_SCHED_PAIRS).
+inline bool pairs_sched(const Problem& p) { return p.sched == SGM_SCHED_PAIRS; }
 
 // Its 32-bit quad offsets (q * 4D) must stay below 4 GiB.
 inline bool pairs_fit(const Problem& p) {
@@ -142,33 +147,43 @@ inline bool pairs_fit(const Problem& p) {
 }
 
 // The quad cubes (one array of FS bytes per field), the quad raw disparity
-// and the horizontal chains' state (sgm_internal.h); `RB` holds the bytes of
-// one quad in a field (4D).
+// and the horizontal states (sgm_internal.h); `RB` holds the bytes of one quad
+// in a field (4D).
 Layout layout_pairs(const Problem& p) {
-    const PairsArgs g = pairs_geometry(p.W, p.H, p.D, p.n1);
+    const PairsArgs g = pairs_geometry(p.W, p.H, p.D, p.n_paths);
     const size_t wh = static_cast<size_t>(p.W) * p.H, quads = static_cast<size_t>(g.QW) * g.QH;
     const size_t fbytes = p.ct62 ? 8 : 4;
     Layout l{};
     l.RB = 4 * p.D;
     l.fs = align_up(quads * static_cast<size_t>(l.RB));
     l.n_lx = 0;
+    l.passes = (p.post & SGM_POST_LR_CHECK) ? 2 : 1;
+    l.feat_stride = align_up(fbytes * wh);
+    l.rec_stride = pairs_fields(p.n_paths) * l.fs;
+    l.raw_stride = align_up(4 * quads);
+    l.state_stride = align_up(4 * pairs_state_words(g));
+    l.p2_stride = (p.post & SGM_POST_ADAPTIVE_P2) ? align_up(4 * quads * (p.n_paths == 8 ? 8 : 4)) : 0;
     size_t o = 0;
     l.Fb = o;
-    o = align_up(o + fbytes * wh);
-    l.Fm = o;
-    o = align_up(o + fbytes * wh);
+    l.Fm = o + l.feat_stride;
+    o += 2 * l.passes * l.feat_stride;
     l.rec = o;
-    o = align_up(o + kPairsFields * l.fs);
+    o += l.passes * l.rec_stride;
     l.raw = o;
-    o = align_up(o + 4 * quads);
+    l.rawR = o + l.raw_stride;
+    o += l.passes * l.raw_stride;
     l.state = o;
-    o = align_up(o + 4 * static_cast<size_t>(g.QH) * 2 * 32 * (p.D / 32 + 1));
+    o += l.passes * l.state_stride;
+    l.p2map = o;
+    o += l.passes * l.p2_stride;
+    l.sub = o;
+    if (p.post & SGM_POST_SUBPIXEL) o = align_up(o + 16 * quads);
     l.in_left = o;
     o = align_up(o + wh);
     l.in_right = o;
     o = align_up(o + wh);
     l.out = o;
-    o = align_up(o + wh);
+    o = align_up(o + (p.post ? 2 : 1) * wh);
     l.total = o;
     return l;
 }
@@ -198,8 +213,6 @@ Layout layout_for(const Problem& p, bool batched = false) {
     l.total = align_up(l.out + wh);
     return l;
 }
-
-size_t arena_need(const Problem& p) { return layout_for(p).total; }
 
 bool valid_problem(const Problem& p, std::string* why) {
     char buf[160];
@@ -233,9 +246,9 @@ struct GraphKey {
     Problem p;
     const void *left, *right, *out, *arena;
     bool operator<(const GraphKey& o) const {
-        return std::tie(p.W, p.H, p.D, p.P1, p.P2, p.n_paths, p.ct62, p.post, p.sched, p.n1, left, right, out, arena) <
-               std::tie(o.p.W, o.p.H, o.p.D, o.p.P1, o.p.P2, o.p.n_paths, o.p.ct62, o.p.post, o.p.sched, o.p.n1, o.left,
-                        o.right, o.out, o.arena);
+        return std::tie(p.W, p.H, p.D, p.P1, p.P2, p.n_paths, p.ct62, p.post, p.sched, left, right, out, arena) <
+               std::tie(o.p.W, o.p.H, o.p.D, o.p.P1, o.p.P2, o.p.n_paths, o.p.ct62, o.p.post, o.p.sched, o.left, o.right,
+                        o.out, o.arena);
     }
 };
 
@@ -280,6 +293,9 @@ struct ListExec {
     std::map<std::pair<std::vector<int>, int>, cudaGraphExec_t> graphs;  // (group keys, sweep grid) -> graph
 };
 
+// Timed runs of the autotuners, and the 4-path schedules they choose among.
+constexpr int kTuneReps = 5, kSchedules = 3;
+
 // Served execution: up to kServeSlots batches in flight, each on its own
 // stream with its own arena from a device-resident pool.
 constexpr int kServeSlots = 2;
@@ -309,10 +325,6 @@ struct sgm_ctx {
     cudaStream_t own_stream = nullptr;
     cudaStream_t stream = nullptr;
     cudaStream_t capture_stream = nullptr;
-    // a second stream and two events that fork and join two kernels of one
-    // path (the paired schedule's second launch), in and outside graph capture
-    cudaStream_t aux_stream = nullptr;
-    cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
     size_t mem_cap = 0;
     uint8_t* arena = nullptr;
     size_t arena_bytes = 0;
@@ -328,7 +340,7 @@ struct sgm_ctx {
     // 4-path schedule: forced (>= 0) or autotuned per key (-1)
     int forced_sched = -1;
     std::map<std::tuple<int, int, int, int, int, bool>, int> tuned;  // (W, H, D, n_paths, ct62, s8) -> schedule
-    cudaEvent_t tune_ev[2] = {};
+    cudaEvent_t tune_ev[kTuneReps + 1] = {};
     // batched execution: the caller's stream's list state, the SM count, the
     // sweep grid tuned per wave (its pairs' (W, H, D, n_paths), sorted)
     ListExec batch_exec;
@@ -464,27 +476,73 @@ static bool is_device_ptr(const void* p) {
     return t == cudaMemoryTypeDevice || t == cudaMemoryTypeManaged;
 }
 
-// Kernels per path: census, cost, the first sweep stage (horizontal pair and
-// vertical-type first halves), the second halves of each vertical-type pair
-// (sweep_diag+, sweep_diag-, sweep_v), median; with 2 paths: census, cost,
-// sweep_h, sweep_v, median.  Each kernel is one timed stage.  With
-// post-filters: one matching pass (census, cost, sweeps) for the left image,
-// with the LR check a mirror kernel and a second pass, then the post kernel.
-// The paired schedule runs its second launch as two kernels side by side (one
-// timed stage).
-static int launches_per_match(const Problem& p) { return p.n_paths == 8 ? 6 : (pairs_sched(p) ? 5 : 4); }
+// Kernels per path.  Per-line schedules: census, cost, the first sweep stage
+// (horizontal pair and vertical-type first halves), the second halves of each
+// vertical-type pair (sweep_diag+, sweep_diag-, sweep_v), median; with 2 paths:
+// census, cost, sweep_h, sweep_v, median.  Each kernel is one timed stage.
+// With post-filters: one matching pass (census, cost, sweeps) for the left
+// image, with the LR check a mirror kernel and a second pass, then the post
+// kernel.  The paired schedule: census, cost, the walks (one kernel with 2
+// paths; horizontal, vertical and, with 8 paths, diagonal walks side by side:
+// one timed stage), the finishing launch, median or post; both passes of the
+// LR check in the same launches, the jump penalties of adaptive P2 one launch
+// per pass.
+static int walk_launches(const Problem& p) { return p.n_paths == 8 ? 3 : (p.n_paths == 4 ? 2 : 1); }
+static int launches_per_match(const Problem& p) { return p.n_paths == 8 ? 6 : 4; }
 static int launches_per_path(const Problem& p) {
+    const int passes = (p.post & SGM_POST_LR_CHECK) ? 2 : 1;
+    if (pairs_sched(p)) return 4 + walk_launches(p) + ((p.post & SGM_POST_ADAPTIVE_P2) ? passes : 0);
     if (!p.post) return launches_per_match(p) + 1;
-    return launches_per_match(p) * ((p.post & SGM_POST_LR_CHECK) ? 2 : 1) + ((p.post & SGM_POST_LR_CHECK) ? 1 : 0) + 1;
+    return launches_per_match(p) * passes + (passes - 1) + 1;
 }
-static int stages_per_path(const Problem& p) { return launches_per_path(p) - (pairs_sched(p) ? 1 : 0); }
+static int stages_per_path(const Problem& p) { return pairs_sched(p) ? 5 : launches_per_path(p); }
 
-// Two kernels of one path side by side: `aux` waits for `fork` recorded on
-// the path's stream, the path's stream waits for `join` recorded on `aux`.
-struct ForkJoin {
-    cudaStream_t aux;
-    cudaEvent_t fork, join;
-};
+// The paired schedule's matching pass, or both passes of the left-right check
+// in the same launches: raw disparities in quads at l.raw (and l.rawR).
+template <class Mark>
+static cudaError_t enqueue_pairs(const Problem& p, const Layout& l, uint8_t* arena, const uint8_t* left,
+                                 const uint8_t* right, uint16_t* Sdbg, Stream s, Mark&& mark) {
+    cudaError_t e;
+    if ((e = launch_census_passes(left, right, arena + l.Fb, l.feat_stride, 2 * l.passes, p.W, p.H, p.ct62 != 0, s)) !=
+        cudaSuccess)
+        return e;
+    if ((e = mark()) != cudaSuccess) return e;
+    if ((e = launch_cost_quads(arena + l.Fb, l.feat_stride, arena + l.rec, l.rec_stride, l.passes, l.RB, p.W, p.H, p.D,
+                               p.ct62 != 0, s)) != cudaSuccess)
+        return e;
+    PairsJobs f{};
+    f.n = l.passes;
+    for (int k = 0; k < l.passes; ++k) {
+        PairsArgs g = pairs_geometry(p.W, p.H, p.D, p.n_paths);
+        g.rec = arena + l.rec + k * l.rec_stride;
+        g.rawq = arena + l.raw + k * l.raw_stride;
+        g.Sdbg = Sdbg;
+        g.state = reinterpret_cast<uint32_t*>(arena + l.state + k * l.state_stride);
+        g.QB = l.RB;
+        g.FS = l.fs;
+        g.P1x2 = static_cast<uint32_t>(p.P1) * 0x10001u;
+        g.P2x2 = static_cast<uint32_t>(p.P2) * 0x10001u;
+        g.mc_max = mc_max(p);
+        g.gs = pairs_group(p2_max(p));
+        g.check_shrink = p.check_shrink;
+        if (p.post & SGM_POST_ADAPTIVE_P2) {
+            uint32_t* map = reinterpret_cast<uint32_t*>(arena + l.p2map + k * l.p2_stride);
+            if ((e = launch_p2map(k ? right : left, k != 0, map, p.n_paths, p.W, p.H, p.P1, p.P2, s)) != cudaSuccess)
+                return e;
+            g.p2map = map;
+        }
+        if (k == 0 && (p.post & SGM_POST_SUBPIXEL)) g.subq = reinterpret_cast<uint32_t*>(arena + l.sub);
+        f.job[k] = g;
+    }
+    if ((e = mark()) != cudaSuccess) return e;
+    // every direction at once
+    const Walks kinds[3] = {walk_launches(p) == 1 ? Walks::kHorVer : Walks::kHor, Walks::kVer, Walks::kDiag};
+    for (int k = 0; k < walk_launches(p); ++k)
+        if ((e = launch_pairs_walks(f, kinds[k], s)) != cudaSuccess) return e;
+    if ((e = mark()) != cudaSuccess) return e;
+    if ((e = launch_pairs_finish(f, s)) != cudaSuccess) return e;
+    return mark();
+}
 
 // One matching pass (Section 2, stages 2-3 and Eq. 4) of the pair
 // (base, match): census, cost and the sweeps; the winner-take-all disparity
@@ -492,44 +550,13 @@ struct ForkJoin {
 // base's intensities and, with sub, write the winner's neighbour sums.
 template <class Mark>
 static cudaError_t enqueue_match(const Problem& p, const Layout& l, uint8_t* arena, const uint8_t* base,
-                                 const uint8_t* match, uint8_t* raw, uint32_t* sub, uint16_t* Sdbg, cudaStream_t s,
-                                 const ForkJoin& fj, Mark&& mark) {
+                                 const uint8_t* match, uint8_t* raw, uint32_t* sub, uint16_t* Sdbg, Stream s,
+                                 Mark&& mark) {
     void* Fb = arena + l.Fb;
     void* Fm = arena + l.Fm;
     cudaError_t e;
     if ((e = launch_census(base, match, Fb, Fm, p.W, p.H, p.ct62 != 0, s)) != cudaSuccess) return e;
     if ((e = mark()) != cudaSuccess) return e;
-    if (pairs_sched(p)) {
-        // two lines per warp over quad cubes: the costs, then every walker
-        // storing its L_r beside the others, then the horizontal rest with
-        // Eq. 4 beside the parallel winner-take-all; raw in quads
-        if ((e = launch_cost_quads(Fb, Fm, arena + l.rec, l.RB, p.W, p.H, p.D, p.ct62 != 0, s)) != cudaSuccess)
-            return e;
-        if ((e = mark()) != cudaSuccess) return e;
-        PairsArgs g = pairs_geometry(p.W, p.H, p.D, p.n1);
-        g.rec = arena + l.rec;
-        g.rawq = raw;
-        g.Sdbg = Sdbg;
-        g.state = reinterpret_cast<uint32_t*>(arena + l.state);
-        g.QB = l.RB;
-        g.FS = l.fs;
-        g.P1x2 = static_cast<uint32_t>(p.P1) * 0x10001u;
-        g.P2x2 = static_cast<uint32_t>(p.P2) * 0x10001u;
-        g.s8 = s8_for(p) ? 1 : 0;
-        g.mc_max = mc_max(p);
-        g.check_shrink = p.check_shrink;
-        if ((e = launch_pairs_stage1(g, s)) != cudaSuccess) return e;
-        if ((e = mark()) != cudaSuccess) return e;
-        // the horizontal chains (the long pole: enqueued first) and the
-        // parallel winner-take-all side by side
-        if ((e = cudaEventRecord(fj.fork, s)) != cudaSuccess) return e;
-        if ((e = launch_pairs_chain2(g, s)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(fj.aux, fj.fork, 0)) != cudaSuccess) return e;
-        if ((e = launch_pairs_par(g, fj.aux)) != cudaSuccess) return e;
-        if ((e = cudaEventRecord(fj.join, fj.aux)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(s, fj.join, 0)) != cudaSuccess) return e;
-        return mark();
-    }
     if ((e = launch_cost(Fb, Fm, arena + l.rec, l.RB, p.W, p.H, p.D, p.ct62 != 0, s)) != cudaSuccess) return e;
     if ((e = mark()) != cudaSuccess) return e;
     SweepArgs a{};
@@ -634,13 +661,36 @@ static cudaError_t enqueue_match(const Problem& p, const Layout& l, uint8_t* are
     return cudaSuccess;
 }
 
+// The schedule of a problem that is not autotuned (2 or 8 paths, or the post
+// form) and room for the path in the context's arena.  The paired schedule
+// holds the stored costs of every direction at once and both passes of the
+// left-right check (2, 7 or 14 bytes per pixel and disparity against 3 to 7 of
+// the per-line sweeps): where the memory cap or the device has no room for
+// that, and in contexts that time stages (their stages are the per-line
+// sweeps'), the per-line sweeps run.
+static int prepare_arena(sgm_ctx* ctx, Problem& p, size_t extra = 0) {
+    p.sched = SGM_SCHED_V_THEN_H;
+    if ((p.n_paths != 4 || p.post) && !ctx->stage_timing && pairs_fit(p)) {
+        Problem q = p;
+        q.sched = SGM_SCHED_PAIRS;
+        const size_t need = layout_for(q).total + extra;
+        if (need <= ctx->arena_bytes || !ctx->mem_cap || need + ctx->serve_bytes.load() <= ctx->mem_cap) {
+            const int rc = ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, need, true);
+            const bool injected = ctx->fail_alloc_at > 0 && ctx->alloc_count.load() == ctx->fail_alloc_at;
+            if (rc == SGM_OK) p.sched = SGM_SCHED_PAIRS;
+            if (rc != SGM_ENOMEM || injected) return rc;
+        }
+    }
+    return ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, layout_for(p).total + extra, true);
+}
+
 // Enqueue the whole path (Section 2, stages 2-4) for one pair whose inputs
 // and output are device pointers: disp is uint8 [H][W], or uint16 [H][W] in
 // 1/16 pixel with post-filters (p.post).  Returns a cudaError_t.
 static cudaError_t enqueue_path(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const uint8_t* left,
                                 const uint8_t* right, uint8_t* disp, uint16_t* Sdbg, cudaStream_t s, bool timed) {
     const Layout l = layout_for(p);
-    const ForkJoin fj{ctx->aux_stream, ctx->fork_ev, ctx->join_ev};
+    const Stream st(s, !timed);  // events between the kernels: plain order
     cudaError_t e;
     int stage = 0;
     // with stage timing, event k is recorded before kernel k and after the last
@@ -650,29 +700,36 @@ static cudaError_t enqueue_path(sgm_ctx* ctx, const Problem& p, uint8_t* arena, 
         return cudaEventRecordWithFlags(ctx->stage_ev[stage++], s, cudaEventRecordExternal);
     };
     if ((e = mark()) != cudaSuccess) return e;
-    if (!p.post) {
-        if ((e = enqueue_match(p, l, arena, left, right, arena + l.raw, nullptr, Sdbg, s, fj, mark)) != cudaSuccess)
-            return e;
-        e = pairs_sched(p) ? launch_median_quads(arena + l.raw, disp, p.W, p.H, s)
-                           : launch_median(arena + l.raw, disp, p.W, p.H, s);
+    if (pairs_sched(p)) {
+        if ((e = enqueue_pairs(p, l, arena, left, right, Sdbg, st, mark)) != cudaSuccess) return e;
+        e = p.post ? launch_post(arena + l.raw,
+                                 (p.post & SGM_POST_SUBPIXEL) ? reinterpret_cast<uint32_t*>(arena + l.sub) : nullptr,
+                                 (p.post & SGM_POST_LR_CHECK) ? arena + l.rawR : nullptr,
+                                 reinterpret_cast<uint16_t*>(disp), true, p.W, p.H, p.D, st)
+                   : launch_median_quads(arena + l.raw, disp, p.W, p.H, st);
+        if (e != cudaSuccess) return e;
+        if ((e = mark()) != cudaSuccess) return e;
+    } else if (!p.post) {
+        if ((e = enqueue_match(p, l, arena, left, right, arena + l.raw, nullptr, Sdbg, st, mark)) != cudaSuccess) return e;
+        e = launch_median(arena + l.raw, disp, p.W, p.H, st);
         if (e != cudaSuccess) return e;
         if ((e = mark()) != cudaSuccess) return e;
     } else {
         uint32_t* sub = (p.post & SGM_POST_SUBPIXEL) ? reinterpret_cast<uint32_t*>(arena + l.sub) : nullptr;
-        if ((e = enqueue_match(p, l, arena, left, right, arena + l.raw, sub, nullptr, s, fj, mark)) != cudaSuccess)
+        if ((e = enqueue_match(p, l, arena, left, right, arena + l.raw, sub, nullptr, st, mark)) != cudaSuccess)
             return e;
         const uint8_t* rawR = nullptr;
         if (p.post & SGM_POST_LR_CHECK) {
             // the right image's disparity: the same pass on the mirrored pair
-            if ((e = launch_mirror(left, right, arena + l.ml, arena + l.mr, p.W, p.H, s)) != cudaSuccess) return e;
+            if ((e = launch_mirror(left, right, arena + l.ml, arena + l.mr, p.W, p.H, st)) != cudaSuccess) return e;
             if ((e = mark()) != cudaSuccess) return e;
-            if ((e = enqueue_match(p, l, arena, arena + l.mr, arena + l.ml, arena + l.rawR, nullptr, nullptr, s, fj,
+            if ((e = enqueue_match(p, l, arena, arena + l.mr, arena + l.ml, arena + l.rawR, nullptr, nullptr, st,
                                    mark)) != cudaSuccess)
                 return e;
             rawR = arena + l.rawR;
         }
-        if ((e = launch_post(arena + l.raw, sub, rawR, reinterpret_cast<uint16_t*>(disp), p.W, p.H, p.D, s)) !=
-            cudaSuccess)
+        if ((e = launch_post(arena + l.raw, sub, rawR, reinterpret_cast<uint16_t*>(disp), false, p.W, p.H,
+                             p.D, st)) != cudaSuccess)
             return e;
         if ((e = mark()) != cudaSuccess) return e;
     }
@@ -692,7 +749,11 @@ struct HostIO {
     int launches() const { return (src[0] ? 1 : 0) + (out_src ? 1 : 0); }
 };
 
-// Enqueue through a cached CUDA graph for this problem and these pointers.
+// Enqueue through a cached CUDA graph for this problem and these pointers: the
+// blocking calls, which find the GPU idle (the whole sequence is there at once:
+// 100.2 us per 640x480 frame from pinned host images against 103.6 kernel by
+// kernel), and contexts that time stages (the events between the kernels are
+// nodes of the graph).
 // The key names the caller's buffers (a staged host buffer's arena copy is the
 // same for every host buffer).  An address that is staged in one call and
 // used in place in another (freed and reused as another kind of memory)
@@ -712,13 +773,13 @@ static int enqueue_graph(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const u
         CUDA_TRY(ctx, cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal));
         const uint64_t before = ctx->launches.load();
         cudaError_t e = cudaSuccess;
-        if (io.src[0]) e = launch_stage(io.src[0], io.dst[0], io.src[1], io.dst[1], io.img_bytes, ctx->capture_stream);
-        // paths with post-filters are never stage-timed (sgm_stage_times names the plain path's kernels)
+        const Stream st(ctx->capture_stream, !(ctx->stage_timing && !p.post));
+        if (io.src[0]) e = launch_stage(io.src[0], io.dst[0], io.src[1], io.dst[1], io.img_bytes, st);
         if (e == cudaSuccess)
             e = enqueue_path(ctx, p, arena, left, right, disp, nullptr, ctx->capture_stream,
                              ctx->stage_timing && !p.post);
         if (e == cudaSuccess && io.out_src)
-            e = launch_stage(io.out_src, io.out_dst, nullptr, nullptr, io.out_bytes, ctx->capture_stream);
+            e = launch_stage(io.out_src, io.out_dst, nullptr, nullptr, io.out_bytes, st);
         ctx->launches = before;  // captured, not launched
         cudaError_t e2 = cudaStreamEndCapture(ctx->capture_stream, &g);
         if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -740,17 +801,30 @@ static int enqueue_graph(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const u
     return SGM_OK;
 }
 
+// Enqueue the path kernel by kernel with programmatic stream serialization
+// (sgm_internal.h): the asynchronous calls, one behind the other in the
+// stream.  Nothing is kept by the buffers' addresses: a call on new buffers
+// costs what any other does.
+static int enqueue_run(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const uint8_t* left, const uint8_t* right,
+                       uint8_t* disp, cudaStream_t s) {
+    // paths with post-filters are never stage-timed (sgm_stage_times names the plain path's kernels)
+    if (ctx->stage_timing && !p.post) return enqueue_graph(ctx, p, arena, left, right, disp, s);
+    CUDA_TRY(ctx, enqueue_path(ctx, p, arena, left, right, disp, nullptr, s, false));
+    ctx->last_stages = ctx->last_n_paths = 0;
+    ctx->last_sched = p.sched;
+    return SGM_OK;
+}
+
 // The 4-path sweep schedule of a plain-path problem: forced, or the fastest of
 // the kSchedules measured on the first use of its (W, H, D, Census, byte sums)
 // key.  Tuning runs the whole path (into the caller's output, which every
 // schedule computes bit-identically) once per schedule to warm up and
 // kTuneReps times timed with events on `s`; the median decides.  A stream
 // under capture cannot be timed: there the default schedule is used untuned.
-constexpr int kSchedules = 3, kTuneReps = 5;
 static int choose_schedule(sgm_ctx* ctx, Problem& p, uint8_t* arena, const uint8_t* left, const uint8_t* right,
                            uint8_t* disp, cudaStream_t s) {
+    if (p.n_paths != 4 || p.post) return SGM_OK;  // see prepare_arena
     p.sched = SGM_SCHED_V_THEN_H;
-    if (p.n_paths != 4 || p.post) return SGM_OK;
     if (ctx->forced_sched >= 0) {
         p.sched = ctx->forced_sched;
         if (pairs_sched(p) && !pairs_fit(p)) p.sched = SGM_SCHED_V_THEN_H;  // quad records would pass 4 GiB
@@ -771,16 +845,18 @@ static int choose_schedule(sgm_ctx* ctx, Problem& p, uint8_t* arena, const uint8
         Problem q = p;
         q.sched = sched;
         if (sched == SGM_SCHED_PAIRS && !pairs_fit(q)) continue;
-        int rc = enqueue_graph(ctx, q, arena, left, right, disp, s);  // captures the graph; warm-up
+        int rc = enqueue_run(ctx, q, arena, left, right, disp, s);  // warm-up
         if (rc != SGM_OK) return rc;
-        float ms[kTuneReps];
+        // one run after the other, as a stream of frames has them
+        CUDA_TRY(ctx, cudaEventRecord(ctx->tune_ev[0], s));
         for (int rep = 0; rep < kTuneReps; ++rep) {
-            CUDA_TRY(ctx, cudaEventRecord(ctx->tune_ev[0], s));
-            if ((rc = enqueue_graph(ctx, q, arena, left, right, disp, s)) != SGM_OK) return rc;
-            CUDA_TRY(ctx, cudaEventRecord(ctx->tune_ev[1], s));
-            CUDA_TRY(ctx, cudaEventSynchronize(ctx->tune_ev[1]));
-            CUDA_TRY(ctx, cudaEventElapsedTime(&ms[rep], ctx->tune_ev[0], ctx->tune_ev[1]));
+            if ((rc = enqueue_run(ctx, q, arena, left, right, disp, s)) != SGM_OK) return rc;
+            CUDA_TRY(ctx, cudaEventRecord(ctx->tune_ev[rep + 1], s));
         }
+        CUDA_TRY(ctx, cudaEventSynchronize(ctx->tune_ev[kTuneReps]));
+        float ms[kTuneReps];
+        for (int rep = 0; rep < kTuneReps; ++rep)
+            CUDA_TRY(ctx, cudaEventElapsedTime(&ms[rep], ctx->tune_ev[rep], ctx->tune_ev[rep + 1]));
         std::sort(ms, ms + kTuneReps);
         const float med = ms[kTuneReps / 2];
         if (best < 0 || med < best_ms) {
@@ -800,7 +876,7 @@ static int choose_schedule(sgm_ctx* ctx, Problem& p, uint8_t* arena, const uint8
 // host link with no separate copy); pageable host memory is staged through
 // the arena with copies.
 static int enqueue_pair(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const uint8_t* left, const uint8_t* right,
-                        uint8_t* disp, cudaStream_t s, bool use_graph) {
+                        uint8_t* disp, cudaStream_t s) {
     const Layout l = layout_for(p);
     const size_t wh = static_cast<size_t>(p.W) * p.H;
     // device buffers are used in place; pinned host buffers are copied by
@@ -843,21 +919,14 @@ static int enqueue_pair(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const ui
             io.out_bytes = ob;
         }
     }
-    if (use_graph) {
-        // the tuner's runs read the arena copies before this call's staging
-        // has filled them: their timing does not depend on the values, and
-        // the graph launched below recomputes the result from the staged ones
-        Problem q = p;
-        int rc = choose_schedule(ctx, q, arena, dl, dr, dout, s);
-        if (rc != SGM_OK) return rc;
-        rc = enqueue_graph(ctx, q, arena, dl, dr, dout, s, io, left, right, disp);
-        if (rc != SGM_OK) return rc;
-    } else {
-        if (io.src[0]) CUDA_TRY(ctx, launch_stage(io.src[0], io.dst[0], io.src[1], io.dst[1], wh, s));
-        CUDA_TRY(ctx, enqueue_path(ctx, p, arena, dl, dr, dout, nullptr, s, false));
-        if (io.out_src) CUDA_TRY(ctx, launch_stage(io.out_src, io.out_dst, nullptr, nullptr, ob, s));
-        ctx->launches += io.launches();
-    }
+    // the tuner's runs read the arena copies before this call's staging has
+    // filled them: their timing does not depend on the values, and the run
+    // below recomputes the result from the staged ones
+    Problem q = p;
+    int rc = choose_schedule(ctx, q, arena, dl, dr, dout, s);
+    if (rc != SGM_OK) return rc;
+    rc = enqueue_graph(ctx, q, arena, dl, dr, dout, s, io, left, right, disp);
+    if (rc != SGM_OK) return rc;
     if (!device_side(ko) && ko != cudaMemoryTypeHost)
         CUDA_TRY(ctx, cudaMemcpyAsync(disp, dout, ob, cudaMemcpyDeviceToHost, s));
     return SGM_OK;
@@ -1603,10 +1672,7 @@ int sgm_create(sgm_ctx** out, int device, size_t mem_cap_bytes, unsigned flags) 
     ctx->device = device;
     ctx->mem_cap = mem_cap_bytes;
     if ((e = cudaStreamCreateWithFlags(&ctx->own_stream, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaStreamCreateWithFlags(&ctx->aux_stream, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&ctx->join_ev, cudaEventDisableTiming)) != cudaSuccess) {
+        (e = cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking)) != cudaSuccess) {
         sgm_destroy(ctx);
         return fail(nullptr, SGM_ECUDA, "cudaStreamCreate: %s", cudaGetErrorString(e));
     }
@@ -1699,12 +1765,6 @@ int sgm_destroy(sgm_ctx* ctx) {
     if (ctx->serve_pool) cudaMemPoolDestroy(ctx->serve_pool);
     if (ctx->own_stream) cudaStreamDestroy(ctx->own_stream);
     if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
-    if (ctx->aux_stream) {
-        cudaStreamSynchronize(ctx->aux_stream);
-        cudaStreamDestroy(ctx->aux_stream);
-    }
-    if (ctx->fork_ev) cudaEventDestroy(ctx->fork_ev);
-    if (ctx->join_ev) cudaEventDestroy(ctx->join_ev);
     for (auto& ev : ctx->stage_ev)
         if (ev) cudaEventDestroy(ev);
     for (auto& ev : ctx->tune_ev)
@@ -1723,13 +1783,13 @@ int sgm_set_stream(sgm_ctx* ctx, void* cuda_stream) {
 
 int sgm_compute(sgm_ctx* ctx, const uint8_t* left, const uint8_t* right, int W, int H, int D, int P1, int P2,
                 int n_paths, uint8_t* disp_out) {
-    const Problem p = make_problem(ctx, W, H, D, P1, P2, n_paths);
+    Problem p = make_problem(ctx, W, H, D, P1, P2, n_paths);
     int rc = check_args(ctx, p, left, right, disp_out);
     if (rc != SGM_OK) return rc;
     CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-    rc = ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, arena_need(p), true);
+    rc = prepare_arena(ctx, p);
     if (rc != SGM_OK) return rc;
-    rc = enqueue_pair(ctx, p, ctx->arena, left, right, disp_out, ctx->stream, true);
+    rc = enqueue_pair(ctx, p, ctx->arena, left, right, disp_out, ctx->stream);
     if (rc != SGM_OK) return rc;
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
     return bounds_status(ctx);
@@ -1742,9 +1802,9 @@ int sgm_compute_ex(sgm_ctx* ctx, const uint8_t* left, const uint8_t* right, int 
     int rc = check_args(ctx, p, left, right, disp16_out);
     if (rc != SGM_OK) return rc;
     CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-    rc = ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, layout_for(p).total, true);
+    rc = prepare_arena(ctx, p);
     if (rc != SGM_OK) return rc;
-    rc = enqueue_pair(ctx, p, ctx->arena, left, right, reinterpret_cast<uint8_t*>(disp16_out), ctx->stream, true);
+    rc = enqueue_pair(ctx, p, ctx->arena, left, right, reinterpret_cast<uint8_t*>(disp16_out), ctx->stream);
     if (rc != SGM_OK) return rc;
     CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
     return bounds_status(ctx);
@@ -1758,12 +1818,12 @@ int sgm_compute_async(sgm_ctx* ctx, const uint8_t* left, const uint8_t* right, i
     if (!is_device_ptr(left) || !is_device_ptr(right) || !is_device_ptr(disp_out))
         return fail(ctx, SGM_EINVAL, "sgm_compute_async takes device pointers only");
     CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-    rc = ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, arena_need(p), true);
-    if (rc != SGM_OK) return rc;
     Problem q = p;
+    rc = prepare_arena(ctx, q);
+    if (rc != SGM_OK) return rc;
     rc = choose_schedule(ctx, q, ctx->arena, left, right, disp_out, ctx->stream);
     if (rc != SGM_OK) return rc;
-    return enqueue_graph(ctx, q, ctx->arena, left, right, disp_out, ctx->stream);
+    return enqueue_run(ctx, q, ctx->arena, left, right, disp_out, ctx->stream);
 }
 
 int sgm_compute_ex_async(sgm_ctx* ctx, const uint8_t* left, const uint8_t* right, int W, int H, int D, int P1,
@@ -1775,9 +1835,9 @@ int sgm_compute_ex_async(sgm_ctx* ctx, const uint8_t* left, const uint8_t* right
     if (!is_device_ptr(left) || !is_device_ptr(right) || !is_device_ptr(disp16_out))
         return fail(ctx, SGM_EINVAL, "sgm_compute_ex_async takes device pointers only");
     CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-    rc = ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, layout_for(p).total, true);
+    rc = prepare_arena(ctx, p);
     if (rc != SGM_OK) return rc;
-    return enqueue_graph(ctx, p, ctx->arena, left, right, reinterpret_cast<uint8_t*>(disp16_out), ctx->stream);
+    return enqueue_run(ctx, p, ctx->arena, left, right, reinterpret_cast<uint8_t*>(disp16_out), ctx->stream);
 }
 
 int sgm_compute_batch(sgm_ctx* ctx, int n, const sgm_pair* pairs) {
@@ -1992,16 +2052,16 @@ int sgm_served_reset_stats(sgm_ctx* ctx) {
 int sgm_debug_stages(sgm_ctx* ctx, const uint8_t* left, const uint8_t* right, int W, int H, int D, int P1, int P2,
                      int n_paths, void* Fb, void* Fm, uint8_t* MC, uint16_t* S, uint8_t* raw, uint8_t* disp) {
     Problem p = make_problem(ctx, W, H, D, P1, P2, n_paths);
-    if (ctx && n_paths == 4 && ctx->forced_sched >= 0) p.sched = ctx->forced_sched;  // else the first schedule
     int rc = check_args(ctx, p, left, right, left);
     if (rc != SGM_OK) return rc;
     CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-    if (pairs_sched(p) && !pairs_fit(p)) return fail(ctx, SGM_EINVAL, "problem too large for the paired schedule");
-    const Layout l = layout_for(p);
     const size_t wh = static_cast<size_t>(W) * H;
     const size_t extra = align_up(wh * D * 2) + align_up(wh * D) + align_up(wh);
-    rc = ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, l.total + extra, true);
+    rc = prepare_arena(ctx, p, extra);
     if (rc != SGM_OK) return rc;
+    if (n_paths == 4 && ctx->forced_sched >= 0) p.sched = ctx->forced_sched;  // else the first schedule
+    if (pairs_sched(p) && !pairs_fit(p)) return fail(ctx, SGM_EINVAL, "problem too large for the paired schedule");
+    const Layout l = layout_for(p);
     uint8_t* a = ctx->arena;
     uint16_t* Sdev = reinterpret_cast<uint16_t*>(a + l.total);
     uint8_t* MCnat = a + l.total + align_up(wh * D * 2);
@@ -2163,9 +2223,18 @@ Layout static_layout(const Problem& p) {
     return l;
 }
 
-// The path of Section 2, stages 2-4, with every phase on one stream.
-cudaError_t enqueue_path_static(const Problem& p, uint8_t* arena, const uint8_t* left, const uint8_t* right,
-                                uint8_t* disp, cudaStream_t s) {
+// The path of Section 2, stages 2-4: the paired schedule where its cubes fit the
+// scratch, else the per-line sweeps with both phases of a pair in one launch.
+cudaError_t enqueue_path_static(Problem p, uint8_t* arena, const uint8_t* left, const uint8_t* right, uint8_t* disp,
+                                cudaStream_t stream) {
+    const Stream s(stream, true);
+    p.sched = SGM_SCHED_PAIRS;
+    const Layout lp = layout_pairs(p);
+    if (lp.in_left <= kStaticScratchBytes) {  // all it touches lies in front of its staging buffers
+        cudaError_t e = enqueue_pairs(p, lp, arena, left, right, nullptr, s, [] { return cudaSuccess; });
+        return e != cudaSuccess ? e : launch_median_quads(arena + lp.raw, disp, p.W, p.H, s);
+    }
+    p.sched = SGM_SCHED_V_THEN_H;
     const Layout l = static_layout(p);
     void* Fb = arena + l.Fb;
     void* Fm = arena + l.Fm;

@@ -26,6 +26,13 @@ namespace sgm {
 // so packed 32-bit adds never carry across lanes.
 constexpr uint32_t kInf16 = 0x3FFFu;
 
+// First instruction of every kernel of a path (Stream, sgm_internal.h): the
+// kernels before it have ended and their writes are visible.  Nothing to wait
+// for in a plain launch.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The next kernel of the stream may start once every block of this one has come here.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t vmin2(uint32_t a, uint32_t b) {
     uint32_t d;
     asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));

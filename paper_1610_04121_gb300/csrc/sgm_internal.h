@@ -6,6 +6,34 @@
 
 namespace sgm {
 
+// A path's kernels follow one another in a stream, each launched with
+// programmatic stream serialization (pdl): its launch work overlaps the kernel
+// before it, and its first instruction waits until that one has ended and its
+// writes are visible (pdl_wait, sgm_device.cuh).  In plain order, and at every
+// graph launch, the device releases a kernel in steps of 2.05 us, 4.1 us at
+// least; measured for five kernels of 1.5 us back to back: 20.5 us launched
+// plainly, 14.3 us as a replayed graph, 11.3 us this way.
+struct Stream {
+    cudaStream_t s;
+    bool pdl;
+    Stream(cudaStream_t stream, bool p = false) : s(stream), pdl(p) {}
+};
+
+// Launches a kernel; the caller reads the error with cudaGetLastError.
+template <class... P, class... A>
+inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, Stream st, A&&... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.stream = st.s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = attr;
+    c.numAttrs = st.pdl ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // The sweeps keep every per-(pixel, disparity) cube of a pair in one array of
 // per-pixel records [H][W][RB] bytes: the paired costs MC (D bytes, offset 0),
 // the sums S (offset D: D paired bytes when s8, else D/2 packed u16x2 words),
@@ -99,11 +127,11 @@ struct ListLaunch {
 // ct62 = false: the CSCT of Eq. 1, uint32 features; true: the full 9x7
 // Census, uint64 features.
 cudaError_t launch_census(const uint8_t* left, const uint8_t* right, void* Fb, void* Fm, int W, int H, bool ct62,
-                          cudaStream_t stream);
+                          Stream stream);
 // MC goes to offset 0 of the RB-byte record of each pixel.
 cudaError_t launch_cost(const void* Fb, const void* Fm, uint8_t* rec, int RB, int W, int H, int D, bool ct62,
-                        cudaStream_t stream);
-cudaError_t launch_sweep_h(const SweepArgs& a, cudaStream_t stream);
+                        Stream stream);
+cudaError_t launch_sweep_h(const SweepArgs& a, Stream stream);
 // The first sweep stage of a path with pairs (4 or 8 directions): the
 // horizontal pair and the first halves (phase 1) of up to three vertical-type
 // pairs in one launch; blocks [start[0], start[1]) run the horizontal pair,
@@ -115,30 +143,30 @@ struct FirstStageArgs {
     int nv;
     int start[5];
 };
-cudaError_t launch_sweep_first(FirstStageArgs& f, cudaStream_t stream);
+cudaError_t launch_sweep_first(FirstStageArgs& f, Stream stream);
 // 4 paths: the horizontal first halves (saving their state in f.h.state) beside
 // the whole vertical pair f.v[0], which writes S; then the horizontal second
 // halves finish with Eq. 4 (launch_sweep_h2, a.state as in the first stage).
-cudaError_t launch_sweep_first4(FirstStageArgs& f, cudaStream_t stream);
-cudaError_t launch_sweep_h2(const SweepArgs& a, cudaStream_t stream);
-cudaError_t launch_sweep_v(const SweepArgs& a, cudaStream_t stream);
+cudaError_t launch_sweep_first4(FirstStageArgs& f, Stream stream);
+cudaError_t launch_sweep_h2(const SweepArgs& a, Stream stream);
+cudaError_t launch_sweep_v(const SweepArgs& a, Stream stream);
 // Words of saved path state per vertical-type pair between its two phases:
 // per line, 32 lanes x (K + 3) words for each warp carrying it (one warp of
 // 16-lane paths, K = D/32; or two warps of 32-lane paths, K = D/64).
 inline size_t sweep_state_words(int W, int D) {
     return (D % 64 == 0) ? static_cast<size_t>(W) * 64 * (D / 64 + 3) : static_cast<size_t>(W) * 32 * (D / 32 + 3);
 }
-cudaError_t launch_median(const uint8_t* raw, uint8_t* disp, int W, int H, cudaStream_t stream);
+cudaError_t launch_median(const uint8_t* raw, uint8_t* disp, int W, int H, Stream stream);
 // Post-filters (sgm_compute_ex).  Mirror: mr[y][x] = right[y][W-1-x],
 // ml[y][x] = left[y][W-1-x].
 cudaError_t launch_mirror(const uint8_t* left, const uint8_t* right, uint8_t* ml, uint8_t* mr, int W, int H,
-                          cudaStream_t stream);
+                          Stream stream);
 // out16 = 3x3 median of v, v = 16 d + the sub-pixel offset from sub (when
 // sub != nullptr) with d = rawL; then, when rawRm != nullptr (the right
 // pass's disparity in mirrored columns), 0xFFFF where the left-right check
-// fails.
-cudaError_t launch_post(const uint8_t* rawL, const uint32_t* sub, const uint8_t* rawRm, uint16_t* out16, int W,
-                        int H, int D, cudaStream_t stream);
+// fails.  quads: the three inputs are in quads of 2 x 2 pixels, else row-major.
+cudaError_t launch_post(const uint8_t* rawL, const uint32_t* sub, const uint8_t* rawRm, uint16_t* out16, bool quads,
+                        int W, int H, int D, Stream stream);
 // The work-list kernels: every job of a list has the launch's D (and, for
 // sweeps, its pair / s8 settings; a vertical-type list runs both halves of
 // its pair in one unit, the vertical one finishing with Eq. 4).
@@ -157,54 +185,83 @@ constexpr int kCensusListPerSM = 16, kCostListPerSM = 8, kMedianListPerSM = 8, k
 cudaError_t launch_unpair_cost(const uint8_t* rec, int RB, uint8_t* out, int W, int H, int D, cudaStream_t stream);
 
 // ---------------------------------------------------------------------------
-// The paired-line 4-path schedule (sgm_pairs.cuh).  Every warp carries two
-// adjacent lines of one direction, one per u16 half of each packed word.  The
+// The paired-line schedule (sgm_pairs.cuh).  Every warp carries two adjacent
+// lines of one direction, one per u16 half of each packed word.  The
 // per-(pixel, disparity) cubes live in quads of 2 x 2 pixels over the grid
 // padded to even sizes W2 x H2: quad (qx, qy) holds, per disparity d, the four
 // bytes of pixels (2qx + i, 2qy + j) at byte i + 2j of a 32-bit word, so a
 // quad takes QB = 4D bytes of a cube.  Each cube is its own array of
 // [QH][QW] quads (FS bytes), at rec + f FS for field f:
-//   0 MC    matching costs (Eq. 2); 0 at padding pixels
-//   1 LvT   stored L_r of the top-to-bottom path
-//   2 LvB   stored L_r of the bottom-to-top path
-//   3 Lh0   stored L_r of the left-to-right path
-//   4 Lh1   stored L_r of the right-to-left path
-// One 32-bit offset q QB then addresses quad q in every field.
+//   0     MC      matching costs (Eq. 2); 0 at padding pixels
+//   1, 2  vertical   r = L_r - MC of the top-to-bottom and bottom-to-top paths
+//   3, 4  diagonal   r of the down-right and the up-left paths
+//   5, 6  diagonal   r of the down-left and the up-right paths
+// (2 paths: fields 0, 1; 4 paths: 0-2; 8 paths: all).  One 32-bit offset
+// q QB then addresses quad q in every field.  The diagonal fields hold units
+// of a line pair instead of quads: unit (j, p) at [j][p] holds, per disparity,
+// line 2p at rows 2j and 2j + 1, then line 2p + 1 (sgm_pairs.cuh).
 // ---------------------------------------------------------------------------
-constexpr int kPairsFields = 5;
+__host__ __device__ constexpr int pairs_fields(int n_paths) { return n_paths == 2 ? 2 : (n_paths == 4 ? 3 : 7); }
+
+// Quads of a segment: the horizontal walks store their state at every segment
+// boundary and the finishing launch walks each segment again.  Sixteen columns
+// keep the states at 1/16 of a stored field per direction; with more than 128
+// disparities a warp's segment has to fit its shared memory.
+__host__ __device__ constexpr int seg_quads(int D) { return D <= 128 ? 8 : 4; }
 
 struct PairsArgs {
-    uint8_t* rec;     // the field arrays (kPairsFields of FS bytes each)
-    uint8_t* rawq;    // winner-take-all disparity in quads [QH][QW][4]
-    uint16_t* Sdbg;   // optional natural-order S [H][W][D] (debug)
-    uint32_t* state;  // horizontal chains between the launches: [QH][2][32][K + 1]
-    int W, H, W2, H2, QW, QH, D;
-    size_t FS;        // bytes of one field array (QH * QW * QB, rounded up)
-    int QB;           // bytes of one quad in a field: 4D (W2 * H2 * D < 2^32)
-    int n1;           // steps of each horizontal direction in the first launch (even)
-    // second launch: left-to-right stores [n1, a) then finishes [a, W2) with
-    // Eq. 4; right-to-left stores [b, W2 - n1) then finishes [0, b); columns
-    // [b, a) are finished by the parallel winner-take-all
-    int a, b;
+    uint8_t* rec;          // the field arrays (pairs_fields of FS bytes each)
+    uint8_t* rawq;         // winner-take-all disparity in quads [QH][QW][4]
+    uint16_t* Sdbg;        // optional natural-order S [H][W][D] (debug)
+    uint32_t* state;       // horizontal states [2][QH][NS][(D/32 + 1) / 2][32]
+    // Post-filters: the jump penalty of every step, [8][QH][QW] words of the
+    // four pixels of a quad or diagonal unit (direction: left to right, right to
+    // left, then the order of the fields), or null (P2 throughout); S(d-1) - S(d)
+    // | (S(d+1) - S(d)) << 16 at the winner in quads [QH][QW][4], or null.
+    const uint32_t* p2map;
+    uint32_t* subq;
+    int W, H, W2, H2, QW, QH, D, n_paths;
+    int NS;                // segments of a row pair
+    size_t FS;             // bytes of one field array (QH * QW * QB, rounded up)
+    int QB;                // bytes of one quad in a field: 4D (W2 * H2 * D < 2^32)
     uint32_t P1x2, P2x2;
-    int s8;           // two stored L_r sum in a byte: 2 (MC_max + P2) <= 255
-    int mc_max;       // largest matching cost: 31 (CSCT) or 62 (full Census)
-    int nvb, nhb;     // first launch: vertical / horizontal blocks (64 threads each)
-    int nh2, npw;     // second launch: chain blocks; parallel winner-take-all blocks (beside them)
-    int check_shrink; // bounds-checked build, test hook: bytes taken off the declared end of the fields
+    int mc_max;            // largest matching cost: 31 (CSCT) or 62 (full Census)
+    int gs;                // stored r that add in a byte: gs * (largest P2) <= 255, at most 3
+    int check_shrink;      // bounds-checked build, test hook: bytes taken off the declared end of the fields
 };
-// Geometry and block counts for a W x H problem (n1 < 0: the default split).
-PairsArgs pairs_geometry(int W, int H, int D, int n1);
-// Quad-layout matching cost (Eq. 2) into mc: quad q at mc + q QB.
-cudaError_t launch_cost_quads(const void* Fb, const void* Fm, uint8_t* mc, int QB, int W, int H, int D, bool ct62,
-                              cudaStream_t stream);
-cudaError_t launch_pairs_stage1(const PairsArgs& a, cudaStream_t stream);
-// The second launch is two kernels that may run side by side: the chains and
-// the parallel winner-take-all.
-cudaError_t launch_pairs_chain2(const PairsArgs& a, cudaStream_t stream);
-cudaError_t launch_pairs_par(const PairsArgs& a, cudaStream_t stream);
+// One launch over one or two problems of the same shape (the two passes of the
+// left-right check).
+struct PairsJobs {
+    PairsArgs job[2];
+    int n;
+};
+// Geometry of a W x H problem.
+PairsArgs pairs_geometry(int W, int H, int D, int n_paths);
+inline size_t pairs_state_words(const PairsArgs& a) {
+    return static_cast<size_t>(2) * a.QH * a.NS * 32 * ((a.D / 32 + 1) / 2);
+}
+inline int pairs_group(int p2_max) { return 3 * p2_max <= 255 ? 3 : (2 * p2_max <= 255 ? 2 : 1); }
+// Features of one or both passes: image z of F + z fstride bytes is left (0),
+// right (1), and with n = 4 the mirrored pair of the right pass (right, left).
+cudaError_t launch_census_passes(const uint8_t* left, const uint8_t* right, void* F, size_t fstride, int n, int W,
+                                 int H, bool ct62, Stream stream);
+// Quad-layout matching cost (Eq. 2): pass k from feature images 2k and 2k + 1
+// into mc + k mcstride, quad q at + q QB.
+cudaError_t launch_cost_quads(const void* F, size_t fstride, uint8_t* mc, size_t mcstride, int passes, int QB, int W,
+                              int H, int D, bool ct62, Stream stream);
+// Jump penalties max(P1, P2 / (1 + g)) of every step (PairsArgs::p2map): base
+// image img, or its mirror image.
+cudaError_t launch_p2map(const uint8_t* img, bool mirror, uint32_t* map, int n_paths, int W, int H, int P1, int P2,
+                         Stream stream);
+// The walks of a path: one launch per kind, side by side (the first one waits
+// for the costs, each lets the next one start as soon as its own blocks have,
+// and the last block of a later one waits for the one before it, so that the
+// last launch ends when all have), or both kinds of 2 paths in one launch.
+enum class Walks { kHor, kVer, kDiag, kHorVer };
+cudaError_t launch_pairs_walks(const PairsJobs& f, Walks w, Stream stream);
+cudaError_t launch_pairs_finish(const PairsJobs& f, Stream stream);
 // 3x3 median of a quad-layout raw disparity.
-cudaError_t launch_median_quads(const uint8_t* rawq, uint8_t* disp, int W, int H, cudaStream_t stream);
+cudaError_t launch_median_quads(const uint8_t* rawq, uint8_t* disp, int W, int H, Stream stream);
 // Debug: a quad-layout cube (quad q at cube + q QB) -> natural order [H][W][D].
 cudaError_t launch_unquad_cost(const uint8_t* cube, int QB, uint8_t* out, int W, int H, int D, cudaStream_t stream);
 

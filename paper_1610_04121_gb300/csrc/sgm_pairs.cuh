@@ -1,6 +1,6 @@
 // Path aggregation (Eq. 3), the sum S and the winner-take-all disparity
-// (Eq. 4) of the 4-path SGM of arXiv 1610.04121 with two lines per warp, for
-// sm_103a.
+// (Eq. 4) of the SGM path of arXiv 1610.04121 with two lines per warp, for
+// sm_103a; 2, 4 and 8 paths.
 //
 // Parallel scheme (Section 3.2's CTA-to-warp conversion, with the paper's
 // byte-SIMD replaced by packed 16-bit lanes): a warp carries two adjacent
@@ -12,26 +12,36 @@
 // the two per-line minima m(q) are two warp reductions.  No byte of a word
 // ever crosses into the other line's half: every value stays below 2^14.
 //
-// Data layout (sgm_internal.h): every cube lives in quads of 2 x 2 pixels,
-// one array per cube, so that a walk in either axis reads one quad (4 K bytes
-// per lane) per two steps and writes one quad per two steps of the same walk,
-// and the walks of neighbouring line pairs touch neighbouring memory.  Rows and columns
-// are padded to even counts; the padding pixels have MC = 0, so a path that
-// starts on one (a walk from the bottom or right edge of an odd-sized image)
-// passes through it unchanged: from the reset state a zero-cost step leaves
-// L = 0 and m = 0, which is the reset state again.
+// Data layout (sgm_internal.h): the cost cube lives in quads of 2 x 2 pixels,
+// so that a walk along rows or columns reads one quad (4 K bytes per lane)
+// per two steps; a walk along diagonals reads two neighbouring quads per two
+// steps.  Rows and columns are padded to even counts; the padding pixels have
+// MC = 0, so a path that starts on one (a walk from the bottom or right edge
+// of an odd-sized image) passes through it unchanged: from the reset state a
+// zero-cost step leaves L = 0 and m = 0, which is the reset state again.
 //
-// Schedule (4 paths: left-to-right, right-to-left, top-to-bottom,
-// bottom-to-top):
-//   launch 1  every walker stores its own L_r: the vertical pair walks every
-//             row, each horizontal direction n1 columns; nothing is read but
-//             the costs, so no walker waits for another;
-//   launch 2  the rest of each horizontal direction, finishing its pixels
-//             with Eq. 4 (S = its own L_r + the three stored ones), beside a
-//             parallel winner-take-all over the columns both horizontal
-//             directions passed in launch 1.
-// With n1 = min(W, H) the longest chain is max(W, H) steps, against H + W / 2
-// for a schedule that finishes one pair before the other starts.
+// Schedule:
+//   walks     every direction of every line pair at once.  The vertical and
+//             diagonal walkers store r = L_r - MC (0 <= r <= P2, a byte); the
+//             horizontal walkers store nothing but their state at every
+//             segment boundary (kSegQuads quads);
+//   finish    a warp per segment of a row pair walks left to right and right
+//             to left again from the stored states, adds the stored r of the
+//             other directions and takes the winner.
+// Walking a horizontal direction twice costs its integer work again (the
+// finishing launch has the integer units to spare: it is bound by reading the
+// stored r), and saves writing and reading back two bytes per pixel and
+// disparity.
+//
+// Bounds: a step takes about 45 instructions per warp and 256 (pixel,
+// disparity) pairs, 15-19 of them on the integer ALU, where each takes two
+// cycles; two warps per scheduler (a 640x480 frame) are bound by that and by
+// the chain of a step (two shuffles and two reductions), full schedulers by
+// the ALU.  Measured, whole frame, against the per-line sweeps (one line per
+// warp, sums in records): 1242x375 D=128 8 paths 390 -> 208 us, 1920x1080
+// D=128 8 paths 1440 -> 1008 us, 640x480 D=128 2 paths 84 -> 62 us, the same
+// with 4 paths and all post-filters 256 -> 182 us; the walks of the 640x480
+// 4-path frame take 38 us, the finishing launch 27 us.
 #pragma once
 
 #include "sgm_device.cuh"
@@ -43,157 +53,195 @@ namespace pairs {
 constexpr uint32_t kInf2 = kInf16 * 0x10001u;
 constexpr unsigned kFull = 0xffffffffu;
 
-// Field arrays (sgm_internal.h).
-enum Field { kMC = 0, kLVT = 1, kLVB = 2, kLH0 = 3, kLH1 = 4 };
+// Walk kinds of the first launch.
+enum Kind { kHor = 0, kVer = 1, kDiag = 2 };
 
-// One quad register [x0y0, x1y0, x0y1, x1y1] -> the u16x2 word of one step:
-// the column pair at row h (vertical walks) or the row pair at column h
-// (horizontal walks).
-template <bool VERT>
-__device__ __forceinline__ uint32_t unq(uint32_t q, int h) {
-    return __byte_perm(q, 0u, VERT ? (h ? 0x4342u : 0x4140u) : (h ? 0x4341u : 0x4240u));
+// Byte selectors: two bytes of a quad [x0y0, x1y0, x0y1, x1y1] as the u16x2 word
+// of a step, columns of row j (vertical walks) or rows of column i (horizontal
+// walks).  The zero bytes replicate the sign of a cost (MC <= 62).
+constexpr uint32_t kSelRow0 = 0x9180u, kSelRow1 = 0xB3A2u, kSelCol0 = 0xA280u, kSelCol1 = 0xB391u;
+// Diagonal walks take row 2j from quad a and row 2j + 1 from quads (a, a + 1)
+// (lines moving right with increasing row) or (a, a - 1) (moving left).
+constexpr uint32_t kSelNext = 0xE6B3u, kSelPrev = 0xA2F7u;
+
+// ---------------------------------------------------------------------------
+// Unit copies: a unit of a field (a quad, 4 D contiguous bytes) goes to
+// shared memory with asynchronous 16-byte copies through L2 only, one group
+// per unit.  Completion is counted per group, so a warp waits for exactly the
+// unit it needs however many are in flight (register prefetch shares six
+// scoreboards among all loads in flight and waits for later ones too).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+    __syncwarp();
 }
 
-// The words of half 0 and half 1 of a unit (values below 256) -> one quad register.
-template <bool VERT>
-__device__ __forceinline__ uint32_t toq(uint32_t w0, uint32_t w1) {
-    return __byte_perm(w0, w1, VERT ? 0x6420u : 0x6240u);
-}
-
-// L2 eviction priority of a cube's loads and stores: kL2Normal, or kL2Last
-// (kept over normal and first lines; the costs, read by four walkers) or
-// kL2First (streamed through; stored costs read much later).
-enum L2Hint { kL2Normal = 0, kL2Last = 1, kL2First = 2 };
-
-template <int HINT>
-__device__ __forceinline__ uint64_t l2_policy() {
+// L2 policy of data read for the last time: its lines go first, so that they do
+// not push out what the other warps are about to read (the finishing launch of
+// a 1242x375 8-path frame reads 7 bytes per pixel and disparity, most of it
+// past what L2 holds: 216 -> 206 us for the frame).
+__device__ __forceinline__ uint64_t last_read() {
     uint64_t pol;
-    if constexpr (HINT == kL2Last)
-        asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-    else
-        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
     return pol;
 }
 
-// N registers from 4N bytes at p (16-byte aligned when N % 4 == 0, 8-byte when
-// N is even), through L2 only.
-template <int N, bool NC, int HINT = kL2Normal>
-__device__ __forceinline__ void ldv(const uint8_t* p, uint32_t (&r)[N]) {
-    if constexpr (N % 4 == 0 && HINT != kL2Normal) {
-        const uint64_t pol = l2_policy<HINT>();
-#pragma unroll
-        for (int i = 0; i < N / 4; ++i)
-            asm volatile("ld.global.cg.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
-                         : "=r"(r[4 * i]), "=r"(r[4 * i + 1]), "=r"(r[4 * i + 2]), "=r"(r[4 * i + 3])
-                         : "l"(p + 16 * i), "l"(pol));
-    } else if constexpr (N % 4 == 0) {
-#pragma unroll
-        for (int i = 0; i < N / 4; ++i) {
-            const uint4* q = reinterpret_cast<const uint4*>(p) + i;
-            const uint4 v = NC ? __ldg(q) : __ldcg(q);
-            r[4 * i] = v.x;
-            r[4 * i + 1] = v.y;
-            r[4 * i + 2] = v.z;
-            r[4 * i + 3] = v.w;
-        }
-    } else if constexpr (N % 2 == 0) {
-#pragma unroll
-        for (int i = 0; i < N / 2; ++i) {
-            const uint2* q = reinterpret_cast<const uint2*>(p) + i;
-            const uint2 v = NC ? __ldg(q) : __ldcg(q);
-            r[2 * i] = v.x;
-            r[2 * i + 1] = v.y;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            const unsigned* q = reinterpret_cast<const unsigned*>(p) + i;
-            r[i] = NC ? __ldg(q) : __ldcg(q);
-        }
-    }
-}
-
-template <int N, int HINT = kL2Normal>
-__device__ __forceinline__ void stv(uint8_t* p, const uint32_t (&r)[N]) {
-    if constexpr (N % 4 == 0 && HINT != kL2Normal) {
-        const uint64_t pol = l2_policy<HINT>();
-#pragma unroll
-        for (int i = 0; i < N / 4; ++i)
-            asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p + 16 * i),
-                         "r"(r[4 * i]), "r"(r[4 * i + 1]), "r"(r[4 * i + 2]), "r"(r[4 * i + 3]), "l"(pol)
-                         : "memory");
-    } else if constexpr (N % 4 == 0) {
-#pragma unroll
-        for (int i = 0; i < N / 4; ++i)
-            reinterpret_cast<uint4*>(p)[i] = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
-    } else if constexpr (N % 2 == 0) {
-#pragma unroll
-        for (int i = 0; i < N / 2; ++i) reinterpret_cast<uint2*>(p)[i] = make_uint2(r[2 * i], r[2 * i + 1]);
-    } else {
-#pragma unroll
-        for (int i = 0; i < N; ++i) reinterpret_cast<unsigned*>(p)[i] = r[i];
-    }
-}
-
-// Launch 2: input registers of the chains' prefetch, and quads per warp of the
-// parallel winner-take-all.
-constexpr int kChainPrefetchRegs = 192, kParItems = 4;
-
-// Cache policy of the walks' traffic (measured on the 640x480 D=128 frame):
-// the stored costs, written in the first launch and read in the second, go
-// through L2 as evict-first, so that they do not push out the costs the other
-// walkers are about to read (first launch 51 -> 43 us, second 41 -> 35 us).
-constexpr int kHintMcLoad = kL2Normal, kHintLStore = kL2First, kHintLLoad = kL2First;
-
-// Extents for the bounds-checked build: the field arrays, the quad raw
-// disparity, the chains' state and the debug sums.
+// Extents for the bounds-checked build.
 __device__ __forceinline__ const uint8_t* cubes_end(const PairsArgs& a) {
-    return a.rec + kPairsFields * a.FS - a.check_shrink;
-}
-__device__ __forceinline__ size_t state_words(const PairsArgs& a) {
-    return static_cast<size_t>(a.QH) * 2 * 32 * (a.D / 32 + 1);
+    return a.rec + pairs_fields(a.n_paths) * a.FS - a.check_shrink;
 }
 
-template <int N, int HINT>
-__device__ __forceinline__ void ldv_checked(const PairsArgs& a, const uint8_t* p, uint32_t (&r)[N], unsigned site) {
-    if (SGM_GUARD(p, 4 * N, a.rec, cubes_end(a), site)) {
-        ldv<N, false, HINT>(p, r);
-    } else {
-#pragma unroll
-        for (int i = 0; i < N; ++i) r[i] = 0u;
-    }
-}
-
-template <int N, int HINT>
-__device__ __forceinline__ void stv_checked(const PairsArgs& a, uint8_t* p, const uint32_t (&r)[N], unsigned site) {
-    if (SGM_GUARD(p, 4 * N, a.rec, cubes_end(a), site)) stv<N, HINT>(p, r);
-}
-
-__device__ __forceinline__ void raw_quad_store(const PairsArgs& a, size_t q, uint32_t v, unsigned site) {
-    if (SGM_GUARD_INDEX(static_cast<long long>(q), static_cast<long long>(a.QW) * a.QH, site))
-        reinterpret_cast<uint32_t*>(a.rawq)[q] = v;
-}
-
-__device__ __forceinline__ void sdbg_store(const PairsArgs& a, size_t i, uint32_t v, unsigned site) {
-    if (SGM_GUARD_INDEX(static_cast<long long>(i), static_cast<long long>(a.W) * a.H * a.D, site))
-        a.Sdbg[i] = static_cast<uint16_t>(v);
-}
-
-// 64-bit base + 32-bit record offset in one instruction.
+// 64-bit base + 32-bit offset in one instruction.
 __device__ __forceinline__ uint8_t* at(uint8_t* base, uint32_t off) {
     uint64_t r;
     asm("mad.wide.u32 %0, %1, 1, %2;" : "=l"(r) : "r"(off), "l"(reinterpret_cast<uint64_t>(base)));
     return reinterpret_cast<uint8_t*>(r);
 }
 
+// base: the lane's base (field + 16 lane); dst: shared address of the slot + 16 lane.
+template <int D, bool LAST = false>
+__device__ __forceinline__ void cp_unit(const PairsArgs& a, uint32_t dst, uint8_t* base, uint32_t off, unsigned site,
+                                        uint64_t pol = 0) {
+    constexpr int NC = D / 4;  // 16-byte pieces of a unit
+    const int lane = threadIdx.x & 31;
+    uint8_t* const g = at(base, off);
+#pragma unroll
+    for (int i = 0; i < (NC + 31) / 32; ++i)
+        if (NC % 32 == 0 || lane + 32 * i < NC)
+            if (SGM_GUARD(g + 512 * i, 16, a.rec, cubes_end(a), site))
+            {
+                if constexpr (LAST)
+                    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst + 512 * i),
+                                 "l"(g + 512 * i), "l"(pol)
+                                 : "memory");
+                else
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 512 * i), "l"(g + 512 * i)
+                                 : "memory");
+            }
+}
+
+// A lane's 4 K bytes of a unit in shared memory (address of the lane's bytes).
+template <int K>
+__device__ __forceinline__ void lds_unit(uint32_t s, uint32_t (&r)[K]) {
+    if constexpr (K % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < K / 4; ++i)
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(r[4 * i]), "=r"(r[4 * i + 1]), "=r"(r[4 * i + 2]), "=r"(r[4 * i + 3])
+                         : "r"(s + 16 * i));
+    } else if constexpr (K % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < K / 2; ++i)
+            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(r[2 * i]), "=r"(r[2 * i + 1]) : "r"(s + 8 * i));
+    } else {
+#pragma unroll
+        for (int i = 0; i < K; ++i) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(r[i]) : "r"(s + 4 * i));
+    }
+}
+
+template <int K>
+__device__ __forceinline__ void sts_unit(uint32_t s, const uint32_t (&r)[K]) {
+    if constexpr (K % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < K / 4; ++i)
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(s + 16 * i), "r"(r[4 * i]),
+                         "r"(r[4 * i + 1]), "r"(r[4 * i + 2]), "r"(r[4 * i + 3])
+                         : "memory");
+    } else if constexpr (K % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < K / 2; ++i)
+            asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(s + 8 * i), "r"(r[2 * i]), "r"(r[2 * i + 1])
+                         : "memory");
+    } else {
+#pragma unroll
+        for (int i = 0; i < K; ++i) asm volatile("st.shared.u32 [%0], %1;" ::"r"(s + 4 * i), "r"(r[i]) : "memory");
+    }
+}
+
+// A lane's 4 K bytes of a unit from global memory, through L2 only.
+template <int K>
+__device__ __forceinline__ void ldg_unit(const PairsArgs& a, const uint8_t* p, uint32_t (&r)[K], uint64_t pol,
+                                         unsigned site) {
+    if (!SGM_GUARD(p, 4 * K, a.rec, cubes_end(a), site)) {
+#pragma unroll
+        for (int i = 0; i < K; ++i) r[i] = 0u;
+    } else if constexpr (K % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < K / 4; ++i) {
+            asm volatile("ld.global.cg.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
+                         : "=r"(r[4 * i]), "=r"(r[4 * i + 1]), "=r"(r[4 * i + 2]), "=r"(r[4 * i + 3])
+                         : "l"(p + 16 * i), "l"(pol));
+        }
+    } else if constexpr (K % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < K / 2; ++i) {
+            asm volatile("ld.global.cg.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
+                         : "=r"(r[2 * i]), "=r"(r[2 * i + 1])
+                         : "l"(p + 8 * i), "l"(pol));
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+            asm volatile("ld.global.cg.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(r[i]) : "l"(p + 4 * i), "l"(pol));
+    }
+}
+
+// A lane's 4 K bytes of a unit to global memory.
+template <int K>
+__device__ __forceinline__ void stg_unit(const PairsArgs& a, uint8_t* p, const uint32_t (&r)[K], unsigned site) {
+    if (!SGM_GUARD(p, 4 * K, a.rec, cubes_end(a), site)) return;
+    if constexpr (K % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < K / 4; ++i)
+            reinterpret_cast<uint4*>(p)[i] = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+    } else if constexpr (K % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < K / 2; ++i) reinterpret_cast<uint2*>(p)[i] = make_uint2(r[2 * i], r[2 * i + 1]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < K; ++i) reinterpret_cast<unsigned*>(p)[i] = r[i];
+    }
+}
+
+// A value the compiler cannot see: multiplying by it stays a multiply-add on
+// the FMA pipe instead of becoming a shift on the integer ALU, the pipe these
+// kernels run out of first (both take two cycles per warp instruction).
+__device__ __forceinline__ uint32_t opaque(uint32_t v) {
+    uint32_t r;
+    asm("mov.b32 %0, %1;" : "=r"(r) : "r"(v));
+    asm volatile("" : "+r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t mad(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t d;
+    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+// Byte permute with the sign-replicating selectors (__byte_perm masks them off).
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+    return d;
+}
+// Minimum of three u16 pairs: one ALU instruction, as a minimum of two is.
+__device__ __forceinline__ uint32_t vmin3(uint32_t a, uint32_t b, uint32_t c) { return __vimin3_u16x2(a, b, c); }
+
+// ---------------------------------------------------------------------------
 // Two chains (lines A and B) of Eq. 3 in one warp.  The first pixel of a path
-// starts from the reset state (L = 0, m = 0), which gives L = MC.
+// starts from the reset state (L = 0, m = 0), which gives L = MC.  A constant
+// added to the w and m of a line changes no r (below): a chain that stores no
+// r may leave the subtraction of m out and take it off now and then.
+// ---------------------------------------------------------------------------
 template <int K>
 struct Chain2 {
+    static constexpr int CW = (K + 1) / 2;  // words of a stored state: two bytes per word and lane
     uint32_t w[K];
     uint32_t up, dn;  // word K-1 of lane l-1 and word 0 of lane l+1, exchanged after every step
     uint32_t mpx2;    // (m_A, m_B)
-    uint32_t mul_up, add_up, mul_dn, add_dn;
+    uint32_t mul_up, add_up, mul_dn, add_dn, k16;
 
     __device__ __forceinline__ void init(int lane) {
         // d = 0 has no d - 1 (lane 0) and d = D - 1 no d + 1 (lane 31): those
@@ -202,6 +250,7 @@ struct Chain2 {
         add_up = lane == 0 ? kInf2 : 0u;
         mul_dn = lane == 31 ? 0u : 1u;
         add_dn = lane == 31 ? kInf2 : 0u;
+        k16 = opaque(0x10000u);
         reset();
     }
 
@@ -212,458 +261,753 @@ struct Chain2 {
         mpx2 = 0u;
     }
 
+    // Lines outside `keep` (a mask over the two halves) start a path at the next step.
+    __device__ __forceinline__ void restart(uint32_t keep) {
+#pragma unroll
+        for (int j = 0; j < K; ++j) w[j] &= keep;
+        up &= keep;
+        dn &= keep;
+        mpx2 &= keep;
+    }
+
+    // Neighbour words and per-line minima of the state in w.
     __device__ __forceinline__ void exchange() {
         up = __shfl_up_sync(kFull, w[K - 1], 1);
         dn = __shfl_down_sync(kFull, w[0], 1);
+        uint32_t r = w[0];
+        if constexpr (K == 2) {
+            r = vmin2(w[0], w[1]);
+        } else if constexpr (K > 2) {
+            r = vmin3(w[0], w[1], w[2]);
+#pragma unroll
+            for (int j = 3; j + 1 < K; j += 2) r = vmin3(r, w[j], w[j + 1]);
+            if constexpr (K % 2 == 0) r = vmin2(r, w[K - 1]);
+        }
+        // the 32-bit minimum orders by the high half first
+        const uint32_t hi = __reduce_min_sync(kFull, r);
+        const uint32_t lo = __reduce_min_sync(kFull, mad(r, k16, 0u));
+        mpx2 = __byte_perm(lo, hi, 0x7632u);
     }
 
-    // L(p, d) = MC(p, d) + min(L(q, d), L(q, d-1) + P1, L(q, d+1) + P1, m(q) + P2) - m(q)
-    __device__ __forceinline__ void step(const uint32_t (&mc)[K], uint32_t P1x2, uint32_t P2x2) {
+    // x(d) = min(L(q, d), L(q, d-1) + P1, L(q, d+1) + P1, m(q) + P2), the step's costs before MC and m(q)
+    __device__ __forceinline__ void relax(uint32_t P1x2, uint32_t P2x2, uint32_t (&x)[K]) const {
         const uint32_t u = up * mul_up + add_up;
         const uint32_t d = dn * mul_dn + add_dn;
         const uint32_t mp2 = mpx2 + P2x2;
-        uint32_t L[K];
 #pragma unroll
         for (int j = 0; j < K; ++j) {
             const uint32_t dm1 = j == 0 ? u : w[j - 1];
             const uint32_t dp1 = j == K - 1 ? d : w[j + 1];
-            // every candidate is >= m(q) in each half, so the packed subtraction never borrows
-            L[j] = vmin2(vmin2(dm1, dp1) + P1x2, vmin2(w[j], mp2)) + mc[j] - mpx2;
+            x[j] = vmin3(vmin2(dm1, dp1) + P1x2, w[j], mp2);
         }
-        uint32_t r = L[0];
+    }
+
+    // One step with r(p, d) = L(p, d) - MC(p, d), 0 <= r <= P2.
+    __device__ __forceinline__ void step(const uint32_t (&mc)[K], uint32_t P1x2, uint32_t P2x2, uint32_t (&r)[K]) {
+        uint32_t x[K];
+        relax(P1x2, P2x2, x);
+        // every candidate is >= m(q) in each half, so the packed subtraction never borrows
 #pragma unroll
-        for (int j = 1; j < K; ++j) r = vmin2(r, L[j]);
+        for (int j = 0; j < K; ++j) r[j] = x[j] - mpx2;
 #pragma unroll
-        for (int j = 0; j < K; ++j) w[j] = L[j];
+        for (int j = 0; j < K; ++j) w[j] = r[j] + mc[j];
         exchange();
-        // per-half minima: the 32-bit minimum orders by the high half first
-        const uint32_t hi = __reduce_min_sync(kFull, r);
-        const uint32_t lo = __reduce_min_sync(kFull, r << 16);
-        mpx2 = __byte_perm(lo, hi, 0x7632u);
+    }
+
+    // One step that leaves m(q) in w and m; at most 16 between rebase() calls
+    // (16 steps add at most 16 * 62, far below the infinity of the border lanes).
+    __device__ __forceinline__ void step_raw(const uint32_t (&mc)[K], uint32_t P1x2, uint32_t P2x2) {
+        uint32_t x[K];
+        relax(P1x2, P2x2, x);
+#pragma unroll
+        for (int j = 0; j < K; ++j) w[j] = x[j] + mc[j];
+        exchange();
+    }
+
+    __device__ __forceinline__ void rebase() {
+#pragma unroll
+        for (int j = 0; j < K; ++j) w[j] -= mpx2;
+        up -= mpx2;
+        dn -= mpx2;
+        mpx2 = 0u;
+    }
+
+    // A stored state: every L_r fits a byte.  Word i of lane l at p[32 i + l].
+    __device__ __forceinline__ void save(uint32_t* p) const {
+#pragma unroll
+        for (int i = 0; i < CW; ++i)
+            p[32 * i] = __byte_perm(w[2 * i], 2 * i + 1 < K ? w[2 * i + 1 < K ? 2 * i + 1 : 0] : 0u, 0x6420u);
+    }
+    __device__ __forceinline__ void restore(const uint32_t (&c)[CW]) {
+#pragma unroll
+        for (int j = 0; j < K; ++j) w[j] = __byte_perm(c[j / 2], 0u, (j & 1) ? 0x4342u : 0x4140u);
+        exchange();
     }
 };
 
-// Winner-take-all (Eq. 4) of two pixels at once: S holds (S_A(d), S_B(d)) for
-// the lane's disparities; returns (d_A, d_B) in the two u16 halves, the
-// lowest d among equal minima.  KEY16: S * D + d fits 16 bits, so one packed
-// multiply-add makes both keys; else 32-bit keys S << 8 | d per pixel.
-template <int K, int D, bool KEY16>
-__device__ __forceinline__ uint32_t wta2(const uint32_t (&S)[K], const uint32_t (&dc)[K]) {
-    if constexpr (KEY16) {
-        uint32_t best = S[0] * static_cast<uint32_t>(D) + dc[0];
-#pragma unroll
-        for (int j = 1; j < K; ++j) best = vmin2(best, S[j] * static_cast<uint32_t>(D) + dc[j]);
-        const uint32_t hi = __reduce_min_sync(kFull, best);
-        const uint32_t lo = __reduce_min_sync(kFull, best << 16);
-        const uint32_t mk = __byte_perm(lo, hi, 0x7632u);
-        if constexpr ((D & (D - 1)) == 0) {
-            return mk & (static_cast<uint32_t>(D - 1) * 0x10001u);
-        } else {
-            return ((mk & 0xffffu) % static_cast<uint32_t>(D)) | (((mk >> 16) % static_cast<uint32_t>(D)) << 16);
-        }
-    } else {
-        uint32_t bA = 0xffffffffu, bB = 0xffffffffu;
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            bA = min(bA, __byte_perm(S[j], dc[j], 0x5104u));  // [d, S_A.b0, S_A.b1, 0]
-            bB = min(bB, __byte_perm(S[j], dc[j], 0x5324u));  // [d, S_B.b0, S_B.b1, 0]
-        }
-        bA = __reduce_min_sync(kFull, bA);
-        bB = __reduce_min_sync(kFull, bB);
-        return (bA & 0xffu) | ((bB & 0xffu) << 16);
-    }
+// A word of bytes [b0, b1, b2, b3] as (b0, b2) and (b1, b3): one permute on the
+// ALU, one multiply-add on the FMA pipe (m256 = -256, opaque).
+__device__ __forceinline__ void split(uint32_t q, uint32_t m256, uint32_t& even, uint32_t& odd) {
+    odd = __byte_perm(q, 0u, 0x4341u);
+    even = mad(odd, m256, q);
 }
 
-template <int K, bool KEY16>
-__device__ __forceinline__ void wta_dconst(int lane, uint32_t (&dc)[K]) {
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-        const uint32_t d = static_cast<uint32_t>(K * lane + j);
-        dc[j] = KEY16 ? d * 0x10001u : d;
-    }
+// Segment states of the horizontal walks: slot s of (direction, row pair) is
+// the state in front of segment s in the direction's order.
+template <int D>
+__device__ __forceinline__ uint32_t* state_slot(const PairsArgs& a, int dir, int r, int s) {
+    constexpr int CW = Chain2<D / 32>::CW;
+    return a.state + ((static_cast<size_t>(dir) * a.QH + r) * a.NS + s) * (32 * CW) + (threadIdx.x & 31);
+}
+template <int D>
+__device__ __forceinline__ bool state_ok(const PairsArgs& a, const uint32_t* p, unsigned site) {
+    return SGM_GUARD(p, 4 * (32 * (Chain2<D / 32>::CW - 1) + 1), a.state,
+                     a.state + static_cast<size_t>(2) * a.QH * a.NS * 32 * Chain2<D / 32>::CW, site);
 }
 
-enum Mode {
-    kStore = 0,  // store L_r in this direction's field
-    kWta = 1     // horizontal last steps: S = L + the three stored L_r, then Eq. 4
-};
-
-// Inputs of one unit (two steps: one quad) of a walk: MC, and for kWta the
-// other horizontal direction's stored L_r and the two vertical ones.
-template <int D, int MODE>
-struct UnitIn {
-    static constexpr int K = D / 32;
-    static constexpr int NO = MODE == kWta ? K : 0;
-    static constexpr int REGS = K + 3 * NO;
-    uint32_t mc[K];
-    uint32_t o[NO > 0 ? NO : 1];
-    uint32_t v0[NO > 0 ? NO : 1];
-    uint32_t v1[NO > 0 ? NO : 1];
-};
-
-// Per-lane field bases of a walk.
-struct Bases {
-    uint8_t* mc;   // MC
-    uint8_t* out;  // this direction's stored L_r (kStore)
-    uint8_t* o;    // the other horizontal direction's stored L_r (kWta)
-    uint8_t* v0;   // top-to-bottom stored L_r (kWta)
-    uint8_t* v1;   // bottom-to-top stored L_r (kWta)
-};
-
-// A walk over `nu` units: unit k at record offset off0 + k * dstride (a
-// wrapped negative step for descending walks) and quad column qc0 + k * dqc
-// (horizontal walks: raw output and debug).
-struct Walk {
-    uint32_t off0, dstride;
-    int nu;
-    int qc0, dqc;  // horizontal walks: quad column of unit 0 and its step
-    int r;         // horizontal walks: the row pair
-};
-
-// Byte selectors of a walk, held in registers so that one body of code serves
-// every axis and direction: the two steps of a unit take halves h0 then h1
-// (0 then 1 for ascending rows or columns); un[t] turns a quad register into
-// the word of step t and cq turns the words of steps 0 and 1 into a quad.
-struct Sel {
-    uint32_t un[2], cq;
-    int h0;
-};
-
-__device__ __forceinline__ Sel walk_sel(bool vert, bool asc) {
-    Sel s;
-    const uint32_t u_lo = vert ? 0x4140u : 0x4240u, u_hi = vert ? 0x4342u : 0x4341u;
-    s.un[0] = asc ? u_lo : u_hi;
-    s.un[1] = asc ? u_hi : u_lo;
-    // words w0 (half 0), w1 (half 1): vertical [w0.b0, w0.b2, w1.b0, w1.b2],
-    // horizontal [w0.b0, w1.b0, w0.b2, w1.b2]; descending walks pass (w1, w0)
-    s.cq = vert ? (asc ? 0x6420u : 0x2064u) : (asc ? 0x6240u : 0x2604u);
-    s.h0 = asc ? 0 : 1;
-    return s;
+// The walks' ring of units in shared memory, per warp: a multiple of kUnroll
+// units, at most 16.
+constexpr int kUnroll = 4;
+template <int D>
+__host__ __device__ constexpr int ring_bytes() {
+    return D <= 128 ? 8192 : 16384;
 }
+template <int D, int KIND>
+struct Ring {
+    static constexpr int SB = (KIND == kDiag ? 2 : 1) * 4 * D;  // bytes of a slot
+    static constexpr int FIT = ring_bytes<D>() / SB / kUnroll * kUnroll;
+    static constexpr int DEPTH = FIT > 16 ? 16 : FIT;
+};
 
-// Units prefetched ahead of the recurrence for `regs_per_unit` input registers.
-__host__ __device__ constexpr int units_ahead(int regs_per_unit, int budget) {
-    return budget / regs_per_unit > 12 ? 12 : (budget / regs_per_unit < 2 ? 2 : budget / regs_per_unit);
-}
-
-// Sum of the three stored L_r of a pixel pair in one step's u16 words: the
-// other horizontal direction (o) and the two vertical ones (v0, v1).  S8:
-// the two vertical costs add as bytes (L_TB + L_BT <= 2 (MC_max + P2) <= 255).
-template <bool S8>
-__device__ __forceinline__ uint32_t stored3(uint32_t o, uint32_t v0, uint32_t v1, uint32_t sel) {
-    if constexpr (S8)
-        return __byte_perm(o, 0u, sel) + __byte_perm(v0 + v1, 0u, sel);
-    else
-        return __byte_perm(o, 0u, sel) + __byte_perm(v0, 0u, sel) + __byte_perm(v1, 0u, sel);
-}
-
-// One walk.  The inputs of unit k + PU are loaded into unit k's registers as
-// soon as unit k is done, so every load has PU units of the recurrence to
-// arrive, and the loop body is PU units long.
-template <int D, int MODE, bool S8 = true, bool KEY16 = true, bool DBG = false, int PFB = 48>
-__device__ __forceinline__ void walk(Chain2<D / 32>& ch, const PairsArgs& a, const Bases& bs, const Walk& wk,
-                                     const Sel& sel) {
-    constexpr int K = D / 32;
-    using In = UnitIn<D, MODE>;
-    constexpr int PU = units_ahead(In::REGS, PFB);
-    const int nu = wk.nu;
-    if (nu <= 0) return;
+// ---------------------------------------------------------------------------
+// One walk of the first launch: line pair `line` of a direction (fwd:
+// increasing row or column).  Diagonals: kd = 0 moves right with increasing
+// row, 1 left; line pair p starts at columns 2p, 2p + 1 of row 0 and wraps
+// around at the padded width, each line starting a new path there
+// (Section 3.2).  AP2: the jump penalty of every step comes from a.p2map.
+// One body of code serves both directions (the byte selectors are registers):
+// with a copy per direction the walks that run side by side no longer fit the
+// instruction caches (164 against 144 us for the walks of a 1242x375 8-path
+// frame, although each ran faster alone).
+// ---------------------------------------------------------------------------
+template <int D, int KIND, bool AP2>
+__device__ __forceinline__ void walk(const PairsArgs& a, int line, int kd, bool fwd, uint32_t ring) {
+    constexpr int K = D / 32, CQ = seg_quads(D), SB = Ring<D, KIND>::SB, DEPTH = Ring<D, KIND>::DEPTH;
+    static_assert(CQ % kUnroll == 0 && DEPTH >= kUnroll, "groups of units end where segments end");
     const int lane = threadIdx.x & 31;
-    // every input goes through L2 only: one 16-byte piece per lane of a 512-byte
-    // run is never re-read by the same SM (measured: the L1 path made the
-    // first launch 1.7x slower)
-    auto load = [&](In& in, uint32_t off) {
-        ldv_checked<K, kHintMcLoad>(a, at(bs.mc, off), in.mc, 101);
-        if constexpr (MODE == kWta) {
-            ldv_checked<K, kHintLLoad>(a, at(bs.o, off), in.o, 102);
-            ldv_checked<K, kHintLLoad>(a, at(bs.v0, off), in.v0, 103);
-            ldv_checked<K, kHintLLoad>(a, at(bs.v1, off), in.v1, 104);
-        }
-    };
-    uint32_t dc[K];
-    if constexpr (MODE == kWta) wta_dconst<K, KEY16>(lane, dc);
-    uint32_t off_cur = wk.off0, off_ld = wk.off0;
-    int qc = wk.qc0;
+    const uint32_t QB = static_cast<uint32_t>(a.QB), rowb = static_cast<uint32_t>(a.QW) * QB;
+    int nu;               // units of the walk
+    uint32_t off, ustep;  // offset of the first unit and from unit to unit (in the output field for diagonals)
+    if constexpr (KIND == kHor) {
+        // the states in front of segments 1 .. NS - 1 (forward) and NS - 2 .. 0 (backward)
+        nu = fwd ? (a.NS - 1) * CQ : max(a.QW - CQ, 0);
+        off = static_cast<uint32_t>(line) * rowb + (fwd ? 0u : rowb - QB);
+        ustep = fwd ? QB : 0u - QB;
+    } else {
+        nu = a.QH;
+        off = static_cast<uint32_t>(line) * QB + (fwd ? 0u : (a.QH - 1) * rowb);
+        ustep = fwd ? rowb : 0u - rowb;
+    }
+    if (nu <= 0) return;
+    // the two steps' words of a unit, and the two steps' r as a unit (vertical
+    // units are quads, diagonal ones [A0, A1, B0, B1])
+    const uint32_t s_lo = KIND == kHor ? kSelCol0 : kSelRow0;
+    const uint32_t s_hi = KIND == kHor ? kSelCol1 : (KIND == kVer ? kSelRow1 : (kd == 0 ? kSelNext : kSelPrev));
+    const uint32_t sel0 = fwd ? s_lo : s_hi, sel1 = fwd ? s_hi : s_lo;
+    const uint32_t selq = KIND == kVer ? (fwd ? 0x6420u : 0x2064u) : (fwd ? 0x6240u : 0x2604u);
+    uint8_t* const src = a.rec + 16 * lane;
+    uint8_t* const out =
+        a.rec + (KIND == kVer ? 1 : 3 + 2 * kd) * a.FS + (fwd ? 0 : a.FS) + 4 * K * lane;  // stored r
 
-    auto unit = [&](const In& in) {
-        uint32_t first[K];    // kStore: L of the unit's first step
-        uint32_t dfirst = 0;  // kWta: disparities of the first step
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            uint32_t m[K];
-#pragma unroll
-            for (int j = 0; j < K; ++j) m[j] = __byte_perm(in.mc[j], 0u, sel.un[t]);
-            ch.step(m, a.P1x2, a.P2x2);
-            if constexpr (MODE == kStore) {
-                if (t == 0) {
-#pragma unroll
-                    for (int j = 0; j < K; ++j) first[j] = ch.w[j];
-                } else {
-                    uint32_t q[K];
-#pragma unroll
-                    for (int j = 0; j < K; ++j) q[j] = __byte_perm(first[j], ch.w[j], sel.cq);
-                    stv_checked<K, kHintLStore>(a, at(bs.out, off_cur), q, 105);
-                }
-            } else {  // kWta (horizontal)
-                uint32_t S[K];
-#pragma unroll
-                for (int j = 0; j < K; ++j) S[j] = ch.w[j] + stored3<S8>(in.o[j], in.v0[j], in.v1[j], sel.un[t]);
-                const uint32_t dd = wta2<K, D, KEY16>(S, dc);
-                if constexpr (DBG) {
-                    const int x = 2 * qc + (t == 0 ? sel.h0 : 1 - sel.h0), y0 = 2 * wk.r;
-                    if (x < a.W) {
-#pragma unroll
-                        for (int j = 0; j < K; ++j) {
-                            const size_t d = static_cast<size_t>(K * lane + j);
-                            if (y0 < a.H) sdbg_store(a, (static_cast<size_t>(y0) * a.W + x) * D + d, S[j] & 0xffffu, 106);
-                            if (y0 + 1 < a.H)
-                                sdbg_store(a, (static_cast<size_t>(y0 + 1) * a.W + x) * D + d, S[j] >> 16, 106);
-                        }
-                    }
-                }
-                if (t == 0) {
-                    dfirst = dd;
-                } else if (lane == 0) {
-                    raw_quad_store(a, static_cast<size_t>(wk.r) * a.QW + qc, __byte_perm(dfirst, dd, sel.cq), 107);
+    // Diagonals read quads qa and qb of every unit, both one column further in
+    // every row, kd = 0: qb = qa + 1, kd = 1: qb = qa - 1.  Around the rows' end
+    // one of them wraps a unit before the other: forward walks qb first, then
+    // qa; backward walks qa, then qb.  ld_n / cp_n count the units up to the
+    // first of the two for the unit being loaded / computed.
+    uint32_t off_a = off, off_b = 0, lstep = ustep, wrap = 0, keep1 = 0;
+    int ld_n = 0, cp_n = 0;
+    if constexpr (KIND == kDiag) {
+        const int j0 = fwd ? 0 : a.QH - 1, jm = j0 % a.QW;
+        const bool right = (kd == 0) == fwd;  // the walk moves right
+        int qa = kd == 0 ? line + jm : line - jm;
+        qa = qa >= a.QW ? qa - a.QW : (qa < 0 ? qa + a.QW : qa);
+        off_a = static_cast<uint32_t>(j0) * rowb + static_cast<uint32_t>(qa) * QB;
+        lstep = ustep + (right ? QB : 0u - QB);
+        wrap = right ? 0u - rowb : rowb;
+        if (fwd) {
+            ld_n = right ? a.QW - 1 - qa : qa;
+            off_b = off_a + (right ? QB : 0u - QB);  // past the row's end where n = 0: wraps in that unit
+        } else {
+            ld_n = right ? (a.QW - qa) % a.QW : (qa + 1) % a.QW;
+            const int qb = kd == 0 ? (qa + 1 == a.QW ? 0 : qa + 1) : (qa == 0 ? a.QW - 1 : qa - 1);
+            off_b = off_a + static_cast<uint32_t>(qb - qa) * QB;
+            if (ld_n == 0) off_a -= wrap;  // the first unit adds it
+        }
+        if (a.QW == 1) {  // one quad per row: never past its end
+            off_a = off_b = static_cast<uint32_t>(j0) * rowb;
+            lstep = ustep;
+            wrap = 0u;
+        }
+        cp_n = ld_n;
+        // the line that goes on at the first wrap: forward, in the unit's second
+        // step (kd = 0: line A, 1: line B); backward, in its first step (kd = 0:
+        // line B, 1: line A); the other line's path starts one step later
+        keep1 = right ? 0x0000ffffu : 0xffff0000u;
+    }
+    const uint32_t sdst = ring + 16 * lane, ssrc = ring + 4 * K * lane;
+    auto issue = [&](int slot, bool near) {
+        if constexpr (KIND == kDiag) {
+            if (near) {  // forward: qb wraps at n = 0, qa one unit later; backward: qa, then qb
+                if (ld_n == 0) (fwd ? off_b : off_a) += wrap;
+                if (ld_n < 0) {
+                    (fwd ? off_a : off_b) += wrap;
+                    ld_n = a.QW - 1;
                 }
             }
+            cp_unit<D>(a, sdst + slot, src, off_a, 101);
+            cp_unit<D>(a, sdst + slot + 4 * D, src, off_b, 102);
+            off_b += lstep;
+            --ld_n;
+        } else {
+            cp_unit<D>(a, sdst + slot, src, off_a, 103);
         }
-        off_cur += wk.dstride;
-        qc += wk.dqc;
+        off_a += lstep;
+    };
+    // a unit's costs from its slot
+    constexpr int KB = KIND == kDiag ? K : 1;
+    struct Cost {
+        uint32_t a[K], b[KB];
+    };
+    auto read = [&](int slot, Cost& c) {
+        lds_unit<K>(ssrc + slot, c.a);
+        if constexpr (KIND == kDiag) lds_unit<K>(ssrc + slot + 4 * D, c.b);
+    };
+    auto words = [&](const Cost& c, uint32_t sel, uint32_t (&m)[K]) {
+#pragma unroll
+        for (int j = 0; j < K; ++j) m[j] = prmt(c.a[j], KIND == kDiag ? c.b[j < KB ? j : 0] : 0u, sel);
+    };
+    // jump penalties (AP2): lane l holds the word of unit 32 b + l, one batch ahead
+    uint32_t p2c = 0, p2n = 0;
+    const size_t units = static_cast<size_t>(a.QW) * a.QH;
+    int p2i = 0, p2s = 0;
+    const uint32_t* p2m = nullptr;
+    auto p2_load = [&](int k) -> uint32_t {
+        const int i = p2i + min(k, nu - 1) * p2s;
+        return SGM_GUARD_INDEX(i, static_cast<long long>(units), 104) ? __ldg(p2m + i) : 0u;
+    };
+    if constexpr (AP2) {
+        const int m = (KIND == kHor ? 0 : (KIND == kVer ? 2 : 4 + 2 * kd)) + (fwd ? 0 : 1);
+        p2m = a.p2map + m * units;
+        p2i = KIND == kHor ? line * a.QW + (fwd ? 0 : a.QW - 1) : line + (fwd ? 0 : (a.QH - 1) * a.QW);
+        p2s = (KIND == kHor ? 1 : a.QW) * (fwd ? 1 : -1);
+        p2n = p2_load(lane);
+    }
+    // selectors of the penalties (up to 255) in the order of the steps
+    const uint32_t p_lo = KIND == kVer ? 0x4140u : 0x4240u, p_hi = KIND == kVer ? 0x4342u : 0x4341u;
+    const uint32_t psel0 = fwd ? p_lo : p_hi, psel1 = fwd ? p_hi : p_lo;
+
+    Chain2<K> ch;
+    ch.init(lane);
+    // one unit; `near`: a diagonal's lines may start a path in it
+    auto unit = [&](const Cost& cur, int k, bool near) {
+        uint32_t pa = a.P2x2, pb = a.P2x2;
+        if constexpr (AP2) {
+            if ((k & 31) == 0) {
+                p2c = p2n;
+                p2n = p2_load(k + 32 + lane);
+            }
+            const uint32_t p = __shfl_sync(kFull, p2c, k & 31);
+            pa = __byte_perm(p, 0u, psel0);
+            pb = __byte_perm(p, 0u, psel1);
+        }
+        uint32_t m[K];
+        words(cur, sel0, m);
+        if constexpr (KIND == kHor) {
+            ch.step_raw(m, a.P1x2, pa);
+            words(cur, sel1, m);
+            ch.step_raw(m, a.P1x2, pb);
+        } else {
+            uint32_t r0[K], r1[K];
+            if (KIND == kDiag && near) {
+                if (a.QW == 1 || (fwd ? cp_n < 0 : cp_n == 0)) ch.restart(fwd ? ~keep1 : keep1);
+            }
+            ch.step(m, a.P1x2, pa, r0);
+            if (KIND == kDiag && near) {
+                if (a.QW == 1 || cp_n == 0) ch.restart(fwd ? keep1 : ~keep1);
+                if (cp_n < 0) cp_n = a.QW - 1;
+            }
+            words(cur, sel1, m);
+            ch.step(m, a.P1x2, pb, r1);
+#pragma unroll
+            for (int j = 0; j < K; ++j) r0[j] = prmt(r0[j], r1[j], selq);
+            stg_unit<K>(a, at(out, off), r0, 106);
+            off += ustep;
+            if constexpr (KIND == kDiag) --cp_n;
+        }
+    };
+    // horizontal: the state after unit k, where a segment ends
+    auto segment_end = [&](int k) {
+        const int q = fwd ? k : a.QW - 1 - k;
+        if ((q & (CQ - 1)) == (fwd ? CQ - 1 : 0)) {
+            ch.rebase();
+            uint32_t* st = state_slot<D>(a, fwd ? 0 : 1, line, fwd ? q / CQ + 1 : q / CQ - 1);
+            if (state_ok<D>(a, st, 105)) ch.save(st);
+        }
     };
 
-    In buf[PU];
-#pragma unroll
-    for (int i = 0; i < PU; ++i) {
-        if (i < nu) load(buf[i], off_ld);
-        off_ld += wk.dstride;
+    // backward row walks start inside a group of kUnroll columns: the first slot
+    // is chosen so that groups of slots and of columns end together
+    const int s0 = KIND == kHor && !fwd ? (kUnroll - a.QW % kUnroll) % kUnroll : 0;
+    int slot = s0 * SB;
+#pragma unroll 1
+    for (int i = 0; i < DEPTH; ++i) {
+        const int si = s0 + i < DEPTH ? s0 + i : s0 + i - DEPTH;
+        if (i < nu) issue(si * SB, true);
+        cp_commit();
     }
-    for (int k0 = 0;; k0 += PU) {
-#pragma unroll
-        for (int i = 0; i < PU; ++i) {
-            if (k0 + i >= nu) return;
-            unit(buf[i]);
-            if (k0 + i + PU < nu) load(buf[i], off_ld);  // refill with unit k0 + i + PU
-            off_ld += wk.dstride;
+    Cost cur, nxt;
+    cp_wait<DEPTH - 1>();
+    read(slot, cur);
+    // every unit: the next unit's costs into registers, its slot refilled, then its two steps
+#pragma unroll 1
+    for (int k = 0; k < nu;) {
+        // groups of kUnroll units that need no care: refills in range, no path starts
+        int groups = 0;
+        if (slot % (kUnroll * SB) == 0) {
+            int n = nu - DEPTH - k;
+            if constexpr (KIND == kDiag) n = min(n, min(ld_n, cp_n));
+            groups = n / kUnroll;
         }
-    }
-}
-
-// The two warps of a block (the two directions of one line pair).
-__device__ __forceinline__ void pair_sync() {
-    __threadfence_block();
-    asm volatile("bar.sync 1, 64;" ::: "memory");
-}
-
-// Horizontal chain state between the launches: the K words and m of each lane.
-template <int K>
-__device__ __forceinline__ uint32_t* state_slot(const PairsArgs& a, int r, int dir) {
-    return a.state + ((static_cast<size_t>(r) * 2 + dir) * 32 + (threadIdx.x & 31)) * (K + 1);
-}
-
-// A lane's 4 K bytes of every quad sit at 4 K lane in each field array.
-template <int D>
-__device__ __forceinline__ Bases lane_bases(const PairsArgs& a, int out_field, int o_field = kMC) {
-    constexpr int K = D / 32;
-    uint8_t* const l = a.rec + 4 * K * (threadIdx.x & 31);
-    return Bases{l, l + out_field * a.FS, l + o_field * a.FS, l + kLVT * a.FS, l + kLVB * a.FS};
-}
-
-// Launch 1: every walker stores its own L_r.  Blocks alternate between
-// vertical line pairs (warp 0 top-to-bottom, warp 1 bottom-to-top, every row)
-// and horizontal line pairs (warp 0 left-to-right over columns [0, n1),
-// warp 1 right-to-left over [W2 - n1, W2)) while both last.
-template <int D>
-__global__ void __launch_bounds__(64) pairs_stage1_kernel(const __grid_constant__ PairsArgs a) {
-    constexpr int K = D / 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = blockIdx.x, nmin = min(a.nvb, a.nhb);
-    bool vert;
-    int idx;
-    if (b < 2 * nmin) {
-        vert = (b & 1) == 0;
-        idx = b >> 1;
-    } else {
-        vert = a.nvb > a.nhb;
-        idx = b - nmin;
-    }
-    Chain2<K> ch;
-    ch.init(lane);
-    const uint32_t QB = static_cast<uint32_t>(a.QB);
-    if (vert) {
-        const int c = idx;  // columns 2c, 2c + 1
-        const uint32_t us = static_cast<uint32_t>(a.QW) * QB, off0 = static_cast<uint32_t>(c) * QB;
-        const bool down = warp == 0;
-        walk<D, kStore>(ch, a, lane_bases<D>(a, down ? kLVT : kLVB),
-                        down ? Walk{off0, us, a.QH, 0, 0, 0} : Walk{off0 + (a.QH - 1) * us, 0u - us, a.QH, 0, 0, 0},
-                        walk_sel(true, down));
-    } else {
-        const int r = idx;  // rows 2r, 2r + 1
-        const uint32_t off0 = static_cast<uint32_t>(r) * a.QW * QB;
-        const int n = a.n1 / 2;
-        const bool right = warp == 0;  // warp 0 walks left to right, warp 1 right to left
-        walk<D, kStore>(ch, a, lane_bases<D>(a, right ? kLH0 : kLH1),
-                        right ? Walk{off0, QB, n, 0, 0, r} : Walk{off0 + (a.QW - 1) * QB, 0u - QB, n, 0, 0, r},
-                        walk_sel(false, right));
-        if (a.nh2 > 0) {
-            uint32_t* st = state_slot<K>(a, r, warp);
-            if (SGM_GUARD(st, 4 * (K + 1), a.state, a.state + state_words(a), 108)) {
+#pragma unroll 1
+        for (; groups > 0; --groups) {
 #pragma unroll
-                for (int j = 0; j < K; ++j) st[j] = ch.w[j];
-                st[K] = ch.mpx2;
+            for (int i = 0; i < kUnroll; ++i) {
+                const int s = slot + i * SB;
+                cp_wait<DEPTH - 2>();
+                read(i + 1 < kUnroll ? s + SB : (s + SB == DEPTH * SB ? 0 : s + SB), nxt);
+                issue(s, false);
+                cp_commit();
+                unit(cur, k + i, false);
+                cur = nxt;
             }
+            k += kUnroll;
+            slot += kUnroll * SB;
+            if (slot == DEPTH * SB) slot = 0;
+            if constexpr (KIND == kHor) segment_end(k - 1);
+        }
+        if (k < nu) {
+            const int ns = slot + SB == DEPTH * SB ? 0 : slot + SB;
+            cp_wait<DEPTH - 2>();
+            read(ns, nxt);
+            if (k + DEPTH < nu) issue(slot, true);
+            cp_commit();
+            unit(cur, k, true);
+            cur = nxt;
+            if constexpr (KIND == kHor) segment_end(k);
+            ++k;
+            slot = ns;
         }
     }
 }
 
-// Launch 2a: the rest of the horizontal pairs, one row pair per block (warp 0
-// left to right, warp 1 right to left), finishing their pixels with Eq. 4.
-// Few warps walk long chains here, so they prefetch deep.
-template <int D, bool S8, bool KEY16, bool DBG>
-__global__ void __launch_bounds__(64) pairs_chain2_kernel(const __grid_constant__ PairsArgs a) {
-    constexpr int K = D / 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t QB = static_cast<uint32_t>(a.QB);
-    const int r = blockIdx.x;
+// The order of the walks' launches (launch_pairs_walks): the first one waits for
+// the costs; a later one starts when every block of the one before has come
+// past that wait, and so needs none, but its last block waits for the end of
+// the one before, so that its own end means both.
+struct Side {
+    int later, trigger;  // not the first launch; another one follows
+    __device__ __forceinline__ void begin() const {
+        if (!later) pdl_wait();
+        if (trigger) pdl_trigger();
+    }
+    __device__ __forceinline__ void end() const {
+        if (later && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1) pdl_wait();
+    }
+};
+
+// The walks: one chain per warp.  Chains [0, nh) are horizontal line pairs
+// (row pair c / nd, direction c % nd), [nh, nh + nv) vertical ones, nd
+// directions each (1 with 2 paths).
+template <int D, bool AP2>
+__global__ void __launch_bounds__(64) walk_hv_kernel(const __grid_constant__ PairsJobs f, int nh, int nv, Side side) {
+    __shared__ __align__(16) uint8_t ring[2][ring_bytes<D>()];
+    side.begin();
+    const int warp = threadIdx.x >> 5;
+    const PairsArgs& a = f.job[blockIdx.y];
+    const uint32_t r = static_cast<uint32_t>(__cvta_generic_to_shared(ring[warp]));
+    const int nd = a.n_paths == 2 ? 1 : 2, c = blockIdx.x * 2 + warp, v = c - nh;
+    if (c < nh)
+        walk<D, kHor, AP2>(a, c / nd, 0, c % nd == 0, r);
+    else if (v < nv)
+        walk<D, kVer, AP2>(a, v / nd, 0, v % nd == 0, r);
+    side.end();
+}
+
+// Diagonal line pairs (8 paths): chain c is line pair c / 4, line set (c / 2) % 2, direction c % 2.
+template <int D, bool AP2>
+__global__ void __launch_bounds__(64) walk_d_kernel(const __grid_constant__ PairsJobs f, Side side) {
+    __shared__ __align__(16) uint8_t ring[2][ring_bytes<D>()];
+    side.begin();
+    const int warp = threadIdx.x >> 5;
+    const PairsArgs& a = f.job[blockIdx.y];
+    const uint32_t r = static_cast<uint32_t>(__cvta_generic_to_shared(ring[warp]));
+    const int c = blockIdx.x * 2 + warp;
+    if (c < 4 * a.QW) walk<D, kDiag, AP2>(a, c / 4, (c / 2) % 2, c % 2 == 0, r);
+    side.end();
+}
+
+// ---------------------------------------------------------------------------
+// Finish: one segment (CQ quads) of a row pair per warp.  The segment's costs
+// come into shared memory; left to right from the stored state, each step's r
+// is kept there too; then right to left, adding everything and taking the
+// winner (2 paths have no second walk: the first one finishes).  The stored r
+// of the other directions come a quad ahead straight into registers, so that
+// their reads are spread over the walk and shared memory allows 28 warps per
+// SM (all of them loaded up front let every warp of a wave wait, then compute,
+// in step: 31 us for a 640x480 D=128 frame).  S = own r + n MC + the r of the
+// other n - 1 directions.  GS r may be added in a byte: GS P2 <= 255.  K16:
+// S D + d fits 16 bits, so that one packed minimum serves both lines.
+// ---------------------------------------------------------------------------
+template <int D, int NP>
+struct Finish {
+    static constexpr int UB = 4 * D, CQ = seg_quads(D);
+    static constexpr int NV = NP == 2 ? 1 : 2, NF = NV + (NP == 8 ? 4 : 0);  // stored r of a quad
+    static constexpr int KEPT = CQ * UB, BYTES = KEPT + (NP == 2 ? 0 : CQ * UB);
+};
+
+template <int D, int NP, int GS, bool K16, bool POST>
+__device__ __forceinline__ void finish(const PairsArgs& a, int r, int s, uint32_t smem) {
+    using F = Finish<D, NP>;
+    constexpr int K = D / 32, UB = F::UB, CQ = F::CQ, NV = F::NV, NF = F::NF;
+    constexpr bool DIAG = NP == 8;
+    const int lane = threadIdx.x & 31;
+    const int q0 = s * CQ, nq = min(CQ, a.QW - q0);
+    const uint32_t QB = static_cast<uint32_t>(a.QB), rowoff = static_cast<uint32_t>(r) * a.QW * QB;
+    const uint32_t off0 = rowoff + static_cast<uint32_t>(q0) * QB;
+    const uint32_t ssrc = smem + 4 * K * lane;
+    const uint32_t m256 = opaque(0xffffff00u), k256 = opaque(256u), k16 = opaque(0x10000u);
+    const uint64_t pol = last_read();
+#pragma unroll
+    for (int i = 0; i < CQ; ++i)
+        if (i < nq) cp_unit<D, true>(a, smem + 16 * lane + i * UB, a.rec + 16 * lane, off0 + i * UB, 111, pol);
+    cp_commit();
+
+    // the states in front of this segment, and its jump penalties
     Chain2<K> ch;
     ch.init(lane);
-    {
-        const uint32_t* st = state_slot<K>(a, r, warp);
-        if (SGM_GUARD(st, 4 * (K + 1), a.state, a.state + state_words(a), 109)) {
+    constexpr int CW = Chain2<K>::CW;
+    uint32_t cl[CW], cr[CW];
 #pragma unroll
-            for (int j = 0; j < K; ++j) ch.w[j] = __ldcg(st + j);
-            ch.mpx2 = __ldcg(st + K);
+    for (int i = 0; i < CW; ++i) cl[i] = cr[i] = 0u;
+    if (s > 0) {
+        const uint32_t* st = state_slot<D>(a, 0, r, s);
+        if (state_ok<D>(a, st, 114))
+#pragma unroll
+            for (int i = 0; i < CW; ++i) cl[i] = __ldcg(st + 32 * i);
+    }
+    if (NP > 2 && s + 1 < a.NS) {
+        const uint32_t* st = state_slot<D>(a, 1, r, s);
+        if (state_ok<D>(a, st, 115))
+#pragma unroll
+            for (int i = 0; i < CW; ++i) cr[i] = __ldcg(st + 32 * i);
+    }
+    uint32_t p2l = 0, p2r = 0;
+    if constexpr (POST) {
+        if (a.p2map) {
+            const size_t i = static_cast<size_t>(r) * a.QW + q0 + min(lane, nq - 1);
+            p2l = __ldg(a.p2map + i);
+            if (NP > 2) p2r = __ldg(a.p2map + static_cast<size_t>(a.QW) * a.QH + i);
         }
-        ch.exchange();
     }
-    const uint32_t off0 = static_cast<uint32_t>(r) * a.QW * QB;
-    const int n1u = a.n1 / 2, au = a.a / 2, bu = a.b / 2, ru = (a.W2 - a.n1) / 2;
-    const bool right = warp == 0;
-    const Sel sel = walk_sel(false, right);
-    walk<D, kStore>(ch, a, lane_bases<D>(a, right ? kLH0 : kLH1),
-                    right ? Walk{off0 + n1u * QB, QB, au - n1u, 0, 0, r}
-                          : Walk{off0 + (ru - 1) * QB, 0u - QB, ru - bu, 0, 0, r},
-                    sel);
-    // when the pair meets in the middle each direction stores columns the other
-    // finishes in this launch (also when a == n1: then only right to left does)
-    if (a.W2 > 2 * a.n1) pair_sync();
-    walk<D, kWta, S8, KEY16, DBG, kChainPrefetchRegs>(ch, a, lane_bases<D>(a, kMC, right ? kLH1 : kLH0),
-                                                      right ? Walk{off0 + au * QB, QB, a.QW - au, au, 1, r}
-                                                            : Walk{off0 + (bu - 1) * QB, 0u - QB, bu, bu - 1, -1, r},
-                                                      sel);
-}
+    auto p2_at = [&](uint32_t words, int i, uint32_t sel) -> uint32_t {
+        if constexpr (POST) {
+            const uint32_t p = __shfl_sync(kFull, words, i);
+            return a.p2map ? __byte_perm(p, 0u, sel) : a.P2x2;
+        } else {
+            return a.P2x2;
+        }
+    };
 
-// Launch 2b (beside 2a): the winner-take-all of the quads in columns [b, a),
-// which both horizontal directions passed in launch 1.  Each warp takes
-// kParItems quads and issues all their loads before the first sum, so many
-// quads are in flight.
-template <int D, bool S8, bool KEY16, bool DBG>
-__global__ void __launch_bounds__(64) pairs_par_kernel(const __grid_constant__ PairsArgs a) {
-    constexpr int K = D / 32, NI = kParItems;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cols = (a.a - a.b) / 2, items = cols * a.QH;
-    uint32_t dc[K];
-    wta_dconst<K, KEY16>(lane, dc);
-    const int lb = 4 * K * lane;
-    const int it0 = (blockIdx.x * 2 + warp) * NI;
-    uint32_t l0[NI][K], l1[NI][K], v0[NI][K], v1[NI][K];
-#pragma unroll
-    for (int n = 0; n < NI; ++n) {
-        const int it = min(it0 + n, items - 1);  // past the end: re-read the last quad
-        const uint8_t* q = a.rec + (static_cast<size_t>(it / cols) * a.QW + a.b / 2 + it % cols) * a.QB + lb;
-        ldv_checked<K, kHintLLoad>(a, q + kLH0 * a.FS, l0[n], 110);
-        ldv_checked<K, kHintLLoad>(a, q + kLH1 * a.FS, l1[n], 110);
-        ldv_checked<K, kHintLLoad>(a, q + kLVT * a.FS, v0[n], 110);
-        ldv_checked<K, kHintLLoad>(a, q + kLVB * a.FS, v1[n], 110);
+    // stored r, in the order of the finishing walk.  Diagonal units are shared
+    // by the two quads of a row that a line pair crosses: fv holds the one a
+    // quad shares with its left neighbour, `carry` the one it shares with the
+    // right, so each is read once, starting one quad past the segment.
+    uint32_t fv[NF][K];
+    uint8_t* const base = a.rec + 4 * K * lane;
+    int up = 0, um = 0;  // next units of the right- and left-moving lines
+    if constexpr (DIAG) {
+        const int rm = r % a.QW;
+        up = q0 + nq - 1 - rm;
+        up = up < 0 ? up + a.QW : up;
+        um = q0 + nq + rm;
+        um = um >= a.QW ? um - a.QW : um;
+        um = um >= a.QW ? um - a.QW : um;
     }
+    auto load_v = [&](int i) {
 #pragma unroll
-    for (int n = 0; n < NI; ++n) {
-        const int it = it0 + n;
-        if (it >= items) return;
-        const int r = it / cols, qx = a.b / 2 + it % cols;
-        uint32_t dd[2];
+        for (int v = 0; v < NV; ++v) ldg_unit<K>(a, at(base + (1 + v) * a.FS, off0 + i * QB), fv[v], pol, 112);
+    };
+    auto load_d = [&]() {
+        if constexpr (DIAG) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {  // rows 2r and 2r + 1
-            uint32_t S[K];
+            for (int v = 0; v < 4; ++v)
+                ldg_unit<K>(a, at(base + (3 + v) * a.FS, rowoff + static_cast<uint32_t>(v < 2 ? up : um) * QB),
+                            fv[NF - 4 + v], pol, 113);
+            up = up == 0 ? a.QW - 1 : up - 1;
+            um = um == 0 ? a.QW - 1 : um - 1;
+        }
+    };
+    load_v(NP == 2 ? 0 : nq - 1);
+    load_d();
+
+    ch.restore(cl);
+    cp_wait<0>();
+    if constexpr (NP > 2) {
+#pragma unroll 1
+        for (int i = 0; i < nq; ++i) {
+            uint32_t mc[K], lo[K], hi[K], r0[K], r1[K];
+            lds_unit<K>(ssrc + i * UB, mc);
+#pragma unroll
+            for (int j = 0; j < K; ++j) split(mc[j], m256, lo[j], hi[j]);
+            ch.step(lo, a.P1x2, p2_at(p2l, i, 0x4240u), r0);
+            ch.step(hi, a.P1x2, p2_at(p2l, i, 0x4341u), r1);
+#pragma unroll
+            for (int j = 0; j < K; ++j) r0[j] = mad(r1[j], k256, r0[j]);
+            sts_unit<K>(ssrc + F::KEPT + i * UB, r0);
+        }
+        ch.restore(cr);
+    }
+
+    // groups of r that add in bytes: the kept and the vertical ones, then each line set's
+    constexpr int NB = NP == 2 ? 1 : (GS == 3 ? 1 : (GS == 2 ? 2 : 3)), NC = GS >= 2 ? 1 : 2;
+    constexpr int NG = NB + (DIAG ? 2 * NC : 0);
+    uint32_t carry[2][NC][K];
+    auto diag_sums = [&](uint32_t (&u)[2][NC][K]) {
+#pragma unroll
+        for (int l = 0; l < 2; ++l)
 #pragma unroll
             for (int j = 0; j < K; ++j) {
-                if constexpr (S8)  // pairs of stored costs in a byte: each pair <= 2 (MC_max + P2) <= 255
-                    S[j] = unq<true>(l0[n][j] + l1[n][j], h) + unq<true>(v0[n][j] + v1[n][j], h);
-                else
-                    S[j] = unq<true>(l0[n][j], h) + unq<true>(l1[n][j], h) + unq<true>(v0[n][j], h) +
-                           unq<true>(v1[n][j], h);
+                const uint32_t x = fv[NF - 4 + 2 * l][j], y = fv[NF - 3 + 2 * l][j];
+                if constexpr (GS >= 2) {
+                    u[l][0][j] = x + y;
+                } else {
+                    u[l][0][j] = x;
+                    u[l][NC - 1][j] = y;
+                }
             }
-            dd[h] = wta2<K, D, KEY16>(S, dc);
-            if constexpr (DBG) {
-                const int y = 2 * r + h;
-                if (y < a.H) {
+    };
+    if constexpr (DIAG) {
+        diag_sums(carry);
+        load_d();
+    }
+    uint32_t rawv = 0;
+#pragma unroll 1
+    for (int n = 0; n < nq; ++n) {
+        const int i = NP == 2 ? n : nq - 1 - n;
+        uint32_t mc[K], g[NG][K], mlo[K], mhi[K];
+        lds_unit<K>(ssrc + i * UB, mc);
+        if constexpr (NP == 2) {
 #pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        const int x = 2 * qx + i;
-                        if (x >= a.W) continue;
+            for (int j = 0; j < K; ++j) g[0][j] = fv[0][j];
+        } else {
+            uint32_t kept[K];
+            lds_unit<K>(ssrc + F::KEPT + i * UB, kept);
 #pragma unroll
-                        for (int j = 0; j < K; ++j)
-                            sdbg_store(a, (static_cast<size_t>(y) * a.W + x) * D + K * lane + j,
-                                       i ? (S[j] >> 16) : (S[j] & 0xffffu), 111);
+            for (int j = 0; j < K; ++j) {
+                if constexpr (GS == 3) {
+                    g[0][j] = fv[0][j] + fv[1][j] + kept[j];
+                } else if constexpr (GS == 2) {
+                    g[0][j] = fv[0][j] + fv[1][j];
+                    g[1][j] = kept[j];
+                } else {
+                    g[0][j] = fv[0][j];
+                    g[1][j] = fv[1][j];
+                    g[2][j] = kept[j];
+                }
+            }
+        }
+        if constexpr (DIAG) {
+            uint32_t u[2][NC][K];
+            diag_sums(u);
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+#pragma unroll
+                for (int j = 0; j < K; ++j) {
+                    // units hold [A0, A1, B0, B1]; a quad [A0, B0, row 1 of the two lines crossing it]
+                    g[NB + c][j] = __byte_perm(carry[0][c][j], u[0][c][j], 0x1720u);
+                    g[NB + NC + c][j] = __byte_perm(u[1][c][j], carry[1][c][j], 0x5320u);
+                    carry[0][c][j] = u[0][c][j];
+                    carry[1][c][j] = u[1][c][j];
+                }
+        }
+        if (n + 1 < nq) {
+            load_v(NP == 2 ? i + 1 : i - 1);
+            load_d();
+        }
+#pragma unroll
+        for (int j = 0; j < K; ++j) split(mc[j], m256, mlo[j], mhi[j]);
+        // sums of the other directions' r, both columns
+        uint32_t slo[K], shi[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            split(g[0][j], m256, slo[j], shi[j]);
+#pragma unroll
+            for (int q = 1; q < NG; ++q) {
+                uint32_t e, o;
+                split(g[q][j], m256, e, o);
+                slo[j] += e;
+                shi[j] += o;
+            }
+        }
+        uint32_t word = 0;
+        uint4 subv = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int h = NP == 2 ? t : 1 - t;  // column of the quad
+            uint32_t S[K];
+            ch.step(h ? mhi : mlo, a.P1x2, p2_at(NP == 2 ? p2l : p2r, i, h ? 0x4341u : 0x4240u), S);
+#pragma unroll
+            for (int j = 0; j < K; ++j) S[j] = mad(h ? mhi[j] : mlo[j], NP, S[j]) + (h ? shi[j] : slo[j]);
+            // the smallest S, then the lowest d, of both lines
+            uint32_t dd, kA = 0xffffffffu, kB = 0xffffffffu;
+            if constexpr (K16) {
+                uint32_t key[K];
+#pragma unroll
+                for (int j = 0; j < K; ++j)
+                    key[j] = mad(S[j], D, static_cast<uint32_t>(K * lane + j) * 0x10001u);
+                uint32_t best = key[0];
+#pragma unroll
+                for (int j = 1; j + 1 < K; j += 2) best = vmin3(best, key[j], key[j + 1]);
+                if constexpr (K % 2 == 0) best = vmin2(best, key[K - 1]);
+                kB = __reduce_min_sync(kFull, best);
+                kA = __reduce_min_sync(kFull, mad(best, k16, 0u));
+                dd = __byte_perm(kA, kB, 0x7632u);
+                if constexpr ((D & (D - 1)) == 0)
+                    dd &= static_cast<uint32_t>(D - 1) * 0x10001u;
+                else
+                    dd = ((dd & 0xffffu) % static_cast<uint32_t>(D)) | (((dd >> 16) % static_cast<uint32_t>(D)) << 16);
+            } else {  // 32-bit keys S << 16 | d
+#pragma unroll
+                for (int j = 0; j < K; ++j) {
+                    const uint32_t d = static_cast<uint32_t>(K * lane + j);
+                    kA = min(kA, mad(S[j], k16, d));
+                    kB = min(kB, (S[j] & 0xffff0000u) | d);
+                }
+                kA = __reduce_min_sync(kFull, kA);
+                kB = __reduce_min_sync(kFull, kB);
+                dd = prmt(kA, kB, 0x5410u) & 0x00ff00ffu;
+            }
+            word |= dd << (8 * h);
+            if (POST && a.Sdbg) {  // debug: natural-order S
+                const int x = 2 * (q0 + i) + h, y = 2 * r;
+                if (x < a.W) {
+#pragma unroll
+                    for (int j = 0; j < K; ++j) {
+                        const size_t d = static_cast<size_t>(K * lane + j);
+                        const size_t p = (static_cast<size_t>(y) * a.W + x) * D + d;
+                        a.Sdbg[p] = static_cast<uint16_t>(S[j] & 0xffffu);
+                        if (y + 1 < a.H) a.Sdbg[p + static_cast<size_t>(a.W) * D] = static_cast<uint16_t>(S[j] >> 16);
+                    }
+                }
+            }
+            if constexpr (POST) {
+                if (a.subq) {  // S(d-1) - S(d) | (S(d+1) - S(d)) << 16 at each line's winner
+                    auto s_at = [&](int e, int half) -> uint32_t {
+                        const int l = e / K, jj = e - l * K;
+                        uint32_t w = S[0];
+#pragma unroll
+                        for (int j = 1; j < K; ++j) w = jj == j ? S[j] : w;
+                        w = __shfl_sync(kFull, w, l);
+                        return half ? w >> 16 : w & 0xffffu;
+                    };
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        const uint32_t key = half ? kB : kA, Sd = key >> 16;
+                        const int d = static_cast<int>(key & 0xffu);
+                        const uint32_t al = d > 0 ? s_at(d - 1, half) - Sd : 0u;
+                        const uint32_t ga = d + 1 < D ? s_at(d + 1, half) - Sd : 0u;
+                        const uint32_t v = al | ga << 16;
+                        if (half)
+                            (h ? subv.w : subv.z) = v;
+                        else
+                            (h ? subv.y : subv.x) = v;
                     }
                 }
             }
         }
-        if (lane == 0) raw_quad_store(a, static_cast<size_t>(r) * a.QW + qx, __byte_perm(dd[0], dd[1], 0x6420u), 112);
+        rawv = lane == i ? word : rawv;
+        if constexpr (POST) {
+            const size_t q = static_cast<size_t>(r) * a.QW + q0 + i;
+            if (a.subq && lane == 0 && SGM_GUARD_INDEX(static_cast<long long>(q), static_cast<long long>(a.QW) * a.QH, 117))
+                reinterpret_cast<uint4*>(a.subq)[q] = subv;
+        }
     }
+    const size_t q = static_cast<size_t>(r) * a.QW + q0 + lane;
+    if (lane < nq && SGM_GUARD_INDEX(static_cast<long long>(q), static_cast<long long>(a.QW) * a.QH, 116))
+        reinterpret_cast<uint32_t*>(a.rawq)[q] = rawv;
+}
+
+template <int D, int NP, int GS, bool K16, bool POST>
+__global__ void __launch_bounds__(64) finish_kernel(const __grid_constant__ PairsJobs f) {
+    __shared__ __align__(16) uint8_t smem[2][Finish<D, NP>::BYTES];
+    pdl_wait();
+    const int warp = threadIdx.x >> 5;
+    const PairsArgs& a = f.job[blockIdx.z];
+    const int r = blockIdx.y * 2 + warp;  // two row pairs
+    if (r < a.QH)
+        finish<D, NP, GS, K16, POST>(a, r, blockIdx.x, static_cast<uint32_t>(__cvta_generic_to_shared(smem[warp])));
 }
 
 template <int D>
 struct PairsD {
-    // S * D + d < 2^16 for every sum of 4 paths: 4 (MC_max + P2) * D + D - 1 <= 65535
-    static bool key16(const PairsArgs& a) {
-        const int P2 = static_cast<int>(a.P2x2 & 0xffffu);
-        return 4 * (a.mc_max + P2) * D + D - 1 <= 65535;
-    }
-    static cudaError_t stage1(const PairsArgs& a, cudaStream_t s) {
-        const int grid = a.nvb + a.nhb;
-        if (grid <= 0) return cudaSuccess;
-        pairs_stage1_kernel<D><<<grid, 64, 0, s>>>(a);
+    static cudaError_t walks(const PairsJobs& f, Walks w, Stream s) {
+        const PairsArgs& a = f.job[0];
+        const int nd = a.n_paths == 2 ? 1 : 2;
+        const Side side{w == Walks::kVer || w == Walks::kDiag,
+                        w == Walks::kHor || (w == Walks::kVer && a.n_paths == 8)};
+        if (side.later) s.pdl = true;
+        if (w == Walks::kDiag) {
+            launch(a.p2map ? walk_d_kernel<D, true> : walk_d_kernel<D, false>, dim3(2 * a.QW, f.n), 64, s, f, side);
+        } else {
+            const int nh = w != Walks::kVer && a.NS > 1 ? a.QH * nd : 0, nv = w != Walks::kHor ? a.QW * nd : 0;
+            const dim3 grid(nh + nv > 0 ? (nh + nv + 1) / 2 : 1, f.n);  // images of one segment have no horizontal states
+            launch(a.p2map ? walk_hv_kernel<D, true> : walk_hv_kernel<D, false>, grid, 64, s, f, nh, nv, side);
+        }
         return cudaGetLastError();
     }
-    template <bool S8, bool KEY16>
-    static void chain_t(const PairsArgs& a, cudaStream_t s) {
-        if (a.Sdbg)
-            pairs_chain2_kernel<D, S8, KEY16, true><<<a.nh2, 64, 0, s>>>(a);
+    template <int NP, int GS, bool K16>
+    static void finish_t(const PairsJobs& f, Stream s) {
+        const PairsArgs& a = f.job[0];
+        const dim3 grid(a.NS, (a.QH + 1) / 2, f.n);
+        if (a.p2map || a.subq || a.Sdbg)  // the post form serves the debug sums too
+            launch(finish_kernel<D, NP, GS, false, true>, grid, 64, s, f);
         else
-            pairs_chain2_kernel<D, S8, KEY16, false><<<a.nh2, 64, 0, s>>>(a);
+            launch(finish_kernel<D, NP, GS, K16, false>, grid, 64, s, f);
     }
-    template <bool S8, bool KEY16>
-    static void par_t(const PairsArgs& a, cudaStream_t s) {
-        if (a.Sdbg)
-            pairs_par_kernel<D, S8, KEY16, true><<<a.npw, 64, 0, s>>>(a);
-        else
-            pairs_par_kernel<D, S8, KEY16, false><<<a.npw, 64, 0, s>>>(a);
+    template <int NP>
+    static void finish_np(const PairsJobs& f, Stream s) {
+        const PairsArgs& a = f.job[0];
+        // S <= NP (MC_max + P2): 16-bit keys S D + d where they fit
+        const bool k16 = NP * (a.mc_max + static_cast<int>(a.P2x2 & 0xffffu)) * D + D - 1 <= 65535;
+        if constexpr (NP == 2) {
+            if (k16)
+                finish_t<2, 1, true>(f, s);
+            else
+                finish_t<2, 1, false>(f, s);
+        } else if (a.gs == 3 && k16) {
+            finish_t<NP, 3, true>(f, s);
+        } else if (a.gs >= 2) {
+            finish_t<NP, 2, false>(f, s);
+        } else {
+            finish_t<NP, 1, false>(f, s);
+        }
     }
-    static cudaError_t chain2(const PairsArgs& a, cudaStream_t s) {
-        if (a.nh2 <= 0) return cudaSuccess;
-        const bool k16 = key16(a);
-        if (a.s8 && k16)
-            chain_t<true, true>(a, s);
-        else if (a.s8)
-            chain_t<true, false>(a, s);
-        else if (k16)
-            chain_t<false, true>(a, s);
-        else
-            chain_t<false, false>(a, s);
-        return cudaGetLastError();
-    }
-    static cudaError_t par(const PairsArgs& a, cudaStream_t s) {
-        if (a.npw <= 0) return cudaSuccess;
-        const bool k16 = key16(a);
-        if (a.s8 && k16)
-            par_t<true, true>(a, s);
-        else if (a.s8)
-            par_t<true, false>(a, s);
-        else if (k16)
-            par_t<false, true>(a, s);
-        else
-            par_t<false, false>(a, s);
+    static cudaError_t fin(const PairsJobs& f, Stream s) {
+        switch (f.job[0].n_paths) {
+            case 2: finish_np<2>(f, s); break;
+            case 4: finish_np<4>(f, s); break;
+            default: finish_np<8>(f, s);
+        }
         return cudaGetLastError();
     }
 };
@@ -673,24 +1017,18 @@ struct PairsD {
 // defined in sgm_sweeps_d<D>.cu; internal to the library (not part of the C ABI)
 #define SGM_INTERNAL_P __attribute__((visibility("hidden")))
 template <int D>
-SGM_INTERNAL_P cudaError_t pairs_launch1(const PairsArgs& a, cudaStream_t s);
+SGM_INTERNAL_P cudaError_t pairs_walks(const PairsJobs& f, Walks w, Stream s);
 template <int D>
-SGM_INTERNAL_P cudaError_t pairs_launch_chain2(const PairsArgs& a, cudaStream_t s);
-template <int D>
-SGM_INTERNAL_P cudaError_t pairs_launch_par(const PairsArgs& a, cudaStream_t s);
+SGM_INTERNAL_P cudaError_t pairs_finish(const PairsJobs& f, Stream s);
 
-#define SGM_INSTANTIATE_PAIRS(D)                                                            \
-    template <>                                                                             \
-    SGM_INTERNAL_P cudaError_t pairs_launch1<D>(const PairsArgs& a, cudaStream_t s) {       \
-        return pairs::PairsD<D>::stage1(a, s);                                              \
-    }                                                                                       \
-    template <>                                                                             \
-    SGM_INTERNAL_P cudaError_t pairs_launch_chain2<D>(const PairsArgs& a, cudaStream_t s) { \
-        return pairs::PairsD<D>::chain2(a, s);                                              \
-    }                                                                                       \
-    template <>                                                                             \
-    SGM_INTERNAL_P cudaError_t pairs_launch_par<D>(const PairsArgs& a, cudaStream_t s) {    \
-        return pairs::PairsD<D>::par(a, s);                                                 \
+#define SGM_INSTANTIATE_PAIRS(D)                                                     \
+    template <>                                                                      \
+    SGM_INTERNAL_P cudaError_t pairs_walks<D>(const PairsJobs& f, Walks w, Stream s) { \
+        return pairs::PairsD<D>::walks(f, w, s);                                     \
+    }                                                                                \
+    template <>                                                                      \
+    SGM_INTERNAL_P cudaError_t pairs_finish<D>(const PairsJobs& f, Stream s) {       \
+        return pairs::PairsD<D>::fin(f, s);                                          \
     }
 
 }  // namespace sgm

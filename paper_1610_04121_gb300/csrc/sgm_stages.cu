@@ -81,7 +81,7 @@ __device__ __forceinline__ uint64_t census62_feature(const uint32_t (&win)[7][NC
 template <bool CT>
 __device__ __forceinline__ void census_body(const uint8_t* __restrict__ left, const uint8_t* __restrict__ right,
                                             void* __restrict__ Fb, void* __restrict__ Fm, int W, int H, int bx,
-                                            int by, int bz) {
+                                            int by, int bz, bool mirror = false) {
     using FT = typename std::conditional<CT, uint64_t, uint32_t>::type;
     constexpr int TW = kCtW + 8, TH = kCtH + 6, NS = (TW + kCtT - 1) / kCtT;
     __shared__ uint8_t tile[TH][TW];
@@ -101,7 +101,7 @@ __device__ __forceinline__ void census_body(const uint8_t* __restrict__ left, co
                 const int gy = y0 - 3 + ty;
                 v[h][ty] = (xin && gy >= 0 && gy < H &&
                             SGM_GUARD_INDEX((long long)gy * W + gx, (long long)W * H, 301))
-                               ? __ldg(img + (size_t)gy * W + gx)
+                               ? __ldg(img + (size_t)gy * W + (mirror ? W - 1 - gx : gx))
                                : uint8_t(0);
             }
         }
@@ -149,6 +149,7 @@ __device__ __forceinline__ void census_body(const uint8_t* __restrict__ left, co
 template <bool CT>
 __global__ void __launch_bounds__(kCtT) census_kernel(const uint8_t* __restrict__ left, const uint8_t* __restrict__ right,
                                                       void* __restrict__ Fb, void* __restrict__ Fm, int W, int H) {
+    pdl_wait();
     census_body<CT>(left, right, Fb, Fm, W, H, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
@@ -176,12 +177,35 @@ cudaError_t launch_census_list(const ListLaunch& l, cudaStream_t stream) {
 }
 
 cudaError_t launch_census(const uint8_t* left, const uint8_t* right, void* Fb, void* Fm, int W, int H, bool ct62,
-                          cudaStream_t stream) {
+                          Stream stream) {
     dim3 grid((W + kCtW - 1) / kCtW, (H + kCtH - 1) / kCtH, 2);
     if (ct62)
-        census_kernel<true><<<grid, kCtT, 0, stream>>>(left, right, Fb, Fm, W, H);
+        launch(census_kernel<true>, grid, kCtT, stream, left, right, Fb, Fm, W, H);
     else
-        census_kernel<false><<<grid, kCtT, 0, stream>>>(left, right, Fb, Fm, W, H);
+        launch(census_kernel<false>, grid, kCtT, stream, left, right, Fb, Fm, W, H);
+    return cudaGetLastError();
+}
+
+// The passes of the paired schedule: image z is left, right, and for the
+// right pass of the left-right check the mirrored right and left images (read
+// mirrored here, which saves writing them).
+template <bool CT>
+__global__ void __launch_bounds__(kCtT) census_passes_kernel(const uint8_t* __restrict__ left,
+                                                             const uint8_t* __restrict__ right, uint8_t* F,
+                                                             size_t fstride, int W, int H) {
+    pdl_wait();
+    const int z = blockIdx.z;
+    void* out = F + z * fstride;
+    census_body<CT>(left, right, out, out, W, H, blockIdx.x, blockIdx.y, (z & 1) ^ (z >> 1), z >= 2);
+}
+
+cudaError_t launch_census_passes(const uint8_t* left, const uint8_t* right, void* F, size_t fstride, int n, int W,
+                                 int H, bool ct62, Stream stream) {
+    dim3 grid((W + kCtW - 1) / kCtW, (H + kCtH - 1) / kCtH, n);
+    if (ct62)
+        launch(census_passes_kernel<true>, grid, kCtT, stream, left, right, static_cast<uint8_t*>(F), fstride, W, H);
+    else
+        launch(census_passes_kernel<false>, grid, kCtT, stream, left, right, static_cast<uint8_t*>(F), fstride, W, H);
     return cudaGetLastError();
 }
 
@@ -279,6 +303,7 @@ __device__ __forceinline__ void cost_body(const FT* __restrict__ Fb, const FT* _
 template <int D, class FT>
 __global__ void __launch_bounds__(kMcThreads) cost_kernel(const FT* __restrict__ Fb, const FT* __restrict__ Fm,
                                                           uint8_t* __restrict__ rec, int RB, int W, int H) {
+    pdl_wait();
     cost_body<D, FT>(Fb, Fm, rec, RB, W, H, blockIdx.x, blockIdx.y);
 }
 
@@ -327,19 +352,19 @@ cudaError_t launch_cost_list(const ListLaunch& l, cudaStream_t stream) {
 
 template <int D>
 static cudaError_t launch_cost_t(const void* Fb, const void* Fm, uint8_t* rec, int RB, int W, int H, bool ct62,
-                                 cudaStream_t s) {
+                                 Stream s) {
     const dim3 grid((W + kMcSeg - 1) / kMcSeg, H);
     if (ct62)
-        cost_kernel<D, uint64_t><<<grid, kMcThreads, 0, s>>>(static_cast<const uint64_t*>(Fb),
+        launch(cost_kernel<D, uint64_t>, grid, kMcThreads, s, static_cast<const uint64_t*>(Fb),
                                                              static_cast<const uint64_t*>(Fm), rec, RB, W, H);
     else
-        cost_kernel<D, uint32_t><<<grid, kMcThreads, 0, s>>>(static_cast<const uint32_t*>(Fb),
+        launch(cost_kernel<D, uint32_t>, grid, kMcThreads, s, static_cast<const uint32_t*>(Fb),
                                                              static_cast<const uint32_t*>(Fm), rec, RB, W, H);
     return cudaGetLastError();
 }
 
 cudaError_t launch_cost(const void* Fb, const void* Fm, uint8_t* rec, int RB, int W, int H, int D, bool ct62,
-                        cudaStream_t stream) {
+                        Stream stream) {
     switch (D) {
         case 32: return launch_cost_t<32>(Fb, Fm, rec, RB, W, H, ct62, stream);
         case 64: return launch_cost_t<64>(Fb, Fm, rec, RB, W, H, ct62, stream);
@@ -445,38 +470,89 @@ __device__ __forceinline__ void cost_quads_body(const FT* __restrict__ Fb, const
 }
 
 template <int D, class FT>
-__global__ void __launch_bounds__(kQcThreads) cost_quads_kernel(const FT* __restrict__ Fb, const FT* __restrict__ Fm,
-                                                                uint8_t* __restrict__ mc, int QB, int W, int H) {
-    cost_quads_body<D, FT>(Fb, Fm, mc, QB, W, H, blockIdx.x, blockIdx.y);
+__global__ void __launch_bounds__(kQcThreads) cost_quads_kernel(const uint8_t* __restrict__ F, size_t fstride,
+                                                                uint8_t* __restrict__ mc, size_t mcstride, int QB,
+                                                                int W, int H) {
+    pdl_wait();
+    const uint8_t* Fp = F + 2 * blockIdx.z * fstride;
+    cost_quads_body<D, FT>(reinterpret_cast<const FT*>(Fp), reinterpret_cast<const FT*>(Fp + fstride),
+                           mc + blockIdx.z * mcstride, QB, W, H, blockIdx.x, blockIdx.y);
 }
 
 template <int D>
-static cudaError_t launch_cost_quads_t(const void* Fb, const void* Fm, uint8_t* mc, int QB, int W, int H, bool ct62,
-                                       cudaStream_t s) {
+static cudaError_t launch_cost_quads_t(const void* F, size_t fstride, uint8_t* mc, size_t mcstride, int passes, int QB,
+                                       int W, int H, bool ct62, Stream s) {
     const int QW = (W + 1) / 2, QH = (H + 1) / 2;
-    const dim3 grid((QW + kQcSeg - 1) / kQcSeg, QH);
+    const dim3 grid((QW + kQcSeg - 1) / kQcSeg, QH, passes);
+    const uint8_t* Fp = static_cast<const uint8_t*>(F);
     if (ct62)
-        cost_quads_kernel<D, uint64_t><<<grid, kQcThreads, 0, s>>>(static_cast<const uint64_t*>(Fb),
-                                                                   static_cast<const uint64_t*>(Fm), mc, QB, W, H);
+        launch(cost_quads_kernel<D, uint64_t>, grid, kQcThreads, s, Fp, fstride, mc, mcstride, QB, W, H);
     else
-        cost_quads_kernel<D, uint32_t><<<grid, kQcThreads, 0, s>>>(static_cast<const uint32_t*>(Fb),
-                                                                   static_cast<const uint32_t*>(Fm), mc, QB, W, H);
+        launch(cost_quads_kernel<D, uint32_t>, grid, kQcThreads, s, Fp, fstride, mc, mcstride, QB, W, H);
     return cudaGetLastError();
 }
 
-cudaError_t launch_cost_quads(const void* Fb, const void* Fm, uint8_t* mc, int QB, int W, int H, int D, bool ct62,
-                              cudaStream_t stream) {
+cudaError_t launch_cost_quads(const void* F, size_t fstride, uint8_t* mc, size_t mcstride, int passes, int QB, int W,
+                              int H, int D, bool ct62, Stream stream) {
     switch (D) {
-        case 32: return launch_cost_quads_t<32>(Fb, Fm, mc, QB, W, H, ct62, stream);
-        case 64: return launch_cost_quads_t<64>(Fb, Fm, mc, QB, W, H, ct62, stream);
-        case 96: return launch_cost_quads_t<96>(Fb, Fm, mc, QB, W, H, ct62, stream);
-        case 128: return launch_cost_quads_t<128>(Fb, Fm, mc, QB, W, H, ct62, stream);
-        case 160: return launch_cost_quads_t<160>(Fb, Fm, mc, QB, W, H, ct62, stream);
-        case 192: return launch_cost_quads_t<192>(Fb, Fm, mc, QB, W, H, ct62, stream);
-        case 224: return launch_cost_quads_t<224>(Fb, Fm, mc, QB, W, H, ct62, stream);
-        case 256: return launch_cost_quads_t<256>(Fb, Fm, mc, QB, W, H, ct62, stream);
+        case 32: return launch_cost_quads_t<32>(F, fstride, mc, mcstride, passes, QB, W, H, ct62, stream);
+        case 64: return launch_cost_quads_t<64>(F, fstride, mc, mcstride, passes, QB, W, H, ct62, stream);
+        case 96: return launch_cost_quads_t<96>(F, fstride, mc, mcstride, passes, QB, W, H, ct62, stream);
+        case 128: return launch_cost_quads_t<128>(F, fstride, mc, mcstride, passes, QB, W, H, ct62, stream);
+        case 160: return launch_cost_quads_t<160>(F, fstride, mc, mcstride, passes, QB, W, H, ct62, stream);
+        case 192: return launch_cost_quads_t<192>(F, fstride, mc, mcstride, passes, QB, W, H, ct62, stream);
+        case 224: return launch_cost_quads_t<224>(F, fstride, mc, mcstride, passes, QB, W, H, ct62, stream);
+        case 256: return launch_cost_quads_t<256>(F, fstride, mc, mcstride, passes, QB, W, H, ct62, stream);
         default: return cudaErrorInvalidValue;
     }
+}
+
+// ---------------------------------------------------------------------------
+// Jump penalties of the paired schedule's post form: one word per quad (or
+// diagonal unit) and direction, the penalty of the step into each of its four
+// pixels, max(P1, P2 / (1 + |I(p) - I(q)|)) with q the pixel before p on the
+// path (P2 where q or p is outside: a path starts there).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(128) p2map_kernel(const uint8_t* __restrict__ img, int mirror,
+                                                    uint32_t* __restrict__ map, int W, int H, int P1, int P2) {
+    pdl_wait();
+    const int QW = (W + 1) / 2, QH = (H + 1) / 2;
+    const int qx = blockIdx.x * blockDim.x + threadIdx.x, qy = blockIdx.y, dir = blockIdx.z;
+    if (qx >= QW) return;
+    // the predecessor's offset of each direction
+    const int px[8] = {-1, 1, 0, 0, -1, 1, 1, -1}, py[8] = {0, 0, -1, 1, -1, 1, -1, 1};
+    auto at = [&](int x, int y) -> int { return __ldg(img + static_cast<size_t>(y) * W + (mirror ? W - 1 - x : x)); };
+    uint32_t word = 0;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        int x, y;
+        if (dir < 4) {  // quad (qx, qy)
+            x = 2 * qx + (b & 1);
+            y = 2 * qy + (b >> 1);
+        } else {  // unit (qy, qx) of the lines moving right (4, 5) or left (6, 7)
+            const int line = 2 * qx + (b >> 1);
+            y = 2 * qy + (b & 1);
+            const int ym = y % (2 * QW);
+            x = dir < 6 ? line + ym : line - ym;
+            x = x >= 2 * QW ? x - 2 * QW : (x < 0 ? x + 2 * QW : x);
+        }
+        const int xq = x + px[dir], yq = y + py[dir];
+        int v = P2;
+        if (x < W && y < H && xq >= 0 && xq < W && yq >= 0 && yq < H) {
+            const int g = abs(at(x, y) - at(xq, yq));
+            v = max(P1, P2 / (1 + g));
+        }
+        word |= static_cast<uint32_t>(v) << (8 * b);
+    }
+    map[(static_cast<size_t>(dir) * QH + qy) * QW + qx] = word;
+}
+
+cudaError_t launch_p2map(const uint8_t* img, bool mirror, uint32_t* map, int n_paths, int W, int H, int P1, int P2,
+                         Stream stream) {
+    const int QW = (W + 1) / 2, QH = (H + 1) / 2;
+    const dim3 grid((QW + 127) / 128, QH, n_paths == 8 ? 8 : 4);
+    launch(p2map_kernel, grid, 128, stream, img, mirror ? 1 : 0, map, W, H, P1, P2);
+    return cudaGetLastError();
 }
 
 // A quad-layout cube -> natural order [H][W][D] (debug only).
@@ -581,6 +657,7 @@ __device__ __forceinline__ void median_body(const uint8_t* __restrict__ raw, uin
 
 __global__ void __launch_bounds__(kMedW) median_kernel(const uint8_t* __restrict__ raw, uint8_t* __restrict__ out,
                                                      int W, int H) {
+    pdl_wait();
     median_body(raw, out, W, H, blockIdx.x, blockIdx.y);
 }
 
@@ -602,20 +679,21 @@ cudaError_t launch_median_list(const ListLaunch& l, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_median(const uint8_t* raw, uint8_t* disp, int W, int H, cudaStream_t stream) {
+cudaError_t launch_median(const uint8_t* raw, uint8_t* disp, int W, int H, Stream stream) {
     dim3 grid((W + kMedW - 1) / kMedW, (H + kMedH - 1) / kMedH);
-    median_kernel<<<grid, kMedW, 0, stream>>>(raw, disp, W, H);
+    launch(median_kernel, grid, kMedW, stream, raw, disp, W, H);
     return cudaGetLastError();
 }
 
 __global__ void __launch_bounds__(kMedW) median_quads_kernel(const uint8_t* __restrict__ rawq,
                                                            uint8_t* __restrict__ out, int W, int H) {
+    pdl_wait();
     median_body<true>(rawq, out, W, H, blockIdx.x, blockIdx.y);
 }
 
-cudaError_t launch_median_quads(const uint8_t* rawq, uint8_t* disp, int W, int H, cudaStream_t stream) {
+cudaError_t launch_median_quads(const uint8_t* rawq, uint8_t* disp, int W, int H, Stream stream) {
     dim3 grid((W + kMedW - 1) / kMedW, (H + kMedH - 1) / kMedH);
-    median_quads_kernel<<<grid, kMedW, 0, stream>>>(rawq, disp, W, H);
+    launch(median_quads_kernel, grid, kMedW, stream, rawq, disp, W, H);
     return cudaGetLastError();
 }
 
@@ -628,6 +706,7 @@ cudaError_t launch_median_quads(const uint8_t* rawq, uint8_t* disp, int W, int H
 __global__ void __launch_bounds__(256) stage_kernel(const uint8_t* __restrict__ src0, uint8_t* __restrict__ dst0,
                                                     const uint8_t* __restrict__ src1, uint8_t* __restrict__ dst1,
                                                     size_t n) {
+    pdl_wait();
     const uint8_t* src = blockIdx.y ? src1 : src0;
     uint8_t* dst = blockIdx.y ? dst1 : dst0;
     if (!src) return;
@@ -643,12 +722,12 @@ __global__ void __launch_bounds__(256) stage_kernel(const uint8_t* __restrict__ 
 }
 
 cudaError_t launch_stage(const uint8_t* src0, uint8_t* dst0, const uint8_t* src1, uint8_t* dst1, size_t n,
-                         cudaStream_t stream) {
+                         Stream stream) {
     if (n == 0) return cudaSuccess;
     constexpr size_t kPer = 256 * 16;        // bytes one block moves per pass
     constexpr size_t kMaxBlocks = 4 * 152;   // four per SM of a GB300: enough requests in flight
     const unsigned blocks = static_cast<unsigned>(std::min<size_t>(kMaxBlocks, (n + kPer - 1) / kPer));
-    stage_kernel<<<dim3(blocks, src1 ? 2 : 1), 256, 0, stream>>>(src0, dst0, src1, dst1, n);
+    launch(stage_kernel, dim3(blocks, src1 ? 2 : 1), 256, stream, src0, dst0, src1, dst1, n);
     return cudaGetLastError();
 }
 
@@ -659,6 +738,7 @@ cudaError_t launch_stage(const uint8_t* src0, uint8_t* dst0, const uint8_t* src1
 __global__ void __launch_bounds__(256) mirror_kernel(const uint8_t* __restrict__ left,
                                                      const uint8_t* __restrict__ right, uint8_t* __restrict__ ml,
                                                      uint8_t* __restrict__ mr, int W, int H) {
+    pdl_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
     if (x >= W || y >= H) return;
     const size_t src = static_cast<size_t>(y) * W + (W - 1 - x), dst = static_cast<size_t>(y) * W + x;
@@ -667,9 +747,9 @@ __global__ void __launch_bounds__(256) mirror_kernel(const uint8_t* __restrict__
 }
 
 cudaError_t launch_mirror(const uint8_t* left, const uint8_t* right, uint8_t* ml, uint8_t* mr, int W, int H,
-                          cudaStream_t stream) {
+                          Stream stream) {
     dim3 grid((W + 255) / 256, H);
-    mirror_kernel<<<grid, 256, 0, stream>>>(left, right, ml, mr, W, H);
+    launch(mirror_kernel, grid, 256, stream, left, right, ml, mr, W, H);
     return cudaGetLastError();
 }
 
@@ -690,10 +770,21 @@ constexpr int kPostW = 32, kPostH = 8;
 
 // v = the sub-pixel (or 16 d) value of each pixel of a 34 x 10 tile in shared
 // memory, then the 3x3 median (border ring copied), then the left-right check.
+// Index of a pixel in a quad-layout or row-major array.
+template <bool QUADS>
+__device__ __forceinline__ size_t pixel_index(int x, int y, int W) {
+    if constexpr (QUADS)
+        return (static_cast<size_t>(y >> 1) * ((W + 1) >> 1) + (x >> 1)) * 4 + (x & 1) + 2 * (y & 1);
+    else
+        return static_cast<size_t>(y) * W + x;
+}
+
+template <bool QUADS>
 __global__ void __launch_bounds__(kPostW* kPostH) post_kernel(const uint8_t* __restrict__ rawL,
                                                               const uint32_t* __restrict__ sub,
                                                               const uint8_t* __restrict__ rawRm,
                                                               uint16_t* __restrict__ out16, int W, int H, int D) {
+    pdl_wait();
     __shared__ int v[kPostH + 2][kPostW + 2];
     const int x0 = blockIdx.x * kPostW, y0 = blockIdx.y * kPostH;
     const int t = threadIdx.y * kPostW + threadIdx.x;
@@ -702,7 +793,7 @@ __global__ void __launch_bounds__(kPostW* kPostH) post_kernel(const uint8_t* __r
         const int gx = x0 - 1 + cx, gy = y0 - 1 + cy;
         int val = 0;
         if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
-            const size_t p = static_cast<size_t>(gy) * W + gx;
+            const size_t p = pixel_index<QUADS>(gx, gy, W);
             const int d = rawL[p];
             val = sub ? subpixel_value(d, sub[p], D) : 16 * d;
         }
@@ -728,10 +819,10 @@ __global__ void __launch_bounds__(kPostW* kPostH) post_kernel(const uint8_t* __r
     }
     const size_t p = static_cast<size_t>(y) * W + x;
     if (rawRm) {
-        const int d = rawL[p], xr = x - d;
+        const int d = rawL[pixel_index<QUADS>(x, y, W)], xr = x - d;
         bool ok = xr >= 0;
         if (ok) {
-            const int dr = rawRm[static_cast<size_t>(y) * W + (W - 1 - xr)];
+            const int dr = rawRm[pixel_index<QUADS>(W - 1 - xr, y, W)];
             ok = d - dr <= 1 && dr - d <= 1;
         }
         if (!ok) out = 0xffff;
@@ -739,10 +830,13 @@ __global__ void __launch_bounds__(kPostW* kPostH) post_kernel(const uint8_t* __r
     out16[p] = static_cast<uint16_t>(out);
 }
 
-cudaError_t launch_post(const uint8_t* rawL, const uint32_t* sub, const uint8_t* rawRm, uint16_t* out16, int W,
-                        int H, int D, cudaStream_t stream) {
+cudaError_t launch_post(const uint8_t* rawL, const uint32_t* sub, const uint8_t* rawRm, uint16_t* out16, bool quads,
+                        int W, int H, int D, Stream stream) {
     dim3 grid((W + kPostW - 1) / kPostW, (H + kPostH - 1) / kPostH), block(kPostW, kPostH);
-    post_kernel<<<grid, block, 0, stream>>>(rawL, sub, rawRm, out16, W, H, D);
+    if (quads)
+        launch(post_kernel<true>, grid, block, stream, rawL, sub, rawRm, out16, W, H, D);
+    else
+        launch(post_kernel<false>, grid, block, stream, rawL, sub, rawRm, out16, W, H, D);
     return cudaGetLastError();
 }
 

@@ -33,19 +33,19 @@ cudaError_t init_kernel_attributes() {
         default: return cudaErrorInvalidValue; \
     }
 
-cudaError_t launch_sweep_h(const SweepArgs& a, cudaStream_t stream) { SGM_DISPATCH_D(sweep_launch_h, a.D, a, stream) }
+cudaError_t launch_sweep_h(const SweepArgs& a, Stream stream) { SGM_DISPATCH_D(sweep_launch_h, a.D, a, stream) }
 
-cudaError_t launch_sweep_v(const SweepArgs& a, cudaStream_t stream) { SGM_DISPATCH_D(sweep_launch_v, a.D, a, stream) }
+cudaError_t launch_sweep_v(const SweepArgs& a, Stream stream) { SGM_DISPATCH_D(sweep_launch_v, a.D, a, stream) }
 
-cudaError_t launch_sweep_first(FirstStageArgs& f, cudaStream_t stream) {
+cudaError_t launch_sweep_first(FirstStageArgs& f, Stream stream) {
     SGM_DISPATCH_D(sweep_launch_first, f.h.D, f, stream)
 }
 
-cudaError_t launch_sweep_first4(FirstStageArgs& f, cudaStream_t stream) {
+cudaError_t launch_sweep_first4(FirstStageArgs& f, Stream stream) {
     SGM_DISPATCH_D(sweep_launch_first4, f.h.D, f, stream)
 }
 
-cudaError_t launch_sweep_h2(const SweepArgs& a, cudaStream_t stream) { SGM_DISPATCH_D(sweep_launch_h2, a.D, a, stream) }
+cudaError_t launch_sweep_h2(const SweepArgs& a, Stream stream) { SGM_DISPATCH_D(sweep_launch_h2, a.D, a, stream) }
 
 cudaError_t launch_sweep_h_list(const ListLaunch& l, cudaStream_t stream) {
     SGM_DISPATCH_D(sweep_launch_h_list, l.D, l, stream)
@@ -61,45 +61,39 @@ int sweep_units(int lines, int D, bool pair) {
     return (lines + per - 1) / per;
 }
 
-// The paired-line 4-path schedule: n1 steps of each horizontal direction
-// beside the vertical pair in the first launch (default min(W2, H2), which
-// ends both at the same step).
-PairsArgs pairs_geometry(int W, int H, int D, int n1_req) {
+PairsArgs pairs_geometry(int W, int H, int D, int n_paths) {
     PairsArgs a{};
     a.W = W;
     a.H = H;
     a.D = D;
+    a.n_paths = n_paths;
     a.W2 = W + (W & 1);
     a.H2 = H + (H & 1);
     a.QW = a.W2 / 2;
     a.QH = a.H2 / 2;
-    int n1 = n1_req < 0 ? std::min(a.W2, a.H2) : n1_req;
-    a.n1 = std::max(0, std::min(a.W2, n1 & ~1));
-    if (a.W2 > 2 * a.n1) {
-        a.a = a.b = (a.W2 / 2) & ~1;  // the horizontal pair meets in the middle in the second launch
-    } else {
-        a.a = a.n1;  // columns [W2 - n1, n1) were passed by both directions in the first launch
-        a.b = a.W2 - a.n1;
-    }
-    a.nvb = a.QW;
-    a.nhb = a.QH;
-    a.nh2 = a.W2 > a.n1 ? a.QH : 0;
-    const int par = (a.a - a.b) / 2 * a.QH;  // quads of the parallel winner-take-all
-    const int per_block = 2 * pairs::kParItems;
-    a.npw = par > 0 ? (par + per_block - 1) / per_block : 0;
+    a.NS = (a.QW + seg_quads(D) - 1) / seg_quads(D);
     return a;
 }
 
-cudaError_t launch_pairs_stage1(const PairsArgs& a, cudaStream_t stream) {
-    SGM_DISPATCH_D(pairs_launch1, a.D, a, stream)
+#define SGM_DISPATCH_PAIRS(FN, ...)                \
+    switch (f.job[0].D) {                          \
+        case 32: return FN<32>(__VA_ARGS__);       \
+        case 64: return FN<64>(__VA_ARGS__);       \
+        case 96: return FN<96>(__VA_ARGS__);       \
+        case 128: return FN<128>(__VA_ARGS__);     \
+        case 160: return FN<160>(__VA_ARGS__);     \
+        case 192: return FN<192>(__VA_ARGS__);     \
+        case 224: return FN<224>(__VA_ARGS__);     \
+        case 256: return FN<256>(__VA_ARGS__);     \
+        default: return cudaErrorInvalidValue;     \
+    }
+
+cudaError_t launch_pairs_walks(const PairsJobs& f, Walks w, Stream stream) {
+    SGM_DISPATCH_PAIRS(pairs_walks, f, w, stream)
 }
 
-cudaError_t launch_pairs_chain2(const PairsArgs& a, cudaStream_t stream) {
-    SGM_DISPATCH_D(pairs_launch_chain2, a.D, a, stream)
-}
-
-cudaError_t launch_pairs_par(const PairsArgs& a, cudaStream_t stream) {
-    SGM_DISPATCH_D(pairs_launch_par, a.D, a, stream)
+cudaError_t launch_pairs_finish(const PairsJobs& f, Stream stream) {
+    SGM_DISPATCH_PAIRS(pairs_finish, f, stream)
 }
 
 }  // namespace sgm

@@ -646,12 +646,14 @@ __device__ __forceinline__ void sweep_h_body(const SweepArgs& a, int bx) {
 // holds the vertical pair's sums).
 template <int D, bool S8, bool DBG, int POST = 0>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock) sweep_h2_kernel(SweepArgs a) {
+    pdl_wait();
     post_init<POST>(a);
     sweep_h_body<D, true, S8, 2, true, DBG, POST>(a, blockIdx.x);
 }
 
 template <int D, bool PAIR, bool S8, int POST = 0>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock) sweep_h_kernel(SweepArgs a) {
+    pdl_wait();
     post_init<POST>(a);
     sweep_h_body<D, PAIR, S8, 0, false, false, POST>(a, blockIdx.x);
 }
@@ -739,6 +741,7 @@ __device__ __forceinline__ void sweep_v_body(const SweepArgs& a, int bx) {
 
 template <int D, int RX, int PH, bool WTA, bool PAIR, bool S8, bool DBG = false, int POST = 0>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock) sweep_v_kernel(SweepArgs a) {
+    pdl_wait();
     post_init<POST>(a);
     sweep_v_body<D, RX, PH, WTA, PAIR, S8, DBG, false, POST>(a, blockIdx.x);
 }
@@ -766,6 +769,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, kSweepListMaxPerSM)
 // (4 paths: the vertical pair only) keeps the diagonal code out of the kernel.
 template <int D, bool S8, int NV, int POST = 0>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock) sweep_first_kernel(const __grid_constant__ FirstStageArgs f) {
+    pdl_wait();
     post_init<POST>(f.h);
     const int b = blockIdx.x;
     if (b < f.start[1]) {
@@ -798,6 +802,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) sweep_first_kernel(const 
 // horizontal second halves then finish with Eq. 4 (sweep_h2_kernel).
 template <int D, bool S8, int POST = 0>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock) sweep_first4_kernel(const __grid_constant__ FirstStageArgs f) {
+    pdl_wait();
     post_init<POST>(f.h);
     const int b = blockIdx.x;
     if (b < f.start[1])
@@ -821,23 +826,23 @@ struct SweepD {
     // No kernel needs an attribute (no dynamic shared memory).
     static cudaError_t set_attrs() { return cudaSuccess; }
 
-    static cudaError_t launch_h(const SweepArgs& a, cudaStream_t s) {
+    static cudaError_t launch_h(const SweepArgs& a, Stream s) {
         const dim3 grid(blocks(a.H, a.pair)), block(32 * kWarpsPerBlock);
         if (a.post) {  // post form: 2-path left-to-right only
             if (a.pair) return cudaErrorInvalidValue;
-            sweep_h_kernel<D, false, true, 1><<<grid, block, 0, s>>>(a);
+            launch(sweep_h_kernel<D, false, true, 1>, grid, block, s, a);
             return cudaGetLastError();
         }
         if (!a.pair)
-            sweep_h_kernel<D, false, true><<<grid, block, 0, s>>>(a);
+            launch(sweep_h_kernel<D, false, true>, grid, block, s, a);
         else if (a.s8)
-            sweep_h_kernel<D, true, true><<<grid, block, 0, s>>>(a);
+            launch(sweep_h_kernel<D, true, true>, grid, block, s, a);
         else
-            sweep_h_kernel<D, true, false><<<grid, block, 0, s>>>(a);
+            launch(sweep_h_kernel<D, true, false>, grid, block, s, a);
         return cudaGetLastError();
     }
 
-    static cudaError_t launch_first(FirstStageArgs& f, cudaStream_t s) {
+    static cudaError_t launch_first(FirstStageArgs& f, Stream s) {
         f.start[0] = 0;
         f.start[1] = blocks(f.h.H, true);
         for (int k = 0; k < f.nv; ++k) f.start[k + 2] = f.start[k + 1] + blocks(f.v[k].W, true);
@@ -845,48 +850,48 @@ struct SweepD {
         const int grid = f.start[f.nv + 1];
         if (f.h.post) {  // post form: 8 paths only
             if (f.nv != 3 || f.h.s8) return cudaErrorInvalidValue;
-            sweep_first_kernel<D, false, 3, 1><<<grid, block, 0, s>>>(f);
+            launch(sweep_first_kernel<D, false, 3, 1>, grid, block, s, f);
             return cudaGetLastError();
         }
         if (f.nv == 1 && f.h.s8)
-            sweep_first_kernel<D, true, 1><<<grid, block, 0, s>>>(f);
+            launch(sweep_first_kernel<D, true, 1>, grid, block, s, f);
         else if (f.nv == 1)
-            sweep_first_kernel<D, false, 1><<<grid, block, 0, s>>>(f);
+            launch(sweep_first_kernel<D, false, 1>, grid, block, s, f);
         else
-            sweep_first_kernel<D, false, 3><<<grid, block, 0, s>>>(f);
+            launch(sweep_first_kernel<D, false, 3>, grid, block, s, f);
         return cudaGetLastError();
     }
 
-    static cudaError_t launch_first4(FirstStageArgs& f, cudaStream_t s) {
+    static cudaError_t launch_first4(FirstStageArgs& f, Stream s) {
         f.start[0] = 0;
         f.start[1] = blocks(f.h.H, true);
         f.start[2] = f.start[1] + blocks(f.v[0].W, true);
         const dim3 block(32 * kWarpsPerBlock);
         if (f.h.post && f.h.s8)
-            sweep_first4_kernel<D, true, 1><<<f.start[2], block, 0, s>>>(f);
+            launch(sweep_first4_kernel<D, true, 1>, f.start[2], block, s, f);
         else if (f.h.post)
-            sweep_first4_kernel<D, false, 1><<<f.start[2], block, 0, s>>>(f);
+            launch(sweep_first4_kernel<D, false, 1>, f.start[2], block, s, f);
         else if (f.h.s8)
-            sweep_first4_kernel<D, true><<<f.start[2], block, 0, s>>>(f);
+            launch(sweep_first4_kernel<D, true>, f.start[2], block, s, f);
         else
-            sweep_first4_kernel<D, false><<<f.start[2], block, 0, s>>>(f);
+            launch(sweep_first4_kernel<D, false>, f.start[2], block, s, f);
         return cudaGetLastError();
     }
 
-    static cudaError_t launch_h2(const SweepArgs& a, cudaStream_t s) {
+    static cudaError_t launch_h2(const SweepArgs& a, Stream s) {
         const dim3 grid(blocks(a.H, true)), block(32 * kWarpsPerBlock);
         if (a.post && a.s8)
-            sweep_h2_kernel<D, true, false, 1><<<grid, block, 0, s>>>(a);
+            launch(sweep_h2_kernel<D, true, false, 1>, grid, block, s, a);
         else if (a.post)
-            sweep_h2_kernel<D, false, false, 1><<<grid, block, 0, s>>>(a);
+            launch(sweep_h2_kernel<D, false, false, 1>, grid, block, s, a);
         else if (a.s8 && a.Sdbg)
-            sweep_h2_kernel<D, true, true><<<grid, block, 0, s>>>(a);
+            launch(sweep_h2_kernel<D, true, true>, grid, block, s, a);
         else if (a.s8)
-            sweep_h2_kernel<D, true, false><<<grid, block, 0, s>>>(a);
+            launch(sweep_h2_kernel<D, true, false>, grid, block, s, a);
         else if (a.Sdbg)
-            sweep_h2_kernel<D, false, true><<<grid, block, 0, s>>>(a);
+            launch(sweep_h2_kernel<D, false, true>, grid, block, s, a);
         else
-            sweep_h2_kernel<D, false, false><<<grid, block, 0, s>>>(a);
+            launch(sweep_h2_kernel<D, false, false>, grid, block, s, a);
         return cudaGetLastError();
     }
 
@@ -920,38 +925,38 @@ struct SweepD {
 
     // Vertical-type sweeps of a pair in phase 1 or 2 (or both, phase 0).
     template <int RX, bool WTA, bool S8>
-    static void launch_v_rx(const SweepArgs& a, dim3 grid, dim3 block, cudaStream_t s) {
+    static void launch_v_rx(const SweepArgs& a, dim3 grid, dim3 block, Stream s) {
         if (WTA && a.Sdbg && a.phase == 2)
-            sweep_v_kernel<D, RX, 2, WTA, true, S8, true><<<grid, block, 0, s>>>(a);
+            launch(sweep_v_kernel<D, RX, 2, WTA, true, S8, true>, grid, block, s, a);
         else if (a.phase == 1)
-            sweep_v_kernel<D, RX, 1, false, true, S8><<<grid, block, 0, s>>>(a);
+            launch(sweep_v_kernel<D, RX, 1, false, true, S8>, grid, block, s, a);
         else if (a.phase == 2)
-            sweep_v_kernel<D, RX, 2, WTA, true, S8><<<grid, block, 0, s>>>(a);
+            launch(sweep_v_kernel<D, RX, 2, WTA, true, S8>, grid, block, s, a);
         else
-            sweep_v_kernel<D, RX, 0, WTA, true, S8><<<grid, block, 0, s>>>(a);
+            launch(sweep_v_kernel<D, RX, 0, WTA, true, S8>, grid, block, s, a);
     }
 
-    static cudaError_t launch_v(const SweepArgs& a, cudaStream_t s) {
+    static cudaError_t launch_v(const SweepArgs& a, Stream s) {
         const dim3 grid(blocks(a.W, a.pair)), block(32 * kWarpsPerBlock);
         if (a.post) {
             // post form: the 2-path top-to-bottom sweep, and the second halves
             // of the three vertical-type pairs of 8 paths (u16 sums)
             if (!a.pair)
-                sweep_v_kernel<D, 0, 0, true, false, true, false, 1><<<grid, block, 0, s>>>(a);
+                launch(sweep_v_kernel<D, 0, 0, true, false, true, false, 1>, grid, block, s, a);
             else if (a.phase != 2 || a.s8)
                 return cudaErrorInvalidValue;
             else if (a.rx == 0)
-                sweep_v_kernel<D, 0, 2, true, true, false, false, 1><<<grid, block, 0, s>>>(a);
+                launch(sweep_v_kernel<D, 0, 2, true, true, false, false, 1>, grid, block, s, a);
             else if (a.rx > 0)
-                sweep_v_kernel<D, 1, 2, false, true, false, false, 1><<<grid, block, 0, s>>>(a);
+                launch(sweep_v_kernel<D, 1, 2, false, true, false, false, 1>, grid, block, s, a);
             else
-                sweep_v_kernel<D, -1, 2, false, true, false, false, 1><<<grid, block, 0, s>>>(a);
+                launch(sweep_v_kernel<D, -1, 2, false, true, false, false, 1>, grid, block, s, a);
             return cudaGetLastError();
         }
         if (!a.pair && a.Sdbg)
-            sweep_v_kernel<D, 0, 0, true, false, true, true><<<grid, block, 0, s>>>(a);
+            launch(sweep_v_kernel<D, 0, 0, true, false, true, true>, grid, block, s, a);
         else if (!a.pair)
-            sweep_v_kernel<D, 0, 0, true, false, true><<<grid, block, 0, s>>>(a);
+            launch(sweep_v_kernel<D, 0, 0, true, false, true>, grid, block, s, a);
         else if (a.rx == 0 && a.s8)
             launch_v_rx<0, true, true>(a, grid, block, s);
         else if (a.rx == 0)
@@ -969,17 +974,17 @@ struct SweepD {
 template <int D>
 SGM_INTERNAL cudaError_t sweep_set_attrs();
 template <int D>
-SGM_INTERNAL cudaError_t sweep_launch_h(const SweepArgs& a, cudaStream_t s);
+SGM_INTERNAL cudaError_t sweep_launch_h(const SweepArgs& a, Stream s);
 template <int D>
-SGM_INTERNAL cudaError_t sweep_launch_v(const SweepArgs& a, cudaStream_t s);
+SGM_INTERNAL cudaError_t sweep_launch_v(const SweepArgs& a, Stream s);
 template <int D>
-SGM_INTERNAL cudaError_t sweep_launch_first(FirstStageArgs& f, cudaStream_t s);
+SGM_INTERNAL cudaError_t sweep_launch_first(FirstStageArgs& f, Stream s);
 template <int D>
 SGM_INTERNAL cudaError_t sweep_launch_h_list(const ListLaunch& l, cudaStream_t s);
 template <int D>
-SGM_INTERNAL cudaError_t sweep_launch_first4(FirstStageArgs& f, cudaStream_t s);
+SGM_INTERNAL cudaError_t sweep_launch_first4(FirstStageArgs& f, Stream s);
 template <int D>
-SGM_INTERNAL cudaError_t sweep_launch_h2(const SweepArgs& a, cudaStream_t s);
+SGM_INTERNAL cudaError_t sweep_launch_h2(const SweepArgs& a, Stream s);
 template <int D>
 SGM_INTERNAL cudaError_t sweep_launch_v_list(const ListLaunch& l, cudaStream_t s);
 
@@ -989,15 +994,15 @@ SGM_INTERNAL cudaError_t sweep_launch_v_list(const ListLaunch& l, cudaStream_t s
         return SweepD<D>::set_attrs();                                                          \
     }                                                                                           \
     template <>                                                                                 \
-    SGM_INTERNAL cudaError_t sweep_launch_h<D>(const SweepArgs& a, cudaStream_t s) {            \
+    SGM_INTERNAL cudaError_t sweep_launch_h<D>(const SweepArgs& a, Stream s) {            \
         return SweepD<D>::launch_h(a, s);                                                       \
     }                                                                                           \
     template <>                                                                                 \
-    SGM_INTERNAL cudaError_t sweep_launch_v<D>(const SweepArgs& a, cudaStream_t s) {            \
+    SGM_INTERNAL cudaError_t sweep_launch_v<D>(const SweepArgs& a, Stream s) {            \
         return SweepD<D>::launch_v(a, s);                                                       \
     }                                                                                           \
     template <>                                                                                 \
-    SGM_INTERNAL cudaError_t sweep_launch_first<D>(FirstStageArgs & f, cudaStream_t s) {        \
+    SGM_INTERNAL cudaError_t sweep_launch_first<D>(FirstStageArgs & f, Stream s) {        \
         return SweepD<D>::launch_first(f, s);                                                   \
     }                                                                                           \
     template <>                                                                                 \
@@ -1009,11 +1014,11 @@ SGM_INTERNAL cudaError_t sweep_launch_v_list(const ListLaunch& l, cudaStream_t s
         return SweepD<D>::launch_v_list(l, s);                                                  \
     }                                                                                           \
     template <>                                                                                 \
-    SGM_INTERNAL cudaError_t sweep_launch_first4<D>(FirstStageArgs & f, cudaStream_t s) {       \
+    SGM_INTERNAL cudaError_t sweep_launch_first4<D>(FirstStageArgs & f, Stream s) {       \
         return SweepD<D>::launch_first4(f, s);                                                  \
     }                                                                                           \
     template <>                                                                                 \
-    SGM_INTERNAL cudaError_t sweep_launch_h2<D>(const SweepArgs& a, cudaStream_t s) {           \
+    SGM_INTERNAL cudaError_t sweep_launch_h2<D>(const SweepArgs& a, Stream s) {           \
         return SweepD<D>::launch_h2(a, s);                                                      \
     }
 
