@@ -193,10 +193,12 @@ SGM_API int sgm_compute_async(sgm_ctx *ctx, const uint8_t *left, const uint8_t *
 /*
  * Batched computation of `n` independent pairs of possibly different sizes,
  * D, penalties and path counts (the paper's scaling argument, Section 4,
- * applied to many pairs at once).  Pairs are grouped by (D, path count, sum
- * width); every stage of a group is one persistent grid whose blocks take
- * units (tiles, row segments, blocks of sweep lines) from a device work list
- * covering the group's pairs, longest chains first.  A wave (the pairs whose
+ * applied to many pairs at once).  A pair that fills the GPU by itself (W * H *
+ * D * n_paths above 2^28) runs through the kernels of sgm_compute.  The others
+ * are grouped by (D, path count, schedule and form of the sums); every stage of
+ * a group is one persistent grid whose blocks take units (tiles, row segments,
+ * line pairs) from a device work list covering the group's pairs, longest
+ * chains first.  A wave (the pairs whose
  * buffers fit the memory budget at once, at most 16 groups) is one CUDA
  * graph launch, the groups on concurrent branches; the graph is captured
  * once per wave shape and replayed with the lists rewritten.  The first wave

@@ -189,7 +189,7 @@ Layout layout_pairs(const Problem& p) {
 }
 
 Layout schedule_layout(const Problem& p, bool batched) {
-    if (!batched && pairs_sched(p)) return layout_pairs(p);
+    if (pairs_sched(p)) return layout_pairs(p);
     return layout_for(p.W, p.H, p.D, p.n_paths, batched, p.ct62 != 0, p.post != 0);
 }
 
@@ -273,7 +273,7 @@ struct Request {
 // Blob layout: status word at 0, the counters at kBlobCounters, the WorkList
 // headers at kBlobLists, the descriptors and prefix sums from kBlobHead.
 // ---------------------------------------------------------------------------
-constexpr int kListGroups = 16, kListBranches = 4, kListStages = 5, kListCounters = 8;
+constexpr int kListGroups = 16, kListBranches = 4, kListStages = 6, kListCounters = 8;
 constexpr size_t kBlobCounters = 64, kBlobLists = 1024, kBlobListStride = 32, kBlobHead = 4096;
 static_assert(kBlobCounters + 4 * kListGroups * kListCounters <= kBlobLists, "blob counters");
 static_assert(kBlobLists + kBlobListStride * kListGroups * kListStages <= kBlobHead, "blob list headers");
@@ -286,6 +286,9 @@ struct ListExec {
     cudaStream_t capture = nullptr;
     cudaStream_t branch[kListBranches] = {};
     cudaEvent_t fork = nullptr, join[kListBranches] = {};
+    // 8-path groups walk three lists side by side: two more streams per branch
+    cudaStream_t side[kListBranches][2] = {};
+    cudaEvent_t side_fork[kListBranches] = {}, side_join[kListBranches][2] = {};
     uint8_t* blob_dev = nullptr;
     uint8_t* blob_host = nullptr;     // pinned, blob_cap bytes
     size_t blob_cap = 0;
@@ -483,8 +486,8 @@ static bool is_device_ptr(const void* p) {
 // With post-filters: one matching pass (census, cost, sweeps) for the left
 // image, with the LR check a mirror kernel and a second pass, then the post
 // kernel.  The paired schedule: census, cost, the walks (one kernel with 2
-// paths; horizontal, vertical and, with 8 paths, diagonal walks side by side:
-// one timed stage), the finishing launch, median or post; both passes of the
+// paths; horizontal and vertical walks with 4, horizontal, downward and upward
+// walks with 8 paths side by side: one timed stage), the finishing launch, median or post; both passes of the
 // LR check in the same launches, the jump penalties of adaptive P2 one launch
 // per pass.
 static int walk_launches(const Problem& p) { return p.n_paths == 8 ? 3 : (p.n_paths == 4 ? 2 : 1); }
@@ -522,8 +525,7 @@ static cudaError_t enqueue_pairs(const Problem& p, const Layout& l, uint8_t* are
         g.FS = l.fs;
         g.P1x2 = static_cast<uint32_t>(p.P1) * 0x10001u;
         g.P2x2 = static_cast<uint32_t>(p.P2) * 0x10001u;
-        g.mc_max = mc_max(p);
-        g.gs = pairs_group(p2_max(p));
+        g.cls = pairs_class(p.n_paths, p.D, p2_max(p), mc_max(p));
         g.check_shrink = p.check_shrink;
         if (p.post & SGM_POST_ADAPTIVE_P2) {
             uint32_t* map = reinterpret_cast<uint32_t*>(arena + l.p2map + k * l.p2_stride);
@@ -536,8 +538,11 @@ static cudaError_t enqueue_pairs(const Problem& p, const Layout& l, uint8_t* are
     }
     if ((e = mark()) != cudaSuccess) return e;
     // every direction at once
-    const Walks kinds[3] = {walk_launches(p) == 1 ? Walks::kHorVer : Walks::kHor, Walks::kVer, Walks::kDiag};
-    for (int k = 0; k < walk_launches(p); ++k)
+    const int n = walk_launches(p);
+    const bool rows = walks_by_rows(f.job[0]);
+    const Walks kinds[3] = {n == 1 ? Walks::kHorVer : Walks::kHor, rows ? Walks::kDown : Walks::kVer,
+                            rows ? Walks::kUp : Walks::kDiag};
+    for (int k = 0; k < n; ++k)
         if ((e = launch_pairs_walks(f, kinds[k], s)) != cudaSuccess) return e;
     if ((e = mark()) != cudaSuccess) return e;
     if ((e = launch_pairs_finish(f, s)) != cudaSuccess) return e;
@@ -961,13 +966,45 @@ struct BatchItem {
     size_t offset;  // of the pair's region in the arena
 };
 
-// Items of one group share D, the path count, the sum storage and the Census type.
-static std::tuple<int, int, bool, int> batch_key(const BatchItem& it) {
-    return std::make_tuple(it.p.D, it.p.n_paths, s8_for(it.p), it.p.ct62);
+// The schedule and sum form of a batched pair: 0, 1 = per-line sweeps with u16 or
+// byte sums, 2 + pairs_class = paired lines.
+static int batch_form(const Problem& p) {
+    return pairs_sched(p) ? 2 + pairs_class(p.n_paths, p.D, p.P2, mc_max(p)) : (s8_for(p) ? 1 : 0);
+}
+
+static bool runs_alone(const Problem& p);
+
+// Items of one group share D, the path count, the form and the Census type
+// (form -1: no group, the pair runs alone).
+static std::tuple<int, int, int, int> batch_key(const BatchItem& it) {
+    return std::make_tuple(it.p.D, it.p.n_paths, runs_alone(it.p) ? -1 : batch_form(it.p), it.p.ct62);
 }
 
 static int group_code(const BatchItem& it) {
-    return it.p.D | it.p.n_paths << 9 | (s8_for(it.p) ? 1 : 0) << 13 | it.p.ct62 << 14;
+    return it.p.D | it.p.n_paths << 9 | batch_form(it.p) << 13 | it.p.ct62 << 16;
+}
+
+// A pair that fills the GPU by itself (2^28 path steps) runs through the
+// single-pair kernels in front of the wave's lists: beside others in the lists
+// it only takes L2 and issue slots from them.  us per pair, in lists of eight /
+// one by one: 640x480 D=128 4 paths 76.9 / 79.9, 1242x375 D=128 4 paths 112 /
+// 128, 1242x375 D=64 8 paths 139 / 139, 640x480 D=128 8 paths 145 / 134, 640x480
+// D=256 4 paths 144 / 131, 1242x375 D=128 8 paths 219 / 205.
+static bool runs_alone(const Problem& p) {
+    return pairs_sched(p) && static_cast<double>(p.W) * p.H * p.D * p.n_paths > 268435456.0;
+}
+
+// The schedule of a batched pair within `room` bytes, one of pairs alike with
+// `px` pixels together: paired lines where their cubes fit (2, 3 or 7 bytes per
+// pixel and disparity), else the per-line sweeps (3 or 4).  Up to 4 paths and
+// 2^18 pixels the sweeps' shorter chains win, which meet in the middle: us per
+// pair, paired / per-line, two of 240x180 D=128 4 paths 52.7 / 43.2, two of
+// 320x240 59.0 / 55.4, 32 of 96x64 5.6 / 5.3; 32 of 240x180 13.5 / 14.7; with 8
+// paths the paired lines lead from 64x48 on (5.7 / 6.1).
+static int batch_sched(Problem p, size_t room, double px) {
+    if (p.n_paths != 8 && px < 262144.0) return SGM_SCHED_V_THEN_H;
+    p.sched = SGM_SCHED_PAIRS;
+    return pairs_fit(p) && layout_for(p, true).total <= room ? SGM_SCHED_PAIRS : SGM_SCHED_V_THEN_H;
 }
 
 static int launches_per_group(int n_paths) { return 4 + (n_paths == 8 ? 3 : 1); }
@@ -978,6 +1015,11 @@ static int list_exec_init(sgm_ctx* ctx, ListExec& x) {
     for (int b = 0; b < kListBranches; ++b) {
         CUDA_TRY(ctx, cudaStreamCreateWithFlags(&x.branch[b], cudaStreamNonBlocking));
         CUDA_TRY(ctx, cudaEventCreateWithFlags(&x.join[b], cudaEventDisableTiming));
+        CUDA_TRY(ctx, cudaEventCreateWithFlags(&x.side_fork[b], cudaEventDisableTiming));
+        for (int k = 0; k < 2; ++k) {
+            CUDA_TRY(ctx, cudaStreamCreateWithFlags(&x.side[b][k], cudaStreamNonBlocking));
+            CUDA_TRY(ctx, cudaEventCreateWithFlags(&x.side_join[b][k], cudaEventDisableTiming));
+        }
     }
     void* q = nullptr;
     CUDA_TRY(ctx, ctx_malloc_host(ctx, &q, sizeof(uint32_t)));
@@ -999,6 +1041,11 @@ static void list_exec_release(ListExec& x) {
     for (int b = 0; b < kListBranches; ++b) {
         if (x.branch[b]) cudaStreamDestroy(x.branch[b]);
         if (x.join[b]) cudaEventDestroy(x.join[b]);
+        if (x.side_fork[b]) cudaEventDestroy(x.side_fork[b]);
+        for (int k = 0; k < 2; ++k) {
+            if (x.side[b][k]) cudaStreamDestroy(x.side[b][k]);
+            if (x.side_join[b][k]) cudaEventDestroy(x.side_join[b][k]);
+        }
     }
     if (x.fork) cudaEventDestroy(x.fork);
     if (x.capture) cudaStreamDestroy(x.capture);
@@ -1024,14 +1071,14 @@ static int list_exec_reserve(sgm_ctx* ctx, ListExec& x, size_t bytes) {
     return SGM_OK;
 }
 
-// The groups of a wave: [first item, end) per group, at most kListGroups
+// The groups of a wave's lists: [first item, end) per group, at most kListGroups
 // (items sorted by batch_key; a longer run of groups goes to the next wave).
 static std::vector<std::pair<size_t, size_t>> wave_groups(const std::vector<BatchItem>& items, size_t b, size_t e) {
     std::vector<std::pair<size_t, size_t>> g;
     for (size_t g0 = b; g0 < e;) {
         size_t g1 = g0;
         while (g1 < e && batch_key(items[g1]) == batch_key(items[g0])) ++g1;
-        g.emplace_back(g0, g1);
+        if (!runs_alone(items[g0].p)) g.emplace_back(g0, g1);
         g0 = g1;
     }
     return g;
@@ -1045,8 +1092,9 @@ static size_t build_lists(sgm_ctx* ctx, ListExec& x, const std::vector<BatchItem
     size_t need = kBlobHead;
     for (const auto& g : groups) {
         const size_t n = g.second - g.first;
-        need += up8(n * sizeof(CensusJob)) + up8(n * sizeof(CostJob)) + 2 * up8(n * sizeof(SweepArgs)) +
-                up8(n * sizeof(MedianJob)) + kListStages * up8((n + 1) * sizeof(uint32_t));
+        need += up8(n * sizeof(CensusJob)) + up8(n * sizeof(CostJob)) + up8(n * sizeof(MedianJob)) +
+                2 * up8(n * std::max(sizeof(SweepArgs), sizeof(PairsArgs))) +
+                kListStages * up8((n + 1) * sizeof(uint32_t));
     }
     if ((*rc = list_exec_reserve(ctx, x, need)) != SGM_OK) return 0;
     std::memset(x.blob_host, 0, kBlobHead);
@@ -1061,8 +1109,58 @@ static size_t build_lists(sgm_ctx* ctx, ListExec& x, const std::vector<BatchItem
         WorkList<CensusJob> w{static_cast<const CensusJob*>(job), static_cast<const uint32_t*>(start), n};
         std::memcpy(x.blob_host + kBlobLists + (g * kListStages + stage) * kBlobListStride, &w, sizeof w);
     };
+    static_assert(sizeof(CostQuadsJob) <= sizeof(CostJob), "room for the cost descriptors");
     for (size_t g = 0; g < groups.size(); ++g) {
         const size_t g0 = groups[g].first, n = groups[g].second - g0;
+        if (pairs_sched(items[g0].p)) {
+            // paired lines: every list in the order of the longest chains
+            std::vector<size_t> o(n);
+            for (size_t k = 0; k < n; ++k) o[k] = g0 + k;
+            auto chain = [&](size_t i) { return std::max(items[i].p.W, items[i].p.H); };
+            std::stable_sort(o.begin(), o.end(), [&](size_t i, size_t j) { return chain(i) > chain(j); });
+            std::vector<CensusJob> cj(n);
+            std::vector<CostQuadsJob> mj(n);
+            std::vector<PairsArgs> pj(n);
+            std::vector<MedianJob> dj(n);
+            std::vector<uint32_t> st[kListStages];  // census, cost, rows' and columns' walks, row walks, finish, median
+            for (auto& v : st) v.assign(n + 1, 0);
+            for (size_t k = 0; k < n; ++k) {
+                const BatchItem& it = items[o[k]];
+                const Problem& p = it.p;
+                const Layout l = layout_for(p, true);
+                uint8_t* base = arena + it.offset;
+                cj[k] = CensusJob{it.left, it.right, base + l.Fb, base + l.Fm, p.W, p.H};
+                mj[k] = CostQuadsJob{base + l.Fb, base + l.Fm, base + l.rec, l.RB, p.W, p.H, p.D};
+                PairsArgs a = pairs_geometry(p.W, p.H, p.D, p.n_paths);
+                a.rec = base + l.rec;
+                a.rawq = base + l.raw;
+                a.state = reinterpret_cast<uint32_t*>(base + l.state);
+                a.QB = l.RB;
+                a.FS = l.fs;
+                a.P1x2 = static_cast<uint32_t>(p.P1) * 0x10001u;
+                a.P2x2 = static_cast<uint32_t>(p.P2) * 0x10001u;
+                a.cls = pairs_class(p.n_paths, p.D, p.P2, mc_max(p));
+                a.run = pairs_finish_run(a);
+                pj[k] = a;
+                dj[k] = MedianJob{base + l.raw, is_device_ptr(it.out) ? it.out : base + l.out, p.W, p.H};
+                const int units[kListStages] = {census_units(p.W, p.H), cost_quads_units(p.W, p.H),
+                                                pairs_hv_units(a, p.n_paths != 8), a.QW, pairs_finish_units(a),
+                                                median_units(p.W, p.H)};
+                for (int i = 0; i < kListStages; ++i) st[i][k + 1] = st[i][k] + units[i];
+            }
+            const int ni = static_cast<int>(n);
+            const void* jobs = place(pj.data(), n * sizeof(PairsArgs));
+            if (g == 0 && ctx->bad_job_waves.load() > 0) {  // test hook: a descriptor its kernel must reject
+                --ctx->bad_job_waves;
+                pj[0].D += 32;
+            }
+            const void* walks = place(pj.data(), n * sizeof(PairsArgs));
+            const void* job[kListStages] = {place(cj.data(), n * sizeof(CensusJob)),
+                                            place(mj.data(), n * sizeof(CostQuadsJob)), walks, jobs, jobs,
+                                            place(dj.data(), n * sizeof(MedianJob))};
+            for (int i = 0; i < kListStages; ++i) header(g, i, job[i], place(st[i].data(), (n + 1) * 4), ni);
+            continue;
+        }
         std::vector<CensusJob> cj(n);
         std::vector<CostJob> mj(n);
         std::vector<SweepArgs> hj, vj;
@@ -1148,8 +1246,11 @@ static int list_graph(sgm_ctx* ctx, ListExec& x, const std::vector<int>& keys, i
             ListLaunch l{};
             l.status = status;
             l.D = D;
-            l.s8 = ((keys[g] >> 13) & 1) != 0;
-            l.ct62 = ((keys[g] >> 14) & 1) != 0;
+            const int form = (keys[g] >> 13) & 7;
+            l.s8 = form == 1;
+            l.cls = form - 2;
+            l.n_paths = n_paths;
+            l.ct62 = ((keys[g] >> 16) & 1) != 0;
             l.pair = n_paths >= 4;
             auto at = [&](int stage, int counter) {
                 l.list = x.blob_dev + kBlobLists + (g * kListStages + stage) * kBlobListStride;
@@ -1160,6 +1261,36 @@ static int list_graph(sgm_ctx* ctx, ListExec& x, const std::vector<int>& keys, i
             if ((e = launch_census_list(l, s)) != cudaSuccess) return e;
             at(1, 1);
             l.grid = kCostListPerSM * ctx->n_sm;
+            if (form >= 2) {
+                l.grid = kCostQuadsListPerSM * ctx->n_sm;
+                if ((e = launch_cost_quads_list(l, s)) != cudaSuccess) return e;
+                // the sweep grid counts 128 threads a block
+                at(2, 2);
+                l.grid = 2 * sweep_grid * ctx->n_sm;
+                const int b = g % kListBranches;
+                if (n_paths == 8) {
+                    if ((e = cudaEventRecord(x.side_fork[b], s)) != cudaSuccess) return e;
+                    if ((e = launch_pairs_walks_list(l, Walks::kHor, s)) != cudaSuccess) return e;
+                    l.grid = (4 * sweep_grid + 2) / 3 * ctx->n_sm;
+                    for (int k = 0; k < 2; ++k) {
+                        cudaStream_t ss = x.side[b][k];
+                        at(3, 3 + k);
+                        if ((e = cudaStreamWaitEvent(ss, x.side_fork[b], 0)) != cudaSuccess) return e;
+                        if ((e = launch_pairs_walks_list(l, k ? Walks::kUp : Walks::kDown, ss)) != cudaSuccess) return e;
+                        if ((e = cudaEventRecord(x.side_join[b][k], ss)) != cudaSuccess) return e;
+                        if ((e = cudaStreamWaitEvent(s, x.side_join[b][k], 0)) != cudaSuccess) return e;
+                    }
+                } else if ((e = launch_pairs_walks_list(l, Walks::kHorVer, s)) != cudaSuccess) {
+                    return e;
+                }
+                at(4, 5);
+                l.grid = kFinishListPerSM * ctx->n_sm;
+                if ((e = launch_pairs_finish_list(l, s)) != cudaSuccess) return e;
+                at(5, 6);
+                l.grid = kMedianListPerSM * ctx->n_sm;
+                if ((e = launch_median_quads_list(l, s)) != cudaSuccess) return e;
+                continue;
+            }
             if ((e = launch_cost_list(l, s)) != cudaSuccess) return e;
             at(2, 2);
             l.grid = sweep_grid * ctx->n_sm;
@@ -1260,47 +1391,58 @@ static int enqueue_wave(sgm_ctx* ctx, ListExec& x, std::vector<BatchItem>& items
             ctx->launches += 1;
         }
     }
+    for (size_t i = b; i < e; ++i) {
+        const BatchItem& it = items[i];
+        if (!runs_alone(it.p)) continue;
+        uint8_t* const base = arena + it.offset;
+        uint8_t* const dst = is_device_ptr(it.out) ? it.out : base + layout_for(it.p, true).out;
+        CUDA_TRY(ctx, enqueue_path(ctx, it.p, base, it.left, it.right, dst, nullptr, s, false));
+    }
     const auto groups = wave_groups(items, b, e);
     std::vector<int> keys;
     for (const auto& g : groups) keys.push_back(group_code(items[g.first]));
     int rc = SGM_OK;
-    const size_t used = build_lists(ctx, x, items, groups, arena, &rc);
-    if (rc != SGM_OK) return rc;
-    CUDA_TRY(ctx, cudaMemcpyAsync(x.blob_dev, x.blob_host, used, cudaMemcpyHostToDevice, s));
-    const int per_wave = wave_launches(items, groups);
-    int grid = kDefaultSweepGrid;  // served batches (the scheduler thread) take the default grid
-    const std::vector<int> sig = tune ? wave_signature(items, b, e) : std::vector<int>{};
-    if (tune && ctx->list_tuned.count(sig)) {
-        grid = ctx->list_tuned[sig];
-    } else if (tune) {
-        float best = 0.0f;
-        for (int cand : kSweepGrids) {
-            cudaGraphExec_t g = nullptr;
-            if ((rc = list_graph(ctx, x, keys, cand, &g)) != SGM_OK) return rc;
-            std::vector<float> ms;
-            for (int r = 0; r <= kTuneReps; ++r) {
-                CUDA_TRY(ctx, cudaEventRecord(ctx->tune_ev[0], s));
-                CUDA_TRY(ctx, cudaGraphLaunch(g, s));
-                CUDA_TRY(ctx, cudaEventRecord(ctx->tune_ev[1], s));
-                CUDA_TRY(ctx, cudaEventSynchronize(ctx->tune_ev[1]));
-                ctx->launches += per_wave;
-                float t = 0.0f;
-                CUDA_TRY(ctx, cudaEventElapsedTime(&t, ctx->tune_ev[0], ctx->tune_ev[1]));
-                if (r > 0) ms.push_back(t);  // run 0 warms up
+    if (groups.empty()) {
+        *x.status_host = 0;  // nothing of an earlier wave is on its way
+    } else {
+        const size_t used = build_lists(ctx, x, items, groups, arena, &rc);
+        if (rc != SGM_OK) return rc;
+        CUDA_TRY(ctx, cudaMemcpyAsync(x.blob_dev, x.blob_host, used, cudaMemcpyHostToDevice, s));
+        const int per_wave = wave_launches(items, groups);
+        int grid = kDefaultSweepGrid;  // served batches (the scheduler thread) take the default grid
+        const std::vector<int> sig = tune ? wave_signature(items, b, e) : std::vector<int>{};
+        if (tune && ctx->list_tuned.count(sig)) {
+            grid = ctx->list_tuned[sig];
+        } else if (tune) {
+            float best = 0.0f;
+            for (int cand : kSweepGrids) {
+                cudaGraphExec_t g = nullptr;
+                if ((rc = list_graph(ctx, x, keys, cand, &g)) != SGM_OK) return rc;
+                std::vector<float> ms;
+                for (int r = 0; r <= kTuneReps; ++r) {
+                    CUDA_TRY(ctx, cudaEventRecord(ctx->tune_ev[0], s));
+                    CUDA_TRY(ctx, cudaGraphLaunch(g, s));
+                    CUDA_TRY(ctx, cudaEventRecord(ctx->tune_ev[1], s));
+                    CUDA_TRY(ctx, cudaEventSynchronize(ctx->tune_ev[1]));
+                    ctx->launches += per_wave;
+                    float t = 0.0f;
+                    CUDA_TRY(ctx, cudaEventElapsedTime(&t, ctx->tune_ev[0], ctx->tune_ev[1]));
+                    if (r > 0) ms.push_back(t);  // run 0 warms up
+                }
+                std::sort(ms.begin(), ms.end());
+                const float med = ms[ms.size() / 2];
+                if (cand == kSweepGrids[0] || med < best) {
+                    best = med;
+                    grid = cand;
+                }
             }
-            std::sort(ms.begin(), ms.end());
-            const float med = ms[ms.size() / 2];
-            if (cand == kSweepGrids[0] || med < best) {
-                best = med;
-                grid = cand;
-            }
+            ctx->list_tuned[sig] = grid;
         }
-        ctx->list_tuned[sig] = grid;
+        cudaGraphExec_t g = nullptr;
+        if ((rc = list_graph(ctx, x, keys, grid, &g)) != SGM_OK) return rc;
+        CUDA_TRY(ctx, cudaGraphLaunch(g, s));
+        ctx->launches += per_wave;
     }
-    cudaGraphExec_t g = nullptr;
-    if ((rc = list_graph(ctx, x, keys, grid, &g)) != SGM_OK) return rc;
-    CUDA_TRY(ctx, cudaGraphLaunch(g, s));
-    ctx->launches += per_wave;
     for (size_t i = b; i < e; ++i) {
         const BatchItem& it = items[i];
         if (!is_device_ptr(it.out)) {
@@ -1331,9 +1473,6 @@ static int wave_status(sgm_ctx* ctx, const ListExec& x) {
 // once per wave.
 static int run_batch(sgm_ctx* ctx, ListExec& x, std::vector<BatchItem>& items, uint8_t** arena, size_t* arena_bytes,
                      bool clear_graphs, cudaStream_t s, bool tune) {
-    std::stable_sort(items.begin(), items.end(), [](const BatchItem& a, const BatchItem& c) {
-        return batch_key(a) < batch_key(c);
-    });
     size_t free_b = 0, total_b = 0;
     CUDA_TRY(ctx, cudaMemGetInfo(&free_b, &total_b));
     size_t budget = (free_b + *arena_bytes) / 10 * 9;
@@ -1341,6 +1480,12 @@ static int run_batch(sgm_ctx* ctx, ListExec& x, std::vector<BatchItem>& items, u
         const size_t other = ctx->serve_bytes.load();
         budget = std::min(budget, ctx->mem_cap > other ? ctx->mem_cap - other : 0);
     }
+    std::map<std::pair<int, int>, double> px;  // pixels of the pairs of one D and path count
+    for (const BatchItem& it : items) px[{it.p.D, it.p.n_paths}] += static_cast<double>(it.p.W) * it.p.H;
+    for (BatchItem& it : items) it.p.sched = batch_sched(it.p, budget, px[{it.p.D, it.p.n_paths}]);
+    std::stable_sort(items.begin(), items.end(), [](const BatchItem& a, const BatchItem& c) {
+        return batch_key(a) < batch_key(c);
+    });
     size_t b = 0;
     while (b < items.size()) {
         size_t e = b, total = 0;
@@ -1587,9 +1732,10 @@ static void serve_loop(sgm_ctx* ctx) {
         int rc = slot_budget(ctx, *sl, &budget);
         lk.lock();
         size_t used = 0;
-        std::set<std::tuple<int, int, bool, int>> keys;
+        std::set<std::tuple<int, int, int, int>> keys;
         while (rc == SGM_OK && !ctx->queue.empty() && sl->reqs.size() < static_cast<size_t>(kServeMaxPairs)) {
-            const Request& r = ctx->queue.front();
+            Request& r = ctx->queue.front();
+            r.p.sched = batch_sched(r.p, budget - used, 8.0 * r.p.W * r.p.H);  // a stream of requests like this one
             const size_t sz = layout_for(r.p, true).total;
             const auto key = batch_key(BatchItem{r.p, nullptr, nullptr, nullptr, 0});
             if (used + sz > budget || (!keys.count(key) && keys.size() == static_cast<size_t>(kListGroups))) break;

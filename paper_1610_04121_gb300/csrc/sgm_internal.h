@@ -121,6 +121,7 @@ struct ListLaunch {
     int D;
     bool ct62, pair, s8;
     int rx;            // vertical-type sweeps: 0 (vertical, finishing with Eq. 4), +1 / -1 (diagonals)
+    int n_paths, cls;  // paired schedule: paths and class of the sums (pairs_class)
 };
 
 // Each launcher enqueues one kernel on `stream` and returns the launch error.
@@ -225,8 +226,8 @@ struct PairsArgs {
     size_t FS;             // bytes of one field array (QH * QW * QB, rounded up)
     int QB;                // bytes of one quad in a field: 4D (W2 * H2 * D < 2^32)
     uint32_t P1x2, P2x2;
-    int mc_max;            // largest matching cost: 31 (CSCT) or 62 (full Census)
-    int gs;                // stored r that add in a byte: gs * (largest P2) <= 255, at most 3
+    int cls;               // class of the sums (pairs_class)
+    int run;               // batched: segments of a unit of the finishing list
     int check_shrink;      // bounds-checked build, test hook: bytes taken off the declared end of the fields
 };
 // One launch over one or two problems of the same shape (the two passes of the
@@ -240,7 +241,17 @@ PairsArgs pairs_geometry(int W, int H, int D, int n_paths);
 inline size_t pairs_state_words(const PairsArgs& a) {
     return static_cast<size_t>(2) * a.QH * a.NS * 32 * ((a.D / 32 + 1) / 2);
 }
-inline int pairs_group(int p2_max) { return 3 * p2_max <= 255 ? 3 : (2 * p2_max <= 255 ? 2 : 1); }
+// How the finishing launch sums and takes the winner.  4 and 8 paths: 0 = three
+// r add in a byte (3 P2 <= 255) and the keys S D + d fit 16 bits, 1 = two r add
+// in a byte, 2 = neither; 2 paths: 0 = 16-bit keys, 1 = 32-bit keys.
+// S <= n_paths (MC_max + P2).
+inline int pairs_class(int n_paths, int D, int p2_max, int mc_max) {
+    const bool k16 = n_paths * (mc_max + p2_max) * D + D - 1 <= 65535;
+    if (n_paths == 2) return k16 ? 0 : 1;
+    return 3 * p2_max <= 255 && k16 ? 0 : (2 * p2_max <= 255 ? 1 : 2);
+}
+// A cube (or a field) that the 126 MB L2 does not hold beside what streams through it.
+__host__ __device__ inline bool larger_than_l2(size_t bytes) { return bytes > (size_t(96) << 20); }
 // Features of one or both passes: image z of F + z fstride bytes is left (0),
 // right (1), and with n = 4 the mirrored pair of the right pass (right, left).
 cudaError_t launch_census_passes(const uint8_t* left, const uint8_t* right, void* F, size_t fstride, int n, int W,
@@ -253,13 +264,35 @@ cudaError_t launch_cost_quads(const void* F, size_t fstride, uint8_t* mc, size_t
 // image img, or its mirror image.
 cudaError_t launch_p2map(const uint8_t* img, bool mirror, uint32_t* map, int n_paths, int W, int H, int P1, int P2,
                          Stream stream);
-// The walks of a path: one launch per kind, side by side (the first one waits
-// for the costs, each lets the next one start as soon as its own blocks have,
-// and the last block of a later one waits for the one before it, so that the
-// last launch ends when all have), or both kinds of 2 paths in one launch.
-enum class Walks { kHor, kVer, kDiag, kHorVer };
+// The walks of a path, side by side: horizontal, vertical and, with 8 paths,
+// diagonal pairs; with 8 paths over a cube larger than L2, horizontal pair,
+// directions that go down and directions that go up; or both directions of 2
+// paths in one launch.  The first launch waits for the costs, each lets the
+// next one start as soon as its own blocks have, and the last block of a later
+// one waits for the one before it, so that the last launch ends when all have.
+enum class Walks { kHor, kVer, kDiag, kDown, kUp, kHorVer };
+inline bool walks_by_rows(const PairsArgs& a) { return a.n_paths == 8 && larger_than_l2(a.FS); }
 cudaError_t launch_pairs_walks(const PairsJobs& f, Walks w, Stream stream);
 cudaError_t launch_pairs_finish(const PairsJobs& f, Stream stream);
+// Work-list forms.  Walks: kHorVer (2 and 4 paths), or kHor, kDown and kUp (8
+// paths; kHor and kHorVer take pairs_hv_units, kDown and kUp QW units a pair).
+struct CostQuadsJob {
+    const void *Fb, *Fm;
+    uint8_t* mc;
+    int QB, W, H, D;
+};
+constexpr int kCostQuadsRun = 4; // 32-quad segments of a unit of the cost list
+cudaError_t launch_cost_quads_list(const ListLaunch& l, cudaStream_t stream);
+cudaError_t launch_pairs_walks_list(const ListLaunch& l, Walks w, cudaStream_t stream);
+cudaError_t launch_pairs_finish_list(const ListLaunch& l, cudaStream_t stream);
+cudaError_t launch_median_quads_list(const ListLaunch& l, cudaStream_t stream);
+int cost_quads_units(int W, int H);
+int pairs_hv_units(const PairsArgs& a, bool ver);
+// Segments a warp takes at once: four, unless that leaves a pair with fewer
+// units than the list's grid has warps.
+inline int pairs_finish_run(const PairsArgs& a) { return a.QH * a.NS >= 16384 ? 4 : (a.QH * a.NS >= 8192 ? 2 : 1); }
+inline int pairs_finish_units(const PairsArgs& a) { return a.QH * ((a.NS + a.run - 1) / a.run); }
+constexpr int kFinishListPerSM = 14, kCostQuadsListPerSM = 12;
 // 3x3 median of a quad-layout raw disparity.
 cudaError_t launch_median_quads(const uint8_t* rawq, uint8_t* disp, int W, int H, Stream stream);
 // Debug: a quad-layout cube (quad q at cube + q QB) -> natural order [H][W][D].

@@ -161,6 +161,12 @@ __device__ __forceinline__ void sts_unit(uint32_t s, const uint32_t (&r)[K]) {
     }
 }
 
+// n contiguous bytes (a multiple of 16) from DRAM into L2.
+__device__ __forceinline__ void prefetch_l2(const PairsArgs& a, const uint8_t* p, uint32_t n, unsigned site) {
+    if (SGM_GUARD(p, n, a.rec, cubes_end(a), site))
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(n) : "memory");
+}
+
 // A lane's 4 K bytes of a unit from global memory, through L2 only.
 template <int K>
 __device__ __forceinline__ void ldg_unit(const PairsArgs& a, const uint8_t* p, uint32_t (&r)[K], uint64_t pol,
@@ -189,20 +195,39 @@ __device__ __forceinline__ void ldg_unit(const PairsArgs& a, const uint8_t* p, u
     }
 }
 
+// L2 policy of the stored r: of a cube larger than L2 they are gone before they
+// are read, so their lines make way for the costs that the other walkers read
+// (1920x1080 D=128 8 paths 974 -> 965 us); of a smaller one they stay.
+__device__ __forceinline__ uint64_t store_policy(const PairsArgs& a) {
+    uint64_t pol;
+    if (larger_than_l2(a.FS))
+        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    else
+        asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+    return pol;
+}
+
 // A lane's 4 K bytes of a unit to global memory.
 template <int K>
-__device__ __forceinline__ void stg_unit(const PairsArgs& a, uint8_t* p, const uint32_t (&r)[K], unsigned site) {
+__device__ __forceinline__ void stg_unit(const PairsArgs& a, uint8_t* p, const uint32_t (&r)[K], uint64_t pol,
+                                         unsigned site) {
     if (!SGM_GUARD(p, 4 * K, a.rec, cubes_end(a), site)) return;
     if constexpr (K % 4 == 0) {
 #pragma unroll
         for (int i = 0; i < K / 4; ++i)
-            reinterpret_cast<uint4*>(p)[i] = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+            asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p + 16 * i),
+                         "r"(r[4 * i]), "r"(r[4 * i + 1]), "r"(r[4 * i + 2]), "r"(r[4 * i + 3]), "l"(pol)
+                         : "memory");
     } else if constexpr (K % 2 == 0) {
 #pragma unroll
-        for (int i = 0; i < K / 2; ++i) reinterpret_cast<uint2*>(p)[i] = make_uint2(r[2 * i], r[2 * i + 1]);
+        for (int i = 0; i < K / 2; ++i)
+            asm volatile("st.global.L2::cache_hint.v2.u32 [%0], {%1, %2}, %3;" ::"l"(p + 8 * i), "r"(r[2 * i]),
+                         "r"(r[2 * i + 1]), "l"(pol)
+                         : "memory");
     } else {
 #pragma unroll
-        for (int i = 0; i < K; ++i) reinterpret_cast<unsigned*>(p)[i] = r[i];
+        for (int i = 0; i < K; ++i)
+            asm volatile("st.global.L2::cache_hint.u32 [%0], %1, %2;" ::"l"(p + 4 * i), "r"(r[i]), "l"(pol) : "memory");
     }
 }
 
@@ -246,9 +271,10 @@ struct Chain2 {
     __device__ __forceinline__ void init(int lane) {
         // d = 0 has no d - 1 (lane 0) and d = D - 1 no d + 1 (lane 31): those
         // neighbours read "infinity" through a multiply-add on the FMA pipe
-        mul_up = lane == 0 ? 0u : 1u;
+        // (opaque: a known 0 or 1 becomes a select on the ALU)
+        mul_up = opaque(lane == 0 ? 0u : 1u);
         add_up = lane == 0 ? kInf2 : 0u;
-        mul_dn = lane == 31 ? 0u : 1u;
+        mul_dn = opaque(lane == 31 ? 0u : 1u);
         add_dn = lane == 31 ? kInf2 : 0u;
         k16 = opaque(0x10000u);
         reset();
@@ -291,8 +317,8 @@ struct Chain2 {
 
     // x(d) = min(L(q, d), L(q, d-1) + P1, L(q, d+1) + P1, m(q) + P2), the step's costs before MC and m(q)
     __device__ __forceinline__ void relax(uint32_t P1x2, uint32_t P2x2, uint32_t (&x)[K]) const {
-        const uint32_t u = up * mul_up + add_up;
-        const uint32_t d = dn * mul_dn + add_dn;
+        const uint32_t u = mad(up, mul_up, add_up);
+        const uint32_t d = mad(dn, mul_dn, add_dn);
         const uint32_t mp2 = mpx2 + P2x2;
 #pragma unroll
         for (int j = 0; j < K; ++j) {
@@ -365,18 +391,25 @@ __device__ __forceinline__ bool state_ok(const PairsArgs& a, const uint32_t* p, 
                      a.state + static_cast<size_t>(2) * a.QH * a.NS * 32 * Chain2<D / 32>::CW, site);
 }
 
-// The walks' ring of units in shared memory, per warp: a multiple of kUnroll
-// units, at most 16.
-constexpr int kUnroll = 4;
+// The walks' ring of units in shared memory, per warp, at most 16 units.  D >
+// 128: 16 KB, which also keeps the warps of an SM at twelve and their reads near
+// one another (1920x1080 D=256 4 paths 893 us per frame; 12 KB 944, 8 KB 924,
+// 24 KB 905); 8 KB for each of the three warps of a block that walks rows (8
+// and 12 KB measure alike).  A walk's loop is UN units long: eight (640x480
+// D=128 frame 79.5 us, four 81.8), four for D > 128 (1920x1080 D=256 892 us,
+// eight 905), but two for diagonals that run beside the other walks (1242x375 8
+// paths 204 us; eight no longer fit the instruction caches with them: 214), and
+// no more than a segment or the ring holds.
 template <int D>
-__host__ __device__ constexpr int ring_bytes() {
-    return D <= 128 ? 8192 : 16384;
+__host__ __device__ constexpr int ring_bytes(bool rows = false) {
+    return D <= 128 || rows ? 8192 : 16384;
 }
-template <int D, int KIND>
+template <int D, int KIND, bool ROWS>
 struct Ring {
     static constexpr int SB = (KIND == kDiag ? 2 : 1) * 4 * D;  // bytes of a slot
-    static constexpr int FIT = ring_bytes<D>() / SB / kUnroll * kUnroll;
-    static constexpr int DEPTH = FIT > 16 ? 16 : FIT;
+    static constexpr int WANT = KIND == kDiag && !ROWS ? 2 : (D <= 128 ? 8 : 4), FIT = ring_bytes<D>(ROWS) / SB;
+    static constexpr int UN = WANT <= FIT && (KIND != kHor || WANT <= seg_quads(D)) ? WANT : (WANT < 4 ? WANT : 4);
+    static constexpr int DEPTH = FIT / UN * UN > 16 ? 16 : FIT / UN * UN;
 };
 
 // ---------------------------------------------------------------------------
@@ -390,10 +423,11 @@ struct Ring {
 // instruction caches (164 against 144 us for the walks of a 1242x375 8-path
 // frame, although each ran faster alone).
 // ---------------------------------------------------------------------------
-template <int D, int KIND, bool AP2>
+template <int D, int KIND, bool AP2, bool ROWS = false>
 __device__ __forceinline__ void walk(const PairsArgs& a, int line, int kd, bool fwd, uint32_t ring) {
-    constexpr int K = D / 32, CQ = seg_quads(D), SB = Ring<D, KIND>::SB, DEPTH = Ring<D, KIND>::DEPTH;
-    static_assert(CQ % kUnroll == 0 && DEPTH >= kUnroll, "groups of units end where segments end");
+    constexpr int K = D / 32, CQ = seg_quads(D), SB = Ring<D, KIND, ROWS>::SB,
+                  DEPTH = Ring<D, KIND, ROWS>::DEPTH, UN = Ring<D, KIND, ROWS>::UN;
+    static_assert((KIND != kHor || CQ % UN == 0) && DEPTH >= UN, "groups of units end where segments end");
     const int lane = threadIdx.x & 31;
     const uint32_t QB = static_cast<uint32_t>(a.QB), rowb = static_cast<uint32_t>(a.QW) * QB;
     int nu;               // units of the walk
@@ -415,6 +449,7 @@ __device__ __forceinline__ void walk(const PairsArgs& a, int line, int kd, bool 
     const uint32_t s_hi = KIND == kHor ? kSelCol1 : (KIND == kVer ? kSelRow1 : (kd == 0 ? kSelNext : kSelPrev));
     const uint32_t sel0 = fwd ? s_lo : s_hi, sel1 = fwd ? s_hi : s_lo;
     const uint32_t selq = KIND == kVer ? (fwd ? 0x6420u : 0x2064u) : (fwd ? 0x6240u : 0x2604u);
+    const uint64_t pol = store_policy(a);
     uint8_t* const src = a.rec + 16 * lane;
     uint8_t* const out =
         a.rec + (KIND == kVer ? 1 : 3 + 2 * kd) * a.FS + (fwd ? 0 : a.FS) + 4 * K * lane;  // stored r
@@ -540,24 +575,31 @@ __device__ __forceinline__ void walk(const PairsArgs& a, int line, int kd, bool 
             ch.step(m, a.P1x2, pb, r1);
 #pragma unroll
             for (int j = 0; j < K; ++j) r0[j] = prmt(r0[j], r1[j], selq);
-            stg_unit<K>(a, at(out, off), r0, 106);
+            stg_unit<K>(a, at(out, off), r0, pol, 106);
             off += ustep;
             if constexpr (KIND == kDiag) --cp_n;
         }
     };
-    // horizontal: the state after unit k, where a segment ends
-    auto segment_end = [&](int k) {
-        const int q = fwd ? k : a.QW - 1 - k;
-        if ((q & (CQ - 1)) == (fwd ? CQ - 1 : 0)) {
+    // horizontal: the state where a segment ends, seg_n units further on
+    int seg_n = 0;
+    uint32_t* seg_st = nullptr;
+    if constexpr (KIND == kHor) {
+        seg_n = fwd ? CQ : (a.QW - 1) % CQ + 1;
+        seg_st = state_slot<D>(a, fwd ? 0 : 1, line, fwd ? 1 : (a.QW - 1) / CQ - 1);
+    }
+    auto segment_end = [&](int n) {
+        seg_n -= n;
+        if (seg_n == 0) {
+            seg_n = CQ;
             ch.rebase();
-            uint32_t* st = state_slot<D>(a, fwd ? 0 : 1, line, fwd ? q / CQ + 1 : q / CQ - 1);
-            if (state_ok<D>(a, st, 105)) ch.save(st);
+            if (state_ok<D>(a, seg_st, 105)) ch.save(seg_st);
+            seg_st += (fwd ? 32 : -32) * Chain2<K>::CW;
         }
     };
 
-    // backward row walks start inside a group of kUnroll columns: the first slot
+    // backward row walks start inside a group of UN columns: the first slot
     // is chosen so that groups of slots and of columns end together
-    const int s0 = KIND == kHor && !fwd ? (kUnroll - a.QW % kUnroll) % kUnroll : 0;
+    const int s0 = KIND == kHor && !fwd ? (UN - a.QW % UN) % UN : 0;
     int slot = s0 * SB;
 #pragma unroll 1
     for (int i = 0; i < DEPTH; ++i) {
@@ -571,29 +613,29 @@ __device__ __forceinline__ void walk(const PairsArgs& a, int line, int kd, bool 
     // every unit: the next unit's costs into registers, its slot refilled, then its two steps
 #pragma unroll 1
     for (int k = 0; k < nu;) {
-        // groups of kUnroll units that need no care: refills in range, no path starts
+        // groups of UN units that need no care: refills in range, no path starts
         int groups = 0;
-        if (slot % (kUnroll * SB) == 0) {
+        if (slot % (UN * SB) == 0) {
             int n = nu - DEPTH - k;
             if constexpr (KIND == kDiag) n = min(n, min(ld_n, cp_n));
-            groups = n / kUnroll;
+            groups = n / UN;
         }
 #pragma unroll 1
         for (; groups > 0; --groups) {
 #pragma unroll
-            for (int i = 0; i < kUnroll; ++i) {
+            for (int i = 0; i < UN; ++i) {
                 const int s = slot + i * SB;
                 cp_wait<DEPTH - 2>();
-                read(i + 1 < kUnroll ? s + SB : (s + SB == DEPTH * SB ? 0 : s + SB), nxt);
+                read(i + 1 < UN ? s + SB : (s + SB == DEPTH * SB ? 0 : s + SB), nxt);
                 issue(s, false);
                 cp_commit();
                 unit(cur, k + i, false);
                 cur = nxt;
             }
-            k += kUnroll;
-            slot += kUnroll * SB;
+            k += UN;
+            slot += UN * SB;
             if (slot == DEPTH * SB) slot = 0;
-            if constexpr (KIND == kHor) segment_end(k - 1);
+            if constexpr (KIND == kHor) segment_end(UN);
         }
         if (k < nu) {
             const int ns = slot + SB == DEPTH * SB ? 0 : slot + SB;
@@ -603,7 +645,7 @@ __device__ __forceinline__ void walk(const PairsArgs& a, int line, int kd, bool 
             cp_commit();
             unit(cur, k, true);
             cur = nxt;
-            if constexpr (KIND == kHor) segment_end(k);
+            if constexpr (KIND == kHor) segment_end(1);
             ++k;
             slot = ns;
         }
@@ -653,6 +695,26 @@ __global__ void __launch_bounds__(64) walk_d_kernel(const __grid_constant__ Pair
     const uint32_t r = static_cast<uint32_t>(__cvta_generic_to_shared(ring[warp]));
     const int c = blockIdx.x * 2 + warp;
     if (c < 4 * a.QW) walk<D, kDiag, AP2>(a, c / 4, (c / 2) % 2, c % 2 == 0, r);
+    side.end();
+}
+
+// 8 paths, cubes larger than L2: the three directions that go down (fwd) or up
+// from one column pair, a warp each.  They pass every row together, so that
+// its costs come from DRAM once for the three.  Cubes that L2 holds walk the
+// vertical pair beside the diagonals instead (fewer code paths per block and
+// shorter blocks): 1920x1080 D=128 974 against 1008 us per frame, but 1242x375
+// D=128 (60 MB of costs) 216 against 208.
+template <int D, bool AP2>
+__global__ void __launch_bounds__(96) walk_rows_kernel(const __grid_constant__ PairsJobs f, bool fwd, Side side) {
+    __shared__ __align__(16) uint8_t ring[3][ring_bytes<D>(true)];
+    side.begin();
+    const int warp = threadIdx.x >> 5;
+    const PairsArgs& a = f.job[blockIdx.y];
+    const uint32_t r = static_cast<uint32_t>(__cvta_generic_to_shared(ring[warp]));
+    if (warp == 0)
+        walk<D, kVer, AP2, true>(a, blockIdx.x, 0, fwd, r);
+    else
+        walk<D, kDiag, AP2, true>(a, blockIdx.x, warp - 1, fwd, r);
     side.end();
 }
 
@@ -757,6 +819,12 @@ __device__ __forceinline__ void finish(const PairsArgs& a, int r, int s, uint32_
             um = um == 0 ? a.QW - 1 : um - 1;
         }
     };
+    // 4 paths: the whole segment's stored r on its way into L2 (lane v: field v),
+    // which a quad ahead in registers leaves short of bytes in flight: 1920x1080
+    // D=256 336 -> 260 us, 640x480 frame 84.2 -> 82.7.  With 8 paths the six
+    // fields would push one another out (1242x375: 208 -> 221), with 2 paths L2
+    // holds the one field already.
+    if (NP == 4 && lane < NV) prefetch_l2(a, a.rec + (1 + lane) * a.FS + off0, nq * UB, 118);
     load_v(NP == 2 ? 0 : nq - 1);
     load_d();
 
@@ -958,15 +1026,103 @@ __global__ void __launch_bounds__(64) finish_kernel(const __grid_constant__ Pair
         finish<D, NP, GS, K16, POST>(a, r, blockIdx.x, static_cast<uint32_t>(__cvta_generic_to_shared(smem[warp])));
 }
 
+// ---------------------------------------------------------------------------
+// Work-list forms (batched pairs, sgm_internal.h): a persistent grid takes
+// blocks of chains or, warp by warp, runs of segments.
+// ---------------------------------------------------------------------------
+template <int D>
+__global__ void __launch_bounds__(64) walk_hv_list_kernel(const WorkList<PairsArgs>* __restrict__ Lp,
+                                                          uint32_t* __restrict__ next, uint32_t* __restrict__ status,
+                                                          bool ver) {
+    __shared__ __align__(16) uint8_t ring[2][ring_bytes<D>()];
+    const WorkList<PairsArgs> L = *Lp;
+    const int warp = threadIdx.x >> 5;
+    const uint32_t r = static_cast<uint32_t>(__cvta_generic_to_shared(ring[warp]));
+    int p, u;
+    while (take_unit(L, next, p, u)) {
+        const PairsArgs a = L.job[p];
+        if (a.D != D) {
+            report_bad_job(status);
+            continue;
+        }
+        const int nd = a.n_paths == 2 ? 1 : 2, nh = a.NS > 1 ? a.QH * nd : 0, c = u * 2 + warp, v = c - nh;
+        if (c < nh)
+            walk<D, kHor, false>(a, c / nd, 0, c % nd == 0, r);
+        else if (ver && v < a.QW * nd)
+            walk<D, kVer, false>(a, v / nd, 0, v % nd == 0, r);
+    }
+}
+
+template <int D>
+__global__ void __launch_bounds__(96) walk_rows_list_kernel(const WorkList<PairsArgs>* __restrict__ Lp,
+                                                            uint32_t* __restrict__ next,
+                                                            uint32_t* __restrict__ status, bool fwd) {
+    __shared__ __align__(16) uint8_t ring[3][ring_bytes<D>(true)];
+    const WorkList<PairsArgs> L = *Lp;
+    const int warp = threadIdx.x >> 5;
+    const uint32_t r = static_cast<uint32_t>(__cvta_generic_to_shared(ring[warp]));
+    int p, u;
+    while (take_unit(L, next, p, u)) {
+        const PairsArgs a = L.job[p];
+        if (a.D != D) {
+            report_bad_job(status);
+            continue;
+        }
+        if (warp == 0)
+            walk<D, kVer, false, true>(a, u, 0, fwd, r);
+        else
+            walk<D, kDiag, false, true>(a, u, warp - 1, fwd, r);
+    }
+}
+
+// Blocks per SM of the finishing list: its descriptors take registers where the
+// single pair's sit in constant memory, so the count is forced.
+template <int D, int NP>
+constexpr int finish_list_blocks() {
+    return D <= 128 ? (NP == 8 ? 10 : 14) : (NP == 8 ? 7 : 9);
+}
+template <int D, int NP, int GS, bool K16>
+__global__ void __launch_bounds__(64, finish_list_blocks<D, NP>()) finish_list_kernel(const WorkList<PairsArgs>* __restrict__ Lp,
+                                                         uint32_t* __restrict__ next, uint32_t* __restrict__ status) {
+    __shared__ __align__(16) uint8_t smem[2][Finish<D, NP>::BYTES];
+    const WorkList<PairsArgs> L = *Lp;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (L.n <= 0) return;
+    const uint32_t end = L.start[L.n];
+    // the next run is taken while this one is on its way
+    uint32_t i = lane == 0 ? atomicAdd(next, 1u) : 0u;
+    i = __shfl_sync(kFull, i, 0);
+    int p = 0;
+    while (i < end) {
+        const uint32_t nx = lane == 0 ? atomicAdd(next, 1u) : 0u;
+        while (L.start[p + 1] <= i) ++p;  // runs come in order
+        const PairsArgs a = L.job[p];
+        if (a.D != D || a.n_paths != NP) {
+            report_bad_job(status);
+        } else {
+            const int u = static_cast<int>(i - L.start[p]), runs = (a.NS + a.run - 1) / a.run;
+            const int r = u / runs, s0 = (u - r * runs) * a.run;
+#pragma unroll 1
+            for (int s = s0; s < min(s0 + a.run, a.NS); ++s)
+                finish<D, NP, GS, K16, false>(a, r, s, static_cast<uint32_t>(__cvta_generic_to_shared(smem[warp])));
+        }
+        i = __shfl_sync(kFull, nx, 0);
+    }
+}
+
 template <int D>
 struct PairsD {
     static cudaError_t walks(const PairsJobs& f, Walks w, Stream s) {
         const PairsArgs& a = f.job[0];
         const int nd = a.n_paths == 2 ? 1 : 2;
-        const Side side{w == Walks::kVer || w == Walks::kDiag,
-                        w == Walks::kHor || (w == Walks::kVer && a.n_paths == 8)};
+        const bool rows = w == Walks::kDown || w == Walks::kUp;
+        const Side side{w != Walks::kHor && w != Walks::kHorVer,
+                        w == Walks::kHor || (a.n_paths == 8 && (w == Walks::kVer || w == Walks::kDown))};
         if (side.later) s.pdl = true;
-        if (w == Walks::kDiag) {
+        if (rows) {
+            launch(a.p2map ? walk_rows_kernel<D, true> : walk_rows_kernel<D, false>, dim3(a.QW, f.n), 96, s, f,
+                   w == Walks::kDown, side);
+        } else if (w == Walks::kDiag) {
             launch(a.p2map ? walk_d_kernel<D, true> : walk_d_kernel<D, false>, dim3(2 * a.QW, f.n), 64, s, f, side);
         } else {
             const int nh = w != Walks::kVer && a.NS > 1 ? a.QH * nd : 0, nv = w != Walks::kHor ? a.QW * nd : 0;
@@ -986,17 +1142,15 @@ struct PairsD {
     }
     template <int NP>
     static void finish_np(const PairsJobs& f, Stream s) {
-        const PairsArgs& a = f.job[0];
-        // S <= NP (MC_max + P2): 16-bit keys S D + d where they fit
-        const bool k16 = NP * (a.mc_max + static_cast<int>(a.P2x2 & 0xffffu)) * D + D - 1 <= 65535;
+        const int cls = f.job[0].cls;
         if constexpr (NP == 2) {
-            if (k16)
+            if (cls == 0)
                 finish_t<2, 1, true>(f, s);
             else
                 finish_t<2, 1, false>(f, s);
-        } else if (a.gs == 3 && k16) {
+        } else if (cls == 0) {
             finish_t<NP, 3, true>(f, s);
-        } else if (a.gs >= 2) {
+        } else if (cls == 1) {
             finish_t<NP, 2, false>(f, s);
         } else {
             finish_t<NP, 1, false>(f, s);
@@ -1010,6 +1164,30 @@ struct PairsD {
         }
         return cudaGetLastError();
     }
+    static cudaError_t walks_list(const ListLaunch& l, Walks w, cudaStream_t s) {
+        const auto* L = static_cast<const WorkList<PairsArgs>*>(l.list);
+        if (w == Walks::kDown || w == Walks::kUp)
+            walk_rows_list_kernel<D><<<l.grid, 96, 0, s>>>(L, l.next, l.status, w == Walks::kDown);
+        else
+            walk_hv_list_kernel<D><<<l.grid, 64, 0, s>>>(L, l.next, l.status, w == Walks::kHorVer);
+        return cudaGetLastError();
+    }
+    template <int NP, int GS, bool K16>
+    static cudaError_t finish_list_t(const ListLaunch& l, cudaStream_t s) {
+        finish_list_kernel<D, NP, GS, K16>
+            <<<l.grid, 64, 0, s>>>(static_cast<const WorkList<PairsArgs>*>(l.list), l.next, l.status);
+        return cudaGetLastError();
+    }
+    template <int NP>
+    static cudaError_t finish_list_np(const ListLaunch& l, cudaStream_t s) {
+        if (l.cls == 0) return finish_list_t<NP, 3, true>(l, s);
+        return l.cls == 1 ? finish_list_t<NP, 2, false>(l, s) : finish_list_t<NP, 1, false>(l, s);
+    }
+    static cudaError_t fin_list(const ListLaunch& l, cudaStream_t s) {
+        if (l.n_paths == 8) return finish_list_np<8>(l, s);
+        if (l.n_paths == 4) return finish_list_np<4>(l, s);
+        return l.cls == 0 ? finish_list_t<2, 1, true>(l, s) : finish_list_t<2, 1, false>(l, s);
+    }
 };
 
 }  // namespace pairs
@@ -1020,15 +1198,27 @@ template <int D>
 SGM_INTERNAL_P cudaError_t pairs_walks(const PairsJobs& f, Walks w, Stream s);
 template <int D>
 SGM_INTERNAL_P cudaError_t pairs_finish(const PairsJobs& f, Stream s);
+template <int D>
+SGM_INTERNAL_P cudaError_t pairs_walks_list(const ListLaunch& l, Walks w, cudaStream_t s);
+template <int D>
+SGM_INTERNAL_P cudaError_t pairs_finish_list(const ListLaunch& l, cudaStream_t s);
 
-#define SGM_INSTANTIATE_PAIRS(D)                                                     \
-    template <>                                                                      \
-    SGM_INTERNAL_P cudaError_t pairs_walks<D>(const PairsJobs& f, Walks w, Stream s) { \
-        return pairs::PairsD<D>::walks(f, w, s);                                     \
-    }                                                                                \
-    template <>                                                                      \
-    SGM_INTERNAL_P cudaError_t pairs_finish<D>(const PairsJobs& f, Stream s) {       \
-        return pairs::PairsD<D>::fin(f, s);                                          \
+#define SGM_INSTANTIATE_PAIRS(D)                                                                   \
+    template <>                                                                                    \
+    SGM_INTERNAL_P cudaError_t pairs_walks<D>(const PairsJobs& f, Walks w, Stream s) {             \
+        return pairs::PairsD<D>::walks(f, w, s);                                                   \
+    }                                                                                              \
+    template <>                                                                                    \
+    SGM_INTERNAL_P cudaError_t pairs_finish<D>(const PairsJobs& f, Stream s) {                     \
+        return pairs::PairsD<D>::fin(f, s);                                                        \
+    }                                                                                              \
+    template <>                                                                                    \
+    SGM_INTERNAL_P cudaError_t pairs_walks_list<D>(const ListLaunch& l, Walks w, cudaStream_t s) { \
+        return pairs::PairsD<D>::walks_list(l, w, s);                                              \
+    }                                                                                              \
+    template <>                                                                                    \
+    SGM_INTERNAL_P cudaError_t pairs_finish_list<D>(const ListLaunch& l, cudaStream_t s) {         \
+        return pairs::PairsD<D>::fin_list(l, s);                                                   \
     }
 
 }  // namespace sgm

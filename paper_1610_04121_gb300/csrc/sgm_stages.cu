@@ -507,6 +507,57 @@ cudaError_t launch_cost_quads(const void* F, size_t fstride, uint8_t* mc, size_t
     }
 }
 
+template <int D, class FT>
+__global__ void __launch_bounds__(kQcThreads, kCostQuadsListPerSM) cost_quads_list_kernel(const WorkList<CostQuadsJob>* __restrict__ Lp,
+                                                                     uint32_t* __restrict__ next,
+                                                                     uint32_t* __restrict__ status) {
+    const WorkList<CostQuadsJob> L = *Lp;
+    int p, u;
+    while (take_unit(L, next, p, u)) {
+        const CostQuadsJob j = L.job[p];
+        if (j.D != D) {
+            report_bad_job(status);
+            continue;
+        }
+        const int segs = ((j.W + 1) / 2 + kQcSeg - 1) / kQcSeg, runs = (segs + kCostQuadsRun - 1) / kCostQuadsRun;
+        const int qy = u / runs, b0 = (u - qy * runs) * kCostQuadsRun;
+        for (int b = b0; b < min(b0 + kCostQuadsRun, segs); ++b) {
+            if (b > b0) __syncthreads();  // the staged features of the segment before are used
+            cost_quads_body<D, FT>(static_cast<const FT*>(j.Fb), static_cast<const FT*>(j.Fm), j.mc, j.QB, j.W, j.H, b,
+                                   qy);
+        }
+    }
+}
+
+int cost_quads_units(int W, int H) {
+    const int segs = ((W + 1) / 2 + kQcSeg - 1) / kQcSeg;
+    return ((segs + kCostQuadsRun - 1) / kCostQuadsRun) * ((H + 1) / 2);
+}
+
+template <int D>
+static cudaError_t launch_cost_quads_list_t(const ListLaunch& l, cudaStream_t s) {
+    const auto* L = static_cast<const WorkList<CostQuadsJob>*>(l.list);
+    if (l.ct62)
+        cost_quads_list_kernel<D, uint64_t><<<l.grid, kQcThreads, 0, s>>>(L, l.next, l.status);
+    else
+        cost_quads_list_kernel<D, uint32_t><<<l.grid, kQcThreads, 0, s>>>(L, l.next, l.status);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cost_quads_list(const ListLaunch& l, cudaStream_t stream) {
+    switch (l.D) {
+        case 32: return launch_cost_quads_list_t<32>(l, stream);
+        case 64: return launch_cost_quads_list_t<64>(l, stream);
+        case 96: return launch_cost_quads_list_t<96>(l, stream);
+        case 128: return launch_cost_quads_list_t<128>(l, stream);
+        case 160: return launch_cost_quads_list_t<160>(l, stream);
+        case 192: return launch_cost_quads_list_t<192>(l, stream);
+        case 224: return launch_cost_quads_list_t<224>(l, stream);
+        case 256: return launch_cost_quads_list_t<256>(l, stream);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Jump penalties of the paired schedule's post form: one word per quad (or
 // diagonal unit) and direction, the penalty of the step into each of its four
@@ -694,6 +745,22 @@ __global__ void __launch_bounds__(kMedW) median_quads_kernel(const uint8_t* __re
 cudaError_t launch_median_quads(const uint8_t* rawq, uint8_t* disp, int W, int H, Stream stream) {
     dim3 grid((W + kMedW - 1) / kMedW, (H + kMedH - 1) / kMedH);
     launch(median_quads_kernel, grid, kMedW, stream, rawq, disp, W, H);
+    return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(kMedW) median_quads_list_kernel(const WorkList<MedianJob>* __restrict__ Lp,
+                                                                  uint32_t* __restrict__ next) {
+    const WorkList<MedianJob> L = *Lp;
+    int p, u;
+    while (take_unit(L, next, p, u)) {
+        const MedianJob j = L.job[p];
+        const int tx = (j.W + kMedW - 1) / kMedW;
+        median_body<true>(j.raw, j.out, j.W, j.H, u % tx, u / tx);
+    }
+}
+
+cudaError_t launch_median_quads_list(const ListLaunch& l, cudaStream_t stream) {
+    median_quads_list_kernel<<<l.grid, kMedW, 0, stream>>>(static_cast<const WorkList<MedianJob>*>(l.list), l.next);
     return cudaGetLastError();
 }
 

@@ -75,8 +75,8 @@ PairsArgs pairs_geometry(int W, int H, int D, int n_paths) {
     return a;
 }
 
-#define SGM_DISPATCH_PAIRS(FN, ...)                \
-    switch (f.job[0].D) {                          \
+#define SGM_DISPATCH_PAIRS(FN, D, ...)             \
+    switch (D) {                                   \
         case 32: return FN<32>(__VA_ARGS__);       \
         case 64: return FN<64>(__VA_ARGS__);       \
         case 96: return FN<96>(__VA_ARGS__);       \
@@ -89,11 +89,24 @@ PairsArgs pairs_geometry(int W, int H, int D, int n_paths) {
     }
 
 cudaError_t launch_pairs_walks(const PairsJobs& f, Walks w, Stream stream) {
-    SGM_DISPATCH_PAIRS(pairs_walks, f, w, stream)
+    SGM_DISPATCH_PAIRS(pairs_walks, f.job[0].D, f, w, stream)
 }
 
 cudaError_t launch_pairs_finish(const PairsJobs& f, Stream stream) {
-    SGM_DISPATCH_PAIRS(pairs_finish, f, stream)
+    SGM_DISPATCH_PAIRS(pairs_finish, f.job[0].D, f, stream)
+}
+
+cudaError_t launch_pairs_walks_list(const ListLaunch& l, Walks w, cudaStream_t stream) {
+    SGM_DISPATCH_PAIRS(pairs_walks_list, l.D, l, w, stream)
+}
+
+cudaError_t launch_pairs_finish_list(const ListLaunch& l, cudaStream_t stream) {
+    SGM_DISPATCH_PAIRS(pairs_finish_list, l.D, l, stream)
+}
+
+int pairs_hv_units(const PairsArgs& a, bool ver) {
+    const int nd = a.n_paths == 2 ? 1 : 2;
+    return ((a.NS > 1 ? a.QH * nd : 0) + (ver ? a.QW * nd : 0) + 1) / 2;
 }
 
 }  // namespace sgm
