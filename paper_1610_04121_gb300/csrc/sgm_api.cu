@@ -488,13 +488,12 @@ static bool is_device_ptr(const void* p) {
 // kernel.  The paired schedule: census, cost, the walks (one kernel with 2
 // paths; horizontal and vertical walks with 4, horizontal, downward and upward
 // walks with 8 paths side by side: one timed stage), the finishing launch, median or post; both passes of the
-// LR check in the same launches, the jump penalties of adaptive P2 one launch
-// per pass.
+// LR check in the same launches, the jump penalties of adaptive P2 one more.
 static int walk_launches(const Problem& p) { return p.n_paths == 8 ? 3 : (p.n_paths == 4 ? 2 : 1); }
 static int launches_per_match(const Problem& p) { return p.n_paths == 8 ? 6 : 4; }
 static int launches_per_path(const Problem& p) {
     const int passes = (p.post & SGM_POST_LR_CHECK) ? 2 : 1;
-    if (pairs_sched(p)) return 4 + walk_launches(p) + ((p.post & SGM_POST_ADAPTIVE_P2) ? passes : 0);
+    if (pairs_sched(p)) return 4 + walk_launches(p) + ((p.post & SGM_POST_ADAPTIVE_P2) ? 1 : 0);
     if (!p.post) return launches_per_match(p) + 1;
     return launches_per_match(p) * passes + (passes - 1) + 1;
 }
@@ -527,15 +526,14 @@ static cudaError_t enqueue_pairs(const Problem& p, const Layout& l, uint8_t* are
         g.P2x2 = static_cast<uint32_t>(p.P2) * 0x10001u;
         g.cls = pairs_class(p.n_paths, p.D, p2_max(p), mc_max(p));
         g.check_shrink = p.check_shrink;
-        if (p.post & SGM_POST_ADAPTIVE_P2) {
-            uint32_t* map = reinterpret_cast<uint32_t*>(arena + l.p2map + k * l.p2_stride);
-            if ((e = launch_p2map(k ? right : left, k != 0, map, p.n_paths, p.W, p.H, p.P1, p.P2, s)) != cudaSuccess)
-                return e;
-            g.p2map = map;
-        }
+        if (p.post & SGM_POST_ADAPTIVE_P2) g.p2map = reinterpret_cast<uint32_t*>(arena + l.p2map + k * l.p2_stride);
         if (k == 0 && (p.post & SGM_POST_SUBPIXEL)) g.subq = reinterpret_cast<uint32_t*>(arena + l.sub);
         f.job[k] = g;
     }
+    if ((p.post & SGM_POST_ADAPTIVE_P2) &&
+        (e = launch_p2map(left, right, reinterpret_cast<uint32_t*>(arena + l.p2map), l.p2_stride / 4, l.passes,
+                          p.n_paths, p.W, p.H, p.P1, p.P2, s)) != cudaSuccess)
+        return e;
     if ((e = mark()) != cudaSuccess) return e;
     // every direction at once
     const int n = walk_launches(p);

@@ -260,10 +260,11 @@ cudaError_t launch_census_passes(const uint8_t* left, const uint8_t* right, void
 // into mc + k mcstride, quad q at + q QB.
 cudaError_t launch_cost_quads(const void* F, size_t fstride, uint8_t* mc, size_t mcstride, int passes, int QB, int W,
                               int H, int D, bool ct62, Stream stream);
-// Jump penalties max(P1, P2 / (1 + g)) of every step (PairsArgs::p2map): base
-// image img, or its mirror image.
-cudaError_t launch_p2map(const uint8_t* img, bool mirror, uint32_t* map, int n_paths, int W, int H, int P1, int P2,
-                         Stream stream);
+// Jump penalties max(P1, P2 / (1 + g)) of every step (PairsArgs::p2map), pass k
+// into map + k stride words: base image left, and for the second pass the
+// mirrored right image.
+cudaError_t launch_p2map(const uint8_t* left, const uint8_t* right, uint32_t* map, size_t stride, int passes,
+                         int n_paths, int W, int H, int P1, int P2, Stream stream);
 // The walks of a path, side by side: horizontal, vertical and, with 8 paths,
 // diagonal pairs; with 8 paths over a cube larger than L2, horizontal pair,
 // directions that go down and directions that go up; or both directions of 2

@@ -928,7 +928,6 @@ __device__ __forceinline__ void finish(const PairsArgs& a, int r, int s, uint32_
             }
         }
         uint32_t word = 0;
-        uint4 subv = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             const int h = NP == 2 ? t : 1 - t;  // column of the quad
@@ -979,36 +978,31 @@ __device__ __forceinline__ void finish(const PairsArgs& a, int r, int s, uint32_
                 }
             }
             if constexpr (POST) {
-                if (a.subq) {  // S(d-1) - S(d) | (S(d+1) - S(d)) << 16 at each line's winner
-                    auto s_at = [&](int e, int half) -> uint32_t {
-                        const int l = e / K, jj = e - l * K;
-                        uint32_t w = S[0];
-#pragma unroll
-                        for (int j = 1; j < K; ++j) w = jj == j ? S[j] : w;
-                        w = __shfl_sync(kFull, w, l);
-                        return half ? w >> 16 : w & 0xffffu;
-                    };
-#pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        const uint32_t key = half ? kB : kA, Sd = key >> 16;
-                        const int d = static_cast<int>(key & 0xffu);
-                        const uint32_t al = d > 0 ? s_at(d - 1, half) - Sd : 0u;
-                        const uint32_t ga = d + 1 < D ? s_at(d + 1, half) - Sd : 0u;
-                        const uint32_t v = al | ga << 16;
-                        if (half)
-                            (h ? subv.w : subv.z) = v;
-                        else
-                            (h ? subv.y : subv.x) = v;
+                if (a.subq) {
+                    // S(d-1) - S(d) | (S(d+1) - S(d)) << 16 at each line's winner: S by
+                    // disparity in shared memory, lane 2 h takes S(d-1) of line h,
+                    // lane 2 h + 1 S(d+1)
+                    const uint32_t sums = smem + F::BYTES;
+                    __syncwarp();
+                    sts_unit<K>(sums + 4 * K * lane, S);
+                    __syncwarp();
+                    const uint32_t key = lane & 2 ? kB : kA;
+                    const int d = static_cast<int>(key & 0xffu), e = lane & 1 ? d + 1 : d - 1;
+                    uint32_t v = 0;
+                    if (lane < 4 && e >= 0 && e < D) {
+                        uint32_t w;
+                        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w) : "r"(sums + 4 * e));
+                        v = (lane & 2 ? w >> 16 : w & 0xffffu) - (key >> 16);
                     }
+                    v |= __shfl_down_sync(kFull, v, 1) << 16;
+                    const size_t q = 4 * (static_cast<size_t>(r) * a.QW + q0 + i) + h + (lane & 2);
+                    if ((lane == 0 || lane == 2) &&
+                        SGM_GUARD_INDEX(static_cast<long long>(q), 4ll * a.QW * a.QH, 117))
+                        a.subq[q] = v;
                 }
             }
         }
         rawv = lane == i ? word : rawv;
-        if constexpr (POST) {
-            const size_t q = static_cast<size_t>(r) * a.QW + q0 + i;
-            if (a.subq && lane == 0 && SGM_GUARD_INDEX(static_cast<long long>(q), static_cast<long long>(a.QW) * a.QH, 117))
-                reinterpret_cast<uint4*>(a.subq)[q] = subv;
-        }
     }
     const size_t q = static_cast<size_t>(r) * a.QW + q0 + lane;
     if (lane < nq && SGM_GUARD_INDEX(static_cast<long long>(q), static_cast<long long>(a.QW) * a.QH, 116))
@@ -1017,7 +1011,7 @@ __device__ __forceinline__ void finish(const PairsArgs& a, int r, int s, uint32_
 
 template <int D, int NP, int GS, bool K16, bool POST>
 __global__ void __launch_bounds__(64) finish_kernel(const __grid_constant__ PairsJobs f) {
-    __shared__ __align__(16) uint8_t smem[2][Finish<D, NP>::BYTES];
+    __shared__ __align__(16) uint8_t smem[2][Finish<D, NP>::BYTES + (POST ? 4 * D : 0)];  // post form: S of a column
     pdl_wait();
     const int warp = threadIdx.x >> 5;
     const PairsArgs& a = f.job[blockIdx.z];
