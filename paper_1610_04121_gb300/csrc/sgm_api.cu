@@ -1143,7 +1143,7 @@ static size_t build_lists(sgm_ctx* ctx, ListExec& x, const std::vector<BatchItem
                 dj[k] = MedianJob{base + l.raw, is_device_ptr(it.out) ? it.out : base + l.out, p.W, p.H};
                 const int units[kListStages] = {census_units(p.W, p.H), cost_quads_units(p.W, p.H),
                                                 pairs_hv_units(a, p.n_paths != 8), a.QW, pairs_finish_units(a),
-                                                median_units(p.W, p.H)};
+                                                median_quads_units(p.W, p.H)};
                 for (int i = 0; i < kListStages; ++i) st[i][k + 1] = st[i][k] + units[i];
             }
             const int ni = static_cast<int>(n);

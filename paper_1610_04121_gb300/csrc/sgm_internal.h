@@ -181,6 +181,7 @@ int census_units(int W, int H);
 int cost_units(int W, int H);
 int sweep_units(int lines, int D, bool pair);
 int median_units(int W, int H);
+int median_quads_units(int W, int H);
 constexpr int kCensusListPerSM = 16, kCostListPerSM = 8, kMedianListPerSM = 8, kSweepListMaxPerSM = 5;
 // Debug: paired costs (offset 0 of RB-byte records) -> natural order [H][W][D].
 cudaError_t launch_unpair_cost(const uint8_t* rec, int RB, uint8_t* out, int W, int H, int D, cudaStream_t stream);

@@ -676,17 +676,10 @@ __device__ __forceinline__ int med3(int a, int b, int c) { return max(min(a, b),
 // sorted once and shared by the three windows that contain the row.
 constexpr int kMedW = 128, kMedH = 4;
 
-// QUAD: raw in quads of 2 x 2 pixels ([ceil(H/2)][ceil(W/2)][4], pixel (x, y)
-// at byte (x & 1) + 2 (y & 1) of its quad), else row-major [H][W].
-template <bool QUAD = false>
 __device__ __forceinline__ int raw_at(const uint8_t* __restrict__ raw, int W, int x, int y) {
-    if constexpr (QUAD)
-        return __ldg(raw + ((size_t)(y >> 1) * ((W + 1) >> 1) + (x >> 1)) * 4 + (x & 1) + 2 * (y & 1));
-    else
-        return SGM_GUARD_INDEX(x, W, 307) ? __ldg(raw + (size_t)y * W + x) : 0;
+    return SGM_GUARD_INDEX(x, W, 307) ? __ldg(raw + (size_t)y * W + x) : 0;
 }
 
-template <bool QUAD = false>
 __device__ __forceinline__ void median_body(const uint8_t* __restrict__ raw, uint8_t* __restrict__ out, int W, int H,
                                             int bx, int by) {
     const int x = bx * kMedW + threadIdx.x, y0 = by * kMedH;
@@ -696,9 +689,9 @@ __device__ __forceinline__ void median_body(const uint8_t* __restrict__ raw, uin
 #pragma unroll
     for (int r = 0; r < kMedH + 2; ++r) {
         const int gy = min(max(y0 - 1 + r, 0), H - 1);
-        lo[r] = raw_at<QUAD>(raw, W, xl, gy);
-        mid[r] = raw_at<QUAD>(raw, W, x, gy);
-        hi[r] = raw_at<QUAD>(raw, W, xr, gy);
+        lo[r] = raw_at(raw, W, xl, gy);
+        mid[r] = raw_at(raw, W, x, gy);
+        hi[r] = raw_at(raw, W, xr, gy);
     }
     int c[kMedH];  // raw centre values: the border ring keeps them
 #pragma unroll
@@ -751,31 +744,101 @@ cudaError_t launch_median(const uint8_t* raw, uint8_t* disp, int W, int H, Strea
     return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(kMedW) median_quads_kernel(const uint8_t* __restrict__ rawq,
-                                                           uint8_t* __restrict__ out, int W, int H) {
-    pdl_wait();
-    median_body<true>(rawq, out, W, H, blockIdx.x, blockIdx.y);
+// The median of the quad layout ([ceil(H/2)][ceil(W/2)][4], pixel (x, y) at byte
+// (x & 1) + 2 (y & 1) of its quad): a thread takes kMedQH quads of a quad
+// column, two pixels at a time in the halves of a word.  The quads left and
+// right of it complete the three columns of both pixels.
+// Bound: the launch itself (2.9 us at 640x480, 5.0 at 1920x1080).  One pixel per
+// thread column with eighteen byte loads took 3.4 and 9: 640x480 D=128 frame
+// 79.8 -> 79.4 us, 1920x1080 D=128 8 paths 946.9 -> 942.7.
+constexpr int kMedQW = 64, kMedQH = 2;
+
+__device__ __forceinline__ uint32_t vmax2(uint32_t a, uint32_t b) { return __vmaxu2(a, b); }
+__device__ __forceinline__ uint32_t med3_2(uint32_t a, uint32_t b, uint32_t c) {
+    return vmax2(vmin2(a, b), vmin2(vmax2(a, b), c));
 }
 
+__device__ __forceinline__ void median_quads_body(const uint8_t* __restrict__ rawq, uint8_t* __restrict__ out, int W,
+                                                  int H, int bx, int by) {
+    const int QW = (W + 1) / 2, QH = (H + 1) / 2, qx = bx * kMedQW + threadIdx.x, qy0 = by * kMedQH;
+    if (qx >= QW) return;
+    const uint32_t* q = reinterpret_cast<const uint32_t*>(rawq);
+    const int ql = max(qx - 1, 0), qr = min(qx + 1, QW - 1);
+    uint32_t wl[kMedQH + 2], wm[kMedQH + 2], wr[kMedQH + 2];
+#pragma unroll
+    for (int k = 0; k < kMedQH + 2; ++k) {
+        const size_t row = static_cast<size_t>(min(max(qy0 - 1 + k, 0), QH - 1)) * QW;
+        wl[k] = __ldg(q + row + ql);
+        wm[k] = __ldg(q + row + qx);
+        wr[k] = __ldg(q + row + qr);
+    }
+    // rows 2 qy0 - 1 .. 2 qy0 + 2 kMedQH of the image, sorted
+    constexpr int NR = 2 * kMedQH + 2;
+    uint32_t lo[NR], mid[NR], hi[NR], c[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int k = (r + 1) / 2;
+        const bool odd = (r & 1) == 0;  // the second row of its quads
+        c[r] = __byte_perm(wm[k], 0u, odd ? 0x4342u : 0x4140u);                // pixels x, x + 1
+        const uint32_t l = __byte_perm(c[r], wl[k], odd ? 0x1017u : 0x1015u);  // x - 1, x
+        const uint32_t h = __byte_perm(c[r], wr[k], odd ? 0x1612u : 0x1412u);  // x + 1, x + 2
+        const uint32_t a = vmin2(l, c[r]), b = vmax2(l, c[r]), m = vmax2(a, h);
+        lo[r] = vmin2(a, h);
+        mid[r] = vmin2(m, b);
+        hi[r] = vmax2(m, b);
+    }
+    const int x = 2 * qx;
+    const uint32_t inner = (x > 0 && x < W - 1 ? 0xffffu : 0u) | (x + 1 < W - 1 ? 0xffff0000u : 0u);
+    const bool two = x + 1 < W, pairs = (W & 1) == 0 && (reinterpret_cast<uintptr_t>(out) & 1) == 0;
+#pragma unroll
+    for (int k = 0; k < 2 * kMedQH; ++k) {
+        const int y = 2 * qy0 + k;
+        if (y >= H) break;
+        const uint32_t l = vmax2(vmax2(lo[k], lo[k + 1]), lo[k + 2]);
+        const uint32_t m = med3_2(mid[k], mid[k + 1], mid[k + 2]);
+        const uint32_t h = vmin2(vmin2(hi[k], hi[k + 1]), hi[k + 2]);
+        const uint32_t in = y > 0 && y < H - 1 ? inner : 0u;
+        const uint32_t v = (med3_2(l, m, h) & in) | (c[k + 1] & ~in);
+        if (!SGM_GUARD_INDEX((long long)y * W + x + (two ? 1 : 0), (long long)W * H, 308)) continue;
+        uint8_t* o = out + static_cast<size_t>(y) * W + x;
+        if (pairs) {
+            *reinterpret_cast<uint16_t*>(o) = static_cast<uint16_t>(__byte_perm(v, 0u, 0x4420u));
+        } else {
+            o[0] = static_cast<uint8_t>(v);
+            if (two) o[1] = static_cast<uint8_t>(v >> 16);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kMedQW) median_quads_kernel(const uint8_t* __restrict__ rawq,
+                                                              uint8_t* __restrict__ out, int W, int H) {
+    pdl_wait();
+    median_quads_body(rawq, out, W, H, blockIdx.x, blockIdx.y);
+}
+
+static int median_quads_across(int W) { return ((W + 1) / 2 + kMedQW - 1) / kMedQW; }
+static int median_quads_down(int H) { return ((H + 1) / 2 + kMedQH - 1) / kMedQH; }
+
 cudaError_t launch_median_quads(const uint8_t* rawq, uint8_t* disp, int W, int H, Stream stream) {
-    dim3 grid((W + kMedW - 1) / kMedW, (H + kMedH - 1) / kMedH);
-    launch(median_quads_kernel, grid, kMedW, stream, rawq, disp, W, H);
+    launch(median_quads_kernel, dim3(median_quads_across(W), median_quads_down(H)), kMedQW, stream, rawq, disp, W, H);
     return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(kMedW) median_quads_list_kernel(const WorkList<MedianJob>* __restrict__ Lp,
-                                                                  uint32_t* __restrict__ next) {
+__global__ void __launch_bounds__(kMedQW) median_quads_list_kernel(const WorkList<MedianJob>* __restrict__ Lp,
+                                                                   uint32_t* __restrict__ next) {
     const WorkList<MedianJob> L = *Lp;
     int p, u;
     while (take_unit(L, next, p, u)) {
         const MedianJob j = L.job[p];
-        const int tx = (j.W + kMedW - 1) / kMedW;
-        median_body<true>(j.raw, j.out, j.W, j.H, u % tx, u / tx);
+        const int tx = ((j.W + 1) / 2 + kMedQW - 1) / kMedQW;
+        median_quads_body(j.raw, j.out, j.W, j.H, u % tx, u / tx);
     }
 }
 
+int median_quads_units(int W, int H) { return median_quads_across(W) * median_quads_down(H); }
+
 cudaError_t launch_median_quads_list(const ListLaunch& l, cudaStream_t stream) {
-    median_quads_list_kernel<<<l.grid, kMedW, 0, stream>>>(static_cast<const WorkList<MedianJob>*>(l.list), l.next);
+    median_quads_list_kernel<<<l.grid, kMedQW, 0, stream>>>(static_cast<const WorkList<MedianJob>*>(l.list), l.next);
     return cudaGetLastError();
 }
 
