@@ -33,6 +33,16 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // The next kernel of the stream may start once every block of this one has come here.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A value the compiler cannot see: multiplying by it stays a multiply-add on
+// the FMA pipe instead of becoming a shift on the integer ALU, the pipe these
+// kernels run out of first (both take two cycles per warp instruction).
+__device__ __forceinline__ uint32_t opaque(uint32_t v) {
+    uint32_t r;
+    asm("mov.b32 %0, %1;" : "=r"(r) : "r"(v));
+    asm volatile("" : "+r"(r));
+    return r;
+}
+
 __device__ __forceinline__ uint32_t vmin2(uint32_t a, uint32_t b) {
     uint32_t d;
     asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));

@@ -231,15 +231,6 @@ __device__ __forceinline__ void stg_unit(const PairsArgs& a, uint8_t* p, const u
     }
 }
 
-// A value the compiler cannot see: multiplying by it stays a multiply-add on
-// the FMA pipe instead of becoming a shift on the integer ALU, the pipe these
-// kernels run out of first (both take two cycles per warp instruction).
-__device__ __forceinline__ uint32_t opaque(uint32_t v) {
-    uint32_t r;
-    asm("mov.b32 %0, %1;" : "=r"(r) : "r"(v));
-    asm volatile("" : "+r"(r));
-    return r;
-}
 __device__ __forceinline__ uint32_t mad(uint32_t a, uint32_t b, uint32_t c) {
     uint32_t d;
     asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));

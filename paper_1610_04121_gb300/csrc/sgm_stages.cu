@@ -10,87 +10,96 @@ namespace sgm {
 
 // ---------------------------------------------------------------------------
 // Eq. 1: 9x7 center-symmetric Census transform.  A CTA of kCtT threads covers
-// a kCtW x kCtH tile (kCtW = 2 kCtT): the (kCtW+8) x (kCtH+6) bytes around it
+// a tile of kCtW = 2 kCtT columns and kCtH (kCtSmallH) rows: the bytes around it
 // are staged in shared memory (the read-cooperative 2D tiling of Section 3.1)
 // and each thread walks two adjacent columns of the tile downwards with the
 // 7 x 10 window they share in registers, loading one new row of 10 bytes per
 // pair of pixels; blockIdx.z picks the image.  The feature is 0 where the 9x7
-// window leaves the image.
+// window leaves the image.  Bound: latency and instructions (two images of
+// 640x480 5.0 us, of 1920x1080 16.2; 20 one pixel at a time).
 // Bit k follows the printed order of Eq. 1: i = 1..4, j = -3..3 give bit
 // (i-1)*7 + j+3; the i = 0 pairs j = 1..3 give bits 28..30; s(u,v) = u >= v.
-// Each bit costs two instructions: for bytes u, v the value v + ~u = v - u - 1
-// is negative exactly when u >= v, and a funnel shift moves its sign bit in
-// below the bits already collected (highest bit first).  The 31 bits are
-// gathered as four independent 8-bit chains joined by byte permutes, which
-// keeps the dependent chain per pixel short.
 // ---------------------------------------------------------------------------
-constexpr int kCtT = 32, kCtW = 2 * kCtT, kCtH = 4;
+constexpr int kCtT = 32, kCtW = 2 * kCtT, kCtH = 4, kCtSmallH = 2;
 
-// Census feature of the pixel whose 9 window columns start at column c0 of
-// the window rows; row k of the window (image y - 3 + k) is win[(r + k) % 7].
-template <int NC>
-__device__ __forceinline__ uint32_t census_feature(const uint32_t (&win)[7][NC], int r, int c0) {
-    auto diff = [&](int b) -> uint32_t {
-        int i, j;
-        if (b >= 28) {
-            i = 0;
-            j = b - 27;  // bits 28..30: i = 0, j = 1..3
-        } else {
-            i = b / 7 + 1;
-            j = b % 7 - 3;  // bit (i-1)*7 + j+3
+// Two horizontal neighbours at a time, in the halves of a word: for u, v below
+// 256 bit 8 of u - v + 256 is set exactly when u >= v, and a multiply-add (on
+// the FMA pipe, `pow` holding 1, 2 .. 128 as values the compiler does not know)
+// puts it where it belongs: three instructions for two bits, two of them on the
+// ALU (four on the ALU with one pixel at a time; with the word loads below
+// 640x480 D=128 frame 79.4 -> 78.7 us, 1920x1080 D=256 900 -> 892, full Census
+// 641x479 86.9 -> 85.9).
+// win[r % 7][c] holds columns c, c + 1 of window row r; row k of the window
+// (image y - 3 + k) is win[(r + k) % 7].  f0, f1: the features of both pixels.
+template <class FT>
+__device__ __forceinline__ void census_pair(const uint32_t (&win)[7][9], int r, const uint32_t (&pow)[8], FT& f0,
+                                            FT& f1) {
+    constexpr int BITS = sizeof(FT) == 8 ? 62 : 31, NQ = (BITS + 7) / 8;
+    uint32_t c[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        c[q] = 0u;
+#pragma unroll
+        for (int b = q * 8; b < q * 8 + 8 && b < BITS; ++b) {
+            uint32_t u, v;
+            if constexpr (sizeof(FT) == 8) {
+                // full Census: window position b in row-major order, the centre (31) skipped
+                const int idx = b < 31 ? b : b + 1, j = idx / 9 - 3, i = idx % 9 - 4;
+                u = win[(r + 3 + j) % 7][4 + i];
+                v = win[(r + 3) % 7][4];
+            } else {
+                const int i = b >= 28 ? 0 : b / 7 + 1, j = b >= 28 ? b - 27 : b % 7 - 3;
+                u = win[(r + 3 + j) % 7][4 + i];
+                v = win[(r + 3 - j) % 7][4 - i];
+            }
+            const uint32_t bit = (u - v + 0x01000100u) & 0x01000100u;
+            asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(c[q]) : "r"(bit), "r"(pow[b & 7]));
         }
-        // sign bit set when I(x+i, y+j) >= I(x-i, y-j)
-        return win[(r + 3 - j) % 7][c0 + 4 - i] + ~win[(r + 3 + j) % 7][c0 + 4 + i];
+    }
+    auto word = [&](int q, uint32_t lo, uint32_t join) -> uint32_t {  // byte 1 or 3 of four accumulators
+        return __byte_perm(__byte_perm(c[q], c[q + 1], lo), __byte_perm(c[q + 2], c[q + 3], lo), join);
     };
-    uint32_t c[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int b = q * 8 + 7; b >= q * 8; --b)  // highest bit of the byte first
-            if (b < 31) c[q] = __funnelshift_l(diff(b), c[q], 1);
-    return __byte_perm(__byte_perm(c[0], c[1], 0x0040u), __byte_perm(c[2], c[3], 0x0040u), 0x5410u);
-}
-
-// The full 9x7 Census (the CT Section 2 contrasts CSCT with): bit k compares
-// the k-th window pixel in row-major order (rows j = -3..3, columns
-// i = -4..4, the centre skipped) with the centre, s(I(x+i, y+j), I(x, y));
-// 62 bits gathered as eight 8-bit chains (the sign of I(x, y) + ~I(x+i, y+j)
-// is set exactly when I(x+i, y+j) >= I(x, y)).
-template <int NC>
-__device__ __forceinline__ uint64_t census62_feature(const uint32_t (&win)[7][NC], int r, int c0) {
-    auto diff = [&](int b) -> uint32_t {
-        const int idx = b < 31 ? b : b + 1;  // window position, the centre (31) skipped
-        const int j = idx / 9 - 3, i = idx % 9 - 4;
-        return win[(r + 3) % 7][c0 + 4] + ~win[(r + 3 + j) % 7][c0 + 4 + i];
-    };
-    uint32_t c[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-#pragma unroll
-        for (int b = q * 8 + 7; b >= q * 8; --b)  // highest bit of the byte first
-            if (b < 62) c[q] = __funnelshift_l(diff(b), c[q], 1);
-    const uint32_t lo =
-        __byte_perm(__byte_perm(c[0], c[1], 0x0040u), __byte_perm(c[2], c[3], 0x0040u), 0x5410u);
-    const uint32_t hi =
-        __byte_perm(__byte_perm(c[4], c[5], 0x0040u), __byte_perm(c[6], c[7], 0x0040u), 0x5410u);
-    return static_cast<uint64_t>(hi) << 32 | lo;
+    f0 = word(0, 0x0051u, 0x5410u);
+    f1 = word(0, 0x0073u, 0x5410u);
+    if constexpr (sizeof(FT) == 8) {
+        f0 |= static_cast<uint64_t>(word(4, 0x0051u, 0x5410u)) << 32;
+        f1 |= static_cast<uint64_t>(word(4, 0x0073u, 0x5410u)) << 32;
+    }
 }
 
 // CT = false: the CSCT of Eq. 1 into uint32 features; CT = true: the full
 // 9x7 Census into uint64 features.
-template <bool CT>
+template <bool CT, int TILE_H = kCtH>
 __device__ __forceinline__ void census_body(const uint8_t* __restrict__ left, const uint8_t* __restrict__ right,
                                             void* __restrict__ Fb, void* __restrict__ Fm, int W, int H, int bx,
                                             int by, int bz, bool mirror = false) {
     using FT = typename std::conditional<CT, uint64_t, uint32_t>::type;
-    constexpr int TW = kCtW + 8, TH = kCtH + 6, NS = (TW + kCtT - 1) / kCtT;
-    __shared__ uint8_t tile[TH][TW];
+    constexpr int TW = kCtW + 8, TH = TILE_H + 6, NS = (TW + kCtT - 1) / kCtT, TW4 = TW / 4;
+    __shared__ __align__(4) uint8_t tile[TH][TW];
     const uint8_t* img = bz ? right : left;
     FT* F = static_cast<FT*>(bz ? Fm : Fb);
-    const int x0 = bx * kCtW, y0 = by * kCtH;
-    // Thread t stages tile columns t, t + kCtT, ...: all loads are issued
-    // before the first shared-memory store.
-    {
+    const int x0 = bx * kCtW, y0 = by * TILE_H;
+    // All loads are issued before the first shared-memory store: words where
+    // rows and image start on a word boundary (the tile does too: a word lies
+    // within the row or outside it, mirrored or not), else thread t takes the
+    // bytes of tile columns t, t + kCtT, ...
+    if ((W & 3) == 0 && (reinterpret_cast<uintptr_t>(img) & 3) == 0) {
+        constexpr int N4 = (TW4 * TH + kCtT - 1) / kCtT;
+        uint32_t v[N4];
+#pragma unroll
+        for (int h = 0; h < N4; ++h) {
+            const int i = threadIdx.x + h * kCtT, ty = i / TW4, gx = x0 - 4 + 4 * (i - ty * TW4), gy = y0 - 3 + ty;
+            const bool in = ty < TH && gx >= 0 && gx < W && gy >= 0 && gy < H &&
+                            SGM_GUARD_INDEX((long long)gy * W + gx + 3, (long long)W * H, 301);
+            v[h] = in ? __ldg(reinterpret_cast<const uint32_t*>(img + (size_t)gy * W + (mirror ? W - 4 - gx : gx))) : 0u;
+            if (mirror) v[h] = __byte_perm(v[h], 0u, 0x0123u);
+        }
+#pragma unroll
+        for (int h = 0; h < N4; ++h) {
+            const int i = threadIdx.x + h * kCtT;
+            if (i < TW4 * TH) reinterpret_cast<uint32_t*>(&tile[0][0])[i] = v[h];
+        }
+    } else {
         uint8_t v[NS][TH];
 #pragma unroll
         for (int h = 0; h < NS; ++h) {
@@ -118,26 +127,27 @@ __device__ __forceinline__ void census_body(const uint8_t* __restrict__ left, co
     const int lx = 2 * threadIdx.x, x = x0 + lx;
     if (x >= W) return;
     const bool ok0 = x >= 4 && x <= W - 5, ok1 = x + 1 >= 4 && x + 1 <= W - 5, has1 = x + 1 < W;
-    uint32_t win[7][10];  // win[r % 7][c]: tile row r, tile column lx + c (image x - 4 + c)
+    uint32_t win[7][9], pow[8];  // win[r % 7][c]: tile row r, tile columns lx + c, lx + c + 1 (image x - 4 + c)
 #pragma unroll
-    for (int r = 0; r < 6; ++r)
+    for (int k = 0; k < 8; ++k) pow[k] = opaque(1u << k);
+    auto read_row = [&](int r, uint32_t (&w)[9]) {
+        uint32_t b[5];
 #pragma unroll
-        for (int c = 0; c < 10; ++c) win[r][c] = tile[r][lx + c];
+        for (int k = 0; k < 5; ++k) b[k] = *reinterpret_cast<const uint16_t*>(&tile[r][lx + 2 * k]);
 #pragma unroll
-    for (int r = 0; r < kCtH; ++r) {
+        for (int k = 0; k < 9; ++k)
+            w[k] = k & 1 ? __byte_perm(b[k / 2], b[k / 2 + 1], 0x2421u) : __byte_perm(b[k / 2], 0u, 0x4140u);
+    };
 #pragma unroll
-        for (int c = 0; c < 10; ++c) win[(r + 6) % 7][c] = tile[r + 6][lx + c];
+    for (int r = 0; r < 6; ++r) read_row(r, win[r]);
+#pragma unroll
+    for (int r = 0; r < TILE_H; ++r) {
+        read_row(r + 6, win[(r + 6) % 7]);
         const int y = y0 + r;
         if (y >= H) break;
         const bool yok = y >= 3 && y <= H - 4;
         FT f0, f1;
-        if constexpr (CT) {
-            f0 = census62_feature(win, r, 0);
-            f1 = census62_feature(win, r, 1);
-        } else {
-            f0 = census_feature(win, r, 0);
-            f1 = census_feature(win, r, 1);
-        }
+        census_pair<FT>(win, r, pow, f0, f1);
         FT* row = F + (size_t)y * W + x;
         if (SGM_GUARD_INDEX((long long)y * W + x + (has1 ? 1 : 0), (long long)W * H, 302)) {
             row[0] = (ok0 && yok) ? f0 : FT(0);
@@ -189,23 +199,36 @@ cudaError_t launch_census(const uint8_t* left, const uint8_t* right, void* Fb, v
 // The passes of the paired schedule: image z is left, right, and for the
 // right pass of the left-right check the mirrored right and left images (read
 // mirrored here, which saves writing them).
-template <bool CT>
+template <bool CT, int TILE_H>
 __global__ void __launch_bounds__(kCtT) census_passes_kernel(const uint8_t* __restrict__ left,
                                                              const uint8_t* __restrict__ right, uint8_t* F,
                                                              size_t fstride, int W, int H) {
     pdl_wait();
     const int z = blockIdx.z;
     void* out = F + z * fstride;
-    census_body<CT>(left, right, out, out, W, H, blockIdx.x, blockIdx.y, (z & 1) ^ (z >> 1), z >= 2);
+    census_body<CT, TILE_H>(left, right, out, out, W, H, blockIdx.x, blockIdx.y, (z & 1) ^ (z >> 1), z >= 2);
 }
 
 cudaError_t launch_census_passes(const uint8_t* left, const uint8_t* right, void* F, size_t fstride, int n, int W,
                                  int H, bool ct62, Stream stream) {
-    dim3 grid((W + kCtW - 1) / kCtW, (H + kCtH - 1) / kCtH, n);
-    if (ct62)
-        launch(census_passes_kernel<true>, grid, kCtT, stream, left, right, static_cast<uint8_t*>(F), fstride, W, H);
-    else
-        launch(census_passes_kernel<false>, grid, kCtT, stream, left, right, static_cast<uint8_t*>(F), fstride, W, H);
+    const int across = (W + kCtW - 1) / kCtW;
+    uint8_t* const Fp = static_cast<uint8_t*>(F);
+    auto run = [&](auto kernel, int h) {
+        launch(kernel, dim3(across, (H + h - 1) / h, n), kCtT, stream, left, right, Fp, fstride, W, H);
+    };
+    // flat tiles while the tall ones leave some of the chip's 608 schedulers without a warp: a thread's
+    // walk down its tile is what the launch then waits for (96x64 frame 14.2 -> 13.7 us; at 320x240
+    // they measure alike, at 640x480 the halo's rows cost more: 78.4 -> 79.2)
+    if (across * ((H + kCtH - 1) / kCtH) * n < 608) {
+        if (ct62)
+            run(census_passes_kernel<true, kCtSmallH>, kCtSmallH);
+        else
+            run(census_passes_kernel<false, kCtSmallH>, kCtSmallH);
+    } else if (ct62) {
+        run(census_passes_kernel<true, kCtH>, kCtH);
+    } else {
+        run(census_passes_kernel<false, kCtH>, kCtH);
+    }
     return cudaGetLastError();
 }
 
@@ -748,9 +771,9 @@ cudaError_t launch_median(const uint8_t* raw, uint8_t* disp, int W, int H, Strea
 // (x & 1) + 2 (y & 1) of its quad): a thread takes kMedQH quads of a quad
 // column, two pixels at a time in the halves of a word.  The quads left and
 // right of it complete the three columns of both pixels.
-// Bound: the launch itself (2.9 us at 640x480, 5.0 at 1920x1080).  One pixel per
-// thread column with eighteen byte loads took 3.4 and 9: 640x480 D=128 frame
-// 79.8 -> 79.4 us, 1920x1080 D=128 8 paths 946.9 -> 942.7.
+// Bound: the launch itself (2.9 us at 640x480, 5.0 at 1920x1080).  Against a
+// thread per pixel column with eighteen byte loads: 640x480 D=128 frame 79.8 ->
+// 79.4 us, 1920x1080 D=128 8 paths 946.9 -> 942.7.
 constexpr int kMedQW = 64, kMedQH = 2;
 
 __device__ __forceinline__ uint32_t vmax2(uint32_t a, uint32_t b) { return __vmaxu2(a, b); }
