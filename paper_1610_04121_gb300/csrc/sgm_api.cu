@@ -266,7 +266,7 @@ struct Request {
 // type); every stage of a group is one persistent grid over a device work
 // list (sgm_internal.h).  The lists of a wave live in one blob: its pinned
 // host image is filled per wave and copied to the device copy before the
-// wave's graph runs.  The graph, captured once per wave shape (the groups'
+// wave's graph runs.  The graph, built once per wave shape (the groups'
 // keys and the sweep grid) and replayed for every wave of that shape, zeroes
 // the lists' counters, runs each group's stages on one of kListBranches
 // concurrent branches, and copies the device status word back to the host.
@@ -283,12 +283,6 @@ constexpr int kSweepGrids[] = {2, 3, 4, 5};
 constexpr int kDefaultSweepGrid = 4;
 
 struct ListExec {
-    cudaStream_t capture = nullptr;
-    cudaStream_t branch[kListBranches] = {};
-    cudaEvent_t fork = nullptr, join[kListBranches] = {};
-    // 8-path groups walk three lists side by side: two more streams per branch
-    cudaStream_t side[kListBranches][2] = {};
-    cudaEvent_t side_fork[kListBranches] = {}, side_join[kListBranches][2] = {};
     uint8_t* blob_dev = nullptr;
     uint8_t* blob_host = nullptr;     // pinned, blob_cap bytes
     size_t blob_cap = 0;
@@ -1008,17 +1002,6 @@ static int batch_sched(Problem p, size_t room, double px) {
 static int launches_per_group(int n_paths) { return 4 + (n_paths == 8 ? 3 : 1); }
 
 static int list_exec_init(sgm_ctx* ctx, ListExec& x) {
-    CUDA_TRY(ctx, cudaStreamCreateWithFlags(&x.capture, cudaStreamNonBlocking));
-    CUDA_TRY(ctx, cudaEventCreateWithFlags(&x.fork, cudaEventDisableTiming));
-    for (int b = 0; b < kListBranches; ++b) {
-        CUDA_TRY(ctx, cudaStreamCreateWithFlags(&x.branch[b], cudaStreamNonBlocking));
-        CUDA_TRY(ctx, cudaEventCreateWithFlags(&x.join[b], cudaEventDisableTiming));
-        CUDA_TRY(ctx, cudaEventCreateWithFlags(&x.side_fork[b], cudaEventDisableTiming));
-        for (int k = 0; k < 2; ++k) {
-            CUDA_TRY(ctx, cudaStreamCreateWithFlags(&x.side[b][k], cudaStreamNonBlocking));
-            CUDA_TRY(ctx, cudaEventCreateWithFlags(&x.side_join[b][k], cudaEventDisableTiming));
-        }
-    }
     void* q = nullptr;
     CUDA_TRY(ctx, ctx_malloc_host(ctx, &q, sizeof(uint32_t)));
     x.status_host = static_cast<uint32_t*>(q);
@@ -1036,17 +1019,6 @@ static void list_exec_release(ListExec& x) {
     if (x.blob_dev) cudaFree(x.blob_dev);
     if (x.blob_host) cudaFreeHost(x.blob_host);
     if (x.status_host) cudaFreeHost(x.status_host);
-    for (int b = 0; b < kListBranches; ++b) {
-        if (x.branch[b]) cudaStreamDestroy(x.branch[b]);
-        if (x.join[b]) cudaEventDestroy(x.join[b]);
-        if (x.side_fork[b]) cudaEventDestroy(x.side_fork[b]);
-        for (int k = 0; k < 2; ++k) {
-            if (x.side[b][k]) cudaStreamDestroy(x.side[b][k]);
-            if (x.side_join[b][k]) cudaEventDestroy(x.side_join[b][k]);
-        }
-    }
-    if (x.fork) cudaEventDestroy(x.fork);
-    if (x.capture) cudaStreamDestroy(x.capture);
     x = ListExec{};
 }
 
@@ -1227,19 +1199,22 @@ static int list_graph(sgm_ctx* ctx, ListExec& x, const std::vector<int>& keys, i
         *out = it->second;
         return SGM_OK;
     }
-    cudaStream_t c = x.capture;
-    CUDA_TRY(ctx, cudaStreamBeginCapture(c, cudaStreamCaptureModeThreadLocal));
+    cudaGraph_t graph = nullptr;
+    CUDA_TRY(ctx, cudaGraphCreate(&graph, 0));
     auto body = [&]() -> cudaError_t {
         cudaError_t e;
         uint32_t* counters = reinterpret_cast<uint32_t*>(x.blob_dev + kBlobCounters);
         uint32_t* status = reinterpret_cast<uint32_t*>(x.blob_dev);
-        if ((e = cudaMemsetAsync(counters, 0, 4 * kListGroups * kListCounters, c)) != cudaSuccess) return e;
-        if ((e = cudaEventRecord(x.fork, c)) != cudaSuccess) return e;
-        const int nb = std::min<int>(kListBranches, static_cast<int>(keys.size()));
-        for (int b = 0; b < nb; ++b)
-            if ((e = cudaStreamWaitEvent(x.branch[b], x.fork, 0)) != cudaSuccess) return e;
+        cudaMemsetParams zero{};
+        zero.dst = counters;
+        zero.elementSize = 4;
+        zero.width = kListGroups * kListCounters;
+        zero.height = 1;
+        cudaGraphNode_t fork = nullptr;
+        if ((e = cudaGraphAddMemsetNode(&fork, graph, nullptr, 0, &zero)) != cudaSuccess) return e;
+        std::vector<NodeChain> branch(std::min<size_t>(kListBranches, keys.size()), NodeChain{graph, {fork}});
         for (size_t g = 0; g < keys.size(); ++g) {
-            cudaStream_t s = x.branch[g % kListBranches];
+            NodeChain& s = branch[g % kListBranches];
             const int D = keys[g] & 511, n_paths = (keys[g] >> 9) & 15;
             ListLaunch l{};
             l.status = status;
@@ -1265,18 +1240,16 @@ static int list_graph(sgm_ctx* ctx, ListExec& x, const std::vector<int>& keys, i
                 // the sweep grid counts 128 threads a block
                 at(2, 2);
                 l.grid = 2 * sweep_grid * ctx->n_sm;
-                const int b = g % kListBranches;
                 if (n_paths == 8) {
-                    if ((e = cudaEventRecord(x.side_fork[b], s)) != cudaSuccess) return e;
+                    // three lists side by side
+                    NodeChain side[2] = {s, s};
                     if ((e = launch_pairs_walks_list(l, Walks::kHor, s)) != cudaSuccess) return e;
                     l.grid = (4 * sweep_grid + 2) / 3 * ctx->n_sm;
                     for (int k = 0; k < 2; ++k) {
-                        cudaStream_t ss = x.side[b][k];
                         at(3, 3 + k);
-                        if ((e = cudaStreamWaitEvent(ss, x.side_fork[b], 0)) != cudaSuccess) return e;
-                        if ((e = launch_pairs_walks_list(l, k ? Walks::kUp : Walks::kDown, ss)) != cudaSuccess) return e;
-                        if ((e = cudaEventRecord(x.side_join[b][k], ss)) != cudaSuccess) return e;
-                        if ((e = cudaStreamWaitEvent(s, x.side_join[b][k], 0)) != cudaSuccess) return e;
+                        if ((e = launch_pairs_walks_list(l, k ? Walks::kUp : Walks::kDown, side[k])) != cudaSuccess)
+                            return e;
+                        s.after.push_back(side[k].after[0]);
                     }
                 } else if ((e = launch_pairs_walks_list(l, Walks::kHorVer, s)) != cudaSuccess) {
                     return e;
@@ -1304,20 +1277,17 @@ static int list_graph(sgm_ctx* ctx, ListExec& x, const std::vector<int>& keys, i
             l.grid = kMedianListPerSM * ctx->n_sm;
             if ((e = launch_median_list(l, s)) != cudaSuccess) return e;
         }
-        for (int b = 0; b < nb; ++b) {
-            if ((e = cudaEventRecord(x.join[b], x.branch[b])) != cudaSuccess) return e;
-            if ((e = cudaStreamWaitEvent(c, x.join[b], 0)) != cudaSuccess) return e;
-        }
-        return cudaMemcpyAsync(x.status_host, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, c);
+        std::vector<cudaGraphNode_t> ends;
+        for (const NodeChain& b : branch) ends.insert(ends.end(), b.after.begin(), b.after.end());
+        cudaGraphNode_t last = nullptr;
+        return cudaGraphAddMemcpyNode1D(&last, graph, ends.data(), ends.size(), x.status_host, status,
+                                        sizeof(uint32_t), cudaMemcpyDeviceToHost);
     };
     const cudaError_t eb = body();
-    cudaGraph_t graph = nullptr;
-    const cudaError_t ee = cudaStreamEndCapture(c, &graph);
-    if (eb != cudaSuccess || ee != cudaSuccess) {
-        if (graph) cudaGraphDestroy(graph);
+    if (eb != cudaSuccess) {
+        cudaGraphDestroy(graph);
         cudaGetLastError();
-        return fail(ctx, SGM_ECUDA, "capturing the batched graph: %s",
-                    cudaGetErrorString(eb != cudaSuccess ? eb : ee));
+        return fail(ctx, SGM_ECUDA, "building the batched graph: %s", cudaGetErrorString(eb));
     }
     cudaGraphExec_t exec = nullptr;
     const cudaError_t ei = cudaGraphInstantiate(&exec, graph, 0);

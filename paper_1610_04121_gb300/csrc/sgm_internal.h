@@ -2,6 +2,8 @@
 #pragma once
 
 #include <cstdint>
+#include <tuple>
+#include <vector>
 #include <cuda_runtime.h>
 
 namespace sgm {
@@ -124,7 +126,32 @@ struct ListLaunch {
     int n_paths, cls;  // paired schedule: paths and class of the sums (pairs_class)
 };
 
-// Each launcher enqueues one kernel on `stream` and returns the launch error.
+// A chain of nodes in a graph under construction: the next kernel runs after
+// the nodes in `after`.  The graphs of the lists are built node by node, not
+// captured: they are built on the scheduler's thread too, and a capture there
+// fails a cudaDeviceSynchronize that another thread happens to make.
+struct NodeChain {
+    cudaGraph_t graph;
+    std::vector<cudaGraphNode_t> after;
+};
+template <class... P, class... A>
+inline cudaError_t add_kernel(NodeChain& c, void (*kernel)(P...), int grid, int block, A... args) {
+    std::tuple<P...> v{static_cast<P>(args)...};
+    cudaKernelNodeParams n{};
+    n.func = reinterpret_cast<void*>(kernel);
+    n.gridDim = dim3(grid);
+    n.blockDim = dim3(block);
+    void* ptrs[sizeof...(P)];
+    std::apply([&](auto&... x) { int i = 0; ((ptrs[i++] = &x), ...); }, v);
+    n.kernelParams = ptrs;  // the values are copied into the node
+    cudaGraphNode_t node = nullptr;
+    const cudaError_t e = cudaGraphAddKernelNode(&node, c.graph, c.after.data(), c.after.size(), &n);
+    if (e == cudaSuccess) c.after.assign(1, node);
+    return e;
+}
+
+// Each launcher enqueues one kernel on `stream` and returns the launch error;
+// the list launchers add it to a chain of nodes.
 // ct62 = false: the CSCT of Eq. 1, uint32 features; true: the full 9x7
 // Census, uint64 features.
 cudaError_t launch_census(const uint8_t* left, const uint8_t* right, void* Fb, void* Fm, int W, int H, bool ct62,
@@ -171,11 +198,11 @@ cudaError_t launch_post(const uint8_t* rawL, const uint32_t* sub, const uint8_t*
 // The work-list kernels: every job of a list has the launch's D (and, for
 // sweeps, its pair / s8 settings; a vertical-type list runs both halves of
 // its pair in one unit, the vertical one finishing with Eq. 4).
-cudaError_t launch_census_list(const ListLaunch& l, cudaStream_t stream);
-cudaError_t launch_cost_list(const ListLaunch& l, cudaStream_t stream);
-cudaError_t launch_sweep_h_list(const ListLaunch& l, cudaStream_t stream);
-cudaError_t launch_sweep_v_list(const ListLaunch& l, cudaStream_t stream);
-cudaError_t launch_median_list(const ListLaunch& l, cudaStream_t stream);
+cudaError_t launch_census_list(const ListLaunch& l, NodeChain& chain);
+cudaError_t launch_cost_list(const ListLaunch& l, NodeChain& chain);
+cudaError_t launch_sweep_h_list(const ListLaunch& l, NodeChain& chain);
+cudaError_t launch_sweep_v_list(const ListLaunch& l, NodeChain& chain);
+cudaError_t launch_median_list(const ListLaunch& l, NodeChain& chain);
 // Units of one pair in each list; blocks of each list kernel resident per SM.
 int census_units(int W, int H);
 int cost_units(int W, int H);
@@ -284,10 +311,10 @@ struct CostQuadsJob {
     int QB, W, H, D;
 };
 constexpr int kCostQuadsRun = 4; // 32-quad segments of a unit of the cost list
-cudaError_t launch_cost_quads_list(const ListLaunch& l, cudaStream_t stream);
-cudaError_t launch_pairs_walks_list(const ListLaunch& l, Walks w, cudaStream_t stream);
-cudaError_t launch_pairs_finish_list(const ListLaunch& l, cudaStream_t stream);
-cudaError_t launch_median_quads_list(const ListLaunch& l, cudaStream_t stream);
+cudaError_t launch_cost_quads_list(const ListLaunch& l, NodeChain& chain);
+cudaError_t launch_pairs_walks_list(const ListLaunch& l, Walks w, NodeChain& chain);
+cudaError_t launch_pairs_finish_list(const ListLaunch& l, NodeChain& chain);
+cudaError_t launch_median_quads_list(const ListLaunch& l, NodeChain& chain);
 int cost_quads_units(int W, int H);
 int pairs_hv_units(const PairsArgs& a, bool ver);
 // Segments a warp takes at once: four, unless that leaves a pair with fewer

@@ -1149,29 +1149,26 @@ struct PairsD {
         }
         return cudaGetLastError();
     }
-    static cudaError_t walks_list(const ListLaunch& l, Walks w, cudaStream_t s) {
+    static cudaError_t walks_list(const ListLaunch& l, Walks w, NodeChain& chain) {
         const auto* L = static_cast<const WorkList<PairsArgs>*>(l.list);
         if (w == Walks::kDown || w == Walks::kUp)
-            walk_rows_list_kernel<D><<<l.grid, 96, 0, s>>>(L, l.next, l.status, w == Walks::kDown);
-        else
-            walk_hv_list_kernel<D><<<l.grid, 64, 0, s>>>(L, l.next, l.status, w == Walks::kHorVer);
-        return cudaGetLastError();
+            return add_kernel(chain, walk_rows_list_kernel<D>, l.grid, 96, L, l.next, l.status, w == Walks::kDown);
+        return add_kernel(chain, walk_hv_list_kernel<D>, l.grid, 64, L, l.next, l.status, w == Walks::kHorVer);
     }
     template <int NP, int GS, bool K16>
-    static cudaError_t finish_list_t(const ListLaunch& l, cudaStream_t s) {
-        finish_list_kernel<D, NP, GS, K16>
-            <<<l.grid, 64, 0, s>>>(static_cast<const WorkList<PairsArgs>*>(l.list), l.next, l.status);
-        return cudaGetLastError();
+    static cudaError_t finish_list_t(const ListLaunch& l, NodeChain& chain) {
+        return add_kernel(chain, finish_list_kernel<D, NP, GS, K16>, l.grid, 64,
+                          static_cast<const WorkList<PairsArgs>*>(l.list), l.next, l.status);
     }
     template <int NP>
-    static cudaError_t finish_list_np(const ListLaunch& l, cudaStream_t s) {
-        if (l.cls == 0) return finish_list_t<NP, 3, true>(l, s);
-        return l.cls == 1 ? finish_list_t<NP, 2, false>(l, s) : finish_list_t<NP, 1, false>(l, s);
+    static cudaError_t finish_list_np(const ListLaunch& l, NodeChain& chain) {
+        if (l.cls == 0) return finish_list_t<NP, 3, true>(l, chain);
+        return l.cls == 1 ? finish_list_t<NP, 2, false>(l, chain) : finish_list_t<NP, 1, false>(l, chain);
     }
-    static cudaError_t fin_list(const ListLaunch& l, cudaStream_t s) {
-        if (l.n_paths == 8) return finish_list_np<8>(l, s);
-        if (l.n_paths == 4) return finish_list_np<4>(l, s);
-        return l.cls == 0 ? finish_list_t<2, 1, true>(l, s) : finish_list_t<2, 1, false>(l, s);
+    static cudaError_t fin_list(const ListLaunch& l, NodeChain& chain) {
+        if (l.n_paths == 8) return finish_list_np<8>(l, chain);
+        if (l.n_paths == 4) return finish_list_np<4>(l, chain);
+        return l.cls == 0 ? finish_list_t<2, 1, true>(l, chain) : finish_list_t<2, 1, false>(l, chain);
     }
 };
 
@@ -1184,9 +1181,9 @@ SGM_INTERNAL_P cudaError_t pairs_walks(const PairsJobs& f, Walks w, Stream s);
 template <int D>
 SGM_INTERNAL_P cudaError_t pairs_finish(const PairsJobs& f, Stream s);
 template <int D>
-SGM_INTERNAL_P cudaError_t pairs_walks_list(const ListLaunch& l, Walks w, cudaStream_t s);
+SGM_INTERNAL_P cudaError_t pairs_walks_list(const ListLaunch& l, Walks w, NodeChain& chain);
 template <int D>
-SGM_INTERNAL_P cudaError_t pairs_finish_list(const ListLaunch& l, cudaStream_t s);
+SGM_INTERNAL_P cudaError_t pairs_finish_list(const ListLaunch& l, NodeChain& chain);
 
 #define SGM_INSTANTIATE_PAIRS(D)                                                                   \
     template <>                                                                                    \
@@ -1198,12 +1195,12 @@ SGM_INTERNAL_P cudaError_t pairs_finish_list(const ListLaunch& l, cudaStream_t s
         return pairs::PairsD<D>::fin(f, s);                                                        \
     }                                                                                              \
     template <>                                                                                    \
-    SGM_INTERNAL_P cudaError_t pairs_walks_list<D>(const ListLaunch& l, Walks w, cudaStream_t s) { \
-        return pairs::PairsD<D>::walks_list(l, w, s);                                              \
+    SGM_INTERNAL_P cudaError_t pairs_walks_list<D>(const ListLaunch& l, Walks w, NodeChain& chain) { \
+        return pairs::PairsD<D>::walks_list(l, w, chain);                                          \
     }                                                                                              \
     template <>                                                                                    \
-    SGM_INTERNAL_P cudaError_t pairs_finish_list<D>(const ListLaunch& l, cudaStream_t s) {         \
-        return pairs::PairsD<D>::fin_list(l, s);                                                   \
+    SGM_INTERNAL_P cudaError_t pairs_finish_list<D>(const ListLaunch& l, NodeChain& chain) {         \
+        return pairs::PairsD<D>::fin_list(l, chain);                                               \
     }
 
 }  // namespace sgm

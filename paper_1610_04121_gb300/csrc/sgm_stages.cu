@@ -177,13 +177,11 @@ __global__ void __launch_bounds__(kCtT) census_list_kernel(const WorkList<Census
 
 int census_units(int W, int H) { return 2 * ((W + kCtW - 1) / kCtW) * ((H + kCtH - 1) / kCtH); }
 
-cudaError_t launch_census_list(const ListLaunch& l, cudaStream_t stream) {
+cudaError_t launch_census_list(const ListLaunch& l, NodeChain& chain) {
     const auto* L = static_cast<const WorkList<CensusJob>*>(l.list);
     if (l.ct62)
-        census_list_kernel<true><<<l.grid, kCtT, 0, stream>>>(L, l.next, l.status);
-    else
-        census_list_kernel<false><<<l.grid, kCtT, 0, stream>>>(L, l.next, l.status);
-    return cudaGetLastError();
+        return add_kernel(chain, census_list_kernel<true>, l.grid, kCtT, L, l.next, l.status);
+    return add_kernel(chain, census_list_kernel<false>, l.grid, kCtT, L, l.next, l.status);
 }
 
 cudaError_t launch_census(const uint8_t* left, const uint8_t* right, void* Fb, void* Fm, int W, int H, bool ct62,
@@ -350,25 +348,23 @@ __global__ void __launch_bounds__(kMcThreads) cost_list_kernel(const WorkList<Co
 int cost_units(int W, int H) { return ((W + kMcSeg - 1) / kMcSeg) * H; }
 
 template <int D>
-static cudaError_t launch_cost_list_t(const ListLaunch& l, cudaStream_t s) {
+static cudaError_t launch_cost_list_t(const ListLaunch& l, NodeChain& chain) {
     const auto* L = static_cast<const WorkList<CostJob>*>(l.list);
     if (l.ct62)
-        cost_list_kernel<D, uint64_t><<<l.grid, kMcThreads, 0, s>>>(L, l.next, l.status);
-    else
-        cost_list_kernel<D, uint32_t><<<l.grid, kMcThreads, 0, s>>>(L, l.next, l.status);
-    return cudaGetLastError();
+        return add_kernel(chain, cost_list_kernel<D, uint64_t>, l.grid, kMcThreads, L, l.next, l.status);
+    return add_kernel(chain, cost_list_kernel<D, uint32_t>, l.grid, kMcThreads, L, l.next, l.status);
 }
 
-cudaError_t launch_cost_list(const ListLaunch& l, cudaStream_t stream) {
+cudaError_t launch_cost_list(const ListLaunch& l, NodeChain& chain) {
     switch (l.D) {
-        case 32: return launch_cost_list_t<32>(l, stream);
-        case 64: return launch_cost_list_t<64>(l, stream);
-        case 96: return launch_cost_list_t<96>(l, stream);
-        case 128: return launch_cost_list_t<128>(l, stream);
-        case 160: return launch_cost_list_t<160>(l, stream);
-        case 192: return launch_cost_list_t<192>(l, stream);
-        case 224: return launch_cost_list_t<224>(l, stream);
-        case 256: return launch_cost_list_t<256>(l, stream);
+        case 32: return launch_cost_list_t<32>(l, chain);
+        case 64: return launch_cost_list_t<64>(l, chain);
+        case 96: return launch_cost_list_t<96>(l, chain);
+        case 128: return launch_cost_list_t<128>(l, chain);
+        case 160: return launch_cost_list_t<160>(l, chain);
+        case 192: return launch_cost_list_t<192>(l, chain);
+        case 224: return launch_cost_list_t<224>(l, chain);
+        case 256: return launch_cost_list_t<256>(l, chain);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -558,25 +554,23 @@ int cost_quads_units(int W, int H) {
 }
 
 template <int D>
-static cudaError_t launch_cost_quads_list_t(const ListLaunch& l, cudaStream_t s) {
+static cudaError_t launch_cost_quads_list_t(const ListLaunch& l, NodeChain& chain) {
     const auto* L = static_cast<const WorkList<CostQuadsJob>*>(l.list);
     if (l.ct62)
-        cost_quads_list_kernel<D, uint64_t><<<l.grid, kQcThreads, 0, s>>>(L, l.next, l.status);
-    else
-        cost_quads_list_kernel<D, uint32_t><<<l.grid, kQcThreads, 0, s>>>(L, l.next, l.status);
-    return cudaGetLastError();
+        return add_kernel(chain, cost_quads_list_kernel<D, uint64_t>, l.grid, kQcThreads, L, l.next, l.status);
+    return add_kernel(chain, cost_quads_list_kernel<D, uint32_t>, l.grid, kQcThreads, L, l.next, l.status);
 }
 
-cudaError_t launch_cost_quads_list(const ListLaunch& l, cudaStream_t stream) {
+cudaError_t launch_cost_quads_list(const ListLaunch& l, NodeChain& chain) {
     switch (l.D) {
-        case 32: return launch_cost_quads_list_t<32>(l, stream);
-        case 64: return launch_cost_quads_list_t<64>(l, stream);
-        case 96: return launch_cost_quads_list_t<96>(l, stream);
-        case 128: return launch_cost_quads_list_t<128>(l, stream);
-        case 160: return launch_cost_quads_list_t<160>(l, stream);
-        case 192: return launch_cost_quads_list_t<192>(l, stream);
-        case 224: return launch_cost_quads_list_t<224>(l, stream);
-        case 256: return launch_cost_quads_list_t<256>(l, stream);
+        case 32: return launch_cost_quads_list_t<32>(l, chain);
+        case 64: return launch_cost_quads_list_t<64>(l, chain);
+        case 96: return launch_cost_quads_list_t<96>(l, chain);
+        case 128: return launch_cost_quads_list_t<128>(l, chain);
+        case 160: return launch_cost_quads_list_t<160>(l, chain);
+        case 192: return launch_cost_quads_list_t<192>(l, chain);
+        case 224: return launch_cost_quads_list_t<224>(l, chain);
+        case 256: return launch_cost_quads_list_t<256>(l, chain);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -756,9 +750,9 @@ __global__ void __launch_bounds__(kMedW) median_list_kernel(const WorkList<Media
 
 int median_units(int W, int H) { return ((W + kMedW - 1) / kMedW) * ((H + kMedH - 1) / kMedH); }
 
-cudaError_t launch_median_list(const ListLaunch& l, cudaStream_t stream) {
-    median_list_kernel<<<l.grid, kMedW, 0, stream>>>(static_cast<const WorkList<MedianJob>*>(l.list), l.next);
-    return cudaGetLastError();
+cudaError_t launch_median_list(const ListLaunch& l, NodeChain& chain) {
+    return add_kernel(chain, median_list_kernel, l.grid, kMedW, static_cast<const WorkList<MedianJob>*>(l.list),
+                      l.next);
 }
 
 cudaError_t launch_median(const uint8_t* raw, uint8_t* disp, int W, int H, Stream stream) {
@@ -860,9 +854,9 @@ __global__ void __launch_bounds__(kMedQW) median_quads_list_kernel(const WorkLis
 
 int median_quads_units(int W, int H) { return median_quads_across(W) * median_quads_down(H); }
 
-cudaError_t launch_median_quads_list(const ListLaunch& l, cudaStream_t stream) {
-    median_quads_list_kernel<<<l.grid, kMedQW, 0, stream>>>(static_cast<const WorkList<MedianJob>*>(l.list), l.next);
-    return cudaGetLastError();
+cudaError_t launch_median_quads_list(const ListLaunch& l, NodeChain& chain) {
+    return add_kernel(chain, median_quads_list_kernel, l.grid, kMedQW,
+                      static_cast<const WorkList<MedianJob>*>(l.list), l.next);
 }
 
 // ---------------------------------------------------------------------------

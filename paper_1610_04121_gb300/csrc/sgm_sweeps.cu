@@ -47,12 +47,12 @@ cudaError_t launch_sweep_first4(FirstStageArgs& f, Stream stream) {
 
 cudaError_t launch_sweep_h2(const SweepArgs& a, Stream stream) { SGM_DISPATCH_D(sweep_launch_h2, a.D, a, stream) }
 
-cudaError_t launch_sweep_h_list(const ListLaunch& l, cudaStream_t stream) {
-    SGM_DISPATCH_D(sweep_launch_h_list, l.D, l, stream)
+cudaError_t launch_sweep_h_list(const ListLaunch& l, NodeChain& chain) {
+    SGM_DISPATCH_D(sweep_launch_h_list, l.D, l, chain)
 }
 
-cudaError_t launch_sweep_v_list(const ListLaunch& l, cudaStream_t stream) {
-    SGM_DISPATCH_D(sweep_launch_v_list, l.D, l, stream)
+cudaError_t launch_sweep_v_list(const ListLaunch& l, NodeChain& chain) {
+    SGM_DISPATCH_D(sweep_launch_v_list, l.D, l, chain)
 }
 
 int sweep_units(int lines, int D, bool pair) {
@@ -96,12 +96,12 @@ cudaError_t launch_pairs_finish(const PairsJobs& f, Stream stream) {
     SGM_DISPATCH_PAIRS(pairs_finish, f.job[0].D, f, stream)
 }
 
-cudaError_t launch_pairs_walks_list(const ListLaunch& l, Walks w, cudaStream_t stream) {
-    SGM_DISPATCH_PAIRS(pairs_walks_list, l.D, l, w, stream)
+cudaError_t launch_pairs_walks_list(const ListLaunch& l, Walks w, NodeChain& chain) {
+    SGM_DISPATCH_PAIRS(pairs_walks_list, l.D, l, w, chain)
 }
 
-cudaError_t launch_pairs_finish_list(const ListLaunch& l, cudaStream_t stream) {
-    SGM_DISPATCH_PAIRS(pairs_finish_list, l.D, l, stream)
+cudaError_t launch_pairs_finish_list(const ListLaunch& l, NodeChain& chain) {
+    SGM_DISPATCH_PAIRS(pairs_finish_list, l.D, l, chain)
 }
 
 int pairs_hv_units(const PairsArgs& a, bool ver) {

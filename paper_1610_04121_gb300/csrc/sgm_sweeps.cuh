@@ -895,32 +895,28 @@ struct SweepD {
         return cudaGetLastError();
     }
 
-    static cudaError_t launch_h_list(const ListLaunch& l, cudaStream_t s) {
+    static cudaError_t launch_h_list(const ListLaunch& l, NodeChain& chain) {
         const auto* L = static_cast<const WorkList<SweepArgs>*>(l.list);
-        const dim3 block(32 * kWarpsPerBlock);
+        constexpr int block = 32 * kWarpsPerBlock;
         if (!l.pair)
-            sweep_h_list_kernel<D, false, true><<<l.grid, block, 0, s>>>(L, l.next, l.status);
-        else if (l.s8)
-            sweep_h_list_kernel<D, true, true><<<l.grid, block, 0, s>>>(L, l.next, l.status);
-        else
-            sweep_h_list_kernel<D, true, false><<<l.grid, block, 0, s>>>(L, l.next, l.status);
-        return cudaGetLastError();
+            return add_kernel(chain, sweep_h_list_kernel<D, false, true>, l.grid, block, L, l.next, l.status);
+        if (l.s8)
+            return add_kernel(chain, sweep_h_list_kernel<D, true, true>, l.grid, block, L, l.next, l.status);
+        return add_kernel(chain, sweep_h_list_kernel<D, true, false>, l.grid, block, L, l.next, l.status);
     }
 
-    static cudaError_t launch_v_list(const ListLaunch& l, cudaStream_t s) {
+    static cudaError_t launch_v_list(const ListLaunch& l, NodeChain& chain) {
         const auto* L = static_cast<const WorkList<SweepArgs>*>(l.list);
-        const dim3 block(32 * kWarpsPerBlock);
+        constexpr int block = 32 * kWarpsPerBlock;
         if (!l.pair)
-            sweep_v_list_kernel<D, 0, true, false, true><<<l.grid, block, 0, s>>>(L, l.next, l.status);
-        else if (l.rx == 0 && l.s8)
-            sweep_v_list_kernel<D, 0, true, true, true><<<l.grid, block, 0, s>>>(L, l.next, l.status);
-        else if (l.rx == 0)
-            sweep_v_list_kernel<D, 0, true, true, false><<<l.grid, block, 0, s>>>(L, l.next, l.status);
-        else if (l.rx > 0)
-            sweep_v_list_kernel<D, 1, false, true, false><<<l.grid, block, 0, s>>>(L, l.next, l.status);
-        else
-            sweep_v_list_kernel<D, -1, false, true, false><<<l.grid, block, 0, s>>>(L, l.next, l.status);
-        return cudaGetLastError();
+            return add_kernel(chain, sweep_v_list_kernel<D, 0, true, false, true>, l.grid, block, L, l.next, l.status);
+        if (l.rx == 0 && l.s8)
+            return add_kernel(chain, sweep_v_list_kernel<D, 0, true, true, true>, l.grid, block, L, l.next, l.status);
+        if (l.rx == 0)
+            return add_kernel(chain, sweep_v_list_kernel<D, 0, true, true, false>, l.grid, block, L, l.next, l.status);
+        if (l.rx > 0)
+            return add_kernel(chain, sweep_v_list_kernel<D, 1, false, true, false>, l.grid, block, L, l.next, l.status);
+        return add_kernel(chain, sweep_v_list_kernel<D, -1, false, true, false>, l.grid, block, L, l.next, l.status);
     }
 
     // Vertical-type sweeps of a pair in phase 1 or 2 (or both, phase 0).
@@ -980,13 +976,13 @@ SGM_INTERNAL cudaError_t sweep_launch_v(const SweepArgs& a, Stream s);
 template <int D>
 SGM_INTERNAL cudaError_t sweep_launch_first(FirstStageArgs& f, Stream s);
 template <int D>
-SGM_INTERNAL cudaError_t sweep_launch_h_list(const ListLaunch& l, cudaStream_t s);
+SGM_INTERNAL cudaError_t sweep_launch_h_list(const ListLaunch& l, NodeChain& chain);
 template <int D>
 SGM_INTERNAL cudaError_t sweep_launch_first4(FirstStageArgs& f, Stream s);
 template <int D>
 SGM_INTERNAL cudaError_t sweep_launch_h2(const SweepArgs& a, Stream s);
 template <int D>
-SGM_INTERNAL cudaError_t sweep_launch_v_list(const ListLaunch& l, cudaStream_t s);
+SGM_INTERNAL cudaError_t sweep_launch_v_list(const ListLaunch& l, NodeChain& chain);
 
 #define SGM_INSTANTIATE_SWEEPS(D)                                                               \
     template <>                                                                                 \
@@ -1006,12 +1002,12 @@ SGM_INTERNAL cudaError_t sweep_launch_v_list(const ListLaunch& l, cudaStream_t s
         return SweepD<D>::launch_first(f, s);                                                   \
     }                                                                                           \
     template <>                                                                                 \
-    SGM_INTERNAL cudaError_t sweep_launch_h_list<D>(const ListLaunch& l, cudaStream_t s) {      \
-        return SweepD<D>::launch_h_list(l, s);                                                  \
+    SGM_INTERNAL cudaError_t sweep_launch_h_list<D>(const ListLaunch& l, NodeChain& chain) {      \
+        return SweepD<D>::launch_h_list(l, chain);                                              \
     }                                                                                           \
     template <>                                                                                 \
-    SGM_INTERNAL cudaError_t sweep_launch_v_list<D>(const ListLaunch& l, cudaStream_t s) {      \
-        return SweepD<D>::launch_v_list(l, s);                                                  \
+    SGM_INTERNAL cudaError_t sweep_launch_v_list<D>(const ListLaunch& l, NodeChain& chain) {      \
+        return SweepD<D>::launch_v_list(l, chain);                                              \
     }                                                                                           \
     template <>                                                                                 \
     SGM_INTERNAL cudaError_t sweep_launch_first4<D>(FirstStageArgs & f, Stream s) {       \
