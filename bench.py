@@ -48,15 +48,17 @@ BATCHED_LINE_STEPS = 5         # timed steps of the batched object of the defaul
 SERVED_OUT_RING = 4  # output buffers per pool pair (a pair can be in flight more than once)
 # DRAM bytes (read + write) per launch of a kernel, from the ncu captures summarised
 # under profiles/, with the fingerprint of the kernel sources they were taken on;
-# reported as null once those sources have changed since the capture.  The
-# 640x480 frame's figures come from the in-sequence capture (--cache-control
-# none: the L2 flushed once before the frame, as in the timed steps); the
-# 8-path frame's from a capture with ncu's default per-launch cache flush.
+# reported as null once those sources have changed since the capture.  All come
+# from in-sequence captures (--cache-control none: the L2 flushed once before the
+# frame, as in the timed steps); pairs_vh is the sum of its two launches.  The
+# 8-path frame's are the per-line sweeps', which contexts that time stages run.
 MEASURED_TRAFFIC = {
-    ("sgm_1242x375_d128_p8", "sweep_h"): (585012992, "f7a7031745fff723"),
-    ("sgm_1242x375_d128_p8", "sweep_diag+"): (311625472, "f7a7031745fff723"),
-    ("sgm_1242x375_d128_p8", "sweep_diag-"): (311849088, "f7a7031745fff723"),
-    ("sgm_1242x375_d128_p8", "sweep_v"): (241643136, "f7a7031745fff723"),
+    ("sgm_640x480_d128_p4", "pairs_vh"): (92325120, "3dd9b3c6c9537dac"),
+    ("sgm_640x480_d128_p4", "pairs_h_wta"): (52539392, "3dd9b3c6c9537dac"),
+    ("sgm_1242x375_d128_p8", "sweep_h"): (606967552, "3dd9b3c6c9537dac"),
+    ("sgm_1242x375_d128_p8", "sweep_diag+"): (349430784, "3dd9b3c6c9537dac"),
+    ("sgm_1242x375_d128_p8", "sweep_diag-"): (355507200, "3dd9b3c6c9537dac"),
+    ("sgm_1242x375_d128_p8", "sweep_v"): (285914624, "3dd9b3c6c9537dac"),
 }
 KERNEL_SOURCES = ("sgm_sweeps.cuh", "sgm_pairs.cuh", "sgm_device.cuh", "sgm_internal.h")
 
@@ -300,8 +302,7 @@ def workload_config(w, args):
 
 
 def run_post_bench(args, w, ws, rank, local):
-    """The path with post-filters (sgm_compute_ex_async, the captured graph)
-    on the workload's pair, resident in HBM."""
+    """The path with post-filters (sgm_compute_ex_async) on the workload's pair, resident in HBM."""
     import torch
     from paper_1610_04121_gb300 import sgm
 
@@ -511,7 +512,7 @@ def measure_batched(args, ws, rank, local, pg, steps, warmup, cpu_sample=False):
     total_ms = max_over_ranks(sum(a.elapsed_time(b) for a, b in ev), pg, dev)
     value = job_mdes(ws, steps, de, total_ms)
     # the same pairs as plain per-pair launches
-    for t in tuples:  # warm-up: tunes and captures one graph per pair
+    for t in tuples:  # warm-up: tunes every pair's schedule
         sgm.sgm_compute_async(ctx.handle, t[0], t[1], t[3], t[4], t[5], t[6], t[7], t[8], t[2])
     torch.cuda.synchronize(dev)
     a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -916,7 +917,8 @@ def main():
             "roofline": roofline, "frame_roofline": frame_roofline,
             "stage_ms": {k: round(v, 5) for k, v in mean_stage.items()},
             "stage_timing": f"separate pass of {stage_steps} steps with an event between kernels "
-                            "(the events lengthen that pass's frames)",
+                            "(the events lengthen that pass's frames"
+                            + (")" if w.n_paths == 4 else "; its stages are the per-line sweeps')"),
             "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches, "clocks": clocks,
             "batched": batched, "served": served,
         }

@@ -200,7 +200,7 @@ SGM_API int sgm_compute_async(sgm_ctx *ctx, const uint8_t *left, const uint8_t *
  * line pairs) from a device work list covering the group's pairs, longest
  * chains first.  A wave (the pairs whose
  * buffers fit the memory budget at once, at most 16 groups) is one CUDA
- * graph launch, the groups on concurrent branches; the graph is captured
+ * graph launch, the groups on concurrent branches; the graph is built
  * once per wave shape and replayed with the lists rewritten.  The first wave
  * of a new set of pair shapes autotunes the sweep grid (persistent blocks per
  * SM from {2, 3, 4, 5}: one warm-up and five timed runs each, the lowest

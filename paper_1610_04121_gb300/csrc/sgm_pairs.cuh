@@ -38,10 +38,11 @@
 // cycles; two warps per scheduler (a 640x480 frame) are bound by that and by
 // the chain of a step (two shuffles and two reductions), full schedulers by
 // the ALU.  Measured, whole frame, against the per-line sweeps (one line per
-// warp, sums in records): 1242x375 D=128 8 paths 390 -> 208 us, 1920x1080
-// D=128 8 paths 1440 -> 1008 us, 640x480 D=128 2 paths 84 -> 62 us, the same
-// with 4 paths and all post-filters 256 -> 182 us; the walks of the 640x480
-// 4-path frame take 38 us, the finishing launch 27 us.
+// warp, sums in records): 1242x375 D=128 8 paths 390 -> 202 us, 1920x1080
+// D=128 8 paths 1440 -> 935 us, 640x480 D=128 2 paths 84 -> 60 us, the same
+// with 4 paths and all post-filters 257 -> 163 us; alone the horizontal walks of
+// the 640x480 4-path frame take 30 us, the vertical ones 34 us, the finishing
+// launch 27 us.
 #pragma once
 
 #include "sgm_device.cuh"
