@@ -325,7 +325,7 @@ struct sgm_ctx {
     size_t mem_cap = 0;
     uint8_t* arena = nullptr;
     size_t arena_bytes = 0;
-    std::map<GraphKey, cudaGraphExec_t> graphs;
+    std::map<GraphKey, cudaGraphExec_t> graphs;  // null: seen once, no graph yet (enqueue_graph)
     std::string err;
     std::atomic<uint64_t> launches{0};
     bool stage_timing = false;
@@ -432,6 +432,12 @@ static int bounds_status(sgm_ctx* ctx) {
     return SGM_OK;
 }
 
+static void drop_graphs(sgm_ctx* ctx) {
+    for (auto& kv : ctx->graphs)
+        if (kv.second) cudaGraphExecDestroy(kv.second);
+    ctx->graphs.clear();
+}
+
 static int ensure_arena(sgm_ctx* ctx, uint8_t** arena, size_t* bytes, size_t need, bool clear_graphs) {
     if (*bytes >= need) return SGM_OK;
     const size_t used_elsewhere = ctx->serve_bytes.load();
@@ -445,8 +451,7 @@ static int ensure_arena(sgm_ctx* ctx, uint8_t** arena, size_t* bytes, size_t nee
         if (e != cudaSuccess) return fail(ctx, SGM_ECUDA, "cudaFree: %s", cudaGetErrorString(e));
     }
     if (clear_graphs) {
-        for (auto& kv : ctx->graphs) cudaGraphExecDestroy(kv.second);
-        ctx->graphs.clear();
+        drop_graphs(ctx);
     }
     void* p = nullptr;
     cudaError_t e = ctx_malloc(ctx, &p, need);
@@ -748,9 +753,11 @@ struct HostIO {
 
 // Enqueue through a cached CUDA graph for this problem and these pointers: the
 // blocking calls, which find the GPU idle (the whole sequence is there at once:
-// 100.2 us per 640x480 frame from pinned host images against 103.6 kernel by
+// 96.4 us per 640x480 frame from pinned host images against 99.1 kernel by
 // kernel), and contexts that time stages (the events between the kernels are
-// nodes of the graph).
+// nodes of the graph).  Making one takes about 45 us, so the first call with a
+// set of buffers runs kernel by kernel and the second one makes the graph (a
+// call on pinned buffers not seen before: 96x64 71 -> 31 us, 640x480 145 -> 101).
 // The key names the caller's buffers (a staged host buffer's arena copy is the
 // same for every host buffer).  An address that is staged in one call and
 // used in place in another (freed and reused as another kind of memory)
@@ -760,21 +767,31 @@ static int enqueue_graph(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const u
                          uint8_t* disp, cudaStream_t s, const HostIO& io = HostIO{}, const void* key_left = nullptr,
                          const void* key_right = nullptr, const void* key_out = nullptr) {
     GraphKey key{p, key_left ? key_left : left, key_right ? key_right : right, key_out ? key_out : disp, arena};
+    const bool timed = ctx->stage_timing && !p.post;
     auto it = ctx->graphs.find(key);
     if (it == ctx->graphs.end()) {
-        if (ctx->graphs.size() >= 64) {
-            for (auto& kv : ctx->graphs) cudaGraphExecDestroy(kv.second);
-            ctx->graphs.clear();
+        if (ctx->graphs.size() >= 64) drop_graphs(ctx);
+        it = ctx->graphs.emplace(key, nullptr).first;
+        if (!timed) {
+            const Stream st(s, true);
+            if (io.src[0]) CUDA_TRY(ctx, launch_stage(io.src[0], io.dst[0], io.src[1], io.dst[1], io.img_bytes, st));
+            CUDA_TRY(ctx, enqueue_path(ctx, p, arena, left, right, disp, nullptr, s, false));
+            if (io.out_src) CUDA_TRY(ctx, launch_stage(io.out_src, io.out_dst, nullptr, nullptr, io.out_bytes, st));
+            ctx->launches += io.launches();
+            ctx->last_stages = ctx->last_n_paths = 0;
+            ctx->last_sched = p.sched;
+            return SGM_OK;
         }
+    }
+    if (!it->second) {
         cudaGraph_t g = nullptr;
         CUDA_TRY(ctx, cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal));
         const uint64_t before = ctx->launches.load();
         cudaError_t e = cudaSuccess;
-        const Stream st(ctx->capture_stream, !(ctx->stage_timing && !p.post));
+        const Stream st(ctx->capture_stream, !timed);
         if (io.src[0]) e = launch_stage(io.src[0], io.dst[0], io.src[1], io.dst[1], io.img_bytes, st);
         if (e == cudaSuccess)
-            e = enqueue_path(ctx, p, arena, left, right, disp, nullptr, ctx->capture_stream,
-                             ctx->stage_timing && !p.post);
+            e = enqueue_path(ctx, p, arena, left, right, disp, nullptr, ctx->capture_stream, timed);
         if (e == cudaSuccess && io.out_src)
             e = launch_stage(io.out_src, io.out_dst, nullptr, nullptr, io.out_bytes, st);
         ctx->launches = before;  // captured, not launched
@@ -788,12 +805,12 @@ static int enqueue_graph(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const u
         e = cudaGraphInstantiate(&exec, g, 0);
         cudaGraphDestroy(g);
         if (e != cudaSuccess) return fail(ctx, SGM_ECUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
-        it = ctx->graphs.emplace(key, exec).first;
+        it->second = exec;
     }
     CUDA_TRY(ctx, cudaGraphLaunch(it->second, s));
     ctx->launches += launches_per_path(p) + io.launches();
-    ctx->last_stages = (ctx->stage_timing && !p.post) ? stages_per_path(p) : 0;
-    ctx->last_n_paths = (ctx->stage_timing && !p.post) ? p.n_paths : 0;
+    ctx->last_stages = timed ? stages_per_path(p) : 0;
+    ctx->last_n_paths = timed ? p.n_paths : 0;
     ctx->last_sched = p.sched;
     return SGM_OK;
 }
@@ -1864,7 +1881,7 @@ int sgm_destroy(sgm_ctx* ctx) {
     if (ctx->worker.joinable()) ctx->worker.join();
     cudaSetDevice(ctx->device);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
-    for (auto& kv : ctx->graphs) cudaGraphExecDestroy(kv.second);
+    drop_graphs(ctx);
     if (ctx->arena) cudaFree(ctx->arena);
     list_exec_release(ctx->batch_exec);
     for (auto& sl : ctx->slots) {
