@@ -242,13 +242,22 @@ bool valid_problem(const Problem& p, std::string* why) {
     return false;
 }
 
+// How a buffer of a blocking call reaches the device: used in place (device
+// memory), copied by a staging kernel of the call's graph (pinned host memory),
+// or copied by cudaMemcpyAsync outside the graph (pageable host memory).
+enum Way { kInPlace = 0, kStaged = 1, kCopied = 2 };
+
+// `ways`: the Way of left, right and out, two bits each.  One address can be
+// pageable in one call and pinned in the next (registered meanwhile, or freed
+// and allocated again), and the graph's nodes differ with that.
 struct GraphKey {
     Problem p;
     const void *left, *right, *out, *arena;
+    int ways;
     bool operator<(const GraphKey& o) const {
-        return std::tie(p.W, p.H, p.D, p.P1, p.P2, p.n_paths, p.ct62, p.post, p.sched, left, right, out, arena) <
+        return std::tie(p.W, p.H, p.D, p.P1, p.P2, p.n_paths, p.ct62, p.post, p.sched, left, right, out, arena, ways) <
                std::tie(o.p.W, o.p.H, o.p.D, o.p.P1, o.p.P2, o.p.n_paths, o.p.ct62, o.p.post, o.p.sched, o.left, o.right,
-                        o.out, o.arena);
+                        o.out, o.arena, o.ways);
     }
 };
 
@@ -748,6 +757,7 @@ struct HostIO {
     const uint8_t* out_src = nullptr;            // arena output
     uint8_t* out_dst = nullptr;                  // host output
     size_t img_bytes = 0, out_bytes = 0;
+    int ways = 0;                                // GraphKey::ways
     int launches() const { return (src[0] ? 1 : 0) + (out_src ? 1 : 0); }
 };
 
@@ -759,14 +769,11 @@ struct HostIO {
 // set of buffers runs kernel by kernel and the second one makes the graph (a
 // call on pinned buffers not seen before: 96x64 71 -> 31 us, 640x480 145 -> 101).
 // The key names the caller's buffers (a staged host buffer's arena copy is the
-// same for every host buffer).  An address that is staged in one call and
-// used in place in another (freed and reused as another kind of memory)
-// reuses the first call's graph, which is correct for either kind: the copies
-// work on device memory, and the kernels can read pinned host memory.
+// same for every host buffer) and the way each one takes to the device.
 static int enqueue_graph(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const uint8_t* left, const uint8_t* right,
                          uint8_t* disp, cudaStream_t s, const HostIO& io = HostIO{}, const void* key_left = nullptr,
                          const void* key_right = nullptr, const void* key_out = nullptr) {
-    GraphKey key{p, key_left ? key_left : left, key_right ? key_right : right, key_out ? key_out : disp, arena};
+    GraphKey key{p, key_left ? key_left : left, key_right ? key_right : right, key_out ? key_out : disp, arena, io.ways};
     const bool timed = ctx->stage_timing && !p.post;
     auto it = ctx->graphs.find(key);
     if (it == ctx->graphs.end()) {
@@ -884,11 +891,6 @@ static int choose_schedule(sgm_ctx* ctx, Problem& p, uint8_t* arena, const uint8
 }
 
 // Copy-in / path / copy-out for one pair into `arena` (already large enough).
-// Device memory and pinned host memory are read and written in place by the
-// kernels (pinned host memory is mapped into the device's address space, so
-// the census reads the images and the last kernel writes the output over the
-// host link with no separate copy); pageable host memory is staged through
-// the arena with copies.
 static int enqueue_pair(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const uint8_t* left, const uint8_t* right,
                         uint8_t* disp, cudaStream_t s) {
     const Layout l = layout_for(p);
@@ -898,26 +900,31 @@ static int enqueue_pair(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const ui
     // requests; the Census tiles would read every image byte several times
     // over the link), inside the call's graph; pageable host buffers by
     // cudaMemcpyAsync before and after it
-    const cudaMemoryType kl = pointer_kind(left), kr = pointer_kind(right), ko = pointer_kind(disp);
-    auto device_side = [](cudaMemoryType t) { return t == cudaMemoryTypeDevice || t == cudaMemoryTypeManaged; };
+    auto way = [](const void* q) {
+        const cudaMemoryType t = pointer_kind(q);
+        return t == cudaMemoryTypeDevice || t == cudaMemoryTypeManaged ? kInPlace
+                                                                       : (t == cudaMemoryTypeHost ? kStaged : kCopied);
+    };
+    const Way wl = way(left), wr = way(right), wo = way(disp);
     const uint8_t* dl = left;
     const uint8_t* dr = right;
     uint8_t* dout = disp;
     HostIO io;
     io.img_bytes = wh;
+    io.ways = wl | wr << 2 | wo << 4;
     int n_st = 0;
-    if (!device_side(kl)) {
+    if (wl != kInPlace) {
         dl = arena + l.in_left;
-        if (kl == cudaMemoryTypeHost) {
+        if (wl == kStaged) {
             io.src[n_st] = left;
             io.dst[n_st++] = arena + l.in_left;
         } else {
             CUDA_TRY(ctx, cudaMemcpyAsync(arena + l.in_left, left, wh, cudaMemcpyHostToDevice, s));
         }
     }
-    if (!device_side(kr)) {
+    if (wr != kInPlace) {
         dr = arena + l.in_right;
-        if (kr == cudaMemoryTypeHost) {
+        if (wr == kStaged) {
             io.src[n_st] = right;
             io.dst[n_st++] = arena + l.in_right;
         } else {
@@ -925,9 +932,9 @@ static int enqueue_pair(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const ui
         }
     }
     const size_t ob = (p.post ? 2 : 1) * wh;
-    if (!device_side(ko)) {
+    if (wo != kInPlace) {
         dout = arena + l.out;
-        if (ko == cudaMemoryTypeHost) {
+        if (wo == kStaged) {
             io.out_src = dout;
             io.out_dst = disp;
             io.out_bytes = ob;
@@ -941,8 +948,7 @@ static int enqueue_pair(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const ui
     if (rc != SGM_OK) return rc;
     rc = enqueue_graph(ctx, q, arena, dl, dr, dout, s, io, left, right, disp);
     if (rc != SGM_OK) return rc;
-    if (!device_side(ko) && ko != cudaMemoryTypeHost)
-        CUDA_TRY(ctx, cudaMemcpyAsync(disp, dout, ob, cudaMemcpyDeviceToHost, s));
+    if (wo == kCopied) CUDA_TRY(ctx, cudaMemcpyAsync(disp, dout, ob, cudaMemcpyDeviceToHost, s));
     return SGM_OK;
 }
 
