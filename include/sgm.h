@@ -93,7 +93,12 @@ typedef struct sgm_pair {
  * Create a context on CUDA device `device` (makes it current for the calling
  * thread).  `mem_cap_bytes` caps the device memory the context may hold for
  * its work arena and served requests (0 = no cap beyond the device's free
- * memory).  `flags` is 0 or a combination of SGM_FLAG_STAGE_TIMING and
+ * memory).  Without a cap a path may take more memory to run faster: 2 and 8
+ * paths and the post form run the paired lines (SGM_SCHED_PAIRS) with 2 and 7
+ * bytes per pixel and disparity, twice that with the left-right check, in place
+ * of the per-line sweeps' 3 and 7 (a batched or served pair of 8 paths 7 in
+ * place of 4).  Under a cap every path takes at most what the per-line sweeps
+ * need, and runs these where the paired lines need more.  `flags` is 0 or a combination of SGM_FLAG_STAGE_TIMING and
  * SGM_FLAG_CENSUS_FULL; the Census type holds for every entry point of the
  * context (sgm_compute_static always uses the CSCT).  On success *out
  * receives the context.
@@ -375,7 +380,8 @@ SGM_API const char *sgm_stage_label(const sgm_ctx *ctx, int i);
  * schedule s; -1 restores autotuning.  Paths of 2 and 8 directions and the
  * post form (sgm_compute_ex) run the paired lines too (with 8 paths the
  * diagonals store their costs as the vertical pair does), or the per-line
- * sweeps where the paired cubes do not fit the memory cap or the device.
+ * sweeps where the device has no room for the paired cubes or the context has
+ * a memory cap that they would strain (sgm_create).
  * Errors: SGM_EINVAL (null context, unknown schedule).
  */
 #define SGM_SCHED_V_THEN_H 0

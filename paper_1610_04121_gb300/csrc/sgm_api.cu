@@ -676,23 +676,26 @@ static cudaError_t enqueue_match(const Problem& p, const Layout& l, uint8_t* are
 // form) and room for the path in the context's arena.  The paired schedule
 // holds the stored costs of every direction at once and both passes of the
 // left-right check (2, 7 or 14 bytes per pixel and disparity against 3 to 7 of
-// the per-line sweeps): where the memory cap or the device has no room for
-// that, and in contexts that time stages (their stages are the per-line
-// sweeps'), the per-line sweeps run.
+// the per-line sweeps): where the device has no room for that, and in contexts
+// that time stages (their stages are the per-line sweeps'), the per-line sweeps
+// run.  Under a memory cap the arena never grows past what the per-line sweeps
+// need, so that whatever a served request or a batch finds left below the cap
+// does not depend on the schedule.
 static int prepare_arena(sgm_ctx* ctx, Problem& p, size_t extra = 0) {
     p.sched = SGM_SCHED_V_THEN_H;
+    const size_t base = layout_for(p).total + extra;
     if ((p.n_paths != 4 || p.post) && !ctx->stage_timing && pairs_fit(p)) {
         Problem q = p;
         q.sched = SGM_SCHED_PAIRS;
         const size_t need = layout_for(q).total + extra;
-        if (need <= ctx->arena_bytes || !ctx->mem_cap || need + ctx->serve_bytes.load() <= ctx->mem_cap) {
+        if (!ctx->mem_cap || need <= std::max(ctx->arena_bytes, base)) {
             const int rc = ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, need, true);
             const bool injected = ctx->fail_alloc_at > 0 && ctx->alloc_count.load() == ctx->fail_alloc_at;
             if (rc == SGM_OK) p.sched = SGM_SCHED_PAIRS;
             if (rc != SGM_ENOMEM || injected) return rc;
         }
     }
-    return ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, layout_for(p).total + extra, true);
+    return ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, base, true);
 }
 
 // Enqueue the whole path (Section 2, stages 2-4) for one pair whose inputs
@@ -1011,13 +1014,17 @@ static bool runs_alone(const Problem& p) {
 
 // The schedule of a batched pair within `room` bytes, one of pairs alike with
 // `px` pixels together: paired lines where their cubes fit (2, 3 or 7 bytes per
-// pixel and disparity), else the per-line sweeps (3 or 4).  Up to 4 paths and
+// pixel and disparity), else the per-line sweeps (3 or 4).  Under a memory cap
+// (`capped`) a pair takes no more than the per-line sweeps would: see
+// prepare_arena.  Up to 4 paths and
 // 2^18 pixels the sweeps' shorter chains win, which meet in the middle: us per
 // pair, paired / per-line, two of 240x180 D=128 4 paths 52.7 / 43.2, two of
 // 320x240 59.0 / 55.4, 32 of 96x64 5.6 / 5.3; 32 of 240x180 13.5 / 14.7; with 8
 // paths the paired lines lead from 64x48 on (5.7 / 6.1).
-static int batch_sched(Problem p, size_t room, double px) {
+static int batch_sched(Problem p, size_t room, double px, bool capped) {
     if (p.n_paths != 8 && px < 262144.0) return SGM_SCHED_V_THEN_H;
+    p.sched = SGM_SCHED_V_THEN_H;
+    if (capped) room = std::min(room, layout_for(p, true).total);
     p.sched = SGM_SCHED_PAIRS;
     return pairs_fit(p) && layout_for(p, true).total <= room ? SGM_SCHED_PAIRS : SGM_SCHED_V_THEN_H;
 }
@@ -1473,7 +1480,7 @@ static int run_batch(sgm_ctx* ctx, ListExec& x, std::vector<BatchItem>& items, u
     }
     std::map<std::pair<int, int>, double> px;  // pixels of the pairs of one D and path count
     for (const BatchItem& it : items) px[{it.p.D, it.p.n_paths}] += static_cast<double>(it.p.W) * it.p.H;
-    for (BatchItem& it : items) it.p.sched = batch_sched(it.p, budget, px[{it.p.D, it.p.n_paths}]);
+    for (BatchItem& it : items) it.p.sched = batch_sched(it.p, budget, px[{it.p.D, it.p.n_paths}], ctx->mem_cap != 0);
     std::stable_sort(items.begin(), items.end(), [](const BatchItem& a, const BatchItem& c) {
         return batch_key(a) < batch_key(c);
     });
@@ -1726,7 +1733,8 @@ static void serve_loop(sgm_ctx* ctx) {
         std::set<std::tuple<int, int, int, int>> keys;
         while (rc == SGM_OK && !ctx->queue.empty() && sl->reqs.size() < static_cast<size_t>(kServeMaxPairs)) {
             Request& r = ctx->queue.front();
-            r.p.sched = batch_sched(r.p, budget - used, 8.0 * r.p.W * r.p.H);  // a stream of requests like this one
+            // a stream of requests like this one
+            r.p.sched = batch_sched(r.p, budget - used, 8.0 * r.p.W * r.p.H, ctx->mem_cap != 0);
             const size_t sz = layout_for(r.p, true).total;
             const auto key = batch_key(BatchItem{r.p, nullptr, nullptr, nullptr, 0});
             if (used + sz > budget || (!keys.count(key) && keys.size() == static_cast<size_t>(kListGroups))) break;
