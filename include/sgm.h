@@ -108,7 +108,9 @@ typedef struct sgm_pair {
  * needed it returns SGM_ENOMEM, or sgm_create itself for its own first
  * allocations, and the context stays usable); SGM_TEST_BAD_JOB=n gives the
  * first n batched waves one sweep descriptor with a wrong D, which its kernel
- * skips and reports through the device status word (SGM_EDEVICE).
+ * skips and reports through the device status word (SGM_EDEVICE);
+ * SGM_TEST_ALLOC_LIMIT=n makes device allocations of more than n bytes fail as
+ * if the device had no room for them.
  * Errors: SGM_EINVAL (null out, bad device, unknown flag), SGM_ENOMEM,
  * SGM_ECUDA.
  */

@@ -6,6 +6,7 @@
 #include <chrono>
 #include <condition_variable>
 #include <cstdarg>
+#include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -334,6 +335,11 @@ struct sgm_ctx {
     size_t mem_cap = 0;
     uint8_t* arena = nullptr;
     size_t arena_bytes = 0;
+    // arenas that a larger one replaced for the paired schedule alone: graphs
+    // that the caller captured may still use them (prepare_arena); and the
+    // smallest arena that the device refused for it
+    std::vector<uint8_t*> replaced;
+    size_t refused_bytes = SIZE_MAX;
     std::map<GraphKey, cudaGraphExec_t> graphs;  // null: seen once, no graph yet (enqueue_graph)
     std::string err;
     std::atomic<uint64_t> launches{0};
@@ -355,8 +361,10 @@ struct sgm_ctx {
 
     // test hooks, read at sgm_create: SGM_TEST_FAIL_ALLOC=n fails the n-th
     // allocation; SGM_TEST_BAD_JOB=n gives n waves one descriptor with a D its
-    // kernel rejects (through the device status word)
+    // kernel rejects (through the device status word); SGM_TEST_ALLOC_LIMIT=n
+    // fails device allocations of more than n bytes
     int fail_alloc_at = 0;
+    size_t alloc_limit = SIZE_MAX;
     std::atomic<int> alloc_count{0};
     // bounds-checked build: SGM_TEST_BOUNDS_SHRINK=1 declares the paired
     // schedule's cube arrays one quad shorter than they are, so that a guard
@@ -422,7 +430,7 @@ static bool injected_alloc_failure(sgm_ctx* ctx) {
 }
 
 static cudaError_t ctx_malloc(sgm_ctx* ctx, void** p, size_t bytes) {
-    return injected_alloc_failure(ctx) ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+    return injected_alloc_failure(ctx) || bytes > ctx->alloc_limit ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
 }
 
 static cudaError_t ctx_malloc_host(sgm_ctx* ctx, void** p, size_t bytes) {
@@ -447,6 +455,11 @@ static void drop_graphs(sgm_ctx* ctx) {
     ctx->graphs.clear();
 }
 
+static void free_replaced(sgm_ctx* ctx) {
+    for (uint8_t* a : ctx->replaced) cudaFree(a);
+    ctx->replaced.clear();
+}
+
 static int ensure_arena(sgm_ctx* ctx, uint8_t** arena, size_t* bytes, size_t need, bool clear_graphs) {
     if (*bytes >= need) return SGM_OK;
     const size_t used_elsewhere = ctx->serve_bytes.load();
@@ -461,6 +474,7 @@ static int ensure_arena(sgm_ctx* ctx, uint8_t** arena, size_t* bytes, size_t nee
     }
     if (clear_graphs) {
         drop_graphs(ctx);
+        free_replaced(ctx);
     }
     void* p = nullptr;
     cudaError_t e = ctx_malloc(ctx, &p, need);
@@ -681,6 +695,14 @@ static cudaError_t enqueue_match(const Problem& p, const Layout& l, uint8_t* are
 // run.  Under a memory cap the arena never grows past what the per-line sweeps
 // need, so that whatever a served request or a batch finds left below the cap
 // does not depend on the schedule.
+//
+// What the per-line sweeps need decides when the arena has to grow; it is freed
+// for that, and the larger of the two is tried first.  An arena that holds the
+// per-line sweeps already is only ever replaced by one in hand, half as large
+// again where the device has it (so that the replaced ones together stay below
+// twice the last one), never in a stream under capture, and not for a size that
+// the device has refused since the arena last had to grow: the call then runs in
+// the arena as it is.
 static int prepare_arena(sgm_ctx* ctx, Problem& p, size_t extra = 0) {
     p.sched = SGM_SCHED_V_THEN_H;
     const size_t base = layout_for(p).total + extra;
@@ -688,11 +710,36 @@ static int prepare_arena(sgm_ctx* ctx, Problem& p, size_t extra = 0) {
         Problem q = p;
         q.sched = SGM_SCHED_PAIRS;
         const size_t need = layout_for(q).total + extra;
-        if (!ctx->mem_cap || need <= std::max(ctx->arena_bytes, base)) {
+        if (need <= ctx->arena_bytes) {
+            p.sched = SGM_SCHED_PAIRS;
+            return SGM_OK;
+        }
+        if (base > ctx->arena_bytes && (!ctx->mem_cap || need <= base)) {
             const int rc = ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, need, true);
             const bool injected = ctx->fail_alloc_at > 0 && ctx->alloc_count.load() == ctx->fail_alloc_at;
             if (rc == SGM_OK) p.sched = SGM_SCHED_PAIRS;
+            if (rc == SGM_OK) ctx->refused_bytes = SIZE_MAX;  // the device has memory again
             if (rc != SGM_ENOMEM || injected) return rc;
+            ctx->refused_bytes = std::min(ctx->refused_bytes, need);
+        } else if (base <= ctx->arena_bytes && !ctx->mem_cap && need < ctx->refused_bytes) {
+            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+            CUDA_TRY(ctx, cudaStreamIsCapturing(ctx->stream, &cs));
+            if (cs != cudaStreamCaptureStatusNone) return SGM_OK;
+            size_t grown = std::max(need, ctx->arena_bytes + ctx->arena_bytes / 2);
+            void* a = nullptr;
+            cudaError_t e = ctx_malloc(ctx, &a, grown);
+            if (e != cudaSuccess && grown > need) e = ctx_malloc(ctx, &a, grown = need);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                ctx->refused_bytes = need;
+                return SGM_OK;
+            }
+            drop_graphs(ctx);
+            ctx->replaced.push_back(ctx->arena);
+            ctx->arena = static_cast<uint8_t*>(a);
+            ctx->arena_bytes = grown;
+            p.sched = SGM_SCHED_PAIRS;
+            return SGM_OK;
         }
     }
     return ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, base, true);
@@ -1850,6 +1897,7 @@ int sgm_create(sgm_ctx** out, int device, size_t mem_cap_bytes, unsigned flags) 
         return fail(nullptr, SGM_ECUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
     }
     if (const char* v = std::getenv("SGM_TEST_FAIL_ALLOC")) ctx->fail_alloc_at = std::atoi(v);
+    if (const char* v = std::getenv("SGM_TEST_ALLOC_LIMIT")) ctx->alloc_limit = std::strtoull(v, nullptr, 10);
     if (const char* v = std::getenv("SGM_TEST_BAD_JOB")) ctx->bad_job_waves = std::atoi(v);
 #ifdef SGM_BOUNDS_CHECK
     if (const char* v = std::getenv("SGM_TEST_BOUNDS_SHRINK")) ctx->bounds_shrink = std::atoi(v) != 0;
@@ -1897,6 +1945,7 @@ int sgm_destroy(sgm_ctx* ctx) {
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     drop_graphs(ctx);
     if (ctx->arena) cudaFree(ctx->arena);
+    free_replaced(ctx);
     list_exec_release(ctx->batch_exec);
     for (auto& sl : ctx->slots) {
         if (sl.arena) cudaFreeAsync(sl.arena, sl.stream);
