@@ -325,8 +325,8 @@ SGM_API int sgm_debug_stages(sgm_ctx *ctx, const uint8_t *left, const uint8_t *r
  * (the horizontal second halves with the winner-take-all).  With 8 paths:
  * sweep_h (the horizontal pair with the first halves of the three
  * vertical-type pairs), sweep_diag+, sweep_diag-, sweep_v.  A context created
- * with SGM_FLAG_STAGE_TIMING runs these per-line sweeps for 2 and 8 paths and
- * for the post form.
+ * with SGM_FLAG_STAGE_TIMING runs these per-line sweeps for 2 and 8 paths, so
+ * its times are not those of the paired lines that other contexts run.
  */
 SGM_API int sgm_stage_times(sgm_ctx *ctx, float *ms_out, int n);
 

@@ -690,11 +690,12 @@ static cudaError_t enqueue_match(const Problem& p, const Layout& l, uint8_t* are
 // form) and room for the path in the context's arena.  The paired schedule
 // holds the stored costs of every direction at once and both passes of the
 // left-right check (2, 7 or 14 bytes per pixel and disparity against 3 to 7 of
-// the per-line sweeps): where the device has no room for that, and in contexts
-// that time stages (their stages are the per-line sweeps'), the per-line sweeps
-// run.  Under a memory cap the arena never grows past what the per-line sweeps
-// need, so that whatever a served request or a batch finds left below the cap
-// does not depend on the schedule.
+// the per-line sweeps): where the device has no room for that, and for 2 and 8
+// paths in contexts that time stages (the stages they name are the per-line
+// sweeps'; the post form is never timed), the per-line sweeps run.  Under a
+// memory cap the arena never grows past what the per-line sweeps need, so that
+// whatever a served request or a batch finds left below the cap does not depend
+// on the schedule.
 //
 // What the per-line sweeps need decides when the arena has to grow; it is freed
 // for that, and the larger of the two is tried first.  An arena that holds the
@@ -706,7 +707,7 @@ static cudaError_t enqueue_match(const Problem& p, const Layout& l, uint8_t* are
 static int prepare_arena(sgm_ctx* ctx, Problem& p, size_t extra = 0) {
     p.sched = SGM_SCHED_V_THEN_H;
     const size_t base = layout_for(p).total + extra;
-    if ((p.n_paths != 4 || p.post) && !ctx->stage_timing && pairs_fit(p)) {
+    if (((p.n_paths != 4 && !ctx->stage_timing) || p.post) && pairs_fit(p)) {
         Problem q = p;
         q.sched = SGM_SCHED_PAIRS;
         const size_t need = layout_for(q).total + extra;
