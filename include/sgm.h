@@ -335,10 +335,14 @@ SGM_API const char *sgm_stage_name(int n_paths, int i);
 
 /*
  * The bounds-checked build (the library compiled with -DSGM_BOUNDS_CHECK,
- * `python -m paper_1610_04121_gb300.build --bounds-check`): every global
- * access of the kernels, and the shared-memory feature indices of the cost
- * kernels, is tested against the extent of its array; a violation records a
- * site number in a device fault word and skips the access (no trap).  The
+ * `python -m paper_1610_04121_gb300.build --bounds-check`): every access of the
+ * kernels to images, features, costs, path states, penalties, sums and
+ * disparities (all but the work lists' headers, the staging copies and the
+ * unpacking kernels of sgm_debug_stages), and the shared-memory feature indices
+ * of the cost kernels, is tested against the extent of its array; a violation
+ * records a site number in a device fault word and skips the access (no trap).
+ * SGM_TEST_BOUNDS_SITE=n in the environment of sgm_create makes the guard at
+ * site n report every access (a test hook; nothing leaves its array).  The
  * synchronous calls (sgm_compute, sgm_compute_ex, sgm_compute_batch,
  * sgm_debug_stages, and sgm_poll for served requests) then return
  * SGM_EDEVICE.  sgm_bounds_checked() is 1 in that build, else 0;

@@ -43,6 +43,14 @@ unsigned take_bounds_fault() {
     }
     return first;
 }
+static std::vector<void (*)(unsigned)>& bounds_sites() {
+    static std::vector<void (*)(unsigned)> setters;
+    return setters;
+}
+void register_bounds_site(void (*setter)(unsigned)) { bounds_sites().push_back(setter); }
+void set_bounds_site(unsigned site) {
+    for (auto setter : bounds_sites()) setter(site);
+}
 // sgm_stages.cu: copy n bytes src0 -> dst0 and, when src1 is not null,
 // src1 -> dst1 (pinned host buffers to or from the work arena).
 cudaError_t launch_stage(const uint8_t* src0, uint8_t* dst0, const uint8_t* src1, uint8_t* dst1, size_t n,
@@ -1902,6 +1910,7 @@ int sgm_create(sgm_ctx** out, int device, size_t mem_cap_bytes, unsigned flags) 
     if (const char* v = std::getenv("SGM_TEST_BAD_JOB")) ctx->bad_job_waves = std::atoi(v);
 #ifdef SGM_BOUNDS_CHECK
     if (const char* v = std::getenv("SGM_TEST_BOUNDS_SHRINK")) ctx->bounds_shrink = std::atoi(v) != 0;
+    if (const char* v = std::getenv("SGM_TEST_BOUNDS_SITE")) set_bounds_site(static_cast<unsigned>(std::atoi(v)));
 #endif
     {
         int rc = list_exec_init(ctx, ctx->batch_exec);

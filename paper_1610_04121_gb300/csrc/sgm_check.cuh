@@ -5,7 +5,12 @@
 // word and the access is skipped (a load yields zeros).  Nothing traps.  The
 // host reads and clears the fault words after every synchronous call and
 // reports SGM_EDEVICE.  In the ordinary build every guard is the constant
-// true and compiles away.
+// true and compiles away.  Not guarded: the work lists' headers, the staging
+// copies and the debug unpacking kernels, whose loops run to the same extents.
+//
+// Sites: 1xx the paired lines, 2xx the per-line sweeps, 3xx the stages.  A test
+// hook (SGM_TEST_BOUNDS_SITE=n at sgm_create) makes the guard at site n take
+// every access for a violation: nothing is accessed out of range.
 #pragma once
 
 #include <cstddef>
@@ -18,19 +23,22 @@ namespace sgm {
 // wins, all words are cleared); 0 when none fired.
 void register_bounds_reader(unsigned (*reader)());
 unsigned take_bounds_fault();
+// Host: the site whose guard fires on every access (0: none), in every translation unit.
+void register_bounds_site(void (*setter)(unsigned));
+void set_bounds_site(unsigned site);
 
 #ifdef SGM_BOUNDS_CHECK
-static __device__ unsigned int g_bounds_fault = 0;
+static __device__ unsigned int g_bounds_fault = 0, g_bounds_site = 0;
 
 __device__ __forceinline__ bool bounds_guard(const void* p, size_t n, const void* lo, const void* hi, unsigned site) {
     const char* q = static_cast<const char*>(p);
-    if (q >= static_cast<const char*>(lo) && q + n <= static_cast<const char*>(hi)) return true;
+    if (q >= static_cast<const char*>(lo) && q + n <= static_cast<const char*>(hi) && site != g_bounds_site) return true;
     atomicCAS(&g_bounds_fault, 0u, site);
     return false;
 }
 
 __device__ __forceinline__ bool bounds_guard_index(long long i, long long n, unsigned site) {
-    if (i >= 0 && i < n) return true;
+    if (i >= 0 && i < n && site != g_bounds_site) return true;
     atomicCAS(&g_bounds_fault, 0u, site);
     return false;
 }
@@ -42,8 +50,12 @@ unsigned take_bounds_fault_here() {
     if (v != 0) cudaMemcpyToSymbol(g_bounds_fault, &z, sizeof z);
     return v;
 }
+void set_bounds_site_here(unsigned site) { cudaMemcpyToSymbol(g_bounds_site, &site, sizeof site); }
 struct BoundsReaderRegistrar {
-    BoundsReaderRegistrar() { register_bounds_reader(&take_bounds_fault_here); }
+    BoundsReaderRegistrar() {
+        register_bounds_reader(&take_bounds_fault_here);
+        register_bounds_site(&set_bounds_site_here);
+    }
 };
 const BoundsReaderRegistrar g_bounds_registrar;
 }  // namespace

@@ -769,8 +769,11 @@ __device__ __forceinline__ void finish(const PairsArgs& a, int r, int s, uint32_
     if constexpr (POST) {
         if (a.p2map) {
             const size_t i = static_cast<size_t>(r) * a.QW + q0 + min(lane, nq - 1);
-            p2l = __ldg(a.p2map + i);
-            if (NP > 2) p2r = __ldg(a.p2map + static_cast<size_t>(a.QW) * a.QH + i);
+            const size_t units = static_cast<size_t>(a.QW) * a.QH;
+            if (SGM_GUARD_INDEX(static_cast<long long>(i), static_cast<long long>(units), 119)) {
+                p2l = __ldg(a.p2map + i);
+                if (NP > 2) p2r = __ldg(a.p2map + units + i);
+            }
         }
     }
     auto p2_at = [&](uint32_t words, int i, uint32_t sel) -> uint32_t {
@@ -959,13 +962,16 @@ __device__ __forceinline__ void finish(const PairsArgs& a, int r, int s, uint32_
             word |= dd << (8 * h);
             if (POST && a.Sdbg) {  // debug: natural-order S
                 const int x = 2 * (q0 + i) + h, y = 2 * r;
+                auto put = [&](size_t p, uint32_t v) {
+                    if (SGM_GUARD_INDEX(static_cast<long long>(p), static_cast<long long>(a.W) * a.H * D, 120))
+                        a.Sdbg[p] = static_cast<uint16_t>(v);
+                };
                 if (x < a.W) {
 #pragma unroll
                     for (int j = 0; j < K; ++j) {
-                        const size_t d = static_cast<size_t>(K * lane + j);
-                        const size_t p = (static_cast<size_t>(y) * a.W + x) * D + d;
-                        a.Sdbg[p] = static_cast<uint16_t>(S[j] & 0xffffu);
-                        if (y + 1 < a.H) a.Sdbg[p + static_cast<size_t>(a.W) * D] = static_cast<uint16_t>(S[j] >> 16);
+                        const size_t p = (static_cast<size_t>(y) * a.W + x) * D + static_cast<size_t>(K * lane + j);
+                        put(p, S[j] & 0xffffu);
+                        if (y + 1 < a.H) put(p + static_cast<size_t>(a.W) * D, S[j] >> 16);
                     }
                 }
             }

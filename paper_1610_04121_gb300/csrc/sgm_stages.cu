@@ -266,6 +266,7 @@ __device__ __forceinline__ void cost_body(const FT* __restrict__ Fb, const FT* _
     __shared__ __align__(16) FT fb[kMcSeg];
     const int x0 = seg * kMcSeg;
     const FT* fmrow = Fm + (size_t)y * W;
+    [[maybe_unused]] const long long rows = H;
     {
         // every load is issued before the first shared-memory store
         constexpr int NI = (NF + kMcThreads - 1) / kMcThreads, NB = kMcSeg / kMcThreads;
@@ -273,12 +274,16 @@ __device__ __forceinline__ void cost_body(const FT* __restrict__ Fb, const FT* _
 #pragma unroll
         for (int it = 0; it < NI; ++it) {
             const int i = threadIdx.x + it * kMcThreads, gx = x0 - D + i;
-            vm[it] = (i < NF && gx >= 0 && gx < W) ? __ldg(fmrow + gx) : FT(0);
+            vm[it] = (i < NF && gx >= 0 && gx < W && SGM_GUARD_INDEX((long long)y * W + gx, rows * W, 309))
+                         ? __ldg(fmrow + gx)
+                         : FT(0);
         }
 #pragma unroll
         for (int it = 0; it < NB; ++it) {
             const int i = threadIdx.x + it * kMcThreads;
-            vb[it] = (x0 + i < W) ? __ldg(Fb + (size_t)y * W + x0 + i) : FT(0);
+            vb[it] = (x0 + i < W && SGM_GUARD_INDEX((long long)y * W + x0 + i, rows * W, 309))
+                         ? __ldg(Fb + (size_t)y * W + x0 + i)
+                         : FT(0);
         }
 #pragma unroll
         for (int it = 0; it < NI; ++it) {
@@ -423,12 +428,16 @@ __device__ __forceinline__ void cost_quads_body(const FT* __restrict__ Fb, const
 #pragma unroll
         for (int it = 0; it < NI; ++it) {
             const int i = threadIdx.x + it * kQcThreads, j = i / NF, k = i - j * NF, gx = x0 - D + k, y = 2 * qy + j;
-            vm[it] = (i < 2 * NF && gx >= 0 && gx < W && y < H) ? __ldg(Fm + (size_t)y * W + gx) : FT(0);
+            const bool in = i < 2 * NF && gx >= 0 && gx < W && y < H;
+            vm[it] = in && SGM_GUARD_INDEX((long long)y * W + gx, (long long)W * H, 310) ? __ldg(Fm + (size_t)y * W + gx)
+                                                                                        : FT(0);
         }
 #pragma unroll
         for (int it = 0; it < NB; ++it) {
             const int i = threadIdx.x + it * kQcThreads, j = i / SW, k = i - j * SW, gx = x0 + k, y = 2 * qy + j;
-            vb[it] = (i < 2 * SW && gx < W && y < H) ? __ldg(Fb + (size_t)y * W + gx) : FT(0);
+            const bool in = i < 2 * SW && gx < W && y < H;
+            vb[it] = in && SGM_GUARD_INDEX((long long)y * W + gx, (long long)W * H, 310) ? __ldg(Fb + (size_t)y * W + gx)
+                                                                                        : FT(0);
         }
 #pragma unroll
         for (int it = 0; it < NI; ++it) {
@@ -601,19 +610,24 @@ __global__ void __launch_bounds__(128) p2map_kernel(const uint8_t* __restrict__ 
     auto at = [&](int x, int y) -> int {
         x = min(max(x, 0), W - 1);
         y = min(max(y, 0), H - 1);
-        return __ldg(img + static_cast<size_t>(y) * W + (pass ? W - 1 - x : x));
+        const size_t p = static_cast<size_t>(y) * W + (pass ? W - 1 - x : x);
+        return SGM_GUARD_INDEX(static_cast<long long>(p), static_cast<long long>(W) * H, 311) ? __ldg(img + p) : 0;
     };
     auto pen = [&](int u, int v) -> uint32_t { return tab[abs(u - v)]; };
     const size_t field = static_cast<size_t>(QW) * QH, idx = static_cast<size_t>(qy) * QW + qx;
     uint32_t* map = map0 + pass * stride + idx;
+    auto put = [&](int k, uint32_t v) {  // direction k, within the pass's 4 (8 paths: 8) fields
+        if (SGM_GUARD_INDEX(static_cast<long long>(k * field + idx), static_cast<long long>((parts + 3) * field), 312))
+            map[k * field] = v;
+    };
     if (part == 0) {
         const int x = 2 * qx, y = 2 * qy;
         const int a0 = at(x, y), a1 = at(x + 1, y), b0 = at(x, y + 1), b1 = at(x + 1, y + 1);
         const uint32_t ha = pen(a0, a1), hb = pen(b0, b1), v0 = pen(a0, b0), v1 = pen(a1, b1);
-        map[0] = pen(at(x - 1, y), a0) | ha << 8 | pen(at(x - 1, y + 1), b0) << 16 | hb << 24;
-        map[field] = ha | pen(at(x + 2, y), a1) << 8 | hb << 16 | pen(at(x + 2, y + 1), b1) << 24;
-        map[2 * field] = pen(at(x, y - 1), a0) | pen(at(x + 1, y - 1), a1) << 8 | v0 << 16 | v1 << 24;
-        map[3 * field] = v0 | v1 << 8 | pen(at(x, y + 2), b0) << 16 | pen(at(x + 1, y + 2), b1) << 24;
+        put(0, pen(at(x - 1, y), a0) | ha << 8 | pen(at(x - 1, y + 1), b0) << 16 | hb << 24);
+        put(1, ha | pen(at(x + 2, y), a1) << 8 | hb << 16 | pen(at(x + 2, y + 1), b1) << 24);
+        put(2, pen(at(x, y - 1), a0) | pen(at(x + 1, y - 1), a1) << 8 | v0 << 16 | v1 << 24);
+        put(3, v0 | v1 << 8 | pen(at(x, y + 2), b0) << 16 | pen(at(x + 1, y + 2), b1) << 24);
         return;
     }
     // unit (qy, qx) of the lines moving right (parts 1, 2: down, up) or left (3, 4: down, up)
@@ -627,7 +641,7 @@ __global__ void __launch_bounds__(128) p2map_kernel(const uint8_t* __restrict__ 
         x = x >= 2 * QW ? x - 2 * QW : (x < 0 ? x + 2 * QW : x);
         word |= pen(at(x, y), at(x - dx, y - dy)) << (8 * b);
     }
-    map[(3 + part) * field] = word;
+    put(3 + part, word);
 }
 
 cudaError_t launch_p2map(const uint8_t* left, const uint8_t* right, uint32_t* map, size_t stride, int passes,
@@ -785,9 +799,13 @@ __device__ __forceinline__ void median_quads_body(const uint8_t* __restrict__ ra
 #pragma unroll
     for (int k = 0; k < kMedQH + 2; ++k) {
         const size_t row = static_cast<size_t>(min(max(qy0 - 1 + k, 0), QH - 1)) * QW;
-        wl[k] = __ldg(q + row + ql);
-        wm[k] = __ldg(q + row + qx);
-        wr[k] = __ldg(q + row + qr);
+        auto load = [&](int x) {
+            return SGM_GUARD_INDEX(static_cast<long long>(row + x), static_cast<long long>(QW) * QH, 313) ? __ldg(q + row + x)
+                                                                                                         : 0u;
+        };
+        wl[k] = load(ql);
+        wm[k] = load(qx);
+        wr[k] = load(qr);
     }
     // rows 2 qy0 - 1 .. 2 qy0 + 2 kMedQH of the image, sorted
     constexpr int NR = 2 * kMedQH + 2;
@@ -904,6 +922,9 @@ __global__ void __launch_bounds__(256) mirror_kernel(const uint8_t* __restrict__
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
     if (x >= W || y >= H) return;
     const size_t src = static_cast<size_t>(y) * W + (W - 1 - x), dst = static_cast<size_t>(y) * W + x;
+    if (!SGM_GUARD_INDEX(static_cast<long long>(src), static_cast<long long>(W) * H, 314) ||
+        !SGM_GUARD_INDEX(static_cast<long long>(dst), static_cast<long long>(W) * H, 314))
+        return;
     ml[dst] = __ldg(left + src);
     mr[dst] = __ldg(right + src);
 }
@@ -949,6 +970,8 @@ __global__ void __launch_bounds__(kPostW* kPostH) post_kernel(const uint8_t* __r
     pdl_wait();
     __shared__ int v[kPostH + 2][kPostW + 2];
     const int x0 = blockIdx.x * kPostW, y0 = blockIdx.y * kPostH;
+    // of the raw disparities and the sums beside the winner (whole quads in the quad layout)
+    [[maybe_unused]] const long long pixels = QUADS ? 4ll * ((W + 1) / 2) * ((H + 1) / 2) : static_cast<long long>(W) * H;
     const int t = threadIdx.y * kPostW + threadIdx.x;
     for (int c = t; c < (kPostH + 2) * (kPostW + 2); c += kPostW * kPostH) {
         const int cy = c / (kPostW + 2), cx = c - cy * (kPostW + 2);
@@ -956,8 +979,10 @@ __global__ void __launch_bounds__(kPostW* kPostH) post_kernel(const uint8_t* __r
         int val = 0;
         if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
             const size_t p = pixel_index<QUADS>(gx, gy, W);
-            const int d = rawL[p];
-            val = sub ? subpixel_value(d, sub[p], D) : 16 * d;
+            if (SGM_GUARD_INDEX(static_cast<long long>(p), pixels, 315)) {
+                const int d = rawL[p];
+                val = sub ? subpixel_value(d, sub[p], D) : 16 * d;
+            }
         }
         v[cy][cx] = val;
     }
@@ -984,12 +1009,13 @@ __global__ void __launch_bounds__(kPostW* kPostH) post_kernel(const uint8_t* __r
         const int d = rawL[pixel_index<QUADS>(x, y, W)], xr = x - d;
         bool ok = xr >= 0;
         if (ok) {
-            const int dr = rawRm[pixel_index<QUADS>(W - 1 - xr, y, W)];
+            const size_t q = pixel_index<QUADS>(W - 1 - xr, y, W);
+            const int dr = SGM_GUARD_INDEX(static_cast<long long>(q), pixels, 316) ? rawRm[q] : 0;
             ok = d - dr <= 1 && dr - d <= 1;
         }
         if (!ok) out = 0xffff;
     }
-    out16[p] = static_cast<uint16_t>(out);
+    if (SGM_GUARD_INDEX(static_cast<long long>(p), static_cast<long long>(W) * H, 317)) out16[p] = static_cast<uint16_t>(out);
 }
 
 cudaError_t launch_post(const uint8_t* rawL, const uint32_t* sub, const uint8_t* rawRm, uint16_t* out16, bool quads,
