@@ -190,7 +190,7 @@ SGM_API int sgm_compute_ex_async(sgm_ctx *ctx, const uint8_t *left, const uint8_
  * be device memory; the caller synchronises the stream before reading
  * `disp_out`.  The kernels are launched one by one with programmatic stream
  * serialization, so that calls follow one another in the stream without gaps;
- * the blocking calls replay a CUDA graph captured once for one (W, H, D, P1,
+ * the blocking calls replay a CUDA graph built once for one (W, H, D, P1,
  * P2, n_paths) and one set of pointers, on the second call with them.
  * Errors: SGM_EINVAL (including host pointers), SGM_ENOMEM, SGM_ECUDA.
  */

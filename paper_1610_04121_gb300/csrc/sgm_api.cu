@@ -339,7 +339,6 @@ struct sgm_ctx {
     int device = 0;
     cudaStream_t own_stream = nullptr;
     cudaStream_t stream = nullptr;
-    cudaStream_t capture_stream = nullptr;
     size_t mem_cap = 0;
     uint8_t* arena = nullptr;
     size_t arena_bytes = 0;
@@ -756,18 +755,26 @@ static int prepare_arena(sgm_ctx* ctx, Problem& p, size_t extra = 0) {
 
 // Enqueue the whole path (Section 2, stages 2-4) for one pair whose inputs
 // and output are device pointers: disp is uint8 [H][W], or uint16 [H][W] in
-// 1/16 pixel with post-filters (p.post).  Returns a cudaError_t.
+// 1/16 pixel with post-filters (p.post).  With `chain`, the path becomes nodes
+// of its graph instead (their errors are left in the chain).  Returns a
+// cudaError_t.
 static cudaError_t enqueue_path(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const uint8_t* left,
-                                const uint8_t* right, uint8_t* disp, uint16_t* Sdbg, cudaStream_t s, bool timed) {
+                                const uint8_t* right, uint8_t* disp, uint16_t* Sdbg, cudaStream_t s, bool timed,
+                                NodeChain* chain = nullptr) {
     const Layout l = layout_for(p);
-    const Stream st(s, !timed);  // events between the kernels: plain order
+    const Stream st(s, !timed, chain);  // events between the kernels: plain order
     cudaError_t e;
     int stage = 0;
     // with stage timing, event k is recorded before kernel k and after the last
     auto mark = [&]() -> cudaError_t {
         if (!timed) return cudaSuccess;
-        // External: inside a stream capture this becomes an event-record node of the graph
-        return cudaEventRecordWithFlags(ctx->stage_ev[stage++], s, cudaEventRecordExternal);
+        if (!chain) return cudaEventRecord(ctx->stage_ev[stage++], s);
+        cudaGraphNode_t node = nullptr;
+        const cudaError_t me =
+            cudaGraphAddEventRecordNode(&node, chain->graph, chain->after.data(), chain->after.size(), ctx->stage_ev[stage++]);
+        if (me == cudaSuccess) chain->after.assign(1, node);
+        chain->kernel = false;
+        return me;
     };
     if ((e = mark()) != cudaSuccess) return e;
     if (pairs_sched(p)) {
@@ -803,7 +810,7 @@ static cudaError_t enqueue_path(sgm_ctx* ctx, const Problem& p, uint8_t* arena, 
             return e;
         if ((e = mark()) != cudaSuccess) return e;
     }
-    ctx->launches += launches_per_path(p);
+    if (!chain) ctx->launches += launches_per_path(p);
     return cudaSuccess;
 }
 
@@ -850,27 +857,22 @@ static int enqueue_graph(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const u
         }
     }
     if (!it->second) {
-        cudaGraph_t g = nullptr;
-        CUDA_TRY(ctx, cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal));
-        const uint64_t before = ctx->launches.load();
+        NodeChain chain{};
+        CUDA_TRY(ctx, cudaGraphCreate(&chain.graph, 0));
+        const Stream st(s, !timed, &chain);
         cudaError_t e = cudaSuccess;
-        const Stream st(ctx->capture_stream, !timed);
         if (io.src[0]) e = launch_stage(io.src[0], io.dst[0], io.src[1], io.dst[1], io.img_bytes, st);
-        if (e == cudaSuccess)
-            e = enqueue_path(ctx, p, arena, left, right, disp, nullptr, ctx->capture_stream, timed);
+        if (e == cudaSuccess) e = enqueue_path(ctx, p, arena, left, right, disp, nullptr, s, timed, &chain);
         if (e == cudaSuccess && io.out_src)
             e = launch_stage(io.out_src, io.out_dst, nullptr, nullptr, io.out_bytes, st);
-        ctx->launches = before;  // captured, not launched
-        cudaError_t e2 = cudaStreamEndCapture(ctx->capture_stream, &g);
-        if (e != cudaSuccess || e2 != cudaSuccess) {
-            if (g) cudaGraphDestroy(g);
-            return fail(ctx, SGM_ECUDA, "graph capture failed: %s / %s", cudaGetErrorString(e),
-                        cudaGetErrorString(e2));
-        }
+        if (e == cudaSuccess) e = chain.err;
         cudaGraphExec_t exec = nullptr;
-        e = cudaGraphInstantiate(&exec, g, 0);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) return fail(ctx, SGM_ECUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, chain.graph, 0);
+        cudaGraphDestroy(chain.graph);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return fail(ctx, SGM_ECUDA, "building the call's graph: %s", cudaGetErrorString(e));
+        }
         it->second = exec;
     }
     CUDA_TRY(ctx, cudaGraphLaunch(it->second, s));
@@ -1872,8 +1874,7 @@ int sgm_create(sgm_ctx** out, int device, size_t mem_cap_bytes, unsigned flags) 
     sgm_ctx* ctx = new sgm_ctx();
     ctx->device = device;
     ctx->mem_cap = mem_cap_bytes;
-    if ((e = cudaStreamCreateWithFlags(&ctx->own_stream, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking)) != cudaSuccess) {
+    if ((e = cudaStreamCreateWithFlags(&ctx->own_stream, cudaStreamNonBlocking)) != cudaSuccess) {
         sgm_destroy(ctx);
         return fail(nullptr, SGM_ECUDA, "cudaStreamCreate: %s", cudaGetErrorString(e));
     }
@@ -1968,7 +1969,6 @@ int sgm_destroy(sgm_ctx* ctx) {
     }
     if (ctx->serve_pool) cudaMemPoolDestroy(ctx->serve_pool);
     if (ctx->own_stream) cudaStreamDestroy(ctx->own_stream);
-    if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
     for (auto& ev : ctx->stage_ev)
         if (ev) cudaEventDestroy(ev);
     for (auto& ev : ctx->tune_ev)

@@ -8,6 +8,17 @@
 
 namespace sgm {
 
+// A chain of nodes in a graph under construction: the next kernel runs after
+// the nodes in `after`.  Graphs are built node by node, not captured: they are
+// built on the scheduler's thread and on those of the callers, and a capture
+// there fails a cudaDeviceSynchronize that another thread happens to make.
+struct NodeChain {
+    cudaGraph_t graph;
+    std::vector<cudaGraphNode_t> after;
+    bool kernel = false;            // `after` is the one kernel before
+    cudaError_t err = cudaSuccess;  // the first error of launch()
+};
+
 // A path's kernels follow one another in a stream, each launched with
 // programmatic stream serialization (pdl): its launch work overlaps the kernel
 // before it, and its first instruction waits until that one has ended and its
@@ -15,15 +26,52 @@ namespace sgm {
 // graph launch, the device releases a kernel in steps of 2.05 us, 4.1 us at
 // least; measured for five kernels of 1.5 us back to back: 20.5 us launched
 // plainly, 14.3 us as a replayed graph, 11.3 us this way.
+// With a chain, the kernels become nodes of its graph instead, one after the
+// other, by programmatic edges where the launch would be a programmatic one.
 struct Stream {
     cudaStream_t s;
     bool pdl;
-    Stream(cudaStream_t stream, bool p = false) : s(stream), pdl(p) {}
+    NodeChain* chain;
+    Stream(cudaStream_t stream, bool p = false, NodeChain* c = nullptr) : s(stream), pdl(p), chain(c) {}
 };
 
-// Launches a kernel; the caller reads the error with cudaGetLastError.
+// Adds a kernel to a chain.
+template <class... P, class... A>
+inline cudaError_t add_kernel(NodeChain& c, void (*kernel)(P...), dim3 grid, dim3 block, A&&... args) {
+    std::tuple<P...> v{static_cast<P>(args)...};
+    cudaKernelNodeParams n{};
+    n.func = reinterpret_cast<void*>(kernel);
+    n.gridDim = grid;
+    n.blockDim = block;
+    void* ptrs[sizeof...(P)];
+    std::apply([&](auto&... x) { int i = 0; ((ptrs[i++] = &x), ...); }, v);
+    n.kernelParams = ptrs;  // the values are copied into the node
+    cudaGraphNode_t node = nullptr;
+    const cudaError_t e = cudaGraphAddKernelNode(&node, c.graph, c.after.data(), c.after.size(), &n);
+    if (e == cudaSuccess) c.after.assign(1, node);
+    return e;
+}
+
+// Launches a kernel, or adds it to the stream's chain; the caller reads the
+// error with cudaGetLastError, or in the chain.
 template <class... P, class... A>
 inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, Stream st, A&&... args) {
+    if (st.chain) {
+        NodeChain& c = *st.chain;
+        if (c.err != cudaSuccess) return;
+        const bool side = st.pdl && c.kernel;
+        const std::vector<cudaGraphNode_t> before = c.after;
+        if (side) c.after.clear();
+        c.err = add_kernel(c, kernel, grid, block, args...);
+        if (side && c.err == cudaSuccess) {
+            cudaGraphEdgeData edge{};
+            edge.type = cudaGraphDependencyTypeProgrammatic;
+            edge.from_port = cudaGraphKernelNodePortProgrammatic;
+            c.err = cudaGraphAddDependencies(c.graph, before.data(), c.after.data(), &edge, 1);
+        }
+        c.kernel = true;
+        return;
+    }
     cudaLaunchConfig_t c{};
     c.gridDim = grid;
     c.blockDim = block;
@@ -125,30 +173,6 @@ struct ListLaunch {
     int rx;            // vertical-type sweeps: 0 (vertical, finishing with Eq. 4), +1 / -1 (diagonals)
     int n_paths, cls;  // paired schedule: paths and class of the sums (pairs_class)
 };
-
-// A chain of nodes in a graph under construction: the next kernel runs after
-// the nodes in `after`.  The graphs of the lists are built node by node, not
-// captured: they are built on the scheduler's thread too, and a capture there
-// fails a cudaDeviceSynchronize that another thread happens to make.
-struct NodeChain {
-    cudaGraph_t graph;
-    std::vector<cudaGraphNode_t> after;
-};
-template <class... P, class... A>
-inline cudaError_t add_kernel(NodeChain& c, void (*kernel)(P...), int grid, int block, A... args) {
-    std::tuple<P...> v{static_cast<P>(args)...};
-    cudaKernelNodeParams n{};
-    n.func = reinterpret_cast<void*>(kernel);
-    n.gridDim = dim3(grid);
-    n.blockDim = dim3(block);
-    void* ptrs[sizeof...(P)];
-    std::apply([&](auto&... x) { int i = 0; ((ptrs[i++] = &x), ...); }, v);
-    n.kernelParams = ptrs;  // the values are copied into the node
-    cudaGraphNode_t node = nullptr;
-    const cudaError_t e = cudaGraphAddKernelNode(&node, c.graph, c.after.data(), c.after.size(), &n);
-    if (e == cudaSuccess) c.after.assign(1, node);
-    return e;
-}
 
 // Each launcher enqueues one kernel on `stream` and returns the launch error;
 // the list launchers add it to a chain of nodes.
