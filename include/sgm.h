@@ -373,9 +373,10 @@ SGM_API const char *sgm_stage_label(const sgm_ctx *ctx, int i);
  *   SGM_SCHED_PAIRS     two lines per warp over 2 x 2 pixel quads: all four
  *                       directions at once, the vertical pair storing its
  *                       costs and the horizontal pair its state at every
- *                       16th column (8th for D > 128); then every segment of
- *                       a row pair walks the horizontal pair again from
- *                       those states, sums and takes the winner.  Not
+ *                       16th column (8th for D > 128; 4th or 8th in small
+ *                       frames); then every segment of a row pair walks the
+ *                       horizontal pair again from those states, sums and
+ *                       takes the winner.  Not
  *                       offered when its quad cubes would pass 4 GiB.
  * All give bit-identical results.  By default the context autotunes: the
  * first call for a new (W, H, D, Census type, byte-sum) key runs the path

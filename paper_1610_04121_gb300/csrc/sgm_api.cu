@@ -158,8 +158,8 @@ inline bool pairs_fit(const Problem& p) {
 // The quad cubes (one array of FS bytes per field), the quad raw disparity
 // and the horizontal states (sgm_internal.h); `RB` holds the bytes of one quad
 // in a field (4D).
-Layout layout_pairs(const Problem& p) {
-    const PairsArgs g = pairs_geometry(p.W, p.H, p.D, p.n_paths);
+Layout layout_pairs(const Problem& p, bool lists) {
+    const PairsArgs g = pairs_geometry(p.W, p.H, p.D, p.n_paths, lists);
     const size_t wh = static_cast<size_t>(p.W) * p.H, quads = static_cast<size_t>(g.QW) * g.QH;
     const size_t fbytes = p.ct62 ? 8 : 4;
     Layout l{};
@@ -198,7 +198,7 @@ Layout layout_pairs(const Problem& p) {
 }
 
 Layout schedule_layout(const Problem& p, bool batched) {
-    if (pairs_sched(p)) return layout_pairs(p);
+    if (pairs_sched(p)) return layout_pairs(p, batched);
     return layout_for(p.W, p.H, p.D, p.n_paths, batched, p.ct62 != 0, p.post != 0);
 }
 
@@ -544,7 +544,7 @@ static cudaError_t enqueue_pairs(const Problem& p, const Layout& l, uint8_t* are
     PairsJobs f{};
     f.n = l.passes;
     for (int k = 0; k < l.passes; ++k) {
-        PairsArgs g = pairs_geometry(p.W, p.H, p.D, p.n_paths);
+        PairsArgs g = pairs_geometry(p.W, p.H, p.D, p.n_paths, false);
         g.rec = arena + l.rec + k * l.rec_stride;
         g.rawq = arena + l.raw + k * l.raw_stride;
         g.Sdbg = Sdbg;
@@ -1189,7 +1189,7 @@ static size_t build_lists(sgm_ctx* ctx, ListExec& x, const std::vector<BatchItem
                 uint8_t* base = arena + it.offset;
                 cj[k] = CensusJob{it.left, it.right, base + l.Fb, base + l.Fm, p.W, p.H};
                 mj[k] = CostQuadsJob{base + l.Fb, base + l.Fm, base + l.rec, l.RB, p.W, p.H, p.D};
-                PairsArgs a = pairs_geometry(p.W, p.H, p.D, p.n_paths);
+                PairsArgs a = pairs_geometry(p.W, p.H, p.D, p.n_paths, true);
                 a.rec = base + l.rec;
                 a.rawq = base + l.raw;
                 a.state = reinterpret_cast<uint32_t*>(base + l.state);
@@ -2433,7 +2433,7 @@ cudaError_t enqueue_path_static(Problem p, uint8_t* arena, const uint8_t* left, 
                                 cudaStream_t stream) {
     const Stream s(stream, true);
     p.sched = SGM_SCHED_PAIRS;
-    const Layout lp = layout_pairs(p);
+    const Layout lp = layout_pairs(p, false);
     if (lp.in_left <= kStaticScratchBytes) {  // all it touches lies in front of its staging buffers
         cudaError_t e = enqueue_pairs(p, lp, arena, left, right, nullptr, s, [] { return cudaSuccess; });
         return e != cudaSuccess ? e : launch_median_quads(arena + lp.raw, disp, p.W, p.H, s);

@@ -261,12 +261,14 @@ __host__ __device__ constexpr int pairs_fields(int n_paths) { return n_paths == 
 // keep the states at 1/16 of a stored field per direction; with more than 128
 // disparities a warp's segment has to fit its shared memory.
 __host__ __device__ constexpr int seg_quads(int D) { return D <= 128 ? 8 : 4; }
+// Small frames walk shorter segments, a multiple of kShortSeg quads (pairs_geometry).
+constexpr int kShortSeg = 2;
 
 struct PairsArgs {
     uint8_t* rec;          // the field arrays (pairs_fields of FS bytes each)
     uint8_t* rawq;         // winner-take-all disparity in quads [QH][QW][4]
     uint16_t* Sdbg;        // optional natural-order S [H][W][D] (debug)
-    uint32_t* state;       // horizontal states [2][QH][NS][(D/32 + 1) / 2][32]
+    uint32_t* state;       // horizontal states [2 (1 with 2 paths)][QH][NS][(D/32 + 1) / 2][32]
     // Post-filters: the jump penalty of every step, [8][QH][QW] words of the
     // four pixels of a quad or diagonal unit (direction: left to right, right to
     // left, then the order of the fields), or null (P2 throughout); S(d-1) - S(d)
@@ -274,7 +276,7 @@ struct PairsArgs {
     const uint32_t* p2map;
     uint32_t* subq;
     int W, H, W2, H2, QW, QH, D, n_paths;
-    int NS;                // segments of a row pair
+    int CQ, NS;            // quads of a segment, segments of a row pair
     size_t FS;             // bytes of one field array (QH * QW * QB, rounded up)
     int QB;                // bytes of one quad in a field: 4D (W2 * H2 * D < 2^32)
     uint32_t P1x2, P2x2;
@@ -288,10 +290,10 @@ struct PairsJobs {
     PairsArgs job[2];
     int n;
 };
-// Geometry of a W x H problem.
-PairsArgs pairs_geometry(int W, int H, int D, int n_paths);
-inline size_t pairs_state_words(const PairsArgs& a) {
-    return static_cast<size_t>(2) * a.QH * a.NS * 32 * ((a.D / 32 + 1) / 2);
+// Geometry of a W x H problem; `lists`: as the work lists walk it (segments of seg_quads).
+PairsArgs pairs_geometry(int W, int H, int D, int n_paths, bool lists);
+__host__ __device__ inline size_t pairs_state_words(const PairsArgs& a) {
+    return static_cast<size_t>(a.n_paths == 2 ? 1 : 2) * a.QH * a.NS * 32 * ((a.D / 32 + 1) / 2);
 }
 // How the finishing launch sums and takes the winner.  4 and 8 paths: 0 = three
 // r add in a byte (3 P2 <= 255) and the keys S D + d fit 16 bits, 1 = two r add

@@ -24,7 +24,7 @@
 //   walks     every direction of every line pair at once.  The vertical and
 //             diagonal walkers store r = L_r - MC (0 <= r <= P2, a byte); the
 //             horizontal walkers store nothing but their state at every
-//             segment boundary (kSegQuads quads);
+//             segment boundary (at most seg_quads(D) quads, pairs_geometry);
 //   finish    a warp per segment of a row pair walks left to right and right
 //             to left again from the stored states, adds the stored r of the
 //             other directions and takes the winner.
@@ -380,7 +380,7 @@ __device__ __forceinline__ uint32_t* state_slot(const PairsArgs& a, int dir, int
 template <int D>
 __device__ __forceinline__ bool state_ok(const PairsArgs& a, const uint32_t* p, unsigned site) {
     return SGM_GUARD(p, 4 * (32 * (Chain2<D / 32>::CW - 1) + 1), a.state,
-                     a.state + static_cast<size_t>(2) * a.QH * a.NS * 32 * Chain2<D / 32>::CW, site);
+                     a.state + pairs_state_words(a), site);
 }
 
 // The walks' ring of units in shared memory, per warp, at most 16 units.  D >
@@ -391,17 +391,19 @@ __device__ __forceinline__ bool state_ok(const PairsArgs& a, const uint32_t* p, 
 // D=128 frame 79.5 us, four 81.8), four for D > 128 (1920x1080 D=256 892 us,
 // eight 905), but two for diagonals that run beside the other walks (1242x375 8
 // paths 204 us; eight no longer fit the instruction caches with them: 214), and
-// no more than a segment or the ring holds.
+// no more than a segment or the ring holds.  SHORT (frames with shorter segments,
+// pairs_geometry): rings of one loop only, because a walk's last DEPTH units run
+// outside the loop, one by one (64x100 D=96 frame 15.4 us, with sixteen 16.7).
 template <int D>
 __host__ __device__ constexpr int ring_bytes(bool rows = false) {
     return D <= 128 || rows ? 8192 : 16384;
 }
-template <int D, int KIND, bool ROWS>
+template <int D, int KIND, bool ROWS, bool SHORT>
 struct Ring {
     static constexpr int SB = (KIND == kDiag ? 2 : 1) * 4 * D;  // bytes of a slot
     static constexpr int WANT = KIND == kDiag && !ROWS ? 2 : (D <= 128 ? 8 : 4), FIT = ring_bytes<D>(ROWS) / SB;
     static constexpr int UN = WANT <= FIT && (KIND != kHor || WANT <= seg_quads(D)) ? WANT : (WANT < 4 ? WANT : 4);
-    static constexpr int DEPTH = FIT / UN * UN > 16 ? 16 : FIT / UN * UN;
+    static constexpr int DEPTH = SHORT ? UN : (FIT / UN * UN > 16 ? 16 : FIT / UN * UN);
 };
 
 // ---------------------------------------------------------------------------
@@ -415,11 +417,13 @@ struct Ring {
 // instruction caches (164 against 144 us for the walks of a 1242x375 8-path
 // frame, although each ran faster alone).
 // ---------------------------------------------------------------------------
-template <int D, int KIND, bool AP2, bool ROWS = false>
+template <int D, int KIND, bool AP2, bool ROWS = false, bool SHORT = false>
 __device__ __forceinline__ void walk(const PairsArgs& a, int line, int kd, bool fwd, uint32_t ring) {
-    constexpr int K = D / 32, CQ = seg_quads(D), SB = Ring<D, KIND, ROWS>::SB,
-                  DEPTH = Ring<D, KIND, ROWS>::DEPTH, UN = Ring<D, KIND, ROWS>::UN;
-    static_assert((KIND != kHor || CQ % UN == 0) && DEPTH >= UN, "groups of units end where segments end");
+    using R = Ring<D, KIND, ROWS, SHORT>;
+    constexpr int K = D / 32, SB = R::SB, DEPTH = R::DEPTH, UN = R::UN;
+    static_assert((KIND != kHor || (seg_quads(D) % UN == 0 && UN % kShortSeg == 0)) && DEPTH >= UN,
+                  "segments end where groups of units end, short ones inside them too");
+    const int CQ = SHORT ? a.CQ : seg_quads(D);
     const int lane = threadIdx.x & 31;
     const uint32_t QB = static_cast<uint32_t>(a.QB), rowb = static_cast<uint32_t>(a.QW) * QB;
     int nu;               // units of the walk
@@ -623,11 +627,13 @@ __device__ __forceinline__ void walk(const PairsArgs& a, int line, int kd, bool 
                 cp_commit();
                 unit(cur, k + i, false);
                 cur = nxt;
+                if constexpr (KIND == kHor && SHORT)
+                    if ((i + 1) % kShortSeg == 0) segment_end(kShortSeg);
             }
             k += UN;
             slot += UN * SB;
             if (slot == DEPTH * SB) slot = 0;
-            if constexpr (KIND == kHor) segment_end(UN);
+            if constexpr (KIND == kHor && !SHORT) segment_end(UN);
         }
         if (k < nu) {
             const int ns = slot + SB == DEPTH * SB ? 0 : slot + SB;
@@ -662,7 +668,7 @@ struct Side {
 // The walks: one chain per warp.  Chains [0, nh) are horizontal line pairs
 // (row pair c / nd, direction c % nd), [nh, nh + nv) vertical ones, nd
 // directions each (1 with 2 paths).
-template <int D, bool AP2>
+template <int D, bool AP2, bool SHORT>
 __global__ void __launch_bounds__(64) walk_hv_kernel(const __grid_constant__ PairsJobs f, int nh, int nv, Side side) {
     __shared__ __align__(16) uint8_t ring[2][ring_bytes<D>()];
     side.begin();
@@ -671,9 +677,9 @@ __global__ void __launch_bounds__(64) walk_hv_kernel(const __grid_constant__ Pai
     const uint32_t r = static_cast<uint32_t>(__cvta_generic_to_shared(ring[warp]));
     const int nd = a.n_paths == 2 ? 1 : 2, c = blockIdx.x * 2 + warp, v = c - nh;
     if (c < nh)
-        walk<D, kHor, AP2>(a, c / nd, 0, c % nd == 0, r);
+        walk<D, kHor, AP2, false, SHORT>(a, c / nd, 0, c % nd == 0, r);
     else if (v < nv)
-        walk<D, kVer, AP2>(a, v / nd, 0, v % nd == 0, r);
+        walk<D, kVer, AP2, false, SHORT>(a, v / nd, 0, v % nd == 0, r);
     side.end();
 }
 
@@ -720,7 +726,8 @@ __global__ void __launch_bounds__(96) walk_rows_kernel(const __grid_constant__ P
 // SM (all of them loaded up front let every warp of a wave wait, then compute,
 // in step: 31 us for a 640x480 D=128 frame).  S = own r + n MC + the r of the
 // other n - 1 directions.  GS r may be added in a byte: GS P2 <= 255.  K16:
-// S D + d fits 16 bits, so that one packed minimum serves both lines.
+// S D + d fits 16 bits, so that one packed minimum serves both lines.  SHORT:
+// segments of a.CQ quads, fewer than seg_quads(D).
 // ---------------------------------------------------------------------------
 template <int D, int NP>
 struct Finish {
@@ -729,13 +736,13 @@ struct Finish {
     static constexpr int KEPT = CQ * UB, BYTES = KEPT + (NP == 2 ? 0 : CQ * UB);
 };
 
-template <int D, int NP, int GS, bool K16, bool POST>
+template <int D, int NP, int GS, bool K16, bool POST, bool SHORT>
 __device__ __forceinline__ void finish(const PairsArgs& a, int r, int s, uint32_t smem) {
     using F = Finish<D, NP>;
     constexpr int K = D / 32, UB = F::UB, CQ = F::CQ, NV = F::NV, NF = F::NF;
     constexpr bool DIAG = NP == 8;
     const int lane = threadIdx.x & 31;
-    const int q0 = s * CQ, nq = min(CQ, a.QW - q0);
+    const int q0 = s * (SHORT ? a.CQ : CQ), nq = min(SHORT ? a.CQ : CQ, a.QW - q0);
     const uint32_t QB = static_cast<uint32_t>(a.QB), rowoff = static_cast<uint32_t>(r) * a.QW * QB;
     const uint32_t off0 = rowoff + static_cast<uint32_t>(q0) * QB;
     const uint32_t ssrc = smem + 4 * K * lane;
@@ -1007,7 +1014,7 @@ __device__ __forceinline__ void finish(const PairsArgs& a, int r, int s, uint32_
         reinterpret_cast<uint32_t*>(a.rawq)[q] = rawv;
 }
 
-template <int D, int NP, int GS, bool K16, bool POST>
+template <int D, int NP, int GS, bool K16, bool POST, bool SHORT>
 __global__ void __launch_bounds__(64) finish_kernel(const __grid_constant__ PairsJobs f) {
     __shared__ __align__(16) uint8_t smem[2][Finish<D, NP>::BYTES + (POST ? 4 * D : 0)];  // post form: S of a column
     pdl_wait();
@@ -1015,7 +1022,8 @@ __global__ void __launch_bounds__(64) finish_kernel(const __grid_constant__ Pair
     const PairsArgs& a = f.job[blockIdx.z];
     const int r = blockIdx.y * 2 + warp;  // two row pairs
     if (r < a.QH)
-        finish<D, NP, GS, K16, POST>(a, r, blockIdx.x, static_cast<uint32_t>(__cvta_generic_to_shared(smem[warp])));
+        finish<D, NP, GS, K16, POST, SHORT>(a, r, blockIdx.x,
+                                            static_cast<uint32_t>(__cvta_generic_to_shared(smem[warp])));
 }
 
 // ---------------------------------------------------------------------------
@@ -1096,7 +1104,7 @@ __global__ void __launch_bounds__(64, finish_list_blocks<D, NP>()) finish_list_k
             const int r = u / runs, s0 = (u - r * runs) * a.run;
 #pragma unroll 1
             for (int s = s0; s < min(s0 + a.run, a.NS); ++s)
-                finish<D, NP, GS, K16, false>(a, r, s, static_cast<uint32_t>(__cvta_generic_to_shared(smem[warp])));
+                finish<D, NP, GS, K16, false, false>(a, r, s, static_cast<uint32_t>(__cvta_generic_to_shared(smem[warp])));
         }
         i = __shfl_sync(kFull, nx, 0);
     }
@@ -1119,7 +1127,10 @@ struct PairsD {
         } else {
             const int nh = w != Walks::kVer && a.NS > 1 ? a.QH * nd : 0, nv = w != Walks::kHor ? a.QW * nd : 0;
             const dim3 grid(nh + nv > 0 ? (nh + nv + 1) / 2 : 1, f.n);  // images of one segment have no horizontal states
-            launch(a.p2map ? walk_hv_kernel<D, true> : walk_hv_kernel<D, false>, grid, 64, s, f, nh, nv, side);
+            const auto kernel = a.CQ != seg_quads(D)
+                                    ? (a.p2map ? walk_hv_kernel<D, true, true> : walk_hv_kernel<D, false, true>)
+                                    : (a.p2map ? walk_hv_kernel<D, true, false> : walk_hv_kernel<D, false, false>);
+            launch(kernel, grid, 64, s, f, nh, nv, side);
         }
         return cudaGetLastError();
     }
@@ -1127,10 +1138,13 @@ struct PairsD {
     static void finish_t(const PairsJobs& f, Stream s) {
         const PairsArgs& a = f.job[0];
         const dim3 grid(a.NS, (a.QH + 1) / 2, f.n);
-        if (a.p2map || a.subq || a.Sdbg)  // the post form serves the debug sums too
-            launch(finish_kernel<D, NP, GS, false, true>, grid, 64, s, f);
+        const bool post = a.p2map || a.subq || a.Sdbg;  // the post form serves the debug sums too
+        if (a.CQ == seg_quads(D))
+            launch(post ? finish_kernel<D, NP, GS, false, true, false> : finish_kernel<D, NP, GS, K16, false, false>, grid,
+                   64, s, f);
         else
-            launch(finish_kernel<D, NP, GS, K16, false>, grid, 64, s, f);
+            launch(post ? finish_kernel<D, NP, GS, false, true, true> : finish_kernel<D, NP, GS, K16, false, true>, grid,
+                   64, s, f);
     }
     template <int NP>
     static void finish_np(const PairsJobs& f, Stream s) {

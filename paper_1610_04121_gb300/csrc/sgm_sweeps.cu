@@ -61,7 +61,24 @@ int sweep_units(int lines, int D, bool pair) {
     return (lines + per - 1) / per;
 }
 
-PairsArgs pairs_geometry(int W, int H, int D, int n_paths) {
+// Quads of a segment.  The finishing launch walks a segment in both directions,
+// one step after the other, and with few segments most of the chip is empty
+// meanwhile: they are halved while they give at most two warps for each of the
+// chip's 608 schedulers; beyond that the states cost more than the shorter
+// walks gain.  us per frame, 4 paths, eight / four / two quads, by the warps of
+// eight: 64x48 D=32 (96) 15.7 / 13.2 / 12.9, 64x128 D=96 (256) 20.2 / 17.1 / 16.2,
+// 100x150 D=96 (525) 21.9 / 18.7 / 18.2, 160x120 D=64 (600) 20.3 / 18.8 / 18.8, 200x150
+// D=128 (975) 24.6 / 22.9 / 23.0, 256x160 D=96 (1280) 27.1 / 26.9 / 27.4, 320x240
+// D=64 (2400) 28.1 / 29.1 / 30.2; four / two quads, by the warps of four: 100x100
+// D=192 (650) 21.1 / 18.4, 128x96 D=224 (768) 24.6 / 23.1, 200x100 D=160 (1250)
+// 25.4 / 25.3, 240x200 D=160 (3000) 30.7 / 31.6.
+static int segment_quads(const PairsArgs& a) {
+    int quads = seg_quads(a.D);
+    while (quads > kShortSeg && a.QH * ((a.QW + quads - 1) / quads) <= 2 * 608) quads /= 2;
+    return quads;
+}
+
+PairsArgs pairs_geometry(int W, int H, int D, int n_paths, bool lists) {
     PairsArgs a{};
     a.W = W;
     a.H = H;
@@ -71,7 +88,8 @@ PairsArgs pairs_geometry(int W, int H, int D, int n_paths) {
     a.H2 = H + (H & 1);
     a.QW = a.W2 / 2;
     a.QH = a.H2 / 2;
-    a.NS = (a.QW + seg_quads(D) - 1) / seg_quads(D);
+    a.CQ = lists ? seg_quads(D) : segment_quads(a);
+    a.NS = (a.QW + a.CQ - 1) / a.CQ;
     return a;
 }
 
