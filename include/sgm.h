@@ -202,7 +202,8 @@ SGM_API int sgm_compute_async(sgm_ctx *ctx, const uint8_t *left, const uint8_t *
  * Batched computation of `n` independent pairs of possibly different sizes,
  * D, penalties and path counts (the paper's scaling argument, Section 4,
  * applied to many pairs at once).  A pair that fills the GPU by itself (W * H *
- * D * n_paths above 2^28) runs through the kernels of sgm_compute.  The others
+ * D * n_paths above 2^28) runs through the kernels of sgm_compute; such pairs
+ * work one after the other in one region of the arena.  The others
  * are grouped by (D, path count, schedule and form of the sums); every stage of
  * a group is one persistent grid whose blocks take units (tiles, row segments,
  * line pairs) from a device work list covering the group's pairs, longest

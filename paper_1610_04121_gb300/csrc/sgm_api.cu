@@ -1075,7 +1075,9 @@ struct BatchItem {
     Problem p;
     const uint8_t *left, *right;
     uint8_t* out;
-    size_t offset;  // of the pair's region in the arena
+    // where the pair works in the arena, and its copies of host buffers (in_left,
+    // in_right and out of its layout, in this order)
+    size_t offset = 0, io = 0;
 };
 
 // The schedule and sum form of a batched pair: 0, 1 = per-line sweeps with u16 or
@@ -1101,7 +1103,8 @@ static int group_code(const BatchItem& it) {
 // it only takes L2 and issue slots from them.  us per pair, in lists of eight /
 // one by one: 640x480 D=128 4 paths 76.9 / 79.9, 1242x375 D=128 4 paths 112 /
 // 128, 1242x375 D=64 8 paths 139 / 139, 640x480 D=128 8 paths 145 / 134, 640x480
-// D=256 4 paths 144 / 131, 1242x375 D=128 8 paths 219 / 205.
+// D=256 4 paths 144 / 131, 1242x375 D=128 8 paths 219 / 205.  (It has at least
+// 4096 segments of eight quads: pairs_geometry is the same for both forms.)
 static bool runs_alone(const Problem& p) {
     return pairs_sched(p) && static_cast<double>(p.W) * p.H * p.D * p.n_paths > 268435456.0;
 }
@@ -1121,6 +1124,36 @@ static int batch_sched(Problem p, size_t room, double px, bool capped) {
     if (capped) room = std::min(room, layout_for(p, true).total);
     p.sched = SGM_SCHED_PAIRS;
     return pairs_fit(p) && layout_for(p, true).total <= room ? SGM_SCHED_PAIRS : SGM_SCHED_V_THEN_H;
+}
+
+// The room of a wave: the pairs that run alone work one after the other in one
+// region (host buffers are copied to and from regions of their own, beside the
+// others' work), the pairs of the lists side by side.
+struct WaveRoom {
+    size_t alone = 0, rest = 0;
+    size_t total() const { return alone + rest; }
+    WaveRoom with(const Problem& p) const {
+        const Layout l = layout_for(p, true);
+        WaveRoom r = *this;
+        if (runs_alone(p)) r.alone = std::max(r.alone, l.in_left);
+        r.rest += runs_alone(p) ? l.total - l.in_left : l.total;
+        return r;
+    }
+};
+
+// Places the pairs of a wave; returns the bytes they take.
+static size_t place_wave(std::vector<BatchItem>& items, size_t b, size_t e) {
+    WaveRoom room;
+    for (size_t i = b; i < e; ++i) room = room.with(items[i].p);
+    size_t at = room.alone;
+    for (size_t i = b; i < e; ++i) {
+        BatchItem& it = items[i];
+        const Layout l = layout_for(it.p, true);
+        it.offset = runs_alone(it.p) ? 0 : at;
+        it.io = runs_alone(it.p) ? at : at + l.in_left;
+        at = it.io + (l.total - l.in_left);
+    }
+    return at;
 }
 
 static int launches_per_group(int n_paths) { return 4 + (n_paths == 8 ? 3 : 1); }
@@ -1236,7 +1269,8 @@ static size_t build_lists(sgm_ctx* ctx, ListExec& x, const std::vector<BatchItem
                 a.cls = pairs_class(p.n_paths, p.D, p.P2, mc_max(p));
                 a.run = pairs_finish_run(a);
                 pj[k] = a;
-                dj[k] = MedianJob{base + l.raw, is_device_ptr(it.out) ? it.out : base + l.out, p.W, p.H};
+                dj[k] = MedianJob{base + l.raw, is_device_ptr(it.out) ? it.out : arena + it.io + (l.out - l.in_left), p.W,
+                                  p.H};
                 const int units[kListStages] = {census_units(p.W, p.H), cost_quads_units(p.W, p.H),
                                                 pairs_hv_units(a, p.n_paths != 8), a.QW, pairs_finish_units(a),
                                                 median_quads_units(p.W, p.H)};
@@ -1282,7 +1316,7 @@ static size_t build_lists(sgm_ctx* ctx, ListExec& x, const std::vector<BatchItem
             a.pair = it.p.n_paths >= 4;
             a.s8 = s8_for(it.p);
             sa[k] = a;
-            uint8_t* dst = is_device_ptr(it.out) ? it.out : base + l.out;
+            uint8_t* dst = is_device_ptr(it.out) ? it.out : arena + it.io + (l.out - l.in_left);
             dj[k] = MedianJob{base + l.raw, dst, it.p.W, it.p.H};
             cs[k + 1] = cs[k] + census_units(it.p.W, it.p.H);
             ms[k + 1] = ms[k] + cost_units(it.p.W, it.p.H);
@@ -1459,8 +1493,7 @@ static int enqueue_wave(sgm_ctx* ctx, ListExec& x, std::vector<BatchItem>& items
         BatchItem& it = items[i];
         const Layout l = layout_for(it.p, true);
         const size_t wh = static_cast<size_t>(it.p.W) * it.p.H;
-        uint8_t* base = arena + it.offset;
-        // host images go to the pair's arena region: pinned ones through a
+        // host images go to the pair's copies in the arena: pinned ones through a
         // staging kernel (each byte over the host link once), pageable ones
         // through cudaMemcpyAsync
         const uint8_t* st_src[2] = {nullptr, nullptr};
@@ -1469,7 +1502,7 @@ static int enqueue_wave(sgm_ctx* ctx, ListExec& x, std::vector<BatchItem>& items
         for (int side = 0; side < 2; ++side) {
             const uint8_t*& img = side ? it.right : it.left;
             if (is_device_ptr(img)) continue;
-            uint8_t* dst = base + (side ? l.in_right : l.in_left);
+            uint8_t* dst = arena + it.io + (side ? l.in_right - l.in_left : 0);
             if (pointer_kind(img) == cudaMemoryTypeHost) {
                 st_src[n_st] = img;
                 st_dst[n_st++] = dst;
@@ -1486,9 +1519,9 @@ static int enqueue_wave(sgm_ctx* ctx, ListExec& x, std::vector<BatchItem>& items
     for (size_t i = b; i < e; ++i) {
         const BatchItem& it = items[i];
         if (!runs_alone(it.p)) continue;
-        uint8_t* const base = arena + it.offset;
-        uint8_t* const dst = is_device_ptr(it.out) ? it.out : base + layout_for(it.p, true).out;
-        CUDA_TRY(ctx, enqueue_path(ctx, it.p, base, it.left, it.right, dst, nullptr, s, false));
+        const Layout l = layout_for(it.p, true);
+        uint8_t* const dst = is_device_ptr(it.out) ? it.out : arena + it.io + (l.out - l.in_left);
+        CUDA_TRY(ctx, enqueue_path(ctx, it.p, arena + it.offset, it.left, it.right, dst, nullptr, s, false));
     }
     const auto groups = wave_groups(items, b, e);
     std::vector<int> keys;
@@ -1541,10 +1574,10 @@ static int enqueue_wave(sgm_ctx* ctx, ListExec& x, std::vector<BatchItem>& items
             const Layout l = layout_for(it.p, true);
             const size_t wh = static_cast<size_t>(it.p.W) * it.p.H;
             if (pointer_kind(it.out) == cudaMemoryTypeHost) {
-                CUDA_TRY(ctx, launch_stage(arena + it.offset + l.out, it.out, nullptr, nullptr, wh, s));
+                CUDA_TRY(ctx, launch_stage(arena + it.io + (l.out - l.in_left), it.out, nullptr, nullptr, wh, s));
                 ctx->launches += 1;
             } else {
-                CUDA_TRY(ctx, cudaMemcpyAsync(it.out, arena + it.offset + l.out, wh, cudaMemcpyDeviceToHost, s));
+                CUDA_TRY(ctx, cudaMemcpyAsync(it.out, arena + it.io + (l.out - l.in_left), wh, cudaMemcpyDeviceToHost, s));
             }
         }
     }
@@ -1580,17 +1613,18 @@ static int run_batch(sgm_ctx* ctx, ListExec& x, std::vector<BatchItem>& items, u
     });
     size_t b = 0;
     while (b < items.size()) {
-        size_t e = b, total = 0;
+        size_t e = b;
+        WaveRoom room;
         int groups = 0;
         while (e < items.size()) {
-            const size_t sz = layout_for(items[e].p, true).total;
+            const WaveRoom next = room.with(items[e].p);
             const bool new_group = e == b || batch_key(items[e]) != batch_key(items[e - 1]);
-            if (e > b && (total + sz > budget || (new_group && groups == kListGroups))) break;
+            if (e > b && (next.total() > budget || (new_group && groups == kListGroups))) break;
             groups += new_group ? 1 : 0;
-            items[e].offset = total;
-            total += sz;
+            room = next;
             ++e;
         }
+        const size_t total = place_wave(items, b, e);
         if (total > budget)
             return fail(ctx, SGM_ENOMEM, "a %dx%d D=%d pair needs %zu bytes, over the memory budget of %zu", items[b].p.W,
                         items[b].p.H, items[b].p.D, total, budget);
@@ -1677,7 +1711,7 @@ static int slot_reserve(sgm_ctx* ctx, ServeSlot& sl, size_t need, size_t budget)
 static int slot_launch(sgm_ctx* ctx, ServeSlot& sl, size_t budget) {
     std::vector<BatchItem> items;
     items.reserve(sl.reqs.size());
-    for (const Request& r : sl.reqs) items.push_back(BatchItem{r.p, r.left, r.right, r.out, 0});
+    for (const Request& r : sl.reqs) items.push_back(BatchItem{r.p, r.left, r.right, r.out});
     // pageable host buffers go through the slot's pinned staging
     auto pageable = [](const void* q) { return pointer_kind(q) == cudaMemoryTypeUnregistered; };
     size_t host = 0;
@@ -1718,11 +1752,7 @@ static int slot_launch(sgm_ctx* ctx, ServeSlot& sl, size_t budget) {
     std::stable_sort(items.begin(), items.end(), [](const BatchItem& x, const BatchItem& y) {
         return batch_key(x) < batch_key(y);
     });
-    size_t total = 0;
-    for (BatchItem& it : items) {
-        it.offset = total;
-        total += layout_for(it.p, true).total;
-    }
+    const size_t total = place_wave(items, 0, items.size());
     int rc = slot_reserve(ctx, sl, total, budget);
     if (rc == SGM_OK) rc = enqueue_wave(ctx, sl.exec, items, 0, items.size(), sl.arena, sl.stream, false);
     if (rc == SGM_OK) CUDA_TRY(ctx, cudaLaunchHostFunc(sl.stream, slot_finished, &sl));
@@ -1823,17 +1853,17 @@ static void serve_loop(sgm_ctx* ctx) {
         size_t budget = 0;
         int rc = slot_budget(ctx, *sl, &budget);
         lk.lock();
-        size_t used = 0;
+        WaveRoom used;
         std::set<std::tuple<int, int, int, int>> keys;
         while (rc == SGM_OK && !ctx->queue.empty() && sl->reqs.size() < static_cast<size_t>(kServeMaxPairs)) {
             Request& r = ctx->queue.front();
             // a stream of requests like this one
-            r.p.sched = batch_sched(r.p, budget - used, 8.0 * r.p.W * r.p.H, ctx->mem_cap != 0);
-            const size_t sz = layout_for(r.p, true).total;
-            const auto key = batch_key(BatchItem{r.p, nullptr, nullptr, nullptr, 0});
-            if (used + sz > budget || (!keys.count(key) && keys.size() == static_cast<size_t>(kListGroups))) break;
+            r.p.sched = batch_sched(r.p, budget - used.total(), 8.0 * r.p.W * r.p.H, ctx->mem_cap != 0);
+            const WaveRoom next = used.with(r.p);
+            const auto key = batch_key(BatchItem{r.p, nullptr, nullptr, nullptr});
+            if (next.total() > budget || (!keys.count(key) && keys.size() == static_cast<size_t>(kListGroups))) break;
             keys.insert(key);
-            used += sz;
+            used = next;
             sl->reqs.push_back(r);
             ctx->queue.pop_front();
         }
@@ -2090,7 +2120,7 @@ int sgm_compute_batch(sgm_ctx* ctx, int n, const sgm_pair* pairs) {
         const Problem p = make_problem(ctx, q.W, q.H, q.D, q.P1, q.P2, q.n_paths);
         int rc = check_args(ctx, p, q.left, q.right, q.disp_out);
         if (rc != SGM_OK) return fail(ctx, rc, "pair %d: %s", i, ctx->err.c_str());
-        items.push_back(BatchItem{p, q.left, q.right, q.disp_out, 0});
+        items.push_back(BatchItem{p, q.left, q.right, q.disp_out});
     }
     CUDA_TRY(ctx, cudaSetDevice(ctx->device));
     int rc = run_batch(ctx, ctx->batch_exec, items, &ctx->arena, &ctx->arena_bytes, true, ctx->stream, true);
