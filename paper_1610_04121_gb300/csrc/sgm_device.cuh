@@ -26,9 +26,10 @@ namespace sgm {
 // so packed 32-bit adds never carry across lanes.
 constexpr uint32_t kInf16 = 0x3FFFu;
 
-// First instruction of every kernel of a path (Stream, sgm_internal.h): the
-// kernels before it have ended and their writes are visible.  Nothing to wait
-// for in a plain launch.
+// First instruction of the kernels of a path (Stream, sgm_internal.h), all but
+// the walks that run beside another walk (Side, sgm_pairs.cuh): the kernels before
+// it have ended and their writes are visible.  Nothing to wait for in a plain
+// launch.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The next kernel of the stream may start once every block of this one has come here.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

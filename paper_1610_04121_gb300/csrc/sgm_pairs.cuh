@@ -28,10 +28,9 @@
 //   finish    a warp per segment of a row pair walks left to right and right
 //             to left again from the stored states, adds the stored r of the
 //             other directions and takes the winner.
-// Walking a horizontal direction twice costs its integer work again (the
-// finishing launch has the integer units to spare: it is bound by reading the
-// stored r), and saves writing and reading back two bytes per pixel and
-// disparity.
+// Walking a horizontal direction twice costs its integer work again (640x480
+// D=128, 4 paths: the finishing launch is bound by issue, not by its 51 MB), and
+// saves writing and reading back two bytes per pixel and disparity.
 //
 // Bounds: a step takes about 45 instructions per warp and 256 (pixel,
 // disparity) pairs, 15-19 of them on the integer ALU, where each takes two
@@ -524,7 +523,7 @@ __device__ __forceinline__ void walk(const PairsArgs& a, int line, int kd, bool 
     const uint32_t* p2m = nullptr;
     auto p2_load = [&](int k) -> uint32_t {
         const int i = p2i + min(k, nu - 1) * p2s;
-        return SGM_GUARD_INDEX(i, static_cast<long long>(units), 104) ? __ldg(p2m + i) : 0u;
+        return SGM_GUARD_INDEX(i, static_cast<long long>(units), 104) ? __ldcg(p2m + i) : 0u;  // see Side
     };
     if constexpr (AP2) {
         const int m = (KIND == kHor ? 0 : (KIND == kVer ? 2 : 4 + 2 * kd)) + (fwd ? 0 : 1);
@@ -652,8 +651,14 @@ __device__ __forceinline__ void walk(const PairsArgs& a, int line, int kd, bool 
 
 // The order of the walks' launches (launch_pairs_walks): the first one waits for
 // the costs; a later one starts when every block of the one before has come
-// past that wait, and so needs none, but its last block waits for the end of
-// the one before, so that its own end means both.
+// past that wait and does without one of its own (which would wait for the end
+// of the walks before, too), but its last block waits for the end of the one
+// before, so that its own end means both.  PTX promises the writes of earlier
+// kernels to a kernel that waits.  What a later walk reads without a wait, the
+// costs and the penalties, was complete and visible to the whole device when the
+// first walk's wait ended, before that walk let this one start; the assumption is
+// that a kernel started after that moment sees it through L2.  So these reads
+// take L2 only, never a line that an L1 may have kept from an earlier frame.
 struct Side {
     int later, trigger;  // not the first launch; another one follows
     __device__ __forceinline__ void begin() const {
