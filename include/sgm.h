@@ -398,8 +398,10 @@ SGM_API const char *sgm_stage_label(const sgm_ctx *ctx, int i);
 #define SGM_SCHED_PAIRS 2
 SGM_API int sgm_set_schedule(sgm_ctx *ctx, int schedule);
 
-/* The schedule the context uses for this problem: the forced one, the tuned
- * one, SGM_SCHED_V_THEN_H for 2 and 8 paths, or -1 when not tuned yet. */
+/* The 4-path schedule the context uses for this problem: the forced one, the
+ * tuned one, or -1 when not tuned yet.  With 2 and 8 paths there is none to
+ * choose and the answer is always SGM_SCHED_V_THEN_H, whichever kernels run (see
+ * sgm_set_schedule). */
 SGM_API int sgm_schedule_for(const sgm_ctx *ctx, int W, int H, int D, int P1, int P2, int n_paths);
 
 /*
@@ -424,11 +426,14 @@ SGM_API const char *sgm_version(void);
  * stream) and returns without waiting.  It needs no context and calls no
  * cudaMalloc, cudaFree or other allocating routine: every intermediate lives
  * in one static device array of 48 MiB that each GPU which loads the library
- * keeps until the process exits.  The intermediates take 8 W H bytes for the
- * features, W H (3 D) bytes (2 paths) or W H (4 D) bytes (4 or 8 paths) for
- * the per-pixel records and W H for the raw disparity; sizes that do not fit
- * are rejected with SGM_EINVAL (320x240 with D = 128 and 8 paths fits, about
- * 40 MB; 640x480 with D = 128 does not).
+ * keeps until the process exits.  With the per-line sweeps the intermediates
+ * take 8 W H bytes for the features, W H (3 D) bytes (2 paths) or W H (4 D)
+ * bytes (4 or 8 paths) for the per-pixel records and W H for the raw disparity;
+ * sizes for which that does not fit are rejected with SGM_EINVAL (320x240 with
+ * D = 128 and 8 paths fits, about 40 MB; 640x480 with D = 128 does not).  The
+ * paired lines (SGM_SCHED_PAIRS), which take 8 W H + 2, 3 or 7 D W H bytes (2, 4
+ * or 8 paths, W and H rounded up to even), the states of the horizontal paths
+ * and W H, run where that fits as well, else the per-line sweeps do.
  *
  * The first call on a device looks up the array's device address and sets
  * kernel attributes; make that first call before any stream capture.  Every
