@@ -391,8 +391,10 @@ __device__ __forceinline__ bool state_ok(const PairsArgs& a, const uint32_t* p, 
 // eight 905), but two for diagonals that run beside the other walks (1242x375 8
 // paths 204 us; eight no longer fit the instruction caches with them: 214), and
 // no more than a segment or the ring holds.  SHORT (frames with shorter segments,
-// pairs_geometry): rings of one loop only, because a walk's last DEPTH units run
-// outside the loop, one by one (64x100 D=96 frame 15.4 us, with sixteen 16.7).
+// pairs_geometry): a walk's last DEPTH units run outside the loop, one by one, so
+// their rings hold eight units, four for D > 128, and their loops are four long
+// (64x100 D=96 frame 14.9 us; rings of sixteen and loops of eight 16.7, eight and
+// eight 15.2, four and four 15.5; 100x100 D=192 18.5, rings of eight 18.9).
 template <int D>
 __host__ __device__ constexpr int ring_bytes(bool rows = false) {
     return D <= 128 || rows ? 8192 : 16384;
@@ -400,9 +402,9 @@ __host__ __device__ constexpr int ring_bytes(bool rows = false) {
 template <int D, int KIND, bool ROWS, bool SHORT>
 struct Ring {
     static constexpr int SB = (KIND == kDiag ? 2 : 1) * 4 * D;  // bytes of a slot
-    static constexpr int WANT = KIND == kDiag && !ROWS ? 2 : (D <= 128 ? 8 : 4), FIT = ring_bytes<D>(ROWS) / SB;
+    static constexpr int WANT = KIND == kDiag && !ROWS ? 2 : (D <= 128 && !SHORT ? 8 : 4), FIT = ring_bytes<D>(ROWS) / SB;
     static constexpr int UN = WANT <= FIT && (KIND != kHor || WANT <= seg_quads(D)) ? WANT : (WANT < 4 ? WANT : 4);
-    static constexpr int DEPTH = SHORT ? UN : (FIT / UN * UN > 16 ? 16 : FIT / UN * UN);
+    static constexpr int DEPTH = SHORT ? (D <= 128 ? 8 : 4) : (FIT / UN * UN > 16 ? 16 : FIT / UN * UN);
 };
 
 // ---------------------------------------------------------------------------
