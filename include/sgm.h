@@ -188,11 +188,11 @@ SGM_API int sgm_compute_ex_async(sgm_ctx *ctx, const uint8_t *left, const uint8_
  * Non-blocking form for device pointers only: enqueues the whole path on the
  * context's stream and returns at once.  `left`, `right` and `disp_out` must
  * be device memory; the caller synchronises the stream before reading
- * `disp_out`.  Behind other work of the stream the kernels are launched one by
- * one with programmatic stream serialization, so that calls follow one another
- * without gaps; on an idle stream, and in the blocking calls, a CUDA graph is
- * replayed that is built once for one (W, H, D, P1, P2, n_paths) and one set of
- * pointers, on the second such call with them.
+ * `disp_out`.  The kernels are launched one by one with programmatic stream
+ * serialization, so that calls follow one another without gaps; the blocking
+ * calls, and a small frame (W * H * D * n_paths up to 2^25) that finds its stream
+ * idle, replay a CUDA graph that is built once for one (W, H, D, P1, P2, n_paths)
+ * and one set of pointers, on the second such call with them.
  * Errors: SGM_EINVAL (including host pointers), SGM_ENOMEM, SGM_ECUDA.
  */
 SGM_API int sgm_compute_async(sgm_ctx *ctx, const uint8_t *left, const uint8_t *right, int W, int H, int D, int P1, int P2,

@@ -839,7 +839,7 @@ struct HostIO {
 };
 
 // Enqueue through a cached CUDA graph for this problem and these pointers: the
-// blocking calls and the asynchronous ones that find their stream idle (the whole
+// blocking calls and small asynchronous ones that find their stream idle (the whole
 // sequence is there at once: 96.4 us per 640x480 frame from pinned host images against 99.1 kernel by
 // kernel), and contexts that time stages (the events between the kernels are
 // nodes of the graph).  Making one takes about 45 us, so the first call with a
@@ -920,16 +920,19 @@ static bool stream_idle(cudaStream_t s) {
     return idle;
 }
 
-// The asynchronous calls: behind work of the stream kernel by kernel (no gaps
-// between the frames), on an idle stream as the blocking calls, so that the host's
-// time for six launches is not part of the result's.  Frames that the caller waits
-// for one by one, from the call to the end, replayed / kernel by kernel: 96x64
-// D=64 26.2 / 28.2 us, 320x240 D=64 40.1 / 41.7, 640x480 D=128 90.7 / 92.7.  The
-// query takes 0.35 us of the host.  One graph for all buffers, its parameters set
-// anew for each call on others, was slower: 0.7 us for each kernel.
+// The asynchronous calls: kernel by kernel, which leaves no gaps between the frames
+// of a stream.  A small frame that finds its stream idle replays a graph as the
+// blocking calls do, because the host's time for six launches is longer than its
+// kernels'.  Frames waited for one by one, from the call to the end, replayed /
+// kernel by kernel: 96x64 D=64 25.8 / 28.2 us, 64x128 D=96 27.5 / 29.0, 320x240 D=64
+// 39.2 / 41.7.  The line lies at 2^25 path steps: a 640x480 frame would gain 2 of 92
+// us when waited for and lose 0.3 of 82.6 behind other work, where the query (0.35
+// us of the host) is all that is left of it.  One graph for all buffers, its
+// parameters set anew for each call on others, was slower: 0.7 us for each kernel.
 static int enqueue_run(sgm_ctx* ctx, const Problem& p, uint8_t* arena, const uint8_t* left, const uint8_t* right,
                        uint8_t* disp, cudaStream_t s) {
-    if (stream_idle(s)) return enqueue_graph(ctx, p, arena, left, right, disp, s);
+    const bool small = static_cast<double>(p.W) * p.H * p.D * p.n_paths <= 33554432.0;
+    if (small && stream_idle(s)) return enqueue_graph(ctx, p, arena, left, right, disp, s);
     return enqueue_kernels(ctx, p, arena, left, right, disp, s);
 }
 
