@@ -53,12 +53,12 @@ SERVED_OUT_RING = 4  # output buffers per pool pair (a pair can be in flight mor
 # frame, as in the timed steps); pairs_vh is the sum of its two launches.  The
 # 8-path frame's are the per-line sweeps', which contexts that time stages run.
 MEASURED_TRAFFIC = {
-    ("sgm_640x480_d128_p4", "pairs_vh"): (92325120, "3dd9b3c6c9537dac"),
-    ("sgm_640x480_d128_p4", "pairs_h_wta"): (52539392, "3dd9b3c6c9537dac"),
-    ("sgm_1242x375_d128_p8", "sweep_h"): (606967552, "3dd9b3c6c9537dac"),
-    ("sgm_1242x375_d128_p8", "sweep_diag+"): (349430784, "3dd9b3c6c9537dac"),
-    ("sgm_1242x375_d128_p8", "sweep_diag-"): (355507200, "3dd9b3c6c9537dac"),
-    ("sgm_1242x375_d128_p8", "sweep_v"): (285914624, "3dd9b3c6c9537dac"),
+    ("sgm_640x480_d128_p4", "pairs_vh"): (92287744, "b6751f1344442dd7"),
+    ("sgm_640x480_d128_p4", "pairs_h_wta"): (52291456, "b6751f1344442dd7"),
+    ("sgm_1242x375_d128_p8", "sweep_h"): (604687104, "b6751f1344442dd7"),
+    ("sgm_1242x375_d128_p8", "sweep_diag+"): (349974784, "b6751f1344442dd7"),
+    ("sgm_1242x375_d128_p8", "sweep_diag-"): (355789696, "b6751f1344442dd7"),
+    ("sgm_1242x375_d128_p8", "sweep_v"): (285923968, "b6751f1344442dd7"),
 }
 KERNEL_SOURCES = ("sgm_sweeps.cuh", "sgm_pairs.cuh", "sgm_device.cuh", "sgm_internal.h")
 
