@@ -36,6 +36,13 @@
  *           or keeps a caller pointer beyond the call, except for
  *           sgm_submit (see there).  The library owns its context, its device
  *           work arena and its CUDA graphs.
+ *  Memory   without a memory cap (sgm_create) a path may take more memory to run
+ *           faster: 2 and 8 paths and the post form run the paired lines
+ *           (SGM_SCHED_PAIRS) with 2 and 7 bytes per pixel and disparity, twice
+ *           that with the left-right check, in place of the per-line sweeps' 3
+ *           and 7 (a batched or served pair of 8 paths 7 in place of 4).  Under a
+ *           cap every path takes at most what the per-line sweeps need, and runs
+ *           these where the paired lines need more.
  *  Errors   every function returns an sgm_status; nothing is thrown across
  *           the ABI.  sgm_last_error(ctx) gives a human-readable reason for
  *           the last failure on that context (thread-local to the context).
@@ -93,15 +100,10 @@ typedef struct sgm_pair {
  * Create a context on CUDA device `device` (makes it current for the calling
  * thread).  `mem_cap_bytes` caps the device memory the context may hold for
  * its work arena and served requests (0 = no cap beyond the device's free
- * memory).  Without a cap a path may take more memory to run faster: 2 and 8
- * paths and the post form run the paired lines (SGM_SCHED_PAIRS) with 2 and 7
- * bytes per pixel and disparity, twice that with the left-right check, in place
- * of the per-line sweeps' 3 and 7 (a batched or served pair of 8 paths 7 in
- * place of 4).  Under a cap every path takes at most what the per-line sweeps
- * need, and runs these where the paired lines need more.  `flags` is 0 or a combination of SGM_FLAG_STAGE_TIMING and
- * SGM_FLAG_CENSUS_FULL; the Census type holds for every entry point of the
- * context (sgm_compute_static always uses the CSCT).  On success *out
- * receives the context.
+ * memory; see Memory above).  `flags` is 0 or a combination of
+ * SGM_FLAG_STAGE_TIMING and SGM_FLAG_CENSUS_FULL; the Census type holds for
+ * every entry point of the context (sgm_compute_static always uses the CSCT).
+ * On success *out receives the context.
  * Test hooks, read from the environment here (host side only; no kernel is
  * made to fault): SGM_TEST_FAIL_ALLOC=n makes the context's n-th device or
  * pinned-host allocation fail as if memory were exhausted (the call that
