@@ -704,8 +704,9 @@ static cudaError_t enqueue_match(const Problem& p, const Layout& l, uint8_t* are
 // whatever a served request or a batch finds left below the cap does not depend
 // on the schedule.
 //
-// What the per-line sweeps need decides when the arena has to grow; it is freed
-// for that, and the larger of the two is tried first.  An arena that holds the
+// What the per-line sweeps need decides when the arena has to grow, and it never
+// gets less (a later call of another shape may be one that the caller captures);
+// it is freed for that, and the larger of the two is tried first.  An arena that holds the
 // per-line sweeps already is only ever replaced by one in hand, half as large
 // again where the device has it (so that the replaced ones together stay below
 // twice the last one), never in a stream under capture, and not for a size that
@@ -723,7 +724,7 @@ static int prepare_arena(sgm_ctx* ctx, Problem& p, size_t extra = 0) {
             return SGM_OK;
         }
         if (base > ctx->arena_bytes && (!ctx->mem_cap || need <= base)) {
-            const int rc = ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, need, true);
+            const int rc = ensure_arena(ctx, &ctx->arena, &ctx->arena_bytes, std::max(need, base), true);
             const bool injected = ctx->fail_alloc_at > 0 && ctx->alloc_count.load() == ctx->fail_alloc_at;
             if (rc == SGM_OK) p.sched = SGM_SCHED_PAIRS;
             if (rc == SGM_OK) ctx->refused_bytes = SIZE_MAX;  // the device has memory again
@@ -733,6 +734,7 @@ static int prepare_arena(sgm_ctx* ctx, Problem& p, size_t extra = 0) {
             cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
             CUDA_TRY(ctx, cudaStreamIsCapturing(ctx->stream, &cs));
             if (cs != cudaStreamCaptureStatusNone) return SGM_OK;
+            CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));  // no graph in flight is destroyed
             size_t grown = std::max(need, ctx->arena_bytes + ctx->arena_bytes / 2);
             void* a = nullptr;
             cudaError_t e = ctx_malloc(ctx, &a, grown);

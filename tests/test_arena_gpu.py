@@ -21,10 +21,10 @@ D = 64
 class Call:
     """One asynchronous call on buffers of its own."""
 
-    def __init__(self, c, W, H, post=None):
+    def __init__(self, c, W, H, post=None, n_paths=8):
         import torch
 
-        self.c, self.W, self.H, self.post = c, W, H, post
+        self.c, self.W, self.H, self.post, self.n_paths = c, W, H, post, n_paths
         self.rng = np.random.default_rng(W)
         self.left, self.right = (torch.zeros((H, W), dtype=torch.uint8, device="cuda") for _ in range(2))
         self.out = torch.zeros((H, W), dtype=torch.uint8 if post is None else torch.int16, device="cuda")
@@ -32,7 +32,7 @@ class Call:
     def run(self):
         from paper_1610_04121_gb300 import sgm
 
-        a = (self.c.handle, self.left, self.right, self.W, self.H, D, 10, 120, 8)
+        a = (self.c.handle, self.left, self.right, self.W, self.H, D, 10, 120, self.n_paths)
         if self.post is None:
             sgm.sgm_compute_async(*a, self.out)
         else:
@@ -51,9 +51,9 @@ class Call:
         torch.cuda.synchronize()
         got = self.out.cpu().numpy()
         if self.post is None:
-            assert (got == oracle.sgm(a, b, D, 10, 120, 8)).all()
+            assert (got == oracle.sgm(a, b, D, 10, 120, self.n_paths)).all()
         else:
-            assert (got.view(np.uint16) == oracle.sgm_ex(a, b, D, 10, 120, 8, self.post)).all()
+            assert (got.view(np.uint16) == oracle.sgm_ex(a, b, D, 10, 120, self.n_paths, self.post)).all()
 
     def capture(self, stream):
         import torch
@@ -126,3 +126,13 @@ def test_graphs_of_the_caller_outlive_a_larger_arena(ctx_on_stream):
         ex.check(ex.run)
         plain.check(g.replay)
         plain.check(plain.run)
+
+
+def test_an_arena_holds_what_the_per_line_sweeps_would(ctx_on_stream):
+    c, st = ctx_on_stream()
+    two = Call(c, 200, 150, n_paths=2)  # per-line sweeps 6.2 MB, paired lines 4.2 MB
+    two.check(two.run)
+    eight = Call(c, 100, 110)  # 5.2 MB
+    g = eight.capture(st)
+    eight.check(g.replay)
+    two.check(two.run)
